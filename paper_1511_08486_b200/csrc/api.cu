@@ -388,8 +388,10 @@ int sfb_destroy(sfb_ctx* c) {
 int sfb_prox(sfb_ctx* c, void* W) {
   if (c == nullptr || W == nullptr || !aligned(W, 16)) return SFB_ERR_ARG;
   if (c->d.model != SFB_SC) return SFB_OK;   // h = 0 for the MLR and DML workloads: identity
-  ACC(launch_prox_unit_columns(c->stream, reinterpret_cast<float*>(W), c->d.J, c->d.D));
-  c->shadow_of = nullptr;   // W changed
+  // a correction operand that mirrors W is rewritten with it (the other sparse-coding paths keep nothing of W)
+  __nv_bfloat16* shadow = c->d.path == SFB_PATH_TF32X3 && c->shadow_of == W ? c->w_shadow : nullptr;
+  if (shadow == nullptr) c->shadow_of = nullptr;   // W changed
+  ACC(launch_prox_unit_columns(c->stream, reinterpret_cast<float*>(W), c->d.J, c->d.D, shadow));
   return SFB_OK;
 }
 

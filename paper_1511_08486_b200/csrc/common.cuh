@@ -45,16 +45,21 @@ struct CorrOut {
   __host__ __device__ CorrOut() : mn(nullptr), km(nullptr), ldc(0), k_bb(32), k_wp(1), k_bpw(1), a_side(0), atoms(0) {}
 };
 #ifdef __CUDACC__
-// values t of pair i (B pairs per worker) at columns j .. j + 3, j a multiple of 4
-__device__ __forceinline__ void corr_store4(const CorrOut& c, int i, int B, int j, float4 t) {
+// Four fp32 values as bf16, and the bf16 remainders of what the tensor core sees of them (see split.cu).
+__device__ __forceinline__ void split4(const float4& t, uint2& val, uint2& rem) {
   const float rx = t.x - __uint_as_float(__float_as_uint(t.x) & 0xFFFFE000u);
   const float ry = t.y - __uint_as_float(__float_as_uint(t.y) & 0xFFFFE000u);
   const float rz = t.z - __uint_as_float(__float_as_uint(t.z) & 0xFFFFE000u);
   const float rw = t.w - __uint_as_float(__float_as_uint(t.w) & 0xFFFFE000u);
   const __nv_bfloat162 v0 = __floats2bfloat162_rn(t.x, t.y), v1 = __floats2bfloat162_rn(t.z, t.w);
   const __nv_bfloat162 r0 = __floats2bfloat162_rn(rx, ry), r1 = __floats2bfloat162_rn(rz, rw);
-  const uint2 val = make_uint2(*reinterpret_cast<const uint32_t*>(&v0), *reinterpret_cast<const uint32_t*>(&v1));
-  const uint2 rem = make_uint2(*reinterpret_cast<const uint32_t*>(&r0), *reinterpret_cast<const uint32_t*>(&r1));
+  val = make_uint2(*reinterpret_cast<const uint32_t*>(&v0), *reinterpret_cast<const uint32_t*>(&v1));
+  rem = make_uint2(*reinterpret_cast<const uint32_t*>(&r0), *reinterpret_cast<const uint32_t*>(&r1));
+}
+// values t of pair i (B pairs per worker) at columns j .. j + 3, j a multiple of 4
+__device__ __forceinline__ void corr_store4(const CorrOut& c, int i, int B, int j, float4 t) {
+  uint2 val, rem;
+  split4(t, val, rem);
   if (c.mn != nullptr && j < c.ldc) {
     const int w = i / B, r = i - w * B;
     long long blk;
@@ -227,7 +232,8 @@ int launch_finish_sc(cudaStream_t s, RowMap z, RowMap u, const float* Xdata, int
                      long long split_stride_bytes = 0, CorrOut corr = CorrOut());
 
 // Column-norm projection: every column of W with 2-norm above 1 is divided by its norm (in place).
-int launch_prox_unit_columns(cudaStream_t s, float* W, int J, int D);
+// shadow (optional, D a multiple of 4): W's correction operand of the compensated path, kept in step with W.
+int launch_prox_unit_columns(cudaStream_t s, float* W, int J, int D, __nv_bfloat16* shadow = nullptr);
 // Minibatch objective: per-sample values from the fp32 rows (z_i for MLR / DML, u_i for SC) into loss_i[K],
 // then their fp64 sum into *total (device).  Two launches.
 int launch_sample_loss(cudaStream_t s, int model, RowMap rows, const int32_t* labels, const uint8_t* similar, float margin,

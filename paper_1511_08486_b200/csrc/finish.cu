@@ -6,7 +6,11 @@
 //
 // One thread block per sample row; the row is staged once in shared memory (when it fits) so HBM
 // sees one read and one write per value; reductions over the J entries use warp shuffles.
+#include <cooperative_groups.h>
+
 #include "common.cuh"
+
+namespace cg = cooperative_groups;
 
 namespace sfb {
 namespace {
@@ -281,33 +285,98 @@ __global__ void __launch_bounds__(256) finish_mlr_fused_kernel(RowMap u, const f
   }
 }
 
-// Unit-ball projection of the columns of W (sparse-coding prox).  One block owns 32 consecutive
-// columns: 32 x 8 threads walk the rows (a warp reads one 128-byte line per row), the squared norms are
-// combined in a fixed order, then the block rescales its columns (second read served by L2).  Columns
-// with norm <= 1 are not written at all.
-__global__ void __launch_bounds__(256) prox_unit_columns_kernel(float* __restrict__ W, int J, int D) {
-  __shared__ float part[8][33];
-  __shared__ float scale[32];
-  const int c = threadIdx.x & 31, r = threadIdx.x >> 5;
-  const int d = blockIdx.x * 32 + c;
-  float acc = 0.f;
-  if (d < D)
-    for (int j = r; j < J; j += 8) {
-      const float w = W[(size_t)j * D + d];
-      acc = fmaf(w, w, acc);
+// Unit-ball projection of the columns of W (sparse-coding prox).  A cluster of CTAs owns a slab of 32 consecutive
+// columns: eight lanes hold a row's 128-byte segment, a CTA takes every 32nd row of its share of the rows and keeps up to
+// PROX_HELD of them per thread in registers between the norm and the rescaling (rows beyond that are read again, from
+// L2).  Squared norms are combined in a fixed order: rows of a thread, threads, CTAs.  Units of four columns none of
+// which is rescaled are not written.
+// shadow (optional): W's correction operand of the compensated tf32 path, [row][atom of 32 columns][32 values | 32
+// remainders]; a slab is one atom, so its line is rewritten from the registers that hold the new W.
+// Bound: HBM, W read once and written once.  (One block per slab with one 4-byte load in flight per thread and a second
+// pass over the slab took 206 us at 4096 x 10000, 1.6 TB/s on its 328 MB; this takes 61 us, 5.4 TB/s, and as long with
+// the 164 MB of the operand, whose stand-alone rebuild before the next forward pass took 45 us.)
+constexpr int PROX_HELD = 16, PROX_THREADS = 256, PROX_ROWS = PROX_THREADS / 8;
+template <bool VEC>
+__global__ void __launch_bounds__(PROX_THREADS, VEC ? 2 : 1) prox_unit_columns_kernel(float* __restrict__ W, int J, int D,
+                                                                            int rows_per_cta, __nv_bfloat16* shadow) {
+  __shared__ float4 part[PROX_ROWS][9];
+  __shared__ float cta_sum[32];
+  cg::cluster_group cluster = cg::this_cluster();
+  const int lq = threadIdx.x & 7, lr = threadIdx.x >> 3;
+  const int ctas = cluster.num_blocks(), slab = blockIdx.x / ctas;
+  const int d = slab * 32 + lq * 4;
+  const int j_lo = (int)cluster.block_rank() * rows_per_cta, j_hi = min(J, j_lo + rows_per_cta);
+  auto load = [&](int j) {
+    const float* w = W + (size_t)j * D + d;
+    float4 t = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (VEC) {
+      if (d < D) t = *reinterpret_cast<const float4*>(w);
+    } else {
+      if (d < D) t.x = w[0];
+      if (d + 1 < D) t.y = w[1];
+      if (d + 2 < D) t.z = w[2];
+      if (d + 3 < D) t.w = w[3];
     }
-  part[r][c] = acc;
-  __syncthreads();
-  if (r == 0) {
-    float n2 = 0.f;
+    return t;
+  };
+  float4 held[PROX_HELD];
 #pragma unroll
-    for (int q = 0; q < 8; ++q) n2 += part[q][c];
-    scale[c] = (n2 > 1.0f) ? 1.0f / sqrtf(n2) : 1.0f;
+  for (int q = 0; q < PROX_HELD; ++q) {
+    const int j = j_lo + lr + q * PROX_ROWS;
+    held[q] = j < j_hi ? load(j) : make_float4(0.f, 0.f, 0.f, 0.f);
   }
+  float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+  auto add = [&](const float4& t) {
+    acc.x = fmaf(t.x, t.x, acc.x); acc.y = fmaf(t.y, t.y, acc.y);
+    acc.z = fmaf(t.z, t.z, acc.z); acc.w = fmaf(t.w, t.w, acc.w);
+  };
+#pragma unroll
+  for (int q = 0; q < PROX_HELD; ++q) add(held[q]);
+  for (int j = j_lo + lr + PROX_HELD * PROX_ROWS; j < j_hi; j += PROX_ROWS) add(load(j));
+  part[lr][lq] = acc;
   __syncthreads();
-  const float sc = scale[c];
-  if (d < D && sc != 1.0f)
-    for (int j = r; j < J; j += 8) W[(size_t)j * D + d] *= sc;
+  if (threadIdx.x < 32) {
+    float n = 0.f;
+#pragma unroll
+    for (int r = 0; r < PROX_ROWS; ++r) n += reinterpret_cast<const float*>(&part[r][0])[threadIdx.x];
+    cta_sum[threadIdx.x] = n;
+  }
+  cluster.sync();
+  float sc[4];
+#pragma unroll
+  for (int e = 0; e < 4; ++e) {
+    float n2 = 0.f;
+    for (int c = 0; c < ctas; ++c) n2 += cluster.map_shared_rank(cta_sum, c)[lq * 4 + e];
+    sc[e] = (n2 > 1.0f) ? 1.0f / sqrtf(n2) : 1.0f;
+  }
+  cluster.sync();   // nobody leaves while its sums may still be read
+  if (sc[0] == 1.0f && sc[1] == 1.0f && sc[2] == 1.0f && sc[3] == 1.0f) return;
+  const int atoms = gridDim.x / ctas;
+  auto store = [&](int j, float4 t) {
+    t.x *= sc[0]; t.y *= sc[1]; t.z *= sc[2]; t.w *= sc[3];
+    float* w = W + (size_t)j * D + d;
+    if (VEC) {
+      if (d < D) *reinterpret_cast<float4*>(w) = t;
+    } else {
+      if (d < D) w[0] = t.x;
+      if (d + 1 < D) w[1] = t.y;
+      if (d + 2 < D) w[2] = t.z;
+      if (d + 3 < D) w[3] = t.w;
+    }
+    if (VEC && shadow != nullptr && d < D) {
+      uint2 val, rem;
+      split4(t, val, rem);
+      uint2* dst = reinterpret_cast<uint2*>(shadow + ((size_t)j * atoms + slab) * 64) + lq;
+      dst[0] = val;
+      dst[8] = rem;
+    }
+  };
+#pragma unroll
+  for (int q = 0; q < PROX_HELD; ++q) {
+    const int j = j_lo + lr + q * PROX_ROWS;
+    if (j < j_hi) store(j, held[q]);
+  }
+  for (int j = j_lo + lr + PROX_HELD * PROX_ROWS; j < j_hi; j += PROX_ROWS) store(j, load(j));
 }
 
 // 16-byte-vectorised row copy; rows are whole numbers of 16-byte units on both sides.
@@ -457,9 +526,23 @@ int launch_finish_mlr_fused(cudaStream_t s, RowMap u, const float2* stats, int n
   return cudaGetLastError() == cudaSuccess ? 1 : SFB_ERR_CUDA;
 }
 
-int launch_prox_unit_columns(cudaStream_t s, float* W, int J, int D) {
-  prox_unit_columns_kernel<<<(D + 31) / 32, 256, 0, s>>>(W, J, D);
-  return cudaGetLastError() == cudaSuccess ? 1 : SFB_ERR_CUDA;
+int launch_prox_unit_columns(cudaStream_t s, float* W, int J, int D, __nv_bfloat16* shadow) {
+  // CTAs per slab: as many as hold the slab in registers, or as are needed to give every SM two, up to eight
+  const int slabs = (D + 31) / 32;
+  int ctas = 1;
+  while (ctas < 8 && (ctas * PROX_HELD * PROX_ROWS < J || (slabs * ctas < 296 && ctas * 2 * PROX_ROWS < J))) ctas *= 2;
+  const int rows = (J + ctas - 1) / ctas;
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = ctas; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
+  cfg.gridDim = dim3(ctas * slabs);
+  cfg.blockDim = dim3(PROX_THREADS);
+  cfg.stream = s;
+  cfg.attrs = at; cfg.numAttrs = 1;
+  const cudaError_t e = (D & 3) == 0 ? cudaLaunchKernelEx(&cfg, prox_unit_columns_kernel<true>, W, J, D, rows, shadow)
+                                     : cudaLaunchKernelEx(&cfg, prox_unit_columns_kernel<false>, W, J, D, rows, shadow);
+  return e == cudaSuccess ? 1 : SFB_ERR_CUDA;
 }
 
 int launch_copy_rows(cudaStream_t s, RowMap src, RowMap dst, int K, int cols, CorrOut corr) {
