@@ -166,8 +166,9 @@ int ensure_shadow(sfb_ctx* c, const void* W) {
 // workers > 0: the minibatch holds only that many workers' samples and u / v / codes start at the first of them.
 // for_apply: the apply of exactly these rows (all K pairs, no compaction in between) follows in the same call, so
 // the compensated path may write the apply's correction operands while it writes the factors.
+// commit (dense v): header and directory of the buffer u and v belong to, written by the finishing pass.
 int factors_into(sfb_ctx* c, const void* W, const void* X, const sfb_aux* aux, RowMap u, RowMap v, CsrView codes,
-                 int workers = 0, bool for_apply = false) {
+                 int workers = 0, bool for_apply = false, const Commit& commit = Commit()) {
   const sfb_desc& d = c->d;
   const int K = workers > 0 ? workers * d.B : c->K;
   const float* Wf = reinterpret_cast<const float*>(W);
@@ -213,10 +214,13 @@ int factors_into(sfb_ctx* c, const void* W, const void* X, const sfb_aux* aux, R
                              c->f32_splits, &ks));
     }
     const RowMap zsrc = ks > 1 ? part : u;
+    FinishExtra extra;
+    extra.commit = commit;
     if (d.model == SFB_MLR)
       ACC(launch_finish_mlr(c->stream, zsrc, u, aux->labels, K, d.J, c->dev_status, ks, sstride,
-                            reinterpret_cast<float*>(aux->dual), aux->sdca_step));
-    else ACC(launch_finish_dml(c->stream, zsrc, u, aux->similar, d.margin, K, d.J, ks, sstride, c->dml_active));
+                            reinterpret_cast<float*>(aux->dual), aux->sdca_step, CorrOut(), extra));
+    else ACC(launch_finish_dml(c->stream, zsrc, u, aux->similar, d.margin, K, d.J, ks, sstride, c->dml_active, CorrOut(),
+                               extra));
     return SFB_OK;
   }
   // tensor-core paths
@@ -224,7 +228,7 @@ int factors_into(sfb_ctx* c, const void* W, const void* X, const sfb_aux* aux, R
     const int r = ensure_shadow(c, W);
     if (r < 0) return r;
   }
-  ACC(umma_forward(c->umma, c->stream, W, c->w_shadow, X, aux, u, v, c->dev_status, workers, for_apply));
+  ACC(umma_forward(c->umma, c->stream, W, c->w_shadow, X, aux, u, v, c->dev_status, workers, for_apply, commit));
   return SFB_OK;
 }
 
@@ -551,13 +555,15 @@ int sfb_pack(sfb_ctx* c, const void* U, const void* V, const sfb_aux* aux, void*
   } else if (V == nullptr || !aligned(V, 16)) {
     return SFB_ERR_ARG;
   }
-  ACC(launch_copy_rows(c->stream, caller_rows(U, c->l.ldu, d.B, c->l.es), stream_u(c, sf_buf), c->K, d.J));
-  if (d.v_sparse)
+  const Commit commit = make_commit(sf_buf, d, c->l, clock, rowptr);
+  if (d.v_sparse) {
+    ACC(launch_copy_rows(c->stream, caller_rows(U, c->l.ldu, d.B, c->l.es), stream_u(c, sf_buf), c->K, d.J));
     ACC(launch_pack_csr(c->stream, sf_buf, d, c->l, aux->rowptr, aux->idx, reinterpret_cast<const float*>(aux->val),
-                        c->dev_status));
-  else
-    ACC(launch_copy_rows(c->stream, caller_rows(V, c->l.ldv, d.B, c->l.es), stream_v(c, sf_buf), c->K, d.D));
-  ACC(launch_write_header(c->stream, sf_buf, d, c->l, clock, rowptr));
+                        c->dev_status, commit));
+  } else {
+    ACC(launch_pack_rows(c->stream, caller_rows(U, c->l.ldu, d.B, c->l.es), stream_u(c, sf_buf), d.J,
+                         caller_rows(V, c->l.ldv, d.B, c->l.es), stream_v(c, sf_buf), d.D, c->K, commit));
+  }
   if (d.compact) ACC(launch_compact(c->stream, sf_buf, d, c->l, c->compact_ws));
   return SFB_OK;
 }
@@ -667,10 +673,12 @@ int sfb_step(sfb_ctx* c, void* W, const void* X, const sfb_aux* aux, void* sf_bu
   memset(&codes, 0, sizeof(codes));
   const int slot = c->prof_n % 128;
   if (c->profiling) cudaEventRecord(c->prof_ev[slot][0], c->stream);
-  // What does not depend on the factors goes to the auxiliary stream, beside the forward pass: the codes into
-  // the buffer, header and directory, and the atom-major re-sort of the codes for the scatter apply.
+  // Sparse v: what does not depend on the factors goes to the auxiliary stream, beside the forward pass: the codes into
+  // the buffer, header and directory, and the atom-major re-sort of the codes for the scatter apply.  (Dense v: the
+  // finishing pass writes the header; a launch and a fork / join of their own cost a small step 5 us of host time.)
   bool forked = false;
-  if (c->aux_ok) {
+  const Commit commit = make_commit(sf_buf, d, c->l, clock, d.v_sparse ? aux->rowptr : nullptr);
+  if (d.v_sparse && c->aux_ok) {
     if (cudaEventRecord(c->aux_fork, c->stream) != cudaSuccess || cudaStreamWaitEvent(c->aux, c->aux_fork, 0) != cudaSuccess)
       return SFB_ERR_CUDA;
     forked = true;
@@ -682,12 +690,11 @@ int sfb_step(sfb_ctx* c, void* W, const void* X, const sfb_aux* aux, void* sf_bu
   auto aux_side = [&]() -> int {
     if (d.v_sparse) {
       ACC(launch_pack_csr(hs, sf_buf, d, c->l, aux->rowptr, aux->idx, reinterpret_cast<const float*>(aux->val),
-                          c->dev_status));
+                          c->dev_status, commit));
       // the forward reads the codes it just committed to the buffer, or, beside the packing, the caller's arrays
       // cut to the same per-worker capacity (so u always belongs to the codes that are on the wire and applied)
       codes = forked ? global_codes(aux, d.B, c->l.cap_p) : stream_codes(c, sf_buf);
     }
-    ACC(launch_write_header(hs, sf_buf, d, c->l, clock, d.v_sparse ? aux->rowptr : nullptr));
     if (forked && d.v_sparse && d.path == SFB_PATH_F32 && c->csc_ws != nullptr) {
       ACC(launch_sc_csc_build(hs, stream_codes(c, sf_buf), K, d.D, (long long)d.nnz_capacity, c->csc_ws, c->dev_status));
       csc_built = true;
@@ -711,7 +718,7 @@ int sfb_step(sfb_ctx* c, void* W, const void* X, const sfb_aux* aux, void* sf_bu
     return SFB_ERR_CUDA;
   }
   r = factors_into(c, W, X, aux, stream_u(c, sf_buf), d.v_sparse ? RowMap() : stream_v(c, sf_buf), codes, 0,
-                   d.path == SFB_PATH_TF32X3 && !d.compact && K == c->K);
+                   d.path == SFB_PATH_TF32X3 && !d.compact && K == c->K, d.v_sparse ? Commit() : commit);
   if (forked && cudaStreamWaitEvent(c->stream, c->aux_join, 0) != cudaSuccess) return SFB_ERR_CUDA;
   if (r < 0) return r;
   // pairs whose u came out as zero are dropped from the message before it is "sent" (and applied)

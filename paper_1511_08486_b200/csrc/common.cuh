@@ -101,6 +101,71 @@ static inline Layout make_layout(const sfb_desc& d) {
   return l;
 }
 
+struct HeaderImage {   // exactly the first 68 bytes of the 128-byte header
+  uint32_t magic;
+  uint16_t version;
+  uint8_t model, dtype;
+  uint32_t flags, P, B, J, D, clock, ldu, ldv;
+  uint64_t stream_stride, total_bytes, streams_off;
+  uint32_t cap_p;
+};
+static_assert(sizeof(HeaderImage) == 72, "header image is 68 bytes of fields plus 4 of tail padding");
+
+// Header and directory of a buffer, for whichever kernel of a call writes them (buf == nullptr: none).
+struct Commit {
+  char* buf;
+  HeaderImage h;
+  long long u_bytes;
+  const uint32_t* rowptr;   // global CSR row pointers (sparse v), or nullptr
+  __host__ __device__ Commit() : buf(nullptr), h(), u_bytes(0), rowptr(nullptr) {}
+};
+Commit make_commit(void* sf_buf, const sfb_desc& d, const Layout& l, uint32_t clock, const uint32_t* rowptr);
+#ifdef __CUDACC__
+// Called by the n threads of one block.
+__device__ __forceinline__ void write_header(const Commit& c, int tid, int n) {
+  uint32_t* w = reinterpret_cast<uint32_t*>(c.buf);
+  const HeaderImage& h = c.h;
+  const uint32_t* src = reinterpret_cast<const uint32_t*>(&h);
+  for (int t = tid; t < 32; t += n) w[t] = (t < 17) ? src[t] : 0u;
+  const int dir_words = (int)((h.streams_off - 128) / 4);
+  for (int t = tid; t < dir_words; t += n) {
+    const int p = t >> 3, f = t & 7;
+    uint32_t val = 0u;
+    if (p < (int)h.P) {
+      const uint64_t u_off = h.streams_off + (uint64_t)p * h.stream_stride;
+      const uint64_t v_off = u_off + (uint64_t)c.u_bytes;
+      switch (f) {
+        case 0: val = (uint32_t)p; break;
+        case 1: val = h.B; break;
+        case 2: val = h.clock; break;
+        case 3:
+          if (c.rowptr != nullptr) {
+            const uint32_t m = c.rowptr[(p + 1) * h.B] - c.rowptr[p * h.B];
+            val = m < h.cap_p ? m : h.cap_p;
+          } else if (h.flags & 1u) {   // no global row pointers: the count the worker's own stream carries
+            val = reinterpret_cast<const uint32_t*>(c.buf + v_off)[h.B];
+          }
+          break;
+        case 4: val = (uint32_t)(u_off & 0xffffffffu); break;
+        case 5: val = (uint32_t)(u_off >> 32); break;
+        case 6: val = (uint32_t)(v_off & 0xffffffffu); break;
+        default: val = (uint32_t)(v_off >> 32); break;
+      }
+    }
+    w[32 + t] = val;
+  }
+}
+#endif
+
+// What a finishing pass does beside its own work: the buffer's header, and (MLR, small batches) the factor v = x.
+struct FinishExtra {
+  Commit commit;
+  RowMap src, dst;   // dst.base == nullptr: no copy
+  int cols;
+  CorrOut corr;
+  FinishExtra() : src(), dst(), cols(0) {}
+};
+
 // cudaFuncSetAttribute acts on the current device only: first() is true once per device (ordinals 0..63)
 // for the static object it is called on.  A repeated call from a racing thread would set the same value.
 struct PerDeviceOnce {
@@ -148,25 +213,31 @@ int launch_apply_f32(cudaStream_t s, float* W, RowMap u, RowMap v, int K, int J,
 // written to u is then the dual step sdca_step * (dual + softmax - onehot).
 int launch_finish_mlr(cudaStream_t s, RowMap z, RowMap u, const int32_t* labels, int K, int J, int* dev_status,
                       int nsplit = 1, long long split_stride_bytes = 0, float* dual = nullptr, float sdca_step = 0.f,
-                      CorrOut corr = CorrOut());
+                      CorrOut corr = CorrOut(), const FinishExtra& extra = FinishExtra());
 
 // DML epilogue: u = +z (similar) or -z * [|z|^2 < margin] (dissimilar).
 // active (optional, [K] bytes): 1 where the pair contributes (similar, or dissimilar inside the margin), 0 where u_i = 0.
 int launch_finish_dml(cudaStream_t s, RowMap z, RowMap u, const uint8_t* similar, float margin, int K, int J,
-                      int nsplit = 1, long long split_stride_bytes = 0, uint8_t* active = nullptr, CorrOut corr = CorrOut());
+                      int nsplit = 1, long long split_stride_bytes = 0, uint8_t* active = nullptr, CorrOut corr = CorrOut(),
+                      const FinishExtra& extra = FinishExtra());
 // idx[0 .. *n_out) = ascending list of the samples i < K with active[i] != 0 (device arrays; one ordered block).
 int launch_compact_active(cudaStream_t s, const uint8_t* active, int K, int* idx, int* n_out);
 
 // Copies K rows of `cols` values from src to dst rows (same value type), zero-filling dst pad columns.
 int launch_copy_rows(cudaStream_t s, RowMap src, RowMap dst, int K, int cols, CorrOut corr = CorrOut());
 
+// The u rows (J values) and v rows (D values) of K pairs into the streams behind u_dst / v_dst, and the header.
+int launch_pack_rows(cudaStream_t s, RowMap u_src, RowMap u_dst, int J, RowMap v_src, RowMap v_dst, int D, int K,
+                     const Commit& commit);
+
 // Writes header and directory of the SF buffer.  `rowptr` (global CSR row pointers) only for sparse v.
 int launch_write_header(cudaStream_t s, void* sf_buf, const sfb_desc& d, const Layout& l, uint32_t clock,
                         const uint32_t* rowptr);
 
-// Copies the CSR codes of every worker into its stream (local row pointers, zero-filled tail).
+// Copies the CSR codes of every worker into its stream (local row pointers, zero-filled tail).  commit (optional): header
+// and directory written by the same launch.
 int launch_pack_csr(cudaStream_t s, void* sf_buf, const sfb_desc& d, const Layout& l, const uint32_t* rowptr,
-                    const uint32_t* idx, const float* val, int* dev_status);
+                    const uint32_t* idx, const float* val, int* dev_status, const Commit& commit = Commit());
 
 // Inactive-pair compaction of a committed dense-v buffer, in place: per worker the pairs with a nonzero u move to
 // the front (same order), the slots behind them are cleared, the directory gets the pair counts and the header

@@ -71,6 +71,37 @@ __device__ __forceinline__ void store_u4(char* row, int j, float4 v, int es) {
   }
 }
 
+// 16 bytes of row i at unit q, copied from src to dst (columns from `cols` on as zeros), with their correction operands.
+__device__ __forceinline__ void copy_unit(const RowMap& src, const RowMap& dst, int i, int q, int cols, const CorrOut& corr) {
+  const int per = 16 / dst.es, c = q * per;
+  uint4 val = make_uint4(0u, 0u, 0u, 0u);
+  if (c < cols && c < src.ld) {
+    val = *reinterpret_cast<const uint4*>(src.row(i) + (size_t)q * 16);
+    if (c + per > cols) {   // mask the tail beyond `cols`
+      if (dst.es == 4) {
+        uint32_t* w = reinterpret_cast<uint32_t*>(&val);
+        for (int e = 0; e < 4; ++e)
+          if (c + e >= cols) w[e] = 0u;
+      } else {
+        uint16_t* h = reinterpret_cast<uint16_t*>(&val);
+        for (int e = 0; e < 8; ++e)
+          if (c + e >= cols) h[e] = 0;
+      }
+    }
+  }
+  *reinterpret_cast<uint4*>(dst.row(i) + (size_t)q * 16) = val;
+  if (corr.mn != nullptr || corr.km != nullptr)   // fp32 rows only (the compensated path)
+    corr_store4(corr, i, dst.B, c, make_float4(__uint_as_float(val.x), __uint_as_float(val.y), __uint_as_float(val.z),
+                                               __uint_as_float(val.w)));
+}
+
+// Block i of a finishing pass: row i of the copy, and block 0 the header.
+__device__ __forceinline__ void finish_extra(const FinishExtra& x, int i) {
+  if (x.commit.buf != nullptr && i == 0) write_header(x.commit, threadIdx.x, blockDim.x);
+  if (x.dst.base != nullptr)
+    for (int q = threadIdx.x; q < x.dst.ld * x.dst.es / 16; q += blockDim.x) copy_unit(x.src, x.dst, i, q, x.cols, x.corr);
+}
+
 // z rows are fp32 with ld a multiple of 4; values beyond J inside the last float4 are ignored.
 // SDCA (dual != nullptr; Section 2.1, "Stochastic DCA"): the factor is the damped dual step
 // du_i = step * (dual_i + g_i) with g_i = softmax(z_i) - onehot(y_i), and dual_i <- dual_i - du_i in place
@@ -91,11 +122,12 @@ __device__ __forceinline__ float4 sdca_step4(float* dual_row, int j, int J, floa
 
 __global__ void __launch_bounds__(1024) finish_mlr_kernel(RowMap z, RowMap u, const int32_t* __restrict__ labels,
                                                                  int K, int J, int cache_floats, int* dev_status, int nsplit, long long zstride,
-                                                                 float* __restrict__ dual, float sdca_step, CorrOut corr) {
+                                                                 float* __restrict__ dual, float sdca_step, CorrOut corr, const __grid_constant__ FinishExtra extra) {
   extern __shared__ __align__(16) float cache[];
   __shared__ float red[32];
   const int i = blockIdx.x;
   if (i >= K) return;
+  finish_extra(extra, i);
   const float* zr = reinterpret_cast<const float*>(z.row(i));
   char* ur = u.row(i);
   const int J4 = (J + 3) >> 2;
@@ -167,11 +199,12 @@ __global__ void __launch_bounds__(1024) finish_mlr_kernel(RowMap z, RowMap u, co
 
 __global__ void __launch_bounds__(1024) finish_dml_kernel(RowMap z, RowMap u, const uint8_t* __restrict__ similar,
                                                                  float margin, int K, int J, int cache_floats, int nsplit, long long zstride,
-                                                                 uint8_t* __restrict__ active, CorrOut corr) {
+                                                                 uint8_t* __restrict__ active, CorrOut corr, const __grid_constant__ FinishExtra extra) {
   extern __shared__ __align__(16) float cache[];
   __shared__ float red[32];
   const int i = blockIdx.x;
   if (i >= K) return;
+  finish_extra(extra, i);
   const float* zr = reinterpret_cast<const float*>(z.row(i));
   char* ur = u.row(i);
   const int J4 = (J + 3) >> 2;
@@ -215,11 +248,12 @@ template <int ES>
 __global__ void __launch_bounds__(256) finish_mlr_fused_kernel(RowMap u, const float2* __restrict__ stats, int n_parts,
                                                                int part_cols, const int32_t* __restrict__ labels, int K,
                                                                int J, int* dev_status, float* __restrict__ dual,
-                                                               float sdca_step) {
+                                                               float sdca_step, const __grid_constant__ FinishExtra extra) {
   extern __shared__ float scale[];   // [n_parts]
   __shared__ float red[32];
   const int i = blockIdx.x;
   if (i >= K) return;
+  finish_extra(extra, i);
   const float kLog2e = 1.4426950408889634f;
   const float2* st = stats + (size_t)i * n_parts;
   float m = -INFINITY;
@@ -382,31 +416,23 @@ __global__ void __launch_bounds__(PROX_THREADS, VEC ? 2 : 1) prox_unit_columns_k
 // 16-byte-vectorised row copy; rows are whole numbers of 16-byte units on both sides.
 __global__ void __launch_bounds__(256) copy_rows_kernel(RowMap src, RowMap dst, int K, int cols, CorrOut corr) {
   const int units_dst = dst.ld * dst.es / 16;
-  const int per = 16 / dst.es;
   const long long total = (long long)K * units_dst;
   for (long long g = blockIdx.x * (long long)blockDim.x + threadIdx.x; g < total;
+       g += (long long)gridDim.x * blockDim.x)
+    copy_unit(src, dst, (int)(g / units_dst), (int)(g % units_dst), cols, corr);
+}
+
+// u and v rows into their streams, and the header, in one launch.
+__global__ void __launch_bounds__(256) pack_rows_kernel(RowMap u_src, RowMap u_dst, int J, RowMap v_src, RowMap v_dst, int D,
+                                                        int K, const __grid_constant__ Commit commit) {
+  if (blockIdx.x == 0) write_header(commit, threadIdx.x, 256);
+  const int uu = u_dst.ld * u_dst.es / 16, units = uu + v_dst.ld * v_dst.es / 16;
+  const long long total = (long long)K * units;
+  for (long long g = blockIdx.x * (long long)blockDim.x + threadIdx.x; g < total;
        g += (long long)gridDim.x * blockDim.x) {
-    const int i = (int)(g / units_dst), q = (int)(g % units_dst);
-    const int c = q * per;
-    uint4 val = make_uint4(0u, 0u, 0u, 0u);
-    if (c < cols && c < src.ld) {
-      val = *reinterpret_cast<const uint4*>(src.row(i) + (size_t)q * 16);
-      if (c + per > cols) {   // mask the tail beyond `cols`
-        if (dst.es == 4) {
-          uint32_t* w = reinterpret_cast<uint32_t*>(&val);
-          for (int e = 0; e < 4; ++e)
-            if (c + e >= cols) w[e] = 0u;
-        } else {
-          uint16_t* h = reinterpret_cast<uint16_t*>(&val);
-          for (int e = 0; e < 8; ++e)
-            if (c + e >= cols) h[e] = 0;
-        }
-      }
-    }
-    *reinterpret_cast<uint4*>(dst.row(i) + (size_t)q * 16) = val;
-    if (corr.mn != nullptr || corr.km != nullptr)   // fp32 rows only (the compensated path)
-      corr_store4(corr, i, dst.B, c, make_float4(__uint_as_float(val.x), __uint_as_float(val.y), __uint_as_float(val.z),
-                                                 __uint_as_float(val.w)));
+    const int i = (int)(g / units), q = (int)(g % units);
+    if (q < uu) copy_unit(u_src, u_dst, i, q, J, CorrOut());
+    else copy_unit(v_src, v_dst, i, q - uu, D, CorrOut());
   }
 }
 
@@ -456,7 +482,8 @@ int fin_cache_floats(int J) {
 }  // namespace
 
 int launch_finish_mlr(cudaStream_t s, RowMap z, RowMap u, const int32_t* labels, int K, int J, int* dev_status,
-                      int nsplit, long long split_stride_bytes, float* dual, float sdca_step, CorrOut corr) {
+                      int nsplit, long long split_stride_bytes, float* dual, float sdca_step, CorrOut corr,
+                      const FinishExtra& extra) {
   const int cf = fin_cache_floats(J);
   static PerDeviceOnce attr_once;   // function attributes are per device
   if (attr_once.first()) {
@@ -464,7 +491,7 @@ int launch_finish_mlr(cudaStream_t s, RowMap z, RowMap u, const int32_t* labels,
     cudaFuncSetAttribute(finish_dml_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, ROW_CACHE_FLOATS * 4);
   }
   finish_mlr_kernel<<<K, fin_threads(J), (size_t)cf * 4, s>>>(z, u, labels, K, J, cf, dev_status, nsplit, split_stride_bytes / 4,
-                                                              dual, sdca_step, corr);
+                                                              dual, sdca_step, corr, extra);
   return cudaGetLastError() == cudaSuccess ? 1 : SFB_ERR_CUDA;
 }
 
@@ -503,7 +530,7 @@ int launch_compact_active(cudaStream_t s, const uint8_t* active, int K, int* idx
 }
 
 int launch_finish_dml(cudaStream_t s, RowMap z, RowMap u, const uint8_t* similar, float margin, int K, int J,
-                      int nsplit, long long split_stride_bytes, uint8_t* active, CorrOut corr) {
+                      int nsplit, long long split_stride_bytes, uint8_t* active, CorrOut corr, const FinishExtra& extra) {
   const int cf = fin_cache_floats(J);
   static PerDeviceOnce attr_once;   // function attributes are per device
   if (attr_once.first()) {
@@ -511,18 +538,19 @@ int launch_finish_dml(cudaStream_t s, RowMap z, RowMap u, const uint8_t* similar
     cudaFuncSetAttribute(finish_dml_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, ROW_CACHE_FLOATS * 4);
   }
   finish_dml_kernel<<<K, fin_threads(J), (size_t)cf * 4, s>>>(z, u, similar, margin, K, J, cf, nsplit, split_stride_bytes / 4,
-                                                              active, corr);
+                                                              active, corr, extra);
   return cudaGetLastError() == cudaSuccess ? 1 : SFB_ERR_CUDA;
 }
 
 int launch_finish_mlr_fused(cudaStream_t s, RowMap u, const float2* stats, int n_parts, int part_cols,
-                            const int32_t* labels, int K, int J, int* dev_status, float* dual, float sdca_step) {
+                            const int32_t* labels, int K, int J, int* dev_status, float* dual, float sdca_step,
+                            const FinishExtra& extra) {
   const size_t smem = (size_t)n_parts * sizeof(float);
   if (smem > 48 * 1024) return SFB_ERR_SHAPE;
   if (u.es == 4)
-    finish_mlr_fused_kernel<4><<<K, 256, smem, s>>>(u, stats, n_parts, part_cols, labels, K, J, dev_status, dual, sdca_step);
+    finish_mlr_fused_kernel<4><<<K, 256, smem, s>>>(u, stats, n_parts, part_cols, labels, K, J, dev_status, dual, sdca_step, extra);
   else
-    finish_mlr_fused_kernel<2><<<K, 256, smem, s>>>(u, stats, n_parts, part_cols, labels, K, J, dev_status, dual, sdca_step);
+    finish_mlr_fused_kernel<2><<<K, 256, smem, s>>>(u, stats, n_parts, part_cols, labels, K, J, dev_status, dual, sdca_step, extra);
   return cudaGetLastError() == cudaSuccess ? 1 : SFB_ERR_CUDA;
 }
 
@@ -543,6 +571,14 @@ int launch_prox_unit_columns(cudaStream_t s, float* W, int J, int D, __nv_bfloat
   const cudaError_t e = (D & 3) == 0 ? cudaLaunchKernelEx(&cfg, prox_unit_columns_kernel<true>, W, J, D, rows, shadow)
                                      : cudaLaunchKernelEx(&cfg, prox_unit_columns_kernel<false>, W, J, D, rows, shadow);
   return e == cudaSuccess ? 1 : SFB_ERR_CUDA;
+}
+
+int launch_pack_rows(cudaStream_t s, RowMap u_src, RowMap u_dst, int J, RowMap v_src, RowMap v_dst, int D, int K,
+                     const Commit& commit) {
+  const long long total = (long long)K * ((u_dst.ld + v_dst.ld) * (long long)u_dst.es / 16);
+  const int blocks = (int)((total + 255) / 256 < 148LL * 16 ? (total + 255) / 256 : 148LL * 16);
+  pack_rows_kernel<<<blocks, 256, 0, s>>>(u_src, u_dst, J, v_src, v_dst, D, K, commit);
+  return cudaGetLastError() == cudaSuccess ? 1 : SFB_ERR_CUDA;
 }
 
 int launch_copy_rows(cudaStream_t s, RowMap src, RowMap dst, int K, int cols, CorrOut corr) {

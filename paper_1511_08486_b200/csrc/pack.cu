@@ -6,17 +6,7 @@
 namespace sfb {
 namespace {
 
-struct HeaderImage {   // exactly the first 68 bytes of the 128-byte header
-  uint32_t magic;
-  uint16_t version;
-  uint8_t model, dtype;
-  uint32_t flags, P, B, J, D, clock, ldu, ldv;
-  uint64_t stream_stride, total_bytes, streams_off;
-  uint32_t cap_p;
-};
-static_assert(sizeof(HeaderImage) == 72, "header image is 68 bytes of fields plus 4 of tail padding");
-
-__host__ HeaderImage make_header(const sfb_desc& d, const Layout& l, uint32_t clock) {
+HeaderImage make_header(const sfb_desc& d, const Layout& l, uint32_t clock) {
   HeaderImage h;
   h.magic = 0x31424653u;
   h.version = 1;
@@ -33,39 +23,7 @@ __host__ HeaderImage make_header(const sfb_desc& d, const Layout& l, uint32_t cl
   return h;
 }
 
-// One block: thread t < 32 writes header word t (128 bytes); then threads stride over the directory.
-__global__ void write_header_kernel(char* buf, HeaderImage h, long long u_bytes, const uint32_t* __restrict__ rowptr) {
-  uint32_t* w = reinterpret_cast<uint32_t*>(buf);
-  const uint32_t* src = reinterpret_cast<const uint32_t*>(&h);
-  if (threadIdx.x < 32) w[threadIdx.x] = (threadIdx.x < 17) ? src[threadIdx.x] : 0u;
-  const int dir_words = (int)((h.streams_off - 128) / 4);
-  for (int t = threadIdx.x; t < dir_words; t += blockDim.x) {
-    const int p = t >> 3, f = t & 7;
-    uint32_t val = 0u;
-    if (p < (int)h.P) {
-      const uint64_t u_off = h.streams_off + (uint64_t)p * h.stream_stride;
-      const uint64_t v_off = u_off + (uint64_t)u_bytes;
-      switch (f) {
-        case 0: val = (uint32_t)p; break;
-        case 1: val = h.B; break;
-        case 2: val = h.clock; break;
-        case 3:
-          if (rowptr != nullptr) {
-            const uint32_t n = rowptr[(p + 1) * h.B] - rowptr[p * h.B];
-            val = n < h.cap_p ? n : h.cap_p;
-          } else if (h.flags & 1u) {   // no global row pointers: the count the worker's own stream carries
-            val = reinterpret_cast<const uint32_t*>(buf + v_off)[h.B];
-          }
-          break;
-        case 4: val = (uint32_t)(u_off & 0xffffffffu); break;
-        case 5: val = (uint32_t)(u_off >> 32); break;
-        case 6: val = (uint32_t)(v_off & 0xffffffffu); break;
-        default: val = (uint32_t)(v_off >> 32); break;
-      }
-    }
-    w[32 + t] = val;
-  }
-}
+__global__ void write_header_kernel(const __grid_constant__ Commit c) { write_header(c, threadIdx.x, blockDim.x); }
 
 __global__ void check_header_kernel(const char* buf, HeaderImage h, int* dev_status) {
   const uint32_t* w = reinterpret_cast<const uint32_t*>(buf);
@@ -82,9 +40,10 @@ __global__ void __launch_bounds__(256) pack_csr_kernel(char* buf, long long stre
                                                        long long u_bytes, long long rp_bytes, long long idx_bytes,
                                                        int B, int cap_p, int D, const uint32_t* __restrict__ rowptr,
                                                        const uint32_t* __restrict__ idx, const float* __restrict__ val,
-                                                       int* dev_status) {
+                                                       int* dev_status, const __grid_constant__ Commit commit) {
   const int p = blockIdx.x;
   const int part = blockIdx.y, parts = gridDim.y;   // the worker's words are spread over gridDim.y blocks
+  if (commit.buf != nullptr && p == 0 && part == 0) write_header(commit, threadIdx.x, 256);
   char* vb = buf + streams_off + (long long)p * stream_stride + u_bytes;
   uint32_t* rp = reinterpret_cast<uint32_t*>(vb);
   uint32_t* ix = reinterpret_cast<uint32_t*>(vb + rp_bytes);
@@ -120,9 +79,18 @@ __global__ void __launch_bounds__(256) pack_csr_kernel(char* buf, long long stre
 
 }  // namespace
 
+Commit make_commit(void* sf_buf, const sfb_desc& d, const Layout& l, uint32_t clock, const uint32_t* rowptr) {
+  Commit c;
+  c.buf = reinterpret_cast<char*>(sf_buf);
+  c.h = make_header(d, l, clock);
+  c.u_bytes = l.u_bytes;
+  c.rowptr = rowptr;
+  return c;
+}
+
 int launch_write_header(cudaStream_t s, void* sf_buf, const sfb_desc& d, const Layout& l, uint32_t clock,
                         const uint32_t* rowptr) {
-  write_header_kernel<<<1, 256, 0, s>>>(reinterpret_cast<char*>(sf_buf), make_header(d, l, clock), l.u_bytes, rowptr);
+  write_header_kernel<<<1, 256, 0, s>>>(make_commit(sf_buf, d, l, clock, rowptr));
   return cudaGetLastError() == cudaSuccess ? 1 : SFB_ERR_CUDA;
 }
 
@@ -132,10 +100,10 @@ int launch_check_header(cudaStream_t s, const void* sf_buf, const sfb_desc& d, c
 }
 
 int launch_pack_csr(cudaStream_t s, void* sf_buf, const sfb_desc& d, const Layout& l, const uint32_t* rowptr,
-                    const uint32_t* idx, const float* val, int* dev_status) {
+                    const uint32_t* idx, const float* val, int* dev_status, const Commit& commit) {
   const int parts = (l.cap_p + 2047) / 2048 < 1 ? 1 : ((l.cap_p + 2047) / 2048 > 64 ? 64 : (l.cap_p + 2047) / 2048);
   pack_csr_kernel<<<dim3(d.P, parts), 256, 0, s>>>(reinterpret_cast<char*>(sf_buf), l.streams_off, l.stream_stride, l.u_bytes,
-                                      l.rp_bytes, l.idx_bytes, d.B, l.cap_p, d.D, rowptr, idx, val, dev_status);
+                                      l.rp_bytes, l.idx_bytes, d.B, l.cap_p, d.D, rowptr, idx, val, dev_status, commit);
   return cudaGetLastError() == cudaSuccess ? 1 : SFB_ERR_CUDA;
 }
 

@@ -29,7 +29,8 @@ namespace sfb {
 
 // extra passes implemented in finish.cu
 int launch_finish_mlr_fused(cudaStream_t s, RowMap u, const float2* stats, int n_parts, int part_cols,
-                            const int32_t* labels, int K, int J, int* dev_status, float* dual, float sdca_step);
+                            const int32_t* labels, int K, int J, int* dev_status, float* dual, float sdca_step,
+                            const FinishExtra& extra);
 
 namespace {
 
@@ -872,6 +873,10 @@ struct UmmaPlan {
 constexpr int FWD_GROUP = 8, APPLY_GROUP = 8;
 // 128-byte atoms of the reduction index per pipeline stage wherever three such stages fit in shared memory.
 constexpr int STAGE_ATOMS = 2;
+// MLR: factors v up to this size are copied by the blocks of the finishing pass.  A launch of their own on the side
+// stream hides behind the GEMM but costs a fork and a join: 257 x 1000, K = 200 (0.8 MB)
+// 31.9 -> 30.7 us a step; 4000 x 2056, K = 1000 in bf16 (4.1 MB) 89.9 against 90.3, no difference.
+constexpr long long V_INLINE_BYTES = 2 << 20;
 // Compensated kernels: 128-byte atoms (32 fp32 reduction steps = 4 MMA instructions) one accumulator may take
 // before its range ends: 40 atoms = 160 roundings toward zero, about 2.6e-6 of the sum.
 constexpr int X3_ATOMS_PER_RANGE = 40;
@@ -1206,7 +1211,8 @@ int umma_forward_sc(UmmaPlan* pl, cudaStream_t s, const void* W, RowMap a, RowMa
 }
 
 int umma_forward(UmmaPlan* pl, cudaStream_t s, const void* W, const __nv_bfloat16* w_shadow, const void* X,
-                 const sfb_aux* aux, RowMap u, RowMap v, int* dev_status, int workers, bool for_apply) {
+                 const sfb_aux* aux, RowMap u, RowMap v, int* dev_status, int workers, bool for_apply,
+                 const Commit& commit) {
   const sfb_desc& d = pl->d;
   const int K = (workers > 0 ? workers : d.P) * d.B;
   int launches = 0, r;
@@ -1221,10 +1227,15 @@ int umma_forward(UmmaPlan* pl, cudaStream_t s, const void* W, const __nv_bfloat1
   x_rows.base = const_cast<char*>(reinterpret_cast<const char*>(X));
   x_rows.ld = d.D; x_rows.B = d.B; x_rows.es = pl->es;
   x_rows.worker_stride = (long long)d.B * d.D * pl->es;
+  FinishExtra extra;
+  extra.commit = commit;
   if (d.model == SFB_MLR) {
     const bool bf16 = d.path == SFB_PATH_BF16;
     bool forked = false;
-    if (v.base != nullptr && pl->side_ok) {   // v = x on the side stream, joined before this call returns its work
+    // a small v goes out beside the finishing pass, a large one beside the GEMM
+    const bool v_inline = v.base != nullptr && (long long)K * v.ld * v.es <= V_INLINE_BYTES;
+    if (v_inline) { extra.src = x_rows; extra.dst = v; extra.cols = d.D; extra.corr = cv; }
+    if (v.base != nullptr && !v_inline && pl->side_ok) {   // v = x on the side stream, joined before this call returns its work
       if (cudaEventRecord(pl->fork, s) != cudaSuccess || cudaStreamWaitEvent(pl->side, pl->fork, 0) != cudaSuccess)
         return SFB_ERR_CUDA;
       forked = true;
@@ -1256,7 +1267,7 @@ int umma_forward(UmmaPlan* pl, cudaStream_t s, const void* W, const __nv_bfloat1
           return r;
         launches += r;
         if ((r = launch_finish_mlr(s, pz, u, aux->labels, K, d.J, dev_status, ks, sstride, reinterpret_cast<float*>(aux->dual),
-                                   aux->sdca_step, cu)) < 0)
+                                   aux->sdca_step, cu, extra)) < 0)
           return r;
         launches += r;
         if (emit) { pl->fresh_u = u.base; pl->fresh_K = K; }
@@ -1267,11 +1278,11 @@ int umma_forward(UmmaPlan* pl, cudaStream_t s, const void* W, const __nv_bfloat1
           return r;
         launches += r;
         if ((r = launch_finish_mlr_fused(s, u, pl->stats, n_parts, part_cols, aux->labels, K, d.J, dev_status,
-                                         reinterpret_cast<float*>(aux->dual), aux->sdca_step)) < 0)
+                                         reinterpret_cast<float*>(aux->dual), aux->sdca_step, extra)) < 0)
           return r;
         launches += r;
       }
-      if (!forked && v.base != nullptr) {
+      if (!forked && !v_inline && v.base != nullptr) {
         if ((r = launch_copy_rows(s, x_rows, v, K, d.D, cv)) < 0) return r;
         launches += r;
       }
@@ -1304,7 +1315,7 @@ int umma_forward(UmmaPlan* pl, cudaStream_t s, const void* W, const __nv_bfloat1
                                pl->x3 ? w_shadow : nullptr, pl->x3)) < 0)
       return r;
     launches += r;
-    if ((r = launch_finish_dml(s, pz, u, aux->similar, d.margin, K, d.J, ks, sstride, nullptr, cu)) < 0) return r;
+    if ((r = launch_finish_dml(s, pz, u, aux->similar, d.margin, K, d.J, ks, sstride, nullptr, cu, extra)) < 0) return r;
     if (emit) { pl->fresh_u = u.base; pl->fresh_v = v.base; pl->fresh_K = K; }
     return launches + r;
   }
@@ -1312,7 +1323,7 @@ int umma_forward(UmmaPlan* pl, cudaStream_t s, const void* W, const __nv_bfloat1
                              pl->x3 ? w_shadow : nullptr, pl->x3)) < 0)
     return r;
   launches += r;
-  if ((r = launch_finish_dml(s, u, u, aux->similar, d.margin, K, d.J, 1, 0, nullptr, cu)) < 0) return r;
+  if ((r = launch_finish_dml(s, u, u, aux->similar, d.margin, K, d.J, 1, 0, nullptr, cu, extra)) < 0) return r;
   if (emit) { pl->fresh_u = u.base; pl->fresh_v = v.base; pl->fresh_K = K; }
   return launches + r;
 }
