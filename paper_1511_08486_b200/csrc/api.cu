@@ -673,6 +673,15 @@ int sfb_step(sfb_ctx* c, void* W, const void* X, const sfb_aux* aux, void* sf_bu
   memset(&codes, 0, sizeof(codes));
   const int slot = c->prof_n % 128;
   if (c->profiling) cudaEventRecord(c->prof_ev[slot][0], c->stream);
+  // (the stage times of a profiled step need separate stages)
+  if (d.path == SFB_PATH_F32 && !d.v_sparse && !d.compact && !c->profiling && step_small_fits(c->K, d.J, d.D)) {
+    ACC(launch_step_small(c->stream, d, reinterpret_cast<float*>(W), reinterpret_cast<const float*>(X), aux,
+                          stream_u(c, sf_buf), stream_v(c, sf_buf), c->K, K, eta, c->dev_status,
+                          make_commit(sf_buf, d, c->l, clock, nullptr)));
+    c->last_step_K = K;
+    c->last_step_listed = false;
+    return SFB_OK;
+  }
   // Sparse v: what does not depend on the factors goes to the auxiliary stream, beside the forward pass: the codes into
   // the buffer, header and directory, and the atom-major re-sort of the codes for the scatter apply.  (Dense v: the
   // finishing pass writes the header; a launch and a fork / join of their own cost a small step 5 us of host time.)

@@ -166,6 +166,25 @@ struct FinishExtra {
   FinishExtra() : src(), dst(), cols(0) {}
 };
 
+#ifdef __CUDACC__
+// SDCA (dual != nullptr; Section 2.1, "Stochastic DCA"): the factor is the damped dual step
+// du_i = step * (dual_i + g_i) with g_i = softmax(z_i) - onehot(y_i), and dual_i <- dual_i - du_i in place
+// (dual rows: fp32, ldd = J rounded up to 4 values per row, pad values written as zeros).
+__device__ __forceinline__ float4 sdca_step4(float* dual_row, int j, int J, float4 g, float step, bool bad) {
+  float4 d = *reinterpret_cast<const float4*>(dual_row + j);
+  float4 du = make_float4(0.f, 0.f, 0.f, 0.f);
+  if (!bad) {   // a sample with a bad label takes no step: its dual variables stay as they are
+    du.x = step * (d.x + g.x); du.y = step * (d.y + g.y); du.z = step * (d.z + g.z); du.w = step * (d.w + g.w);
+    d.x -= du.x; d.y -= du.y; d.z -= du.z; d.w -= du.w;
+  }
+  if (j + 1 >= J) { du.y = 0.f; d.y = 0.f; }
+  if (j + 2 >= J) { du.z = 0.f; d.z = 0.f; }
+  if (j + 3 >= J) { du.w = 0.f; d.w = 0.f; }
+  *reinterpret_cast<float4*>(dual_row + j) = d;
+  return du;
+}
+#endif
+
 // cudaFuncSetAttribute acts on the current device only: first() is true once per device (ordinals 0..63)
 // for the static object it is called on.  A repeated call from a racing thread would set the same value.
 struct PerDeviceOnce {
@@ -206,6 +225,12 @@ int launch_apply_f32(cudaStream_t s, float* W, RowMap u, RowMap v, int K, int J,
                      const int* dev_status, const int* row_idx = nullptr, const int* n_rows = nullptr);
 // row_idx / n_rows (optional, device): apply only the factor rows row_idx[0 .. *n_rows), in that order, instead of
 // rows 0 .. K-1 (rows that are known to be all zeros can be left out: the result is bit-identical).
+
+// A whole step (dense fp32, MLR or DML) of a problem that fits in one block: factors of K samples into u and v, header,
+// and the update by the first K_apply pairs.  Same bits as the separate kernels.
+bool step_small_fits(int K, int J, int D);
+int launch_step_small(cudaStream_t s, const sfb_desc& d, float* W, const float* X, const sfb_aux* aux, RowMap u, RowMap v,
+                      int K, int K_apply, float eta, int* dev_status, const Commit& commit);
 
 // MLR epilogue: u = softmax(z) - onehot(label).  z rows are fp32; u rows fp32 or bf16 (u.es).
 // z may be `nsplit` partial products (split s at z + s * split_stride_bytes), summed in split order.

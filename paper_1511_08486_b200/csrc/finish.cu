@@ -103,23 +103,6 @@ __device__ __forceinline__ void finish_extra(const FinishExtra& x, int i) {
 }
 
 // z rows are fp32 with ld a multiple of 4; values beyond J inside the last float4 are ignored.
-// SDCA (dual != nullptr; Section 2.1, "Stochastic DCA"): the factor is the damped dual step
-// du_i = step * (dual_i + g_i) with g_i = softmax(z_i) - onehot(y_i), and dual_i <- dual_i - du_i in place
-// (dual rows: fp32, ldd = J rounded up to 4 values per row, pad values written as zeros).
-__device__ __forceinline__ float4 sdca_step4(float* dual_row, int j, int J, float4 g, float step, bool bad) {
-  float4 d = *reinterpret_cast<const float4*>(dual_row + j);
-  float4 du = make_float4(0.f, 0.f, 0.f, 0.f);
-  if (!bad) {   // a sample with a bad label takes no step: its dual variables stay as they are
-    du.x = step * (d.x + g.x); du.y = step * (d.y + g.y); du.z = step * (d.z + g.z); du.w = step * (d.w + g.w);
-    d.x -= du.x; d.y -= du.y; d.z -= du.z; d.w -= du.w;
-  }
-  if (j + 1 >= J) { du.y = 0.f; d.y = 0.f; }
-  if (j + 2 >= J) { du.z = 0.f; d.z = 0.f; }
-  if (j + 3 >= J) { du.w = 0.f; d.w = 0.f; }
-  *reinterpret_cast<float4*>(dual_row + j) = d;
-  return du;
-}
-
 __global__ void __launch_bounds__(1024) finish_mlr_kernel(RowMap z, RowMap u, const int32_t* __restrict__ labels,
                                                                  int K, int J, int cache_floats, int* dev_status, int nsplit, long long zstride,
                                                                  float* __restrict__ dual, float sdca_step, CorrOut corr, const __grid_constant__ FinishExtra extra) {
