@@ -8,11 +8,11 @@
 //             the output index ("MN-major"); tcgen05 reads them in that form directly from the SF
 //             buffer's worker streams, no transposed copy is made.
 //
-// Warp roles (320 threads): warp 0 issues TMA loads into a shared-memory ring of 3 to 8 stages, warp 1 issues
-// the MMAs (one thread) into one of two TMEM accumulators, warps 2-9 drain the other accumulator
+// Warp roles: warp 0 issues TMA loads into a shared-memory ring of 3 to 8 stages, warp 1 issues
+// the MMAs (one thread) into one of two TMEM accumulators, eight warps drain the other accumulator
 // (tcgen05.ld) and run the epilogue, so the write-back of tile t overlaps the MMAs of tile t+1.
-// The error-compensated kernels (SPLIT, fp32-grade results from tf32 MMAs) add warps 10-13, which split every
-// operand stage into what the tensor core sees of it and the exact remainder.
+// The error-compensated kernels (SPLIT, fp32-grade results from tf32 MMAs) keep a second accumulator per tile for the
+// correction products.
 // Every wait on an mbarrier is bounded; a wait that runs out sets SFB_DEV_TIMEOUT and the CTA leaves
 // through the common exit (TMEM freed) instead of hanging.
 #include <cuda.h>
@@ -35,7 +35,10 @@ int launch_finish_mlr_fused(cudaStream_t s, RowMap u, const float2* stats, int n
 namespace {
 
 constexpr int BM = 128;          // rows per CTA tile = TMEM lanes
-constexpr int NUM_THREADS = 320;         // TMA warp, MMA warp, 8 epilogue warps
+// TMA warp, MMA warp, 8 epilogue warps.  Compensated kernels: two idle warps behind the first two, so that the epilogue
+// warps are two whole warpgroups that can take over the registers of the first (setmaxnreg).
+constexpr int num_threads(bool split) { return split ? 384 : 320; }
+constexpr int SPLIT_LAUNCH_REGS = 168;   // per thread: 384 of them fill the register file
 constexpr int EPI_STAGE_BYTES = 8 * 4096;  // one swizzled 32 x 32 fp32 block per epilogue warp
 constexpr int RING_BYTES = 192 * 1024;   // shared memory given to the operand ring
 constexpr int MAX_STAGES = 8;
@@ -142,7 +145,7 @@ __device__ __forceinline__ void tile_coords(const GemmParams& p, int tile, int& 
 //          instruction (measured: a sum of n instructions comes out short by about n * 2^-26): the small
 //          corrections must not cost the large sum more roundings.
 template <int ES, bool APPLY, int BN, int CG, int KA, bool FOLD, int EPI, bool SPLIT>
-__global__ void __launch_bounds__(NUM_THREADS, 1)
+__global__ void __launch_bounds__(num_threads(SPLIT), 1)
 umma_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                  const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUtensorMap tmAc,
                  const __grid_constant__ CUtensorMap tmBc, const GemmParams p) {
@@ -166,6 +169,8 @@ umma_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
   constexpr uint32_t IDESC_C = ptx::instr_desc(1u, APPLY ? 1u : 0u, APPLY ? 1u : 0u, BM * CG, BN);   // SPLIT: bf16 corrections
   static_assert(!SPLIT || KA == 1, "the correction tiles hold one atom of the reduction");
   static_assert(STAGES >= 2, "ring too shallow");
+  constexpr int EPI_WARP0 = SPLIT ? 4 : 2;                     // first epilogue warp
+  constexpr int BLOCKS = BN / 64;                              // 32-column blocks an epilogue warp drains per tile
 
   extern __shared__ uint8_t smem_raw[];
   uint8_t* tiles = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -219,8 +224,11 @@ umma_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
   const int k_blocks = APPLY ? ctl->k_total : p.k_blocks;
   const int k_per_split = APPLY ? k_blocks : p.k_per_split;
   const bool by_dir = APPLY && p.dir != nullptr;
-  const int total_work = (APPLY && k_blocks == 0) ? 0 : p.m_tiles * p.n_tiles * p.k_splits;
+  const int tile_count = p.m_tiles * p.n_tiles;
+  const int total_work = (APPLY && k_blocks == 0) ? 0 : tile_count * p.k_splits;
 
+  if (warp < EPI_WARP0) {
+  if (SPLIT) ptx::regs_dec<56>();   // 128 x 56 + 256 x 224 registers = the 384 x 168 of the launch
   if (warp == 0) {
     // ------------------------------------------------------------------ TMA producer (every CTA)
     int s = 0;
@@ -436,13 +444,15 @@ umma_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
         if (++s == STAGES) { s = 0; ph ^= 1u; }
       }
     }
+  }
   } else {
-    // ------------------------------------------------------------------ epilogue (warps 2..9, every CTA)
+    if (SPLIT) ptx::regs_inc<224>();
+    // ------------------------------------------------------------------ epilogue (eight warps, every CTA)
     // A warp may only read the TMEM lanes of its quarter (warp index mod 4).  Two warps share each
     // quarter and split the tile's columns in halves.  Per 32 x 32 block: accumulators come out of
     // TMEM one row per thread, go through an XOR-swizzled 4 KB shared-memory block, and are read back
     // four rows x 128 bytes per warp instruction, so that every global access is a full 128-byte line.
-    const int e = warp - 2;
+    const int e = warp - EPI_WARP0;
     const int quarter = warp & 3;
     const int half = e >> 2;
     float* stage = epi_stage + e * 1024;
@@ -556,35 +566,51 @@ umma_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
             p.stats[(long long)(wp_ * p.B + slot) * p.n_parts + nt * 2 + half] = make_float2(m, ssum);
         }
       } else
-#pragma unroll 1
-      for (int cc = 0; cc < BN / 64; ++cc) {
+      {
+      // this warp's part of the accumulator is in registers: the MMAs may go on
+      auto drained = [&]() {
+        ptx::tc_fence_before();
+        __syncwarp();
+        if (lane == 0) {
+          if (CG == 1 || rank == 0) ptx::mbar_arrive(&ctl->tmem_empty[buf]);
+          else ptx::mbar_arrive_cluster(ptx::map_to_cta(ptx::smem_u32(&ctl->tmem_empty[buf]), 0));
+        }
+      };
+      // Compensated kernels: all of the warp's columns come out of tensor memory first (main accumulator + correction
+      // accumulator, one fp32 addition, round to nearest, per value) and wait in registers for their way to global
+      // memory, so that a tile whose two accumulators fill the tensor memory holds the next tile's MMAs up for the
+      // reads only, not for the stores: apply of 1000 x 20000, K = 1024 168 -> 157 us, of 4096 x 10000 311 -> 281 us
+      uint32_t vs[SPLIT ? BLOCKS : 1][32];
+      if (SPLIT) {
+#pragma unroll
+        for (int cc = 0; cc < BLOCKS; ++cc) {
+          uint32_t lo[32];
+          ptx::tmem_ld32(taddr + half * (BN / 2) + cc * 32, vs[SPLIT ? cc : 0]);
+          ptx::tmem_ld32(taddr + BN + half * (BN / 2) + cc * 32, lo);
+          ptx::tmem_ld_wait();
+#pragma unroll
+          for (int q = 0; q < 32; ++q)
+            vs[SPLIT ? cc : 0][q] = __float_as_uint(__uint_as_float(vs[SPLIT ? cc : 0][q]) + __uint_as_float(lo[q]));
+        }
+        drained();
+      }
+#pragma unroll (SPLIT ? BLOCKS : 1)
+      for (int cc = 0; cc < BLOCKS; ++cc) {
         const int col_in_tile = half * (BN / 2) + cc * 32;
         const int c = cbase + cc * 32;
-        uint32_t v[32];
-        ptx::tmem_ld32(taddr + col_in_tile, v);
+        uint32_t (&v)[32] = vs[SPLIT ? cc : 0];
+        if (!SPLIT) ptx::tmem_ld32(taddr + col_in_tile, v);
         float4 wn[8];   // next block of W, in flight while this block is combined and stored
 #pragma unroll
         for (int g = 0; g < 8; ++g) wn[g] = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (APPLY && cc + 1 < BN / 64) {
+        if (APPLY && cc + 1 < BLOCKS) {
 #pragma unroll
           for (int g = 0; g < 8; ++g)
             if (rowp[g] != nullptr && c + 32 < ncols) wn[g] = __ldcs(reinterpret_cast<const float4*>(rowp[g] + c + 32));
         }
-        ptx::tmem_ld_wait();
-        if (SPLIT) {   // main accumulator + correction accumulator, one fp32 addition (round to nearest) per value
-          uint32_t lo[32];
-          ptx::tmem_ld32(taddr + BN + col_in_tile, lo);
+        if (!SPLIT) {
           ptx::tmem_ld_wait();
-#pragma unroll
-          for (int q = 0; q < 32; ++q) v[q] = __float_as_uint(__uint_as_float(v[q]) + __uint_as_float(lo[q]));
-        }
-        if (cc == BN / 64 - 1) {   // the last of this warp's accumulator columns are in registers: the MMAs may go on
-          ptx::tc_fence_before();
-          __syncwarp();
-          if (lane == 0) {
-            if (CG == 1 || rank == 0) ptx::mbar_arrive(&ctl->tmem_empty[buf]);
-            else ptx::mbar_arrive_cluster(ptx::map_to_cta(ptx::smem_u32(&ctl->tmem_empty[buf]), 0));
-          }
+          if (cc == BLOCKS - 1) drained();
         }
 #pragma unroll
         for (int q = 0; q < 8; ++q)
@@ -640,6 +666,7 @@ umma_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
         }
         __syncwarp();
       }
+      }
       if (!APPLY && EPI == 1) {   // (the other epilogues signal from inside their last block)
         ptx::tc_fence_before();
         __syncwarp();
@@ -651,7 +678,7 @@ umma_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
     }
   }
 
-  if (APPLY && warp >= 2 && lane == 0) ptx::tma_store_wait_all();
+  if (APPLY && warp >= EPI_WARP0 && lane == 0) ptx::tma_store_wait_all();
   ptx::tc_fence_before();
   __syncthreads();
   if (CG == 2) ptx::cluster_sync();   // nobody leaves while its pair may still signal it or read its tiles
@@ -717,7 +744,7 @@ template <int ES, bool APPLY, int BN, int CG, int KA, bool FOLD, int EPI, bool S
 int launch_gemm(cudaStream_t s, const CUtensorMap& a, const CUtensorMap& b, const CUtensorMap& w, const CUtensorMap& ac,
                 const CUtensorMap& bc, const GemmParams& p, int num_sms) {
   constexpr int stage_bytes = (BM + BN / CG) * 128 * KA * (SPLIT ? 2 : 1);
-  constexpr int threads = NUM_THREADS;
+  constexpr int threads = num_threads(SPLIT);
   constexpr int stages = (RING_BYTES / stage_bytes) < MAX_STAGES ? (RING_BYTES / stage_bytes) : MAX_STAGES;
   constexpr int smem = stages * stage_bytes + EPI_STAGE_BYTES + 1024 + (int)sizeof(SharedCtl);
   auto kernel = umma_gemm_kernel<ES, APPLY, BN, CG, KA, FOLD, EPI, SPLIT>;
@@ -726,6 +753,9 @@ int launch_gemm(cudaStream_t s, const CUtensorMap& a, const CUtensorMap& b, cons
   if (attr_once.first()) {
     if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess)
       return SFB_ERR_CUDA;
+    cudaFuncAttributes fa;
+    if (cudaFuncGetAttributes(&fa, kernel) != cudaSuccess) return SFB_ERR_CUDA;
+    if (SPLIT && fa.numRegs != SPLIT_LAUNCH_REGS) return SFB_ERR_CUDA;   // the register split would wait for ever
     if (CG == 2) {   // how many CTA pairs the device can hold at once
       cudaLaunchConfig_t q;
       memset(&q, 0, sizeof(q));
@@ -880,6 +910,7 @@ constexpr long long V_INLINE_BYTES = 2 << 20;
 // Compensated kernels: 128-byte atoms (32 fp32 reduction steps = 4 MMA instructions) one accumulator may take
 // before its range ends: 40 atoms = 160 roundings toward zero, about 2.6e-6 of the sum.
 constexpr int X3_ATOMS_PER_RANGE = 40;
+constexpr int EPI_STAGES = 10;   // stages whose time a tile's stores take
 // ... and pairs one launch of the compensated apply takes (128 instructions: 2e-6 of the sum; measured: 4096 pairs in
 // one launch come out at 1.0e-5, 2048 at 5e-6); larger updates are applied in several launches.
 constexpr int X3_PAIRS_PER_APPLY = 1024;
@@ -1017,7 +1048,9 @@ static Variant pick_variant(const UmmaPlan* pl, int m_units, int N, bool dims_ch
     long long best_cost = -1;
     auto consider = [&](int bn, int cg) {
       const long long stage_kb = (BM + bn / cg) * 256 / 1024;    // fp32 + correction tiles of one CTA
-      const long long epi = (4 * bn > 512) ? 8 * stage_kb : 0;   // exposed epilogue, in KB loaded
+      // a tile's epilogue runs beside the next tile's stages, EPI_STAGES of them; with one accumulator set the reads of
+      // tensor memory come first
+      const long long epi = (4 * bn > 512) ? stage_kb : 0;
       const long long tiles = (long long)((m_units + cg - 1) / cg) * ((N + bn - 1) / bn);
       const long long slots = pl->num_sms / cg;
       long long ks_lo = 1, ks_hi = 1;
@@ -1031,7 +1064,7 @@ static Variant pick_variant(const UmmaPlan* pl, int m_units, int N, bool dims_ch
         const long long per = (k_len + ks - 1) / ks;
         const long long n_ranges = (k_len + per - 1) / per;          // ranges that exist
         const long long waves = (tiles * n_ranges + slots - 1) / slots;
-        const long long cost = waves * (per * stage_kb + epi) + (ranged ? n_ranges * stage_kb * 3 / 8 : 0);
+        const long long cost = waves * ((per > EPI_STAGES ? per : EPI_STAGES) * stage_kb + epi) + (ranged ? n_ranges * stage_kb * 3 / 8 : 0);
         if (best_cost < 0 || cost < best_cost) {
           best_cost = cost;
           v.bn = bn; v.cg = cg;
