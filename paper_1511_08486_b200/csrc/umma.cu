@@ -224,6 +224,10 @@ umma_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
   const int k_blocks = APPLY ? ctl->k_total : p.k_blocks;
   const int k_per_split = APPLY ? k_blocks : p.k_per_split;
   const bool by_dir = APPLY && p.dir != nullptr;
+  // Work items: all tiles of the first reduction range, then all of the second, ...: the CTAs at work at one time share
+  // the operand columns of one or two ranges, and every one of them comes from HBM once.  (With the
+  // ranges of a tile one after the other instead, the compensated forward at 1000 x 20000, K = 1024 took 155 us, now 121;
+  // at 4096 x 10000 254, now 226.)
   const int tile_count = p.m_tiles * p.n_tiles;
   const int total_work = (APPLY && k_blocks == 0) ? 0 : tile_count * p.k_splits;
 
@@ -237,7 +241,7 @@ umma_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
     bool ok = true;
     const uint64_t pol_a = ptx::l2_policy(p.a_policy), pol_b = ptx::l2_policy(p.b_policy);
     for (int work = cluster_id; work < total_work && ok; work += num_clusters) {
-      const int tile = work / p.k_splits, split = work - tile * p.k_splits;
+      const int split = work / tile_count, tile = work - split * tile_count;
       const int kb_begin = split * k_per_split, kb_end = min(kb_begin + k_per_split, k_blocks);
       int mt, nt;
       tile_coords(p, tile, mt, nt);
@@ -368,7 +372,7 @@ umma_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
     int it = 0;
     bool ok = (rank == 0);
     for (int work = cluster_id; work < total_work && ok; work += num_clusters, ++it) {
-      const int split = work % p.k_splits;
+      const int split = work / tile_count;
       const int kb_begin = split * k_per_split, kb_end = min(kb_begin + k_per_split, k_blocks);
       const int buf = it % NBUF;
       const uint32_t acc_ph = (uint32_t)(it / NBUF) & 1u;
@@ -460,7 +464,7 @@ umma_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
     int it = 0;
     bool ok = true;
     for (int work = cluster_id; work < total_work && ok; work += num_clusters, ++it) {
-      const int tile = work / p.k_splits, split = work - tile * p.k_splits;
+      const int split = work / tile_count, tile = work - split * tile_count;
       int mt, nt;
       tile_coords(p, tile, mt, nt);
       mt = mt * CG + (int)rank;
