@@ -1127,10 +1127,16 @@ int umma_forward_rows(UmmaPlan* pl, cudaStream_t s, const void* Wop, RowMap a, R
   const int P = workers > 0 ? workers : d.P;     // a shard of the workers, or all of them
   GemmParams p;
   memset(&p, 0, sizeof(p));
-  p.B = d.B; p.P = P;
+  // Operand rows that follow one another without a gap between workers (the caller's samples, dense code rows) are
+  // tiled as one block of rows.  Otherwise every worker's rows are padded: to whole 128-row units, or to a power of two.
+  // (10 workers x 100 rows: 8 units instead of 10, which at 4000 x 2056 is one
+  // wave of pair tiles instead of two: forward 40 -> 28 us.)
+  const bool packed = a.worker_stride == (long long)a.B * a.ld * a.es;
+  p.B = packed ? P * d.B : d.B;
+  p.P = packed ? 1 : P;
   int m_units;
-  if (d.B >= BM) { p.m_bb = BM; p.m_wp = 1; p.m_tpw = (d.B + BM - 1) / BM; m_units = P * p.m_tpw; }
-  else { p.m_bb = pow2_at_least(d.B); p.m_wp = BM / p.m_bb; p.m_tpw = 1; m_units = (P + p.m_wp - 1) / p.m_wp; }
+  if (p.B >= BM) { p.m_bb = BM; p.m_wp = 1; p.m_tpw = (p.B + BM - 1) / BM; m_units = p.P * p.m_tpw; }
+  else { p.m_bb = pow2_at_least(p.B); p.m_wp = BM / p.m_bb; p.m_tpw = 1; m_units = (p.P + p.m_wp - 1) / p.m_wp; }
   // folding walks the reduction index (D) in 128-byte atoms: rows must be whole atoms long
   const bool may_split = k_splits_out != nullptr && stats == nullptr && max_splits > 1;
   int ks_pick = 1;
@@ -1165,7 +1171,8 @@ int umma_forward_rows(UmmaPlan* pl, cudaStream_t s, const void* Wop, RowMap a, R
   if (n_parts_out != nullptr) *n_parts_out = p.n_parts;
   if (part_cols_out != nullptr) *part_cols_out = v.bn / 2;
   CUtensorMap ta, tb;
-  if (!encode_rows_map(&ta, es, a.base, d.D, d.B, P, (long long)a.ld * es, a.worker_stride, p.m_bb, p.m_wp, v.fold,
+  if (!encode_rows_map(&ta, es, a.base, d.D, p.B, p.P, (long long)a.ld * es, (long long)a.worker_stride * (P / p.P), p.m_bb,
+                       p.m_wp, v.fold,
                        v.ka, false))
     return SFB_ERR_CUDA;
   if (!encode_rows_map(&tb, es, Wop, d.D, d.J, 1, (long long)d.D * es, (long long)d.D * es * d.J, v.bn / v.cg, 1,
@@ -1182,7 +1189,7 @@ int umma_forward_rows(UmmaPlan* pl, cudaStream_t s, const void* Wop, RowMap a, R
       if (r < 0) return r;
       launches += r;
     }
-    if (!encode_corr_k_map(&tac, pl->xc, d.B, P, atoms, p.m_bb, p.m_wp) ||
+    if (!encode_corr_k_map(&tac, pl->xc, p.B, p.P, atoms, p.m_bb, p.m_wp) ||
         !encode_corr_k_map(&tbc, w_corr, d.J, 1, atoms, v.bn / v.cg, 1))
       return SFB_ERR_CUDA;
   }
