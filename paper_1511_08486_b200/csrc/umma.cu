@@ -866,7 +866,7 @@ bool encode_corr_mn_map(CUtensorMap* m, const void* base, long long ldc, long lo
 
 }  // namespace
 
-constexpr int MAX_SPLITS = 8;   // ranges a forward reduction may be cut into (partial buffers of the plan)
+constexpr int MAX_SPLITS = 16;   // ranges a forward reduction may be cut into (partial buffers of the plan)
 constexpr int X3_MAX_SPLITS = 32;   // ... on the compensated path, where the count is also tuned to fill whole waves
 
 struct UmmaPlan {
@@ -1027,7 +1027,7 @@ void umma_plan_destroy(UmmaPlan* p) {
 // max_splits > 1: the caller can take partial products, so a problem with few tiles may cut its reduction
 // (k_atoms 128-byte atoms long) into *splits ranges.  CTA pairs on 256 x 256 tiles need half the operand
 // traffic per flop of single 128 x 128 tiles, so they are preferred as soon as pairs x ranges fill the SMs.
-static Variant pick_variant(const UmmaPlan* pl, int m_units, int N, bool dims_chunk_aligned, int k_atoms = 0,
+static Variant pick_variant(const UmmaPlan* pl, int m_units, int N, bool dims_chunk_aligned, bool apply, int k_atoms,
                             int max_splits = 1, int* splits = nullptr) {
   Variant v;
   v.split = false;
@@ -1086,31 +1086,34 @@ static Variant pick_variant(const UmmaPlan* pl, int m_units, int N, bool dims_ch
     v.fold = v.cg == 2 && dims_chunk_aligned;
     return v;
   }
-  v.bn = (N > 128 && (long long)m_units * ((N + 255) / 256) >= pl->num_sms) ? 256 : 128;
-  // CTA pairs (256-row tiles) once there is enough work to fill the machine with them
-  v.cg = (v.bn == 256 && (long long)((m_units + 1) / 2) * ((N + 255) / 256) >= pl->num_sms / 2) ? 2 : 1;
-  if (v.cg == 1 && k_atoms > 0) {
-    const int k_blocks = (k_atoms + STAGE_ATOMS - 1) / STAGE_ATOMS;
-    auto ranges = [&](long long tiles, int slots) {
-      long long ks = slots / (tiles > 0 ? tiles : 1);
-      if (ks > max_splits) ks = max_splits;
-      while (ks > 1 && k_blocks < 16 * ks) --ks;
-      return (int)(ks < 1 ? 1 : ks);
-    };
-    const long long t_pair = (long long)((m_units + 1) / 2) * ((N + 255) / 256);
-    const int ks_pair = ranges(t_pair, pl->num_sms / 2);
-    const long long t_one = (long long)m_units * ((N + 127) / 128);
-    const int ks_one = ranges(t_one, pl->num_sms);
-    // pairs that fill three quarters of the machine beat single tiles that fill all of it: the single
-    // 128 x 128 tiles are bound by the operand feed (about 50 % tensor-pipe activity with fp32 operands)
-    if (N > 128 && m_units >= 2 && 4 * t_pair * ks_pair >= 3 * (pl->num_sms / 2)) {
-      v.bn = 256; v.cg = 2;
-      if (splits != nullptr) *splits = ks_pair;
-    } else if (t_one < pl->num_sms && splits != nullptr && max_splits > 1) {
-      v.bn = 128; v.cg = 1;
-      *splits = ks_one;
+  // tf32 and bf16 kernels: the candidate with the least estimated clocks of its busiest SM.
+  //   An atom (128 bytes of every operand row) takes 2 clocks of the tensor pipe per tile column, or its bytes at
+  //   50 a clock and SM, whichever is longer: 655 for 256 x 256 pair tiles and for 128 x 128 single ones, which hold a
+  //   quarter of the work (1024 x 4608, K = 4096, tf32: 62 against 83 us, although only 72 pairs have work).
+  //   A tile's epilogue takes about 48 clocks per column (32 without the write-back of W) beside the next tile's atoms;
+  //   the last one, the launch and the pipeline's first loads are on top.
+  //   Ranges of a forward reduction: their partial products go out and come back at 3400 bytes a clock.
+  v.bn = 128; v.cg = 1;
+  double best = -1;
+  auto consider = [&](int bn, int cg) {
+    const double mma = 2.0 * bn, load = (BM + bn / cg) * 128.0 / 50;
+    const double t_atom = mma > load ? mma : load, epi = bn * (apply ? 48.0 : 32.0);
+    const long long tiles = (long long)((m_units + cg - 1) / cg) * ((N + bn - 1) / bn), slots = pl->num_sms / cg;
+    for (int ks = 1; ks <= max_splits && (ks == 1 || k_atoms >= 2 * STAGE_ATOMS * ks); ++ks) {
+      const int per = (k_atoms + ks - 1) / ks, ranges = (k_atoms + per - 1) / per;
+      const double waves = (double)((tiles * ranges + slots - 1) / slots), work = per * t_atom;
+      const double cost = waves * (work > epi ? work : epi) + epi + 8000.0 +
+                          (ks > 1 ? (double)ranges * m_units * BM * N * 8 / 3400 : 0.0);
+      if (best < 0 || cost < best) {
+        best = cost;
+        v.bn = bn; v.cg = cg;
+        if (splits != nullptr) *splits = ks;
+      }
     }
-  }
+  };
+  consider(128, 1);
+  if (N > 128) consider(256, 1);
+  if (N > 128 && m_units >= 2) consider(256, 2);
   v.fold = v.cg == 2 && dims_chunk_aligned;
   // two 128-byte atoms of reduction per stage wherever three such stages fit in shared memory: the
   // per-stage barrier round trip, not the number of TMA instructions, is what costs
@@ -1140,7 +1143,7 @@ int umma_forward_rows(UmmaPlan* pl, cudaStream_t s, const void* Wop, RowMap a, R
   // folding walks the reduction index (D) in 128-byte atoms: rows must be whole atoms long
   const bool may_split = k_splits_out != nullptr && stats == nullptr && max_splits > 1;
   int ks_pick = 1;
-  const Variant v = pick_variant(pl, m_units, d.J, (d.D % CH) == 0 && (a.ld % CH) == 0, (d.D + CH - 1) / CH,
+  const Variant v = pick_variant(pl, m_units, d.J, (d.D % CH) == 0 && (a.ld % CH) == 0, false, (d.D + CH - 1) / CH,
                                  may_split ? (max_splits < pl->max_splits ? max_splits : pl->max_splits) : 1, &ks_pick);
   p.m_tiles = (m_units + v.cg - 1) / v.cg;
   p.n_tiles = (d.J + v.bn - 1) / v.bn;
@@ -1431,7 +1434,7 @@ static int umma_apply_range(UmmaPlan* pl, cudaStream_t s, void* W, __nv_bfloat16
   // stream (the next row, or the stream's V block: always inside the buffer), which only feeds accumulator rows
   // j >= J, and those are never written.  (The V block of the last stream ends the buffer, hence no such
   // licence for D.)
-  const Variant v = pick_variant(pl, m_units, d.D, (d.D % CH) == 0, pl->x3 ? (K + 31) / 32 : 0);
+  const Variant v = pick_variant(pl, m_units, d.D, (d.D % CH) == 0, true, (K + CH - 1) / CH);
   const int BK = CH * v.ka;
   if (d.B >= BK) { p.k_bb = BK; p.k_wp = 1; p.k_bpw = (d.B + BK - 1) / BK; p.k_blocks = workers * p.k_bpw; }
   else { p.k_bb = pow2_at_least(d.B); p.k_wp = BK / p.k_bb; p.k_bpw = 1; p.k_blocks = (workers + p.k_wp - 1) / p.k_wp; }
