@@ -1281,8 +1281,16 @@ int umma_forward(UmmaPlan* pl, cudaStream_t s, const void* W, const __nv_bfloat1
     bool forked = false;
     // a small v goes out beside the finishing pass, a large one beside the GEMM
     const bool v_inline = v.base != nullptr && (long long)K * v.ld * v.es <= V_INLINE_BYTES;
-    if (v_inline) { extra.src = x_rows; extra.dst = v; extra.cols = d.D; extra.corr = cv; }
-    if (v.base != nullptr && !v_inline && pl->side_ok) {   // v = x on the side stream, joined before this call returns its work
+    // compensated path: one pass over the samples writes v and both correction operands of them
+    const bool v_first = pl->x3 && v.base != nullptr;
+    if (v_first) {
+      cv.km = reinterpret_cast<char*>(pl->xc);
+      cv.atoms = (d.D + 31) / 32;
+      if ((r = launch_copy_rows(s, x_rows, v, K, d.D, cv)) < 0) return r;
+      launches += r;
+    }
+    if (v_inline && !v_first) { extra.src = x_rows; extra.dst = v; extra.cols = d.D; extra.corr = cv; }
+    if (v.base != nullptr && !v_inline && !v_first && pl->side_ok) {   // v = x on the side stream, joined before this call returns its work
       if (cudaEventRecord(pl->fork, s) != cudaSuccess || cudaStreamWaitEvent(pl->side, pl->fork, 0) != cudaSuccess)
         return SFB_ERR_CUDA;
       forked = true;
@@ -1310,7 +1318,7 @@ int umma_forward(UmmaPlan* pl, cudaStream_t s, const void* W, const __nv_bfloat1
         const long long sstride = (long long)d.P * d.B * pl->ldp * 4;
         int ks = 1;
         if ((r = umma_forward_rows(pl, s, bf16 ? (const void*)w_shadow : W, x_rows, pz, dev_status, nullptr, nullptr,
-                                   nullptr, &ks, pl->max_splits, sstride, workers, pl->x3 ? w_shadow : nullptr)) < 0)
+                                   nullptr, &ks, pl->max_splits, sstride, workers, pl->x3 ? w_shadow : nullptr, v_first)) < 0)
           return r;
         launches += r;
         if ((r = launch_finish_mlr(s, pz, u, aux->labels, K, d.J, dev_status, ks, sstride, reinterpret_cast<float*>(aux->dual),
@@ -1329,7 +1337,7 @@ int umma_forward(UmmaPlan* pl, cudaStream_t s, const void* W, const __nv_bfloat1
           return r;
         launches += r;
       }
-      if (!forked && !v_inline && v.base != nullptr) {
+      if (!forked && !v_inline && !v_first && v.base != nullptr) {
         if ((r = launch_copy_rows(s, x_rows, v, K, d.D, cv)) < 0) return r;
         launches += r;
       }
