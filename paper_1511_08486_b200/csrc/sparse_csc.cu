@@ -3,18 +3,18 @@
 //   W[:, d] -= eta * sum_{i : a_id != 0} a_id * u_i        (Section 3 update with v_i = a_i sparse)
 //
 // The codes arrive sample-major (CSR, the factor v_i of each sample).  Per step they are re-sorted by
-// atom with a counting sort that is deterministic: counts per (chunk of 8 samples, atom) by integer
+// (slice of samples, atom) with a counting sort that is deterministic: counts per (chunk of 8 samples, atom) by integer
 // atomics, prefix sums over chunks and atoms, then every chunk places its samples one after the other,
-// so inside a column the entries are in sample order whatever the thread schedule.
-// The apply gives each thread block 64 rows of W and keeps the matching 64 columns of a slice of the
-// u_i in shared memory (the samples are taken in as few slices as fit).  A warp takes 16 consecutive
-// atoms: for each atom it walks the slice's entries of the column (coalesced loads staged through a
-// small per-warp strip), accumulating a_id * u_i[j0 + 2 lane .. + 1] from shared memory, parks the sums
-// in a private 16 x 65 tile, and finally updates W with 64-byte row segments.
+// so inside a column the entries are in sample order whatever the thread schedule.  Every column of a slice is padded
+// with zero entries to a multiple of four, so that a warp reads the entries of consecutive atoms as one stream of groups
+// of four.
+// The apply gives each thread block 64 rows of W at a time and keeps the matching 64 columns of a slice of the
+// u_i in shared memory (the samples are taken in as few slices as fit).  A warp takes 8 consecutive
+// atoms: it starts the loads of its part of W, walks the atoms' entries (coalesced loads staged through a
+// small per-warp strip), accumulating a_id * u_i[j0 + 4 q .. + 3] from shared memory, parks the sums
+// in a private 8 x 68 tile, and finally updates W with 32-byte row segments.
 // U is read once and W once per slice; no floating-point atomics; every element of W has one owner and a fixed
 // summation order (bit-reproducible); atoms nobody uses get W + (-eta * 0) = W, bit-identical.
-#include <type_traits>
-
 #include "common.cuh"
 
 namespace sfb {
@@ -70,39 +70,45 @@ __global__ void __launch_bounds__(256) csc_count_kernel(CsrView codes, int K, in
   if (bad && dev_status != nullptr) atomicOr(dev_status, SFB_DEV_BAD_INDEX);
 }
 
-// per atom: counts per chunk -> offsets of each chunk inside the column; column totals
-__global__ void __launch_bounds__(256) csc_chunk_offsets_kernel(int nchunks, int D, int* __restrict__ cnt,
+// per atom: counts per chunk -> offsets of each chunk inside the column's slice; slice totals, rounded up to fours
+__global__ void __launch_bounds__(256) csc_chunk_offsets_kernel(int nchunks, int chunks_per_slice, int D, int* __restrict__ cnt,
                                                                 int* __restrict__ total) {
   const int d = blockIdx.x * 256 + threadIdx.x;
   if (d >= D) return;
-  int run = 0;
+  int run = 0, slice = 0, left = chunks_per_slice;
   for (int c0 = 0; c0 < nchunks; c0 += 8) {   // eight independent loads in flight, then the running sum
     int t[8];
 #pragma unroll
     for (int q = 0; q < 8; ++q) t[q] = (c0 + q < nchunks) ? cnt[(size_t)(c0 + q) * D + d] : 0;
 #pragma unroll
     for (int q = 0; q < 8; ++q) {
-      if (c0 + q < nchunks) cnt[(size_t)(c0 + q) * D + d] = run;
-      run += t[q];
+      if (c0 + q < nchunks) {
+        cnt[(size_t)(c0 + q) * D + d] = run;
+        run += t[q];
+        if (--left == 0) {
+          total[(size_t)slice * D + d] = (run + 3) & ~3;
+          run = 0; ++slice; left = chunks_per_slice;
+        }
+      }
     }
   }
-  total[d] = run;
+  if (left < chunks_per_slice) total[(size_t)slice * D + d] = (run + 3) & ~3;
 }
 
-// colptr = exclusive scan of total (one block, fixed order)
-__global__ void __launch_bounds__(1024) csc_scan_kernel(int D, const int* __restrict__ total, int* __restrict__ colptr) {
+// colptr[0 .. n] = exclusive scan of total[0 .. n) (one block, fixed order)
+__global__ void __launch_bounds__(1024) csc_scan_kernel(int n, const int* __restrict__ total, int* __restrict__ colptr) {
   __shared__ int warp_sum[32];
   __shared__ int carry;
   if (threadIdx.x == 0) carry = 0;
   __syncthreads();
-  for (int base = 0; base < D; base += 1024) {
+  for (int base = 0; base < n; base += 1024) {
     const int d = base + threadIdx.x;
-    const int v = d < D ? total[d] : 0;
+    const int v = d < n ? total[d] : 0;
     int incl = v;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
-      const int n = __shfl_up_sync(0xffffffffu, incl, o);
-      if ((threadIdx.x & 31) >= o) incl += n;
+      const int o_ = __shfl_up_sync(0xffffffffu, incl, o);
+      if ((threadIdx.x & 31) >= o) incl += o_;
     }
     if ((threadIdx.x & 31) == 31) warp_sum[threadIdx.x >> 5] = incl;
     __syncthreads();
@@ -110,27 +116,30 @@ __global__ void __launch_bounds__(1024) csc_scan_kernel(int D, const int* __rest
       int w = warp_sum[threadIdx.x];
 #pragma unroll
       for (int o = 1; o < 32; o <<= 1) {
-        const int n = __shfl_up_sync(0xffffffffu, w, o);
-        if (threadIdx.x >= o) w += n;
+        const int o_ = __shfl_up_sync(0xffffffffu, w, o);
+        if (threadIdx.x >= o) w += o_;
       }
       warp_sum[threadIdx.x] = w;
     }
     __syncthreads();
     const int before = carry + ((threadIdx.x >> 5) > 0 ? warp_sum[(threadIdx.x >> 5) - 1] : 0) + incl - v;
-    if (d < D) colptr[d] = before;
+    if (d < n) colptr[d] = before;
     __syncthreads();
     if (threadIdx.x == 1023) carry = before + v;
     __syncthreads();
   }
-  if (threadIdx.x == 0) colptr[D] = carry;
+  if (threadIdx.x == 0) colptr[n] = carry;
 }
 
 // one block per chunk: its samples are placed one after the other, so a column is in sample order
-__global__ void __launch_bounds__(256) csc_fill_kernel(CsrView codes, int K, int D, int* __restrict__ cnt,
-                                                       const int* __restrict__ colptr, int* __restrict__ ent_i,
-                                                       float* __restrict__ ent_a) {
+// (entry = sample index inside its slice, value)
+__global__ void __launch_bounds__(256) csc_fill_kernel(CsrView codes, int K, int D, int chunks_per_slice,
+                                                       int* __restrict__ cnt, const int* __restrict__ colptr,
+                                                       int2* __restrict__ ent) {
   const int c = blockIdx.x;
+  const int slice = c / chunks_per_slice, i_lo = slice * chunks_per_slice * CSC_CHUNK;
   int* off = cnt + (size_t)c * D;
+  const int* base = colptr + (size_t)slice * D;
   for (int s = 0; s < CSC_CHUNK; ++s) {
     const int i = c * CSC_CHUNK + s;
     if (i < K) {
@@ -138,10 +147,9 @@ __global__ void __launch_bounds__(256) csc_fill_kernel(CsrView codes, int K, int
       for (int k = threadIdx.x; k < row.len; k += 256) {
         if (entry_ok(row, k, D)) {  // indices that pass are unique inside a row: one writer per (chunk, atom) per step
           const uint32_t d = row.idx[k];
-          const int pos = colptr[d] + off[d];
-          off[d] += 1;
-          ent_i[pos] = i;
-          ent_a[pos] = row.val[k];
+          const int o = off[d];
+          off[d] = o + 1;
+          ent[base[d] + o] = make_int2(i - i_lo, __float_as_int(row.val[k]));
         }
       }
     }
@@ -149,130 +157,169 @@ __global__ void __launch_bounds__(256) csc_fill_kernel(CsrView codes, int K, int
   }
 }
 
-constexpr int CSC2_JT = 64;     // rows of W per block of the two-rows-per-lane apply
-constexpr int CSC2_AB = 16;     // atoms per warp block there
-constexpr int CSC2_WARP_FLOATS = 64 + CSC2_AB * 65;   // entry strip (32 x 8 bytes) + [16][65] tile
+constexpr int CSC2_JT = 64;     // rows of W per block, four per lane of a half warp
+constexpr int CSC2_AB = 8;      // atoms per warp block
+constexpr int CSC2_WARPS = 16;
+constexpr int CSC2_STRIP = 128; // entries a warp stages at a time
+constexpr int CSC2_TS = 68;     // row length of the tile: 4 atoms-worth of banks apart, rows 16-byte aligned
+constexpr int CSC2_WARP_FLOATS = 2 * CSC2_STRIP + CSC2_AB * CSC2_TS;   // entry strip + [8][68] tile
 
-// Two rows of W per lane, the samples taken in `passes` slices so that a slice of the u columns
-// (Kh x 256 bytes) fits in shared memory.  Shared-memory bandwidth bounds this kernel: per entry and 64 rows
-// it costs half a broadcast read of the strip (two entries per 16-byte load) and one 256-byte read of u.
-// grid = (ceil(J / 64), atom splits).  cnt holds, after the fill, for every (chunk, atom) the number of
-// entries of the column that belong to samples before the END of the chunk, which gives the slice bounds.
-__global__ void __launch_bounds__(512) csc_apply_kernel(float* __restrict__ W, RowMap u, int K, int J, int D, float eta,
-                                                         const int* __restrict__ colptr, const int* __restrict__ cnt,
-                                                         const int* __restrict__ ent_i, const float* __restrict__ ent_a,
-                                                         int passes, int Kh, const int* __restrict__ status_ro) {
+// The work is the list of (block of 64 rows, block of 8 atoms), rows outermost; every thread block takes an equal run
+// of it, so the SMs are loaded evenly whatever J is (a run rarely touches more than two blocks of rows).
+// A half warp takes every other entry: one 8-byte read of the strip (two addresses) and one 512-byte read of u per two
+// entries, five wavefronts of shared memory, which bounds this kernel.  (Two rows per lane and an entry at a time cost
+// three wavefronts per entry: a 16-byte broadcast read takes two.)
+// 4096 x 10000, K = 1024: 5 % density 742 -> 514 us an apply, 1 % 459 -> 304, against columns staged one by one in rounds
+// of 8, 16 or 32 entries on 64 x 2 blocks with 64-byte segments of W.
+__global__ void __launch_bounds__(CSC2_WARPS * 32) csc_apply_kernel(float* __restrict__ W, RowMap u, int K, int J, int D,
+                                                                    float eta, const int* __restrict__ colptr,
+                                                                    const int2* __restrict__ ent, int passes, int Kh,
+                                                                    const int* __restrict__ status_ro) {
   extern __shared__ __align__(16) float smem[];
   if (status_ro != nullptr && (*status_ro & SFB_DEV_BAD_HEADER)) return;
   float* Us = smem;                                   // [Kh][64]
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nwarps = blockDim.x >> 5;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   float* region = smem + (size_t)Kh * 64 + warp * CSC2_WARP_FLOATS;
   int2* strip = reinterpret_cast<int2*>(region);
-  const int4* strip4 = reinterpret_cast<const int4*>(region);
-  float* T = region + 64;
-  const int j0 = blockIdx.x * CSC2_JT;
-  const int jn = min(CSC2_JT, J - j0);
-  const int nnz = colptr[D];
-  const int nchunks = (K + CSC_CHUNK - 1) / CSC_CHUNK;
+  const int half = lane >> 4, q4 = (lane & 15) * 4;   // this lane's entries and rows
+  float* T = region + 2 * CSC2_STRIP;
   const int nblocks = (D + CSC2_AB - 1) / CSC2_AB;
-  for (int h = 0; h < passes; ++h) {
-    const int i_lo = h * Kh;
-    if (i_lo >= K) break;
-    const int i_n = min(Kh, K - i_lo);
-    __syncthreads();                                  // the previous slice is no longer read
-    for (int i = warp; i < i_n; i += nwarps) {
-      const float* ur = reinterpret_cast<const float*>(u.row(i_lo + i)) + j0;
-      float2 v = make_float2(0.f, 0.f);
-      if (2 * lane + 1 < jn) v = *reinterpret_cast<const float2*>(ur + 2 * lane);
-      else if (2 * lane < jn) v.x = ur[2 * lane];
-      *reinterpret_cast<float2*>(Us + i * 64 + 2 * lane) = v;
-    }
-    __syncthreads();
-    const int c_lo = i_lo / CSC_CHUNK;                               // Kh is a multiple of the chunk size
-    const int c_hi = min(nchunks, (i_lo + Kh) / CSC_CHUNK);
-    for (int ab = blockIdx.y + gridDim.y * warp; ab < nblocks; ab += gridDim.y * nwarps) {
-      const int d0 = ab * CSC2_AB;
-      const int dn = min(CSC2_AB, D - d0);
-      int lo = nnz, hi = nnz;                                        // entry range of atom d0 + lane in this slice
-      if (lane < dn) {
-        const int d = d0 + lane, cp = colptr[d];
-        lo = (c_lo == 0) ? cp : cp + cnt[(size_t)(c_lo - 1) * D + d];
-        hi = cp + cnt[(size_t)(c_hi - 1) * D + d];
+  const long long work = (long long)((J + CSC2_JT - 1) / CSC2_JT) * nblocks;
+  const long long w_lo = work * blockIdx.x / gridDim.x, w_hi = work * (blockIdx.x + 1) / gridDim.x;
+  const int n_ent = colptr[(size_t)passes * D];       // padded entries of all slices
+  for (long long w0 = w_lo; w0 < w_hi;) {
+    const int jb = (int)(w0 / nblocks), ab_lo = (int)(w0 - (long long)jb * nblocks);
+    const int ab_hi = (int)min((long long)nblocks, ab_lo + (w_hi - w0));
+    w0 += ab_hi - ab_lo;
+    const int j0 = jb * CSC2_JT;
+    const int jn = min(CSC2_JT, J - j0);
+    for (int h = 0; h < passes; ++h) {
+      const int i_lo = h * Kh;
+      const int i_n = min(Kh, K - i_lo);
+      __syncthreads();                                  // the previous slice is no longer read
+      // 16-byte asynchronous copies, all in flight together; rows of u are padded to 16 bytes
+      for (int t = threadIdx.x; t < i_n * 16; t += CSC2_WARPS * 32) {
+        const int i = t >> 4, c = (t & 15) * 4;
+        const uint32_t dst = (uint32_t)__cvta_generic_to_shared(Us + i * 64 + c);
+        const bool in = c < jn;
+        const char* src = u.row(i_lo + i) + (in ? (size_t)(j0 + c) * 4 : 0);
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(in ? 16 : 0) : "memory");
       }
-      int pre_i = 0;
-      float pre_a = 0.f;
-      {
-        const int b0 = __shfl_sync(0xffffffffu, lo, 0);
-        if (b0 + lane < nnz) { pre_i = ent_i[b0 + lane]; pre_a = ent_a[b0 + lane]; }
-      }
-      for (int dd = 0; dd < dn; ++dd) {
-        const int beg = __shfl_sync(0xffffffffu, lo, dd);
-        const int stop = __shfl_sync(0xffffffffu, hi, dd);
-        const int next_beg = __shfl_sync(0xffffffffu, lo, dd + 1);   // lane 16 and up hold nnz: nothing to fetch
-        float2 acc0 = make_float2(0.f, 0.f), acc1 = acc0, acc2 = acc0, acc3 = acc0;
-        if (beg >= stop && next_beg + lane < nnz) { pre_i = ent_i[next_beg + lane]; pre_a = ent_a[next_beg + lane]; }
-        for (int base = beg; base < stop; base += 32) {
-          const bool ok = base + lane < stop;
-          // the sample index addresses shared memory: keep it inside the slice whatever the entry arrays hold
-          const int li = min(max(pre_i - i_lo, 0), i_n - 1);
-          strip[lane] = make_int2(ok ? li : 0, __float_as_int(ok ? pre_a : 0.f));
-          const int nxt = (base + 32 < stop) ? base + 32 : next_beg;
-          if (nxt + lane < nnz) { pre_i = ent_i[nxt + lane]; pre_a = ent_a[nxt + lane]; }
-          __syncwarp();
-          // a round holds up to 32 entries; short columns (sparse codes) take the 8- or 16-entry body, so the time of
-          // a column follows its entries, not the round size (the bodies are unrolled: no branch inside them)
-          const int n_here = min(32, stop - base);     // warp-uniform
-          auto body = [&](auto iters) {
+      asm volatile("cp.async.wait_all;" ::: "memory");
+      __syncthreads();
+      // entries of the warp's next block, on their way while the current one is summed
+      constexpr int PRE = CSC2_STRIP / 32;
+      int2 pre[PRE];
+      auto fetch = [&](int from) {
 #pragma unroll
-            for (int k = 0; k < decltype(iters)::value; k += 2) {
-              const int4 p = strip4[k], q = strip4[k + 1];
-              const float2 u0 = *reinterpret_cast<const float2*>(Us + p.x * 64 + 2 * lane);
-              const float2 u1 = *reinterpret_cast<const float2*>(Us + p.z * 64 + 2 * lane);
-              const float2 u2 = *reinterpret_cast<const float2*>(Us + q.x * 64 + 2 * lane);
-              const float2 u3 = *reinterpret_cast<const float2*>(Us + q.z * 64 + 2 * lane);
-              acc0.x = fmaf(__int_as_float(p.y), u0.x, acc0.x); acc0.y = fmaf(__int_as_float(p.y), u0.y, acc0.y);
-              acc1.x = fmaf(__int_as_float(p.w), u1.x, acc1.x); acc1.y = fmaf(__int_as_float(p.w), u1.y, acc1.y);
-              acc2.x = fmaf(__int_as_float(q.y), u2.x, acc2.x); acc2.y = fmaf(__int_as_float(q.y), u2.y, acc2.y);
-              acc3.x = fmaf(__int_as_float(q.w), u3.x, acc3.x); acc3.y = fmaf(__int_as_float(q.w), u3.y, acc3.y);
-            }
-          };
-          if (n_here <= 8) body(std::integral_constant<int, 4>());
-          else if (n_here <= 16) body(std::integral_constant<int, 8>());
-          else body(std::integral_constant<int, 16>());
-          __syncwarp();
+        for (int t = 0; t < PRE; ++t) {
+          const int e = from + 32 * t + lane;
+          pre[t] = e < n_ent ? ent[e] : make_int2(0, 0);
         }
-        T[dd * 65 + 2 * lane] = (acc0.x + acc1.x) + (acc2.x + acc3.x);
-        T[dd * 65 + 2 * lane + 1] = (acc0.y + acc1.y) + (acc2.y + acc3.y);
-      }
-      __syncwarp();
-      // W[j0 + jj][d0 + a] -= eta * T[a][jj]: a warp instruction covers two rows x 16 atoms (64-byte segments)
-      const int a = lane & 15, q = lane >> 4;
-      if (a < dn) {
-        for (int jb = 0; jb < jn; jb += 16) {
-          float wv[8];
+      };
+      // first entry of the atoms of a block: lane a has atom a's, lanes behind the last atom the end of its column
+      const int* cols = colptr + (size_t)h * D;
+      auto starts = [&](int ab) { return ab < ab_hi ? cols[ab * CSC2_AB + min(lane, min(CSC2_AB, D - ab * CSC2_AB))] : n_ent; };
+      int beg_next = starts(ab_lo + warp);
+      fetch(__shfl_sync(0xffffffffu, beg_next, 0));
+      // the warp's part of W of a block: lane = atom lane % 8, rows lane / 8 + 4 t
+      const int wa = lane & (CSC2_AB - 1), wq = lane / CSC2_AB;
+      for (int ab = ab_lo + warp; ab < ab_hi; ab += CSC2_WARPS) {
+        const int d0 = ab * CSC2_AB;
+        const int dn = min(CSC2_AB, D - d0);
+        const int beg = beg_next;
+        beg_next = starts(ab + CSC2_WARPS);
+        int pos = __shfl_sync(0xffffffffu, beg, 0);
+        const int end = __shfl_sync(0xffffffffu, beg, dn);
+        int strip_lo = pos, strip_hi = pos;             // entries in the strip: [strip_lo, strip_hi)
+        auto refill = [&]() {
+          __syncwarp();
+          // the sample index addresses shared memory: keep it inside the slice whatever the entries hold
 #pragma unroll
-          for (int t = 0; t < 8; ++t) {
-            const int jj = jb + 2 * t + q;
-            wv[t] = (jj < jn) ? W[(size_t)(j0 + jj) * D + d0 + a] : 0.f;
+          for (int t = 0; t < PRE; ++t) strip[32 * t + lane] = make_int2(min(max(pre[t].x, 0), i_n - 1), pre[t].y);
+          strip_lo = pos;
+          strip_hi = pos + CSC2_STRIP;
+          const int nxt = __shfl_sync(0xffffffffu, beg_next, 0);
+          fetch(strip_hi < end ? strip_hi : nxt);
+          __syncwarp();
+        };
+        refill();
+        // W is on its way while the entries are summed
+        float wv[CSC2_JT / 4];
+#pragma unroll
+        for (int t = 0; t < CSC2_JT / 4; ++t) {
+          const int jj = 4 * t + wq;
+          wv[t] = (wa < dn && jj < jn) ? W[(size_t)(j0 + jj) * D + d0 + wa] : 0.f;
+        }
+        for (int dd = 0; dd < dn; ++dd) {
+          const int stop = __shfl_sync(0xffffffffu, beg, dd + 1);
+          float4 acc0 = make_float4(0.f, 0.f, 0.f, 0.f), acc1 = acc0;
+          while (pos < stop) {
+            if (pos == strip_hi) refill();              // (warp-uniform)
+            auto four = [&](int k) {
+              const int2 p = strip[k + half], q = strip[k + 2 + half];
+              const float4 u0 = *reinterpret_cast<const float4*>(Us + p.x * 64 + q4);
+              const float4 u1 = *reinterpret_cast<const float4*>(Us + q.x * 64 + q4);
+              const float a0 = __int_as_float(p.y), a1 = __int_as_float(q.y);
+              acc0.x = fmaf(a0, u0.x, acc0.x); acc0.y = fmaf(a0, u0.y, acc0.y);
+              acc0.z = fmaf(a0, u0.z, acc0.z); acc0.w = fmaf(a0, u0.w, acc0.w);
+              acc1.x = fmaf(a1, u1.x, acc1.x); acc1.y = fmaf(a1, u1.y, acc1.y);
+              acc1.z = fmaf(a1, u1.z, acc1.z); acc1.w = fmaf(a1, u1.w, acc1.w);
+            };
+            const int to = min(stop, strip_hi);         // groups of four never straddle a column or the strip
+            int k = pos - strip_lo;
+            const int k_end = to - strip_lo;
+            for (; k + 8 <= k_end; k += 8) { four(k); four(k + 4); }
+            if (k < k_end) four(k);
+            pos = to;
           }
+          acc0.x += acc1.x; acc0.y += acc1.y; acc0.z += acc1.z; acc0.w += acc1.w;
+          acc0.x += __shfl_xor_sync(0xffffffffu, acc0.x, 16); acc0.y += __shfl_xor_sync(0xffffffffu, acc0.y, 16);
+          acc0.z += __shfl_xor_sync(0xffffffffu, acc0.z, 16); acc0.w += __shfl_xor_sync(0xffffffffu, acc0.w, 16);
+          if (half == 0) *reinterpret_cast<float4*>(T + dd * CSC2_TS + q4) = acc0;
+        }
+        __syncwarp();
+        // W[j0 + jj][d0 + wa] -= eta * T[wa][jj]: a warp instruction covers four rows x 8 atoms (32-byte segments)
+        if (wa < dn) {
 #pragma unroll
-          for (int t = 0; t < 8; ++t) {
-            const int jj = jb + 2 * t + q;
-            if (jj < jn) W[(size_t)(j0 + jj) * D + d0 + a] = fmaf(-eta, T[a * 65 + jj], wv[t]);
+          for (int t = 0; t < CSC2_JT / 4; ++t) {
+            const int jj = 4 * t + wq;
+            if (jj < jn) W[(size_t)(j0 + jj) * D + d0 + wa] = fmaf(-eta, T[wa * CSC2_TS + jj], wv[t]);
           }
         }
+        __syncwarp();
       }
-      __syncwarp();
     }
   }
+}
+
+// Slices of the samples: the fewest that let Kh x 256 bytes of u sit beside the warps' tiles.
+struct CscSlices {
+  int passes, Kh;
+};
+CscSlices csc_slices(int K) {
+  const int tiles = CSC2_WARPS * CSC2_WARP_FLOATS * 4;
+  const int kh_max = (220 * 1024 - tiles) / 256 / CSC_CHUNK * CSC_CHUNK;
+  CscSlices s;
+  s.passes = (K + kh_max - 1) / kh_max;
+  s.Kh = ((K + s.passes - 1) / s.passes + CSC_CHUNK - 1) / CSC_CHUNK * CSC_CHUNK;
+  s.passes = (K + s.Kh - 1) / s.Kh;
+  return s;
 }
 
 }  // namespace
 
-// Scratch of the CSC path: counts [nchunks][D] + totals [D] + colptr [D + 1] ints, entries (int + float) x nnz_capacity.
-long long sc_csc_workspace_bytes(int K, int D, long long nnz_capacity) {
+// Scratch of the CSC path: counts [nchunks][D], totals and column starts [slices][D] ints, entries x (nnz_capacity + padding).
+static long long csc_entries(int K, int D, long long nnz_capacity) {
+  return nnz_capacity + 3LL * csc_slices(K).passes * D;
+}
+static long long csc_ints(int K, int D) {
   const long long nchunks = (K + CSC_CHUNK - 1) / CSC_CHUNK;
-  return pad_to((nchunks * D + D + D + 1) * 4, 256) + pad_to(nnz_capacity * 4, 256) * 2;
+  return nchunks * D + 2LL * csc_slices(K).passes * D + 1;
+}
+long long sc_csc_workspace_bytes(int K, int D, long long nnz_capacity) {
+  // (a step over the first workers' samples only takes fewer slices of another length: no more entries or ints)
+  return pad_to(csc_ints(K, D) * 4, 256) + pad_to(csc_entries(K, D, nnz_capacity) * 8, 256);
 }
 
 // The sliced kernel takes any K (more slices); the bound only keeps the chunk tables small.
@@ -280,17 +327,15 @@ bool sc_csc_supported(int K) { return K <= (1 << 14); }
 
 namespace {
 struct CscScratch {
-  int* cnt; int* total; int* colptr; int* ent_i; float* ent_a;
+  int* cnt; int* total; int* colptr; int2* ent;
 };
-CscScratch csc_scratch(void* workspace, int K, int D, long long nnz_capacity) {
-  const int nchunks = (K + CSC_CHUNK - 1) / CSC_CHUNK;
+CscScratch csc_scratch(void* workspace, int K, int D) {
+  const int nchunks = (K + CSC_CHUNK - 1) / CSC_CHUNK, passes = csc_slices(K).passes;
   CscScratch w;
   w.cnt = reinterpret_cast<int*>(workspace);
   w.total = w.cnt + (size_t)nchunks * D;
-  w.colptr = w.total + D;
-  char* ent_base = reinterpret_cast<char*>(workspace) + pad_to(((long long)nchunks * D + D + D + 1) * 4, 256);
-  w.ent_i = reinterpret_cast<int*>(ent_base);
-  w.ent_a = reinterpret_cast<float*>(ent_base + pad_to(nnz_capacity * 4, 256));
+  w.colptr = w.total + (size_t)passes * D;
+  w.ent = reinterpret_cast<int2*>(reinterpret_cast<char*>(workspace) + pad_to(csc_ints(K, D) * 4, 256));
   return w;
 }
 }  // namespace
@@ -300,36 +345,31 @@ CscScratch csc_scratch(void* workspace, int K, int D, long long nnz_capacity) {
 int launch_sc_csc_build(cudaStream_t s, CsrView codes, int K, int D, long long nnz_capacity, void* workspace,
                         int* dev_status) {
   const int nchunks = (K + CSC_CHUNK - 1) / CSC_CHUNK;
-  const CscScratch w = csc_scratch(workspace, K, D, nnz_capacity);
+  const CscSlices sl = csc_slices(K);
+  const CscScratch w = csc_scratch(workspace, K, D);
   if (cudaMemsetAsync(w.cnt, 0, (size_t)nchunks * D * 4, s) != cudaSuccess) return SFB_ERR_CUDA;
+  if (cudaMemsetAsync(w.ent, 0, (size_t)csc_entries(K, D, nnz_capacity) * 8, s) != cudaSuccess) return SFB_ERR_CUDA;
   csc_count_kernel<<<K, 256, 0, s>>>(codes, K, D, w.cnt, dev_status);
-  csc_chunk_offsets_kernel<<<(D + 255) / 256, 256, 0, s>>>(nchunks, D, w.cnt, w.total);
-  csc_scan_kernel<<<1, 1024, 0, s>>>(D, w.total, w.colptr);
-  csc_fill_kernel<<<nchunks, 256, 0, s>>>(codes, K, D, w.cnt, w.colptr, w.ent_i, w.ent_a);
+  csc_chunk_offsets_kernel<<<(D + 255) / 256, 256, 0, s>>>(nchunks, sl.Kh / CSC_CHUNK, D, w.cnt, w.total);
+  csc_scan_kernel<<<1, 1024, 0, s>>>(sl.passes * D, w.total, w.colptr);
+  csc_fill_kernel<<<nchunks, 256, 0, s>>>(codes, K, D, sl.Kh / CSC_CHUNK, w.cnt, w.colptr, w.ent);
   return cudaGetLastError() == cudaSuccess ? 4 : SFB_ERR_CUDA;
 }
 
 // The update from a workspace that launch_sc_csc_build filled for the same K, D and codes.
 int launch_sc_csc_apply(cudaStream_t s, float* W, RowMap u, int K, int J, int D, float eta, long long nnz_capacity,
                         void* workspace, const int* dev_status_ro) {
-  const CscScratch w = csc_scratch(workspace, K, D, nnz_capacity);
-  const int threads = 512;
+  const CscSlices sl = csc_slices(K);
+  const CscScratch w = csc_scratch(workspace, K, D);
   static PerDeviceOnce attr_once;   // function attributes are per device
   if (attr_once.first())
     cudaFuncSetAttribute(csc_apply_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024);
-  // slices of the samples: the fewest that let Kh x 256 bytes of u sit beside the warps' tiles
-  const long long tiles = (long long)(threads / 32) * CSC2_WARP_FLOATS * 4;
-  const int kh_max = (int)((220 * 1024 - tiles) / 256) / CSC_CHUNK * CSC_CHUNK;
-  const int passes = (K + kh_max - 1) / kh_max;
-  const int Kh = ((K + passes - 1) / passes + CSC_CHUNK - 1) / CSC_CHUNK * CSC_CHUNK;
-  const int nj = (J + CSC2_JT - 1) / CSC2_JT;
-  const int nblocks = (D + CSC2_AB - 1) / CSC2_AB;
-  int splits = 148 / nj;                            // atom splits: fill the SMs when J / 64 alone does not
-  if (splits > nblocks / (threads / 32)) splits = nblocks / (threads / 32);
-  if (splits < 1) splits = 1;
-  const size_t smem = (size_t)Kh * 256 + (size_t)tiles;
-  csc_apply_kernel<<<dim3(nj, splits), threads, smem, s>>>(W, u, K, J, D, eta, w.colptr, w.cnt, w.ent_i, w.ent_a, passes,
-                                                          Kh, dev_status_ro);
+  const long long work = (long long)((J + CSC2_JT - 1) / CSC2_JT) * ((D + CSC2_AB - 1) / CSC2_AB);
+  long long blocks = (work + CSC2_WARPS - 1) / CSC2_WARPS;   // at least one block of atoms per warp
+  if (blocks > 148) blocks = 148;
+  const size_t smem = (size_t)sl.Kh * 256 + (size_t)CSC2_WARPS * CSC2_WARP_FLOATS * 4;
+  csc_apply_kernel<<<(unsigned)blocks, CSC2_WARPS * 32, smem, s>>>(W, u, K, J, D, eta, w.colptr, w.ent, sl.passes, sl.Kh,
+                                                                   dev_status_ro);
   return cudaGetLastError() == cudaSuccess ? 1 : SFB_ERR_CUDA;
 }
 
