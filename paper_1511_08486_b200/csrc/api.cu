@@ -166,9 +166,9 @@ int ensure_shadow(sfb_ctx* c, const void* W) {
 // workers > 0: the minibatch holds only that many workers' samples and u / v / codes start at the first of them.
 // for_apply: the apply of exactly these rows (all K pairs, no compaction in between) follows in the same call, so
 // the compensated path may write the apply's correction operands while it writes the factors.
-// commit (dense v): header and directory of the buffer u and v belong to, written by the finishing pass.
+// extra (dense v): what the finishing pass does besides (header of the buffer u and v belong to, flags of nonzero rows).
 int factors_into(sfb_ctx* c, const void* W, const void* X, const sfb_aux* aux, RowMap u, RowMap v, CsrView codes,
-                 int workers = 0, bool for_apply = false, const Commit& commit = Commit()) {
+                 int workers = 0, bool for_apply = false, const FinishExtra& extra = FinishExtra()) {
   const sfb_desc& d = c->d;
   const int K = workers > 0 ? workers * d.B : c->K;
   const float* Wf = reinterpret_cast<const float*>(W);
@@ -214,8 +214,6 @@ int factors_into(sfb_ctx* c, const void* W, const void* X, const sfb_aux* aux, R
                              c->f32_splits, &ks));
     }
     const RowMap zsrc = ks > 1 ? part : u;
-    FinishExtra extra;
-    extra.commit = commit;
     if (d.model == SFB_MLR)
       ACC(launch_finish_mlr(c->stream, zsrc, u, aux->labels, K, d.J, c->dev_status, ks, sstride,
                             reinterpret_cast<float*>(aux->dual), aux->sdca_step, CorrOut(), extra));
@@ -228,7 +226,7 @@ int factors_into(sfb_ctx* c, const void* W, const void* X, const sfb_aux* aux, R
     const int r = ensure_shadow(c, W);
     if (r < 0) return r;
   }
-  ACC(umma_forward(c->umma, c->stream, W, c->w_shadow, X, aux, u, v, c->dev_status, workers, for_apply, commit));
+  ACC(umma_forward(c->umma, c->stream, W, c->w_shadow, X, aux, u, v, c->dev_status, workers, for_apply, extra));
   return SFB_OK;
 }
 
@@ -448,7 +446,7 @@ int sfb_active_pairs(sfb_ctx* c, int32_t* n) {
     const int workers = c->last_step_K / c->d.B;
     int32_t* h = new (std::nothrow) int32_t[workers];
     if (h == nullptr) return SFB_ERR_ALLOC;
-    const char* counts = reinterpret_cast<const char*>(c->compact_ws) + pad_to(c->K, 256) + pad_to((long long)c->K * 4, 256);
+    const char* counts = reinterpret_cast<const char*>(c->compact_ws) + pad_to(c->K, 256);
     const bool ok = cudaMemcpy(h, counts, (size_t)workers * 4, cudaMemcpyDeviceToHost) == cudaSuccess;
     for (int p = 0; ok && p < workers; ++p) *n += h[p];
     delete[] h;
@@ -636,10 +634,13 @@ int sfb_factors_shard(sfb_ctx* c, const void* W, const void* X, const sfb_aux* a
                         c->dev_status));
     codes = stream_codes(c, shard);
   }
-  r = factors_into(c, W, X, aux, stream_u(c, shard), d.v_sparse ? RowMap() : stream_v(c, shard), codes, n_workers);
+  FinishExtra extra;
+  if (d.compact) extra.nonzero = compact_flags(c->compact_ws);
+  r = factors_into(c, W, X, aux, stream_u(c, shard), d.v_sparse ? RowMap() : stream_v(c, shard), codes, n_workers, false,
+                   extra);
   if (r < 0) return r;
   // a process compacts the streams of its own workers before they are sent
-  if (d.compact) ACC(launch_compact(c->stream, sf_buf, d, c->l, c->compact_ws, first_worker, n_workers));
+  if (d.compact) ACC(launch_compact(c->stream, sf_buf, d, c->l, c->compact_ws, first_worker, n_workers, true));
   return SFB_OK;
 }
 
@@ -726,12 +727,15 @@ int sfb_step(sfb_ctx* c, void* W, const void* X, const sfb_aux* aux, void* sf_bu
     join_aux();
     return SFB_ERR_CUDA;
   }
+  FinishExtra extra;
+  if (!d.v_sparse) extra.commit = commit;
+  if (d.compact) extra.nonzero = compact_flags(c->compact_ws);
   r = factors_into(c, W, X, aux, stream_u(c, sf_buf), d.v_sparse ? RowMap() : stream_v(c, sf_buf), codes, 0,
-                   d.path == SFB_PATH_TF32X3 && !d.compact && K == c->K, d.v_sparse ? Commit() : commit);
+                   d.path == SFB_PATH_TF32X3 && !d.compact && K == c->K, extra);
   if (forked && cudaStreamWaitEvent(c->stream, c->aux_join, 0) != cudaSuccess) return SFB_ERR_CUDA;
   if (r < 0) return r;
   // pairs whose u came out as zero are dropped from the message before it is "sent" (and applied)
-  if (d.compact) ACC(launch_compact(c->stream, sf_buf, d, c->l, c->compact_ws));
+  if (d.compact) ACC(launch_compact(c->stream, sf_buf, d, c->l, c->compact_ws, 0, 0, true));
   if (c->profiling) cudaEventRecord(c->prof_ev[slot][1], c->stream);
   const bool listed = !d.compact && d.model == SFB_DML && d.path == SFB_PATH_F32 && c->dml_active != nullptr &&
                       (long long)((d.J + 127) / 128) * ((d.D + 127) / 128) >= 148;   // the large-tile apply takes the list

@@ -157,13 +157,15 @@ __device__ __forceinline__ void write_header(const Commit& c, int tid, int n) {
 }
 #endif
 
-// What a finishing pass does beside its own work: the buffer's header, and (MLR, small batches) the factor v = x.
+// What a finishing pass does beside its own work: the buffer's header, which u rows hold a nonzero wire value (for the
+// compaction), and (MLR, small batches) the factor v = x.
 struct FinishExtra {
   Commit commit;
+  uint8_t* nonzero;  // [rows] or nullptr
   RowMap src, dst;   // dst.base == nullptr: no copy
   int cols;
   CorrOut corr;
-  FinishExtra() : src(), dst(), cols(0) {}
+  FinishExtra() : nonzero(nullptr), src(), dst(), cols(0) {}
 };
 
 #ifdef __CUDACC__
@@ -270,7 +272,10 @@ int launch_pack_csr(cudaStream_t s, void* sf_buf, const sfb_desc& d, const Layou
 // p * B + r, r < count of worker p, of the first `workers` workers (idx [K], n_out one int; device arrays).
 long long compact_workspace_bytes(int K, int P);
 int launch_compact(cudaStream_t s, void* sf_buf, const sfb_desc& d, const Layout& l, void* workspace, int first_worker = 0,
-                   int n_workers = 0);   // n_workers > 0: only those workers' streams (a process's shard)
+                   int n_workers = 0,
+                   bool flags_ready = false);   // n_workers > 0: only those workers' streams (a process's shard)
+// flags_ready: the finishing pass that wrote the u rows left its flags (FinishExtra::nonzero) in compact_flags(workspace).
+uint8_t* compact_flags(void* workspace);
 // Rebuilds the directory's pair counts (and the header flag) from streams that arrived already compacted.
 int launch_count_pairs(cudaStream_t s, void* sf_buf, const sfb_desc& d, const Layout& l, void* workspace);
 int launch_kept_rows(cudaStream_t s, const void* sf_buf, int B, int workers, int* idx, int* n_out);

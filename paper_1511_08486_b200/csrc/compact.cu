@@ -8,15 +8,15 @@
 // bit 1 is set.  Offsets and strides of the buffer do not change.
 //
 // In place and deterministic: a row only ever moves to a lower slot of its own worker, and every block of the
-// move kernel owns one (worker, 256-byte column slice) and walks the rows in waves of 64: a wave is read whole into
+// move kernel owns one (worker, 128-byte column slice) and walks the rows in waves of 256: a wave is read whole into
 // shared memory before any of its rows is written, and the slots it writes were all read by then.
 #include "common.cuh"
 
 namespace sfb {
 namespace {
 
-constexpr int WAVE = 64;          // rows per wave of the move
-constexpr int SLICE_UNITS = 16;   // 16-byte units per column slice (256 B): many small blocks hide the latency
+constexpr int WAVE = 256;         // rows per wave of the move, one per thread
+constexpr int SLICE_UNITS = 8;    // 16-byte units per column slice
 
 // flags[i] = 1 if the wire values of u row i are not all zero (-0 counts as zero).  One warp per row.
 __global__ void __launch_bounds__(256) row_nonzero_kernel(RowMap u, int K, int J, uint8_t* __restrict__ flags) {
@@ -34,74 +34,70 @@ __global__ void __launch_bounds__(256) row_nonzero_kernel(RowMap u, int K, int J
   if (lane == 0) flags[i] = (uint8_t)any;
 }
 
-// One block per worker: dest[i] = new slot of pair i inside its worker (-1: left out); the worker's count goes
-// to counts[p] and to the n_sf field of its directory entry; block 0 sets the header's "compacted" flag.
-__global__ void __launch_bounds__(256) compact_scan_kernel(const uint8_t* __restrict__ flags, int B, int* __restrict__ dest,
-                                                           int* __restrict__ counts, char* buf, int first_worker) {
-  __shared__ int warp_cnt[8];
-  __shared__ int base;
-  const int p = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  if (threadIdx.x == 0) base = 0;
-  __syncthreads();
-  for (int start = 0; start < B; start += 256) {
-    const int r = start + threadIdx.x;
-    const bool f = r < B && flags[(size_t)p * B + r] != 0;
-    const unsigned m = __ballot_sync(0xffffffffu, f);
-    if (lane == 0) warp_cnt[warp] = __popc(m);
-    __syncthreads();
-    int off = base;
-    for (int w = 0; w < warp; ++w) off += warp_cnt[w];
-    if (r < B) dest[(size_t)p * B + r] = f ? off + __popc(m & ((1u << lane) - 1u)) : -1;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      int t = 0;
-      for (int w = 0; w < 8; ++w) t += warp_cnt[w];
-      base += t;
-    }
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) {
-    counts[p] = base;
-    reinterpret_cast<uint32_t*>(buf + 128 + (size_t)(first_worker + p) * 32)[1] = (uint32_t)base;   // directory: n_sf
-    if (p == 0) reinterpret_cast<uint32_t*>(buf)[2] |= 2u;                                            // header flags, bit 1
-  }
-}
-
-// grid = (P, slices of the U rows + slices of the V rows).  Moves this block's 256-byte column slice of every kept
-// row of worker p to its new slot and clears the slice in the slots behind the last kept row.
-__global__ void __launch_bounds__(256) compact_move_kernel(char* streams, long long stream_stride, long long v_off, int B,
-                                                           int u_units, int v_units, int u_slices,
-                                                           const int* __restrict__ dest, const int* __restrict__ counts) {
-  __shared__ uint4 wave[WAVE * SLICE_UNITS];   // 16 KB
+// One block per (slice of the U rows, then of the V rows; worker).  Moves this block's 128-byte column slice of every kept
+// row of worker p to its new slot (the number of kept rows before it: every block counts the worker's flags for itself,
+// a wave at a time) and clears the slice in the slots behind the last kept row.  The first slice's block also leaves the
+// worker's pair count in counts[p] and in the n_sf field of its directory entry, and block 0 sets the header's
+// "compacted" flag.
+// Bound: HBM (kept rows read and written, left-out slots cleared).  A wave is a whole stream of up to 256 pairs, so that
+// all of a block's loads are in flight at once.  600 x 10000, 8 x 256 pairs
+// with three quarters kept: 37 -> 30 us (waves of 64 rows of 256-byte slices before, and 8 us of launches for flags and
+// scan that the finishing pass and this kernel now do on the way).
+__global__ void __launch_bounds__(256) compact_move_kernel(char* buf, char* streams, long long stream_stride, long long v_off,
+                                                           int B, int u_units, int v_units, int u_slices,
+                                                           const uint8_t* __restrict__ flags, int* __restrict__ counts,
+                                                           int first_worker, int n_workers) {
+  __shared__ uint4 wave[WAVE * SLICE_UNITS];   // 32 KB
   __shared__ int s_dest[WAVE];
-  const int p = blockIdx.x;
-  const bool is_v = (int)blockIdx.y >= u_slices;
-  const int slice = is_v ? blockIdx.y - u_slices : blockIdx.y;
+  __shared__ int warp_cnt[WAVE / 32];
+  const int y = blockIdx.x / n_workers, p = blockIdx.x - y * n_workers;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const bool is_v = y >= u_slices;
+  const int slice = is_v ? y - u_slices : y;
   const int row_units = is_v ? v_units : u_units;                 // 16-byte units per row
   const int q0 = slice * SLICE_UNITS;
   const int nq = min(SLICE_UNITS, row_units - q0);                // units of this slice that exist
   uint4* block = reinterpret_cast<uint4*>(streams + (size_t)p * stream_stride + (is_v ? v_off : 0));
-  const int n_keep = counts[p];
-  if (n_keep == B) return;                                        // nothing left out: every row stays where it is
+  int base = 0;                                                   // kept rows before this wave
   for (int r0 = 0; r0 < B; r0 += WAVE) {
-    if (threadIdx.x < WAVE) s_dest[threadIdx.x] = (r0 + threadIdx.x < B) ? dest[(size_t)p * B + r0 + threadIdx.x] : -1;
+    const int r = r0 + threadIdx.x;
+    const bool f = r < B && flags[(size_t)p * B + r] != 0;
+    const unsigned m = __ballot_sync(0xffffffffu, f);
+    if (lane == 0) warp_cnt[warp] = __popc(m);
     __syncthreads();
-    for (int t = threadIdx.x; t < WAVE * SLICE_UNITS; t += 256) {
-      const int r = t / SLICE_UNITS, q = t % SLICE_UNITS;
-      if (q < nq && s_dest[r] >= 0 && s_dest[r] != r0 + r) wave[t] = block[(size_t)(r0 + r) * row_units + q0 + q];
+    int before = base, total = 0;
+#pragma unroll
+    for (int w = 0; w < WAVE / 32; ++w) {
+      if (w < warp) before += warp_cnt[w];
+      total += warp_cnt[w];
+    }
+    // rows that stay where they are, and rows left out, are not moved
+    const int to = f ? before + __popc(m & ((1u << lane) - 1u)) : -1;
+    s_dest[threadIdx.x] = to == r ? -1 : to;
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < SLICE_UNITS; ++k) {
+      const int t = threadIdx.x + k * 256, rr = t / SLICE_UNITS, q = t % SLICE_UNITS;
+      if (q < nq && s_dest[rr] >= 0) wave[t] = block[(size_t)(r0 + rr) * row_units + q0 + q];
     }
     __syncthreads();
-    for (int t = threadIdx.x; t < WAVE * SLICE_UNITS; t += 256) {
-      const int r = t / SLICE_UNITS, q = t % SLICE_UNITS;
-      if (q < nq && s_dest[r] >= 0 && s_dest[r] != r0 + r) block[(size_t)s_dest[r] * row_units + q0 + q] = wave[t];
+#pragma unroll
+    for (int k = 0; k < SLICE_UNITS; ++k) {
+      const int t = threadIdx.x + k * 256, rr = t / SLICE_UNITS, q = t % SLICE_UNITS;
+      if (q < nq && s_dest[rr] >= 0) block[(size_t)s_dest[rr] * row_units + q0 + q] = wave[t];
     }
+    base += total;
     __syncthreads();
   }
   const uint4 zero = make_uint4(0u, 0u, 0u, 0u);
-  const int tail = B - n_keep;
-  for (int t = threadIdx.x; t < tail * nq; t += 256) {
-    const int r = n_keep + t / nq, q = t % nq;
-    block[(size_t)r * row_units + q0 + q] = zero;
+  for (int t = threadIdx.x; t < (B - base) * SLICE_UNITS; t += 256) {
+    const int r = base + t / SLICE_UNITS, q = t % SLICE_UNITS;
+    if (q < nq) block[(size_t)r * row_units + q0 + q] = zero;
+  }
+  if (y == 0 && threadIdx.x == 0) {
+    counts[p] = base;
+    reinterpret_cast<uint32_t*>(buf + 128 + (size_t)(first_worker + p) * 32)[1] = (uint32_t)base;   // directory: n_sf
+    if (p == 0) reinterpret_cast<uint32_t*>(buf)[2] |= 2u;                                            // header flags, bit 1
   }
 }
 
@@ -142,21 +138,22 @@ __global__ void __launch_bounds__(256) count_pairs_kernel(const uint8_t* __restr
 }
 
 struct Scratch {
-  uint8_t* flags; int* dest; int* counts;
+  uint8_t* flags; int* counts;
 };
-// flags [K] bytes, new slots [K] ints, per-worker counts [P] ints; offsets fixed by the full K = P * B
+// flags [K] bytes, per-worker counts [P] ints; offsets fixed by the full K = P * B
 Scratch scratch(void* workspace, int K) {
   Scratch w;
   w.flags = reinterpret_cast<uint8_t*>(workspace);
-  w.dest = reinterpret_cast<int*>(reinterpret_cast<char*>(workspace) + pad_to(K, 256));
-  w.counts = reinterpret_cast<int*>(reinterpret_cast<char*>(w.dest) + pad_to((long long)K * 4, 256));
+  w.counts = reinterpret_cast<int*>(reinterpret_cast<char*>(workspace) + pad_to(K, 256));
   return w;
 }
 
 }  // namespace
 
+uint8_t* compact_flags(void* workspace) { return reinterpret_cast<uint8_t*>(workspace); }
+
 long long compact_workspace_bytes(int K, int P) {
-  return pad_to((long long)K, 256) + pad_to((long long)K * 4, 256) + pad_to((long long)P * 4, 256);
+  return pad_to((long long)K, 256) + pad_to((long long)P * 4, 256);
 }
 
 // Directory pair counts of a buffer whose streams were compacted elsewhere (each process of a sharded step compacts
@@ -176,7 +173,7 @@ int launch_count_pairs(cudaStream_t s, void* sf_buf, const sfb_desc& d, const La
 // inside the kernels are relative to first_worker: streams, directory entries, flags, slots and counts alike
 // (counts[p] of the workspace belongs to worker first_worker + p).
 int launch_compact(cudaStream_t s, void* sf_buf, const sfb_desc& d, const Layout& l, void* workspace, int first_worker,
-                   int n_workers) {
+                   int n_workers, bool flags_ready) {
   if (n_workers <= 0) { first_worker = 0; n_workers = d.P; }
   const int K = n_workers * d.B;
   const Scratch w = scratch(workspace, d.P * d.B);
@@ -184,13 +181,13 @@ int launch_compact(cudaStream_t s, void* sf_buf, const sfb_desc& d, const Layout
   char* streams = buf + l.streams_off + (long long)first_worker * l.stream_stride;
   RowMap u;
   u.base = streams; u.worker_stride = l.stream_stride; u.ld = l.ldu; u.B = d.B; u.es = l.es;
-  row_nonzero_kernel<<<(K + 7) / 8, 256, 0, s>>>(u, K, d.J, w.flags);
-  compact_scan_kernel<<<n_workers, 256, 0, s>>>(w.flags, d.B, w.dest, w.counts, buf, first_worker);
+  if (!flags_ready) row_nonzero_kernel<<<(K + 7) / 8, 256, 0, s>>>(u, K, d.J, w.flags);
   const int u_units = l.ldu * l.es / 16, v_units = l.ldv * l.es / 16;
   const int u_slices = (u_units + SLICE_UNITS - 1) / SLICE_UNITS, v_slices = (v_units + SLICE_UNITS - 1) / SLICE_UNITS;
-  compact_move_kernel<<<dim3(n_workers, u_slices + v_slices), 256, 0, s>>>(streams, l.stream_stride, l.u_bytes, d.B, u_units,
-                                                                           v_units, u_slices, w.dest, w.counts);
-  return cudaGetLastError() == cudaSuccess ? 3 : SFB_ERR_CUDA;
+  compact_move_kernel<<<n_workers * (u_slices + v_slices), 256, 0, s>>>(buf, streams, l.stream_stride, l.u_bytes, d.B,
+                                                                           u_units, v_units, u_slices, w.flags, w.counts,
+                                                                           first_worker, n_workers);
+  return cudaGetLastError() == cudaSuccess ? (flags_ready ? 1 : 2) : SFB_ERR_CUDA;
 }
 
 int launch_kept_rows(cudaStream_t s, const void* sf_buf, int B, int workers, int* idx, int* n_out) {

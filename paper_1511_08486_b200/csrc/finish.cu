@@ -102,6 +102,18 @@ __device__ __forceinline__ void finish_extra(const FinishExtra& x, int i) {
     for (int q = threadIdx.x; q < x.dst.ld * x.dst.es / 16; q += blockDim.x) copy_unit(x.src, x.dst, i, q, x.cols, x.corr);
 }
 
+// Row i of u written: does it hold a nonzero wire value?  (any: this thread's values do)
+__device__ __forceinline__ void flag_row(const FinishExtra& x, int i, bool any) {
+  if (x.nonzero == nullptr) return;
+  any = __syncthreads_or(any);
+  if (threadIdx.x == 0) x.nonzero[i] = any ? 1 : 0;
+}
+__device__ __forceinline__ bool wire_nonzero4(const float4& t, int es) {
+  if (es == 4) return t.x != 0.f || t.y != 0.f || t.z != 0.f || t.w != 0.f;
+  const __nv_bfloat162 lo = __floats2bfloat162_rn(t.x, t.y), hi = __floats2bfloat162_rn(t.z, t.w);
+  return ((*reinterpret_cast<const uint32_t*>(&lo) | *reinterpret_cast<const uint32_t*>(&hi)) & 0x7fff7fffu) != 0u;
+}
+
 // z rows are fp32 with ld a multiple of 4; values beyond J inside the last float4 are ignored.
 __global__ void __launch_bounds__(1024) finish_mlr_kernel(RowMap z, RowMap u, const int32_t* __restrict__ labels,
                                                                  int K, int J, int cache_floats, int* dev_status, int nsplit, long long zstride,
@@ -154,6 +166,7 @@ __global__ void __launch_bounds__(1024) finish_mlr_kernel(RowMap z, RowMap u, co
   const bool bad = (y < 0) || (y >= J);
   if (bad && threadIdx.x == 0) atomicOr(dev_status, SFB_DEV_BAD_LABEL);
   const int ld4 = u.ld >> 2;   // u.ld is a multiple of 4 (fp32) or 8 (bf16)
+  bool any = false;
   for (int q = threadIdx.x; q < ld4; q += blockDim.x) {
     const int j = q * 4;
     float4 t = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -176,8 +189,10 @@ __global__ void __launch_bounds__(1024) finish_mlr_kernel(RowMap z, RowMap u, co
     }
     if (dual != nullptr && q < J4) t = sdca_step4(dual + (size_t)i * (J4 * 4), j, J, t, sdca_step, bad);
     store_u4(ur, j, t, u.es);
+    any |= wire_nonzero4(t, u.es);
     if (corr.mn != nullptr) corr_store4(corr, i, u.B, j, t);
   }
+  flag_row(extra, i, any);
 }
 
 __global__ void __launch_bounds__(1024) finish_dml_kernel(RowMap z, RowMap u, const uint8_t* __restrict__ similar,
@@ -209,6 +224,7 @@ __global__ void __launch_bounds__(1024) finish_dml_kernel(RowMap z, RowMap u, co
   if (active != nullptr && threadIdx.x == 0) active[i] = (g != 0.f) ? 1 : 0;   // u_i is all zeros otherwise
 
   const int ld4 = u.ld >> 2;
+  bool any = false;
   for (int q = threadIdx.x; q < ld4; q += blockDim.x) {
     const int j = q * 4;
     float4 t = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -220,8 +236,10 @@ __global__ void __launch_bounds__(1024) finish_dml_kernel(RowMap z, RowMap u, co
       if (j + 3 >= J) t.w = 0.f;
     }
     store_u4(ur, j, t, u.es);
+    any |= wire_nonzero4(t, u.es);
     if (corr.mn != nullptr) corr_store4(corr, i, u.B, j, t);
   }
+  flag_row(extra, i, any);
 }
 
 // Second half of the fused multiclass-logistic epilogue.  The forward GEMM left e[j] = exp(z[j] - m_p)
@@ -257,6 +275,7 @@ __global__ void __launch_bounds__(256) finish_mlr_fused_kernel(RowMap u, const f
   char* ur = u.row(i);
   constexpr int PER = 16 / ES;          // values per 16-byte unit (part_cols is a multiple of it)
   const int units = u.ld / PER;
+  bool any = false;
   for (int q = threadIdx.x; q < units; q += 256) {
     const int j = q * PER;
     uint4 raw = *reinterpret_cast<const uint4*>(ur + (size_t)q * 16);
@@ -298,8 +317,10 @@ __global__ void __launch_bounds__(256) finish_mlr_fused_kernel(RowMap u, const f
 #pragma unroll
       for (int e = 0; e < PER; ++e) h[e] = __float2bfloat16_rn(vals[e]);
     }
+    any |= ((raw.x | raw.y | raw.z | raw.w) & (ES == 4 ? 0x7fffffffu : 0x7fff7fffu)) != 0u;
     *reinterpret_cast<uint4*>(ur + (size_t)q * 16) = raw;
   }
+  flag_row(extra, i, any);
 }
 
 // Unit-ball projection of the columns of W (sparse-coding prox).  A cluster of CTAs owns a slab of 32 consecutive

@@ -1259,7 +1259,7 @@ int umma_forward_sc(UmmaPlan* pl, cudaStream_t s, const void* W, RowMap a, RowMa
 
 int umma_forward(UmmaPlan* pl, cudaStream_t s, const void* W, const __nv_bfloat16* w_shadow, const void* X,
                  const sfb_aux* aux, RowMap u, RowMap v, int* dev_status, int workers, bool for_apply,
-                 const Commit& commit) {
+                 const FinishExtra& extra_in) {
   const sfb_desc& d = pl->d;
   const int K = (workers > 0 ? workers : d.P) * d.B;
   int launches = 0, r;
@@ -1274,8 +1274,7 @@ int umma_forward(UmmaPlan* pl, cudaStream_t s, const void* W, const __nv_bfloat1
   x_rows.base = const_cast<char*>(reinterpret_cast<const char*>(X));
   x_rows.ld = d.D; x_rows.B = d.B; x_rows.es = pl->es;
   x_rows.worker_stride = (long long)d.B * d.D * pl->es;
-  FinishExtra extra;
-  extra.commit = commit;
+  FinishExtra extra = extra_in;
   if (d.model == SFB_MLR) {
     const bool bf16 = d.path == SFB_PATH_BF16;
     bool forked = false;

@@ -15,10 +15,10 @@ void umma_plan_destroy(UmmaPlan* p);
 // for_apply (compensated path): umma_apply of exactly these u / v rows, all K pairs, follows before anything else
 // changes them: the kernels that write the factors also write the apply's correction operands (one use).
 // workers > 0: only that many workers' samples (X, aux, u, v start at the first of them).
-// commit: header and directory of the buffer the rows belong to, written by the finishing pass.
+// extra: what the finishing pass does besides (header, flags of nonzero rows).
 int umma_forward(UmmaPlan* p, cudaStream_t s, const void* W, const __nv_bfloat16* w_shadow, const void* X,
                  const sfb_aux* aux, RowMap u, RowMap v, int* dev_status, int workers = 0, bool for_apply = false,
-                 const Commit& commit = Commit());
+                 const FinishExtra& extra = FinishExtra());
 
 // Z rows (fp32) = A rows (the path's value type) times Wop^T on the tensor cores; no epilogue beyond the store.
 // w_corr: on the compensated path, W's correction operand (launch_split_k of W's rows, B side); w_shadow plays
