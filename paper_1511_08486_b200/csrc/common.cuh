@@ -187,6 +187,30 @@ __device__ __forceinline__ float4 sdca_step4(float* dual_row, int j, int J, floa
 }
 #endif
 
+// Chained launches (programmatic dependent launch): a kernel of a call's chain may be scheduled while its predecessor on
+// the stream is still running, so that launch latency and set-up overlap with it.  Every such kernel starts with chain(),
+// or, where the set-up touches no memory that another kernel writes, chain_next() first and chain_wait() behind it:
+// nothing before the wait reads or writes global memory, and every thread waits, so each grid is complete, its writes
+// visible, before its successor touches memory, exactly as without the overlap.
+#ifdef __CUDACC__
+__device__ __forceinline__ void chain_next() { asm volatile("griddepcontrol.launch_dependents;"); }
+__device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void chain() {
+  chain_next();
+  chain_wait();
+}
+template <typename... P, typename... A>
+cudaError_t launch_chained(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A&&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = s;
+  cfg.attrs = at; cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+#endif
+
 // cudaFuncSetAttribute acts on the current device only: first() is true once per device (ordinals 0..63)
 // for the static object it is called on.  A repeated call from a racing thread would set the same value.
 struct PerDeviceOnce {

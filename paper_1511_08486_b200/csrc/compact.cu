@@ -20,6 +20,7 @@ constexpr int SLICE_UNITS = 8;    // 16-byte units per column slice
 
 // flags[i] = 1 if the wire values of u row i are not all zero (-0 counts as zero).  One warp per row.
 __global__ void __launch_bounds__(256) row_nonzero_kernel(RowMap u, int K, int J, uint8_t* __restrict__ flags) {
+  chain();
   const int i = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (i >= K) return;
   const int per = 16 / u.es, units = (J + per - 1) / per;     // pad values inside the last unit are zeros
@@ -47,6 +48,7 @@ __global__ void __launch_bounds__(256) compact_move_kernel(char* buf, char* stre
                                                            int B, int u_units, int v_units, int u_slices,
                                                            const uint8_t* __restrict__ flags, int* __restrict__ counts,
                                                            int first_worker, int n_workers) {
+  chain();
   __shared__ uint4 wave[WAVE * SLICE_UNITS];   // 32 KB
   __shared__ int s_dest[WAVE];
   __shared__ int warp_cnt[WAVE / 32];
@@ -104,6 +106,7 @@ __global__ void __launch_bounds__(256) compact_move_kernel(char* buf, char* stre
 // idx[0 .. *n_out) = p * B + r for every worker p < workers and every r < its pair count, in that order.
 __global__ void __launch_bounds__(256) kept_rows_kernel(const char* buf, int B, int workers, int* __restrict__ idx,
                                                         int* __restrict__ n_out) {
+  chain();
   __shared__ int base;
   if (threadIdx.x == 0) base = 0;
   __syncthreads();
@@ -122,6 +125,7 @@ __global__ void __launch_bounds__(256) kept_rows_kernel(const char* buf, int B, 
 // One block per worker: n_sf of its directory entry = number of its u rows flagged nonzero (in a compacted stream
 // the kept pairs are exactly the leading rows); block 0 sets the header's "compacted" flag.
 __global__ void __launch_bounds__(256) count_pairs_kernel(const uint8_t* __restrict__ flags, int B, char* buf) {
+  chain();
   __shared__ int total;
   if (threadIdx.x == 0) total = 0;
   __syncthreads();
@@ -164,8 +168,8 @@ int launch_count_pairs(cudaStream_t s, void* sf_buf, const sfb_desc& d, const La
   char* buf = reinterpret_cast<char*>(sf_buf);
   RowMap u;
   u.base = buf + l.streams_off; u.worker_stride = l.stream_stride; u.ld = l.ldu; u.B = d.B; u.es = l.es;
-  row_nonzero_kernel<<<(K + 7) / 8, 256, 0, s>>>(u, K, d.J, w.flags);
-  count_pairs_kernel<<<d.P, 256, 0, s>>>(w.flags, d.B, buf);
+  launch_chained(row_nonzero_kernel, (K + 7) / 8, 256, 0, s, u, K, d.J, w.flags);
+  launch_chained(count_pairs_kernel, d.P, 256, 0, s, w.flags, d.B, buf);
   return cudaGetLastError() == cudaSuccess ? 2 : SFB_ERR_CUDA;
 }
 
@@ -181,17 +185,17 @@ int launch_compact(cudaStream_t s, void* sf_buf, const sfb_desc& d, const Layout
   char* streams = buf + l.streams_off + (long long)first_worker * l.stream_stride;
   RowMap u;
   u.base = streams; u.worker_stride = l.stream_stride; u.ld = l.ldu; u.B = d.B; u.es = l.es;
-  if (!flags_ready) row_nonzero_kernel<<<(K + 7) / 8, 256, 0, s>>>(u, K, d.J, w.flags);
+  if (!flags_ready) launch_chained(row_nonzero_kernel, (K + 7) / 8, 256, 0, s, u, K, d.J, w.flags);
   const int u_units = l.ldu * l.es / 16, v_units = l.ldv * l.es / 16;
   const int u_slices = (u_units + SLICE_UNITS - 1) / SLICE_UNITS, v_slices = (v_units + SLICE_UNITS - 1) / SLICE_UNITS;
-  compact_move_kernel<<<n_workers * (u_slices + v_slices), 256, 0, s>>>(buf, streams, l.stream_stride, l.u_bytes, d.B,
+  launch_chained(compact_move_kernel, n_workers * (u_slices + v_slices), 256, 0, s, buf, streams, l.stream_stride, l.u_bytes, d.B,
                                                                            u_units, v_units, u_slices, w.flags, w.counts,
                                                                            first_worker, n_workers);
   return cudaGetLastError() == cudaSuccess ? (flags_ready ? 1 : 2) : SFB_ERR_CUDA;
 }
 
 int launch_kept_rows(cudaStream_t s, const void* sf_buf, int B, int workers, int* idx, int* n_out) {
-  kept_rows_kernel<<<1, 256, 0, s>>>(reinterpret_cast<const char*>(sf_buf), B, workers, idx, n_out);
+  launch_chained(kept_rows_kernel, 1, 256, 0, s, reinterpret_cast<const char*>(sf_buf), B, workers, idx, n_out);
   return cudaGetLastError() == cudaSuccess ? 1 : SFB_ERR_CUDA;
 }
 

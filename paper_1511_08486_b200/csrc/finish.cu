@@ -118,6 +118,7 @@ __device__ __forceinline__ bool wire_nonzero4(const float4& t, int es) {
 __global__ void __launch_bounds__(1024) finish_mlr_kernel(RowMap z, RowMap u, const int32_t* __restrict__ labels,
                                                                  int K, int J, int cache_floats, int* dev_status, int nsplit, long long zstride,
                                                                  float* __restrict__ dual, float sdca_step, CorrOut corr, const __grid_constant__ FinishExtra extra) {
+  chain();
   extern __shared__ __align__(16) float cache[];
   __shared__ float red[32];
   const int i = blockIdx.x;
@@ -198,6 +199,7 @@ __global__ void __launch_bounds__(1024) finish_mlr_kernel(RowMap z, RowMap u, co
 __global__ void __launch_bounds__(1024) finish_dml_kernel(RowMap z, RowMap u, const uint8_t* __restrict__ similar,
                                                                  float margin, int K, int J, int cache_floats, int nsplit, long long zstride,
                                                                  uint8_t* __restrict__ active, CorrOut corr, const __grid_constant__ FinishExtra extra) {
+  chain();
   extern __shared__ __align__(16) float cache[];
   __shared__ float red[32];
   const int i = blockIdx.x;
@@ -250,6 +252,7 @@ __global__ void __launch_bounds__(256) finish_mlr_fused_kernel(RowMap u, const f
                                                                int part_cols, const int32_t* __restrict__ labels, int K,
                                                                int J, int* dev_status, float* __restrict__ dual,
                                                                float sdca_step, const __grid_constant__ FinishExtra extra) {
+  chain();
   extern __shared__ float scale[];   // [n_parts]
   __shared__ float red[32];
   const int i = blockIdx.x;
@@ -337,6 +340,7 @@ constexpr int PROX_HELD = 16, PROX_THREADS = 256, PROX_ROWS = PROX_THREADS / 8;
 template <bool VEC>
 __global__ void __launch_bounds__(PROX_THREADS, VEC ? 2 : 1) prox_unit_columns_kernel(float* __restrict__ W, int J, int D,
                                                                             int rows_per_cta, __nv_bfloat16* shadow) {
+  chain();
   __shared__ float4 part[PROX_ROWS][9];
   __shared__ float cta_sum[32];
   cg::cluster_group cluster = cg::this_cluster();
@@ -419,6 +423,7 @@ __global__ void __launch_bounds__(PROX_THREADS, VEC ? 2 : 1) prox_unit_columns_k
 
 // 16-byte-vectorised row copy; rows are whole numbers of 16-byte units on both sides.
 __global__ void __launch_bounds__(256) copy_rows_kernel(RowMap src, RowMap dst, int K, int cols, CorrOut corr) {
+  chain();
   const int units_dst = dst.ld * dst.es / 16;
   const long long total = (long long)K * units_dst;
   for (long long g = blockIdx.x * (long long)blockDim.x + threadIdx.x; g < total;
@@ -429,6 +434,7 @@ __global__ void __launch_bounds__(256) copy_rows_kernel(RowMap src, RowMap dst, 
 // u and v rows into their streams, and the header, in one launch.
 __global__ void __launch_bounds__(256) pack_rows_kernel(RowMap u_src, RowMap u_dst, int J, RowMap v_src, RowMap v_dst, int D,
                                                         int K, const __grid_constant__ Commit commit) {
+  chain();
   if (blockIdx.x == 0) write_header(commit, threadIdx.x, 256);
   const int uu = u_dst.ld * u_dst.es / 16, units = uu + v_dst.ld * v_dst.es / 16;
   const long long total = (long long)K * units;
@@ -443,6 +449,7 @@ __global__ void __launch_bounds__(256) pack_rows_kernel(RowMap u_src, RowMap u_d
 // v rows = Xa - Xb (one fp32 subtraction per element), pad columns zero; 4 values per thread.
 __global__ void __launch_bounds__(256) diff_rows_kernel(const float* __restrict__ Xa, const float* __restrict__ Xb, RowMap v,
                                                         int K, int D, CorrOut corr) {
+  chain();
   const int units = v.ld >> 2;
   const long long total = (long long)K * units;
   for (long long g = blockIdx.x * (long long)blockDim.x + threadIdx.x; g < total;
@@ -465,6 +472,7 @@ __global__ void __launch_bounds__(256) diff_rows_kernel(const float* __restrict_
 
 __global__ void __launch_bounds__(256) cast_bf16_kernel(const float* __restrict__ W, __nv_bfloat16* __restrict__ Wb,
                                                         long long n4) {
+  chain();
   for (long long g = blockIdx.x * (long long)blockDim.x + threadIdx.x; g < n4; g += (long long)gridDim.x * blockDim.x) {
     const float4 t = reinterpret_cast<const float4*>(W)[g];
     __nv_bfloat162 lo = __floats2bfloat162_rn(t.x, t.y), hi = __floats2bfloat162_rn(t.z, t.w);
@@ -494,7 +502,7 @@ int launch_finish_mlr(cudaStream_t s, RowMap z, RowMap u, const int32_t* labels,
     cudaFuncSetAttribute(finish_mlr_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, ROW_CACHE_FLOATS * 4);
     cudaFuncSetAttribute(finish_dml_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, ROW_CACHE_FLOATS * 4);
   }
-  finish_mlr_kernel<<<K, fin_threads(J), (size_t)cf * 4, s>>>(z, u, labels, K, J, cf, dev_status, nsplit, split_stride_bytes / 4,
+  launch_chained(finish_mlr_kernel, K, fin_threads(J), (size_t)cf * 4, s, z, u, labels, K, J, cf, dev_status, nsplit, split_stride_bytes / 4,
                                                               dual, sdca_step, corr, extra);
   return cudaGetLastError() == cudaSuccess ? 1 : SFB_ERR_CUDA;
 }
@@ -502,6 +510,7 @@ int launch_finish_mlr(cudaStream_t s, RowMap z, RowMap u, const int32_t* labels,
 // idx[0 .. n) = the samples i < K with active[i] != 0, in ascending order; *n_out = n.  One block, ordered.
 __global__ void __launch_bounds__(1024) compact_active_kernel(const uint8_t* __restrict__ active, int K, int* __restrict__ idx,
                                                               int* __restrict__ n_out) {
+  chain();
   __shared__ int warp_cnt[32];
   __shared__ int base;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -529,7 +538,7 @@ __global__ void __launch_bounds__(1024) compact_active_kernel(const uint8_t* __r
 }
 
 int launch_compact_active(cudaStream_t s, const uint8_t* active, int K, int* idx, int* n_out) {
-  compact_active_kernel<<<1, 1024, 0, s>>>(active, K, idx, n_out);
+  launch_chained(compact_active_kernel, 1, 1024, 0, s, active, K, idx, n_out);
   return cudaGetLastError() == cudaSuccess ? 1 : SFB_ERR_CUDA;
 }
 
@@ -541,7 +550,7 @@ int launch_finish_dml(cudaStream_t s, RowMap z, RowMap u, const uint8_t* similar
     cudaFuncSetAttribute(finish_mlr_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, ROW_CACHE_FLOATS * 4);
     cudaFuncSetAttribute(finish_dml_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, ROW_CACHE_FLOATS * 4);
   }
-  finish_dml_kernel<<<K, fin_threads(J), (size_t)cf * 4, s>>>(z, u, similar, margin, K, J, cf, nsplit, split_stride_bytes / 4,
+  launch_chained(finish_dml_kernel, K, fin_threads(J), (size_t)cf * 4, s, z, u, similar, margin, K, J, cf, nsplit, split_stride_bytes / 4,
                                                               active, corr, extra);
   return cudaGetLastError() == cudaSuccess ? 1 : SFB_ERR_CUDA;
 }
@@ -552,9 +561,9 @@ int launch_finish_mlr_fused(cudaStream_t s, RowMap u, const float2* stats, int n
   const size_t smem = (size_t)n_parts * sizeof(float);
   if (smem > 48 * 1024) return SFB_ERR_SHAPE;
   if (u.es == 4)
-    finish_mlr_fused_kernel<4><<<K, 256, smem, s>>>(u, stats, n_parts, part_cols, labels, K, J, dev_status, dual, sdca_step, extra);
+    launch_chained(finish_mlr_fused_kernel<4>, K, 256, smem, s, u, stats, n_parts, part_cols, labels, K, J, dev_status, dual, sdca_step, extra);
   else
-    finish_mlr_fused_kernel<2><<<K, 256, smem, s>>>(u, stats, n_parts, part_cols, labels, K, J, dev_status, dual, sdca_step, extra);
+    launch_chained(finish_mlr_fused_kernel<2>, K, 256, smem, s, u, stats, n_parts, part_cols, labels, K, J, dev_status, dual, sdca_step, extra);
   return cudaGetLastError() == cudaSuccess ? 1 : SFB_ERR_CUDA;
 }
 
@@ -565,13 +574,15 @@ int launch_prox_unit_columns(cudaStream_t s, float* W, int J, int D, __nv_bfloat
   while (ctas < 8 && (ctas * PROX_HELD * PROX_ROWS < J || (slabs * ctas < 296 && ctas * 2 * PROX_ROWS < J))) ctas *= 2;
   const int rows = (J + ctas - 1) / ctas;
   cudaLaunchConfig_t cfg = {};
-  cudaLaunchAttribute at[1];
+  cudaLaunchAttribute at[2];
   at[0].id = cudaLaunchAttributeClusterDimension;
   at[0].val.clusterDim.x = ctas; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
+  at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.gridDim = dim3(ctas * slabs);
   cfg.blockDim = dim3(PROX_THREADS);
   cfg.stream = s;
-  cfg.attrs = at; cfg.numAttrs = 1;
+  cfg.attrs = at; cfg.numAttrs = 2;
   const cudaError_t e = (D & 3) == 0 ? cudaLaunchKernelEx(&cfg, prox_unit_columns_kernel<true>, W, J, D, rows, shadow)
                                      : cudaLaunchKernelEx(&cfg, prox_unit_columns_kernel<false>, W, J, D, rows, shadow);
   return e == cudaSuccess ? 1 : SFB_ERR_CUDA;
@@ -581,7 +592,7 @@ int launch_pack_rows(cudaStream_t s, RowMap u_src, RowMap u_dst, int J, RowMap v
                      const Commit& commit) {
   const long long total = (long long)K * ((u_dst.ld + v_dst.ld) * (long long)u_dst.es / 16);
   const int blocks = (int)((total + 255) / 256 < 148LL * 16 ? (total + 255) / 256 : 148LL * 16);
-  pack_rows_kernel<<<blocks, 256, 0, s>>>(u_src, u_dst, J, v_src, v_dst, D, K, commit);
+  launch_chained(pack_rows_kernel, blocks, 256, 0, s, u_src, u_dst, J, v_src, v_dst, D, K, commit);
   return cudaGetLastError() == cudaSuccess ? 1 : SFB_ERR_CUDA;
 }
 
@@ -589,21 +600,21 @@ int launch_copy_rows(cudaStream_t s, RowMap src, RowMap dst, int K, int cols, Co
   const long long total = (long long)K * (dst.ld * dst.es / 16);
   if (total == 0) return 0;
   const int blocks = (int)((total + 255) / 256 < 148LL * 16 ? (total + 255) / 256 : 148LL * 16);
-  copy_rows_kernel<<<blocks, 256, 0, s>>>(src, dst, K, cols, corr);
+  launch_chained(copy_rows_kernel, blocks, 256, 0, s, src, dst, K, cols, corr);
   return cudaGetLastError() == cudaSuccess ? 1 : SFB_ERR_CUDA;
 }
 
 int launch_diff_rows(cudaStream_t s, const float* Xa, const float* Xb, RowMap v, int K, int D, CorrOut corr) {
   const long long total = (long long)K * (v.ld >> 2);
   const int blocks = (int)((total + 255) / 256 < 148LL * 16 ? (total + 255) / 256 : 148LL * 16);
-  diff_rows_kernel<<<blocks, 256, 0, s>>>(Xa, Xb, v, K, D, corr);
+  launch_chained(diff_rows_kernel, blocks, 256, 0, s, Xa, Xb, v, K, D, corr);
   return cudaGetLastError() == cudaSuccess ? 1 : SFB_ERR_CUDA;
 }
 
 int launch_cast_bf16(cudaStream_t s, const float* W, __nv_bfloat16* Wb, long long n) {
   const long long n4 = n / 4;   // J*D is a multiple of 4 on the bf16 path (D % 8 == 0 is required there)
   const int blocks = (int)((n4 + 255) / 256 < 148LL * 16 ? (n4 + 255) / 256 : 148LL * 16);
-  cast_bf16_kernel<<<blocks, 256, 0, s>>>(W, Wb, n4);
+  launch_chained(cast_bf16_kernel, blocks, 256, 0, s, W, Wb, n4);
   return cudaGetLastError() == cudaSuccess ? 1 : SFB_ERR_CUDA;
 }
 

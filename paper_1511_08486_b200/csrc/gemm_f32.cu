@@ -68,6 +68,7 @@ template <int MI, int NI>
 __global__ void __launch_bounds__(256, 2) forward_f32_kernel(const float* __restrict__ W, const float* __restrict__ X,
                                                           const float* __restrict__ Xb, int K, int J, int D,
                                                           RowMap z, RowMap v, int d_per_split, long long split_stride) {
+  chain();
   constexpr int BM = 64 * MI, BN = 64 * NI;
   __shared__ __align__(16) float As[BK][BM + 4];
   __shared__ __align__(16) float Bs[BK][BN + 4];
@@ -156,6 +157,7 @@ __global__ void __launch_bounds__(256, 2) forward_f32_kernel(const float* __rest
 template <int MI, int NI>
 __global__ void __launch_bounds__(256, 2) apply_f32_kernel(float* __restrict__ W, RowMap u, RowMap v, int K, int J,
                                                         int D, float eta, const int* __restrict__ dev_status) {
+  chain();
   constexpr int BM = 64 * MI, BN = 64 * NI;
   __shared__ __align__(16) float As[BK][BM + 4];
   __shared__ __align__(16) float Bs[BK][BN + 4];
@@ -251,6 +253,7 @@ __global__ void __launch_bounds__(256, 2) sgemm_pipe_kernel(float* __restrict__ 
                                                          int D, float eta, const int* __restrict__ dev_status,
                                                          RowMap z, int k_per_range, long long range_stride,
                                                          const int* __restrict__ row_idx, const int* __restrict__ n_rows) {
+  chain();
   constexpr int BM = 128, BN = 128;
   extern __shared__ __align__(16) float ring[];
   if (OUT == 0 && dev_status != nullptr && (*dev_status & SFB_DEV_BAD_HEADER)) return;
@@ -353,6 +356,7 @@ __global__ void __launch_bounds__(256, 2) sgemm_pipe_kernel(float* __restrict__ 
 // zero).  `copy` (optional): the same rows also copied there, pad columns zero (the factor v = x of the MLR model).
 __global__ void __launch_bounds__(256) transpose_rows_kernel(RowMap src, float* __restrict__ dst, int R, int C, int ldr,
                                                              RowMap copy) {
+  chain();
   __shared__ float tile[32][33];
   const int c0 = blockIdx.x * 32, r0 = blockIdx.y * 32;
   const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;   // 32 x 8
@@ -382,6 +386,7 @@ struct TransposeJob {
   RowMap copy;
 };
 __global__ void __launch_bounds__(256) transpose_rows_vec_kernel(TransposeJob j0, TransposeJob j1) {
+  chain();
   __shared__ float tile[64][65];
   const TransposeJob& j = blockIdx.z == 0 ? j0 : j1;
   const int c0 = blockIdx.x * 64, r0 = blockIdx.y * 64;
@@ -437,14 +442,14 @@ int launch_forward_f32(cudaStream_t s, const float* W, const float* X, const flo
   if (ks > 1) {
     const int per = ((D + ks - 1) / ks + BK - 1) / BK * BK;
     dim3 grid((J + 127) / 128, (K + 127) / 128, ks);
-    forward_f32_kernel<2, 2><<<grid, 256, 0, s>>>(W, X, Xb, K, J, D, part, v, per, split_stride);
+    launch_chained(forward_f32_kernel<2, 2>, grid, 256, 0, s, W, X, Xb, K, J, D, part, v, per, split_stride);
     *nsplit_out = ks;
   } else if (big_tiles >= 148) {
     dim3 grid((J + 127) / 128, (K + 127) / 128);
-    forward_f32_kernel<2, 2><<<grid, 256, 0, s>>>(W, X, Xb, K, J, D, z, v, D, 0);
+    launch_chained(forward_f32_kernel<2, 2>, grid, 256, 0, s, W, X, Xb, K, J, D, z, v, D, 0);
   } else {
     dim3 grid((J + 63) / 64, (K + 63) / 64);
-    forward_f32_kernel<1, 1><<<grid, 256, 0, s>>>(W, X, Xb, K, J, D, z, v, D, 0);
+    launch_chained(forward_f32_kernel<1, 1>, grid, 256, 0, s, W, X, Xb, K, J, D, z, v, D, 0);
   }
   return cudaGetLastError() == cudaSuccess ? 1 : SFB_ERR_CUDA;
 }
@@ -458,11 +463,11 @@ int launch_apply_f32(cudaStream_t s, float* W, RowMap u, RowMap v, int K, int J,
     if (attr_once.first()) {
       cudaFuncSetAttribute(sgemm_pipe_kernel<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, PIPE * PIPE_STAGE_FLOATS * 4);
     }
-    sgemm_pipe_kernel<0><<<grid, 256, PIPE * PIPE_STAGE_FLOATS * 4, s>>>(W, u, v, K, J, D, eta, dev_status, RowMap(), 0, 0,
+    launch_chained(sgemm_pipe_kernel<0>, grid, 256, PIPE * PIPE_STAGE_FLOATS * 4, s, W, u, v, K, J, D, eta, dev_status, RowMap(), 0, 0,
                                                                          row_idx, n_rows);
   } else {
     dim3 grid((D + 63) / 64, (J + 63) / 64);
-    apply_f32_kernel<1, 1><<<grid, 256, 0, s>>>(W, u, v, K, J, D, eta, dev_status);
+    launch_chained(apply_f32_kernel<1, 1>, grid, 256, 0, s, W, u, v, K, J, D, eta, dev_status);
   }
   return cudaGetLastError() == cudaSuccess ? 1 : SFB_ERR_CUDA;
 }
@@ -493,11 +498,11 @@ int launch_forward_f32_nn(cudaStream_t s, const float* W, RowMap src, RowMap cop
     jx.src = src; jx.dst = xt; jx.R = K; jx.C = D; jx.ldr = ldk; jx.copy = copy;
     jw.src = wrows; jw.dst = wt; jw.R = J; jw.C = D; jw.ldr = ldj; jw.copy = RowMap();
     const int ry = ((ldk > ldj ? ldk : ldj) + 63) / 64;
-    transpose_rows_vec_kernel<<<dim3((D + 63) / 64, ry, 2), 256, 0, s>>>(jx, jw);
+    launch_chained(transpose_rows_vec_kernel, dim3((D + 63) / 64, ry, 2), 256, 0, s, jx, jw);
     transposes = 1;
   } else {
-    transpose_rows_kernel<<<dim3((D + 31) / 32, (ldk + 31) / 32), 256, 0, s>>>(src, xt, K, D, ldk, copy);
-    transpose_rows_kernel<<<dim3((D + 31) / 32, (ldj + 31) / 32), 256, 0, s>>>(wrows, wt, J, D, ldj, RowMap());
+    launch_chained(transpose_rows_kernel, dim3((D + 31) / 32, (ldk + 31) / 32), 256, 0, s, src, xt, K, D, ldk, copy);
+    launch_chained(transpose_rows_kernel, dim3((D + 31) / 32, (ldj + 31) / 32), 256, 0, s, wrows, wt, J, D, ldj, RowMap());
   }
   int ks = (part.base != nullptr && nsplit_out != nullptr) ? forward_f32_splits(K, J, D) : 1;
   if (ks > max_splits) ks = max_splits;
@@ -511,7 +516,7 @@ int launch_forward_f32_nn(cudaStream_t s, const float* W, RowMap src, RowMap cop
     cudaFuncSetAttribute(sgemm_pipe_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, PIPE * PIPE_STAGE_FLOATS * 4);
   // rows of the output tile = samples (M = K), columns = classes (N = J), reduction over the D features
   dim3 grid((J + 127) / 128, (K + 127) / 128, ks);
-  sgemm_pipe_kernel<1><<<grid, 256, PIPE * PIPE_STAGE_FLOATS * 4, s>>>(nullptr, a, b, D, K, ldj, 0.f, nullptr,
+  launch_chained(sgemm_pipe_kernel<1>, grid, 256, PIPE * PIPE_STAGE_FLOATS * 4, s, nullptr, a, b, D, K, ldj, 0.f, nullptr,
                                                                        ks > 1 ? part : z, per, split_stride, nullptr, nullptr);
   return cudaGetLastError() == cudaSuccess ? transposes + 1 : SFB_ERR_CUDA;
 }

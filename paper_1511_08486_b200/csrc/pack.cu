@@ -23,9 +23,10 @@ HeaderImage make_header(const sfb_desc& d, const Layout& l, uint32_t clock) {
   return h;
 }
 
-__global__ void write_header_kernel(const __grid_constant__ Commit c) { write_header(c, threadIdx.x, blockDim.x); }
+__global__ void write_header_kernel(const __grid_constant__ Commit c) { chain(); write_header(c, threadIdx.x, blockDim.x); }
 
 __global__ void check_header_kernel(const char* buf, HeaderImage h, int* dev_status) {
+  chain();
   const uint32_t* w = reinterpret_cast<const uint32_t*>(buf);
   const uint32_t* ref = reinterpret_cast<const uint32_t*>(&h);
   const int t = threadIdx.x;   // 32 threads
@@ -90,12 +91,12 @@ Commit make_commit(void* sf_buf, const sfb_desc& d, const Layout& l, uint32_t cl
 
 int launch_write_header(cudaStream_t s, void* sf_buf, const sfb_desc& d, const Layout& l, uint32_t clock,
                         const uint32_t* rowptr) {
-  write_header_kernel<<<1, 256, 0, s>>>(make_commit(sf_buf, d, l, clock, rowptr));
+  launch_chained(write_header_kernel, 1, 256, 0, s, make_commit(sf_buf, d, l, clock, rowptr));
   return cudaGetLastError() == cudaSuccess ? 1 : SFB_ERR_CUDA;
 }
 
 int launch_check_header(cudaStream_t s, const void* sf_buf, const sfb_desc& d, const Layout& l, int* dev_status) {
-  check_header_kernel<<<1, 32, 0, s>>>(reinterpret_cast<const char*>(sf_buf), make_header(d, l, 0), dev_status);
+  launch_chained(check_header_kernel, 1, 32, 0, s, reinterpret_cast<const char*>(sf_buf), make_header(d, l, 0), dev_status);
   return cudaGetLastError() == cudaSuccess ? 1 : SFB_ERR_CUDA;
 }
 

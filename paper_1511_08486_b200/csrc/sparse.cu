@@ -48,6 +48,7 @@ __device__ __forceinline__ CsrRow csr_row(const CsrView& c, int i) {
 // Wt[d][j] = W[j][d]; Wt rows have ldt values (J rounded up to 4), pad columns zero.
 __global__ void __launch_bounds__(256) transpose_kernel(const float* __restrict__ W, float* __restrict__ Wt, int J, int D,
                                                         int ldt) {
+  chain();
   __shared__ float tile[32][33];
   const int d0 = blockIdx.x * 32, j0 = blockIdx.y * 32;
   const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;   // 32 x 8
@@ -68,6 +69,7 @@ __global__ void __launch_bounds__(256) transpose_kernel(const float* __restrict_
 __global__ void __launch_bounds__(256) sc_forward_kernel(const float* __restrict__ Wt, int ldt, CsrView codes,
                                                          const float* __restrict__ Xdata, RowMap u, int K, int J, int D,
                                                          int* dev_status) {
+  chain();
   __shared__ uint32_t s_idx[256];
   __shared__ float s_val[256];
   const int i = blockIdx.x;
@@ -123,6 +125,7 @@ __global__ void __launch_bounds__(256) sc_forward_kernel(const float* __restrict
 // One block per sample: zero the dense row, then scatter the sample's nonzeros into it.
 __global__ void __launch_bounds__(256) densify_kernel(CsrView codes, RowMap a, int K, int D, int* dev_status,
                                                       bool round_tf32) {
+  chain();
   const int i = blockIdx.x;
   float* dst = reinterpret_cast<float*>(a.row(i));
   for (int q = threadIdx.x; q < (a.ld >> 2); q += 256) reinterpret_cast<float4*>(dst)[q] = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -145,6 +148,7 @@ __global__ void __launch_bounds__(256) densify_kernel(CsrView codes, RowMap a, i
 // compensated path: the row goes out in whole 16-byte units together with its correction operands.
 __global__ void __launch_bounds__(256) densify_corr_kernel(CsrView codes, RowMap a, int K, int D, int* dev_status,
                                                            CorrOut corr) {
+  chain();
   extern __shared__ __align__(16) float dense[];
   const int i = blockIdx.x;
   const int units = a.ld >> 2;
@@ -167,6 +171,7 @@ __global__ void __launch_bounds__(256) densify_corr_kernel(CsrView codes, RowMap
 
 __global__ void __launch_bounds__(256) finish_sc_kernel(RowMap zr, RowMap u, const float* __restrict__ Xdata, int K, int J,
                                                         int nsplit, long long zstride, CorrOut corr) {
+  chain();
   const int units = u.ld >> 2;
   const long long total = (long long)K * units;
   for (long long g = blockIdx.x * (long long)blockDim.x + threadIdx.x; g < total;
@@ -346,15 +351,15 @@ int launch_sc_forward_ws(cudaStream_t s, const float* W, float* Wt, CsrView code
                          int J, int D, int* dev_status) {
   const int ldt = (int)pad_to(J, 4);
   dim3 tg((D + 31) / 32, (ldt + 31) / 32);
-  transpose_kernel<<<tg, 256, 0, s>>>(W, Wt, J, D, ldt);
+  launch_chained(transpose_kernel, tg, 256, 0, s, W, Wt, J, D, ldt);
   const int cols = ldt > u.ld ? ldt : u.ld;   // pad columns of a wider u row are written (as zeros) too
   dim3 grid(K, (cols + 1023) / 1024);
-  sc_forward_kernel<<<grid, 256, 0, s>>>(Wt, ldt, codes, Xdata, u, K, J, D, dev_status);
+  launch_chained(sc_forward_kernel, grid, 256, 0, s, Wt, ldt, codes, Xdata, u, K, J, D, dev_status);
   return cudaGetLastError() == cudaSuccess ? 2 : SFB_ERR_CUDA;
 }
 
 int launch_densify_codes(cudaStream_t s, CsrView codes, RowMap a, int K, int D, int* dev_status, bool round_tf32) {
-  densify_kernel<<<K, 256, 0, s>>>(codes, a, K, D, dev_status, round_tf32);
+  launch_chained(densify_kernel, K, 256, 0, s, codes, a, K, D, dev_status, round_tf32);
   return cudaGetLastError() == cudaSuccess ? 1 : SFB_ERR_CUDA;
 }
 
@@ -365,7 +370,7 @@ int launch_densify_codes_corr(cudaStream_t s, CsrView codes, RowMap a, int K, in
   static PerDeviceOnce attr_once;   // function attributes are per device
   if (attr_once.first())
     cudaFuncSetAttribute(densify_corr_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-  densify_corr_kernel<<<K, 256, smem, s>>>(codes, a, K, D, dev_status, corr);
+  launch_chained(densify_corr_kernel, K, 256, smem, s, codes, a, K, D, dev_status, corr);
   return cudaGetLastError() == cudaSuccess ? 1 : SFB_ERR_CUDA;
 }
 
@@ -373,7 +378,7 @@ int launch_finish_sc(cudaStream_t s, RowMap z, RowMap u, const float* Xdata, int
                      long long split_stride_bytes, CorrOut corr) {
   const long long total = (long long)K * (u.ld >> 2);
   const int blocks = (int)((total + 255) / 256 < 148LL * 16 ? (total + 255) / 256 : 148LL * 16);
-  finish_sc_kernel<<<blocks, 256, 0, s>>>(z, u, Xdata, K, J, nsplit, split_stride_bytes / 4, corr);
+  launch_chained(finish_sc_kernel, blocks, 256, 0, s, z, u, Xdata, K, J, nsplit, split_stride_bytes / 4, corr);
   return cudaGetLastError() == cudaSuccess ? 1 : SFB_ERR_CUDA;
 }
 

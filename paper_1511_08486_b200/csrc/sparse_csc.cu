@@ -175,6 +175,7 @@ __global__ void __launch_bounds__(CSC2_WARPS * 32) csc_apply_kernel(float* __res
                                                                     float eta, const int* __restrict__ colptr,
                                                                     const int2* __restrict__ ent, int passes, int Kh,
                                                                     const int* __restrict__ status_ro) {
+  chain();
   extern __shared__ __align__(16) float smem[];
   if (status_ro != nullptr && (*status_ro & SFB_DEV_BAD_HEADER)) return;
   float* Us = smem;                                   // [Kh][64]
@@ -368,7 +369,7 @@ int launch_sc_csc_apply(cudaStream_t s, float* W, RowMap u, int K, int J, int D,
   long long blocks = (work + CSC2_WARPS - 1) / CSC2_WARPS;   // at least one block of atoms per warp
   if (blocks > 148) blocks = 148;
   const size_t smem = (size_t)sl.Kh * 256 + (size_t)CSC2_WARPS * CSC2_WARP_FLOATS * 4;
-  csc_apply_kernel<<<(unsigned)blocks, CSC2_WARPS * 32, smem, s>>>(W, u, K, J, D, eta, w.colptr, w.ent, sl.passes, sl.Kh,
+  launch_chained(csc_apply_kernel, (unsigned)blocks, CSC2_WARPS * 32, smem, s, W, u, K, J, D, eta, w.colptr, w.ent, sl.passes, sl.Kh,
                                                                    dev_status_ro);
   return cudaGetLastError() == cudaSuccess ? 1 : SFB_ERR_CUDA;
 }

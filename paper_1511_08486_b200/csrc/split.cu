@@ -42,6 +42,7 @@ __device__ __forceinline__ void split8(const float4& x0, const float4& x1, uint4
 // K-major.  One thread per (row, 8 values); cols is a multiple of 4, rows are 16-byte aligned.
 __global__ void __launch_bounds__(256) split_k_kernel(RowMap src, int rows, int cols, int atoms, uint4* __restrict__ dst,
                                                       int a_side) {
+  chain();
   const long long t = (long long)blockIdx.x * 256 + threadIdx.x;
   const int per_row = atoms * 4;
   const long long row = t / per_row;
@@ -63,6 +64,7 @@ __global__ void __launch_bounds__(256) split_k_kernel(RowMap src, int rows, int 
 // MN-major.  grid = (reduction blocks, groups of 8 units of 8 values along the padded row); block = 32 lines x 8 units.
 __global__ void __launch_bounds__(256) split_mn_kernel(RowMap src, int cols, int workers, int k_bb, int k_wp, int k_bpw,
                                                        uint4* __restrict__ dst, int ldc, int a_side) {
+  chain();
   const int unit = blockIdx.y * 8 + (threadIdx.x & 7);   // 8 values = 16 bytes of bf16
   const int line = threadIdx.x >> 3;                      // 0..31: pair inside the reduction block
   const int blk = blockIdx.x;
@@ -91,7 +93,7 @@ int launch_split_k(cudaStream_t s, RowMap src, int rows, int cols, void* dst, bo
   if (rows <= 0) return 0;
   const int atoms = (cols + 31) / 32;
   const long long threads = (long long)rows * atoms * 4;
-  split_k_kernel<<<(unsigned)((threads + 255) / 256), 256, 0, s>>>(src, rows, cols, atoms, reinterpret_cast<uint4*>(dst),
+  launch_chained(split_k_kernel, (unsigned)((threads + 255) / 256), 256, 0, s, src, rows, cols, atoms, reinterpret_cast<uint4*>(dst),
                                                                   a_side ? 1 : 0);
   return cudaGetLastError() == cudaSuccess ? 1 : SFB_ERR_CUDA;
 }
@@ -100,7 +102,7 @@ int launch_split_mn(cudaStream_t s, RowMap src, int cols, int workers, int k_bb,
                     void* dst, int ldc, bool a_side) {
   if (blocks <= 0) return 0;
   const dim3 grid((unsigned)blocks, (unsigned)((ldc / 8 + 7) / 8));
-  split_mn_kernel<<<grid, 256, 0, s>>>(src, cols, workers, k_bb, k_wp, k_bpw, reinterpret_cast<uint4*>(dst), ldc,
+  launch_chained(split_mn_kernel, grid, 256, 0, s, src, cols, workers, k_bb, k_wp, k_bpw, reinterpret_cast<uint4*>(dst), ldc,
                                        a_side ? 1 : 0);
   return cudaGetLastError() == cudaSuccess ? 1 : SFB_ERR_CUDA;
 }

@@ -39,6 +39,7 @@ __device__ __forceinline__ float warp_sum(float v) {
 }
 
 __global__ void __launch_bounds__(T) step_small_kernel(const __grid_constant__ SmallStep p) {
+  chain();
   extern __shared__ __align__(16) float smem[];
   float* Xs = smem;                       // [K][dp]
   float* Ws = Xs + p.K * p.dp;            // [J][dp]
@@ -193,7 +194,7 @@ int launch_step_small(cudaStream_t s, const sfb_desc& d, float* W, const float* 
   p.dp = odd_units(d.D); p.jp = odd_units(d.J);
   p.dev_status = dev_status;
   p.commit = commit;
-  step_small_kernel<<<1, T, smem_bytes(K, d.J, d.D), s>>>(p);
+  launch_chained(step_small_kernel, 1, T, smem_bytes(K, d.J, d.D), s, p);
   return cudaGetLastError() == cudaSuccess ? 1 : SFB_ERR_CUDA;
 }
 

@@ -178,7 +178,7 @@ umma_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
   SharedCtl* ctl = reinterpret_cast<SharedCtl*>(tiles + STAGES * STAGE_BYTES + EPI_STAGE_BYTES);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  if (p.status_ro != nullptr && (*p.status_ro & SFB_DEV_BAD_HEADER)) return;   // uniform over the grid
+  chain_next();
 
   const uint32_t rank = (CG == 2) ? ptx::cluster_ctarank() : 0u;   // 0 = the CTA that issues the MMAs
   const int cluster_id = blockIdx.x / CG, num_clusters = gridDim.x / CG;
@@ -196,6 +196,7 @@ umma_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
     if (APPLY) {
       int tot = p.k_blocks;
       if (p.dir != nullptr) {   // only with B >= BK and at most MAX_DIR_WORKERS workers (the host checks)
+        chain_wait();
         tot = 0;
         for (int w = 0; w < p.P; ++w) {
           const int n = min((int)p.dir[w * 8 + 1], p.B);
@@ -220,6 +221,8 @@ umma_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
   if (CG == 2) ptx::cluster_sync();   // the peer's barriers exist before anything is signalled remotely
   ptx::tc_fence_after();
   const uint32_t tmem_base = ctl->tmem_base;
+  chain_wait();   // all of the above was set-up; from here on memory that earlier kernels wrote
+  const bool refused = p.status_ro != nullptr && (*p.status_ro & SFB_DEV_BAD_HEADER);   // uniform over the grid
   // apply: every worker contributes its own number of reduction blocks; none at all = nothing to add to W
   const int k_blocks = APPLY ? ctl->k_total : p.k_blocks;
   const int k_per_split = APPLY ? k_blocks : p.k_per_split;
@@ -229,7 +232,7 @@ umma_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
   // ranges of a tile one after the other instead, the compensated forward at 1000 x 20000, K = 1024 took 155 us, now 121;
   // at 4096 x 10000 254, now 226.)
   const int tile_count = p.m_tiles * p.n_tiles;
-  const int total_work = (APPLY && k_blocks == 0) ? 0 : tile_count * p.k_splits;
+  const int total_work = (refused || (APPLY && k_blocks == 0)) ? 0 : tile_count * p.k_splits;
 
   if (warp < EPI_WARP0) {
   if (SPLIT) ptx::regs_dec<56>();   // 128 x 56 + 256 x 224 registers = the 384 x 168 of the launch
@@ -779,19 +782,21 @@ int launch_gemm(cudaStream_t s, const CUtensorMap& a, const CUtensorMap& b, cons
   const int tiles = p.m_tiles * p.n_tiles * p.k_splits;
   if (CG == 1) {
     const int grid = tiles < num_sms ? tiles : num_sms;
-    kernel<<<grid, threads, smem, s>>>(a, b, w, ac, bc, p);
+    if (launch_chained(kernel, grid, threads, smem, s, a, b, w, ac, bc, p) != cudaSuccess) return SFB_ERR_CUDA;
   } else {
     const int clusters = tiles < max_clusters ? tiles : max_clusters;
     cudaLaunchConfig_t cfg;
     memset(&cfg, 0, sizeof(cfg));
-    cudaLaunchAttribute at[1];
+    cudaLaunchAttribute at[2];
     at[0].id = cudaLaunchAttributeClusterDimension;
     at[0].val.clusterDim.x = 2; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
+    at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.gridDim = dim3(2 * clusters, 1, 1);
     cfg.blockDim = dim3(threads, 1, 1);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
-    cfg.attrs = at; cfg.numAttrs = 1;
+    cfg.attrs = at; cfg.numAttrs = 2;
     if (cudaLaunchKernelEx(&cfg, kernel, a, b, w, ac, bc, p) != cudaSuccess) return SFB_ERR_CUDA;
   }
   return cudaGetLastError() == cudaSuccess ? 1 : SFB_ERR_CUDA;
