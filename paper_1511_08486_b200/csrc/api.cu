@@ -166,9 +166,11 @@ int ensure_shadow(sfb_ctx* c, const void* W) {
 // workers > 0: the minibatch holds only that many workers' samples and u / v / codes start at the first of them.
 // for_apply: the apply of exactly these rows (all K pairs, no compaction in between) follows in the same call, so
 // the compensated path may write the apply's correction operands while it writes the factors.
+// defer_v: see umma_forward.
 // extra (dense v): what the finishing pass does besides (header of the buffer u and v belong to, flags of nonzero rows).
 int factors_into(sfb_ctx* c, const void* W, const void* X, const sfb_aux* aux, RowMap u, RowMap v, CsrView codes,
-                 int workers = 0, bool for_apply = false, const FinishExtra& extra = FinishExtra()) {
+                 int workers = 0, bool for_apply = false, const FinishExtra& extra = FinishExtra(),
+                 bool defer_v = false) {
   const sfb_desc& d = c->d;
   const int K = workers > 0 ? workers * d.B : c->K;
   const float* Wf = reinterpret_cast<const float*>(W);
@@ -226,7 +228,7 @@ int factors_into(sfb_ctx* c, const void* W, const void* X, const sfb_aux* aux, R
     const int r = ensure_shadow(c, W);
     if (r < 0) return r;
   }
-  ACC(umma_forward(c->umma, c->stream, W, c->w_shadow, X, aux, u, v, c->dev_status, workers, for_apply, extra));
+  ACC(umma_forward(c->umma, c->stream, W, c->w_shadow, X, aux, u, v, c->dev_status, workers, for_apply, extra, defer_v));
   return SFB_OK;
 }
 
@@ -567,9 +569,10 @@ int sfb_pack(sfb_ctx* c, const void* U, const void* V, const sfb_aux* aux, void*
 }
 
 // csc_built: the atom-major re-sort of this buffer's codes for these K samples is already in the workspace
+// v_rows (tensor-core paths): where the factor rows v can be read instead of in the buffer (the same values)
 // active_rows: c->dml_active describes the u rows of this buffer (set by the factor stage of the same step)
 static int apply_from(sfb_ctx* c, void* W, const void* sf_buf, float eta, int K, bool check, bool csc_built = false,
-                      bool active_rows = false) {
+                      bool active_rows = false, const RowMap* v_rows = nullptr) {
   const sfb_desc& d = c->d;
   if (check) ACC(launch_check_header(c->stream, sf_buf, d, c->l, c->dev_status));
   if (d.v_sparse && d.path == SFB_PATH_F32 && c->csc_ws != nullptr) {
@@ -604,7 +607,8 @@ static int apply_from(sfb_ctx* c, void* W, const void* sf_buf, float eta, int K,
     ACC(launch_apply_f32(c->stream, reinterpret_cast<float*>(W), stream_u(c, sf_buf), stream_v(c, sf_buf), K, d.J, d.D,
                          eta, c->dev_status, idx, n_idx));
   } else {
-    ACC(umma_apply(c->umma, c->stream, W, c->w_shadow, stream_u(c, sf_buf), stream_v(c, sf_buf), eta, K, c->dev_status,
+    ACC(umma_apply(c->umma, c->stream, W, c->w_shadow, stream_u(c, sf_buf),
+                   v_rows != nullptr ? *v_rows : stream_v(c, sf_buf), eta, K, c->dev_status,
                    d.compact ? reinterpret_cast<const char*>(sf_buf) + 128 : nullptr));
     // The apply epilogue rewrote the shadow from the new W.  (A compacted buffer without a single pair launches no
     // tile: W and a shadow that mirrored it stay as they were; a stale shadow stays stale.)
@@ -727,19 +731,24 @@ int sfb_step(sfb_ctx* c, void* W, const void* X, const sfb_aux* aux, void* sf_bu
     join_aux();
     return SFB_ERR_CUDA;
   }
+  // MLR: the factor v is a copy of the samples, so the update can take the samples themselves and the copy into the
+  // buffer only has to be done by the end of the step (a large one runs on the side stream beside both GEMMs: V_INLINE_BYTES)
+  const bool defer_v = d.model == SFB_MLR && !d.compact && (d.path == SFB_PATH_TF32 || d.path == SFB_PATH_BF16);
+  const RowMap x_rows = caller_rows(X, d.D, d.B, c->l.es);
   FinishExtra extra;
   if (!d.v_sparse) extra.commit = commit;
   if (d.compact) extra.nonzero = compact_flags(c->compact_ws);
   r = factors_into(c, W, X, aux, stream_u(c, sf_buf), d.v_sparse ? RowMap() : stream_v(c, sf_buf), codes, 0,
-                   d.path == SFB_PATH_TF32X3 && !d.compact && K == c->K, extra);
+                   d.path == SFB_PATH_TF32X3 && !d.compact && K == c->K, extra, defer_v);
   if (forked && cudaStreamWaitEvent(c->stream, c->aux_join, 0) != cudaSuccess) return SFB_ERR_CUDA;
-  if (r < 0) return r;
+  if (r < 0) return r;   // (umma_forward has joined its side stream)
   // pairs whose u came out as zero are dropped from the message before it is "sent" (and applied)
   if (d.compact) ACC(launch_compact(c->stream, sf_buf, d, c->l, c->compact_ws, 0, 0, true));
   if (c->profiling) cudaEventRecord(c->prof_ev[slot][1], c->stream);
   const bool listed = !d.compact && d.model == SFB_DML && d.path == SFB_PATH_F32 && c->dml_active != nullptr &&
                       (long long)((d.J + 127) / 128) * ((d.D + 127) / 128) >= 148;   // the large-tile apply takes the list
-  r = apply_from(c, W, sf_buf, eta, K, false, csc_built, listed);
+  r = apply_from(c, W, sf_buf, eta, K, false, csc_built, listed, defer_v ? &x_rows : nullptr);
+  if (defer_v && umma_join(c->umma, c->stream) < 0 && r >= 0) r = SFB_ERR_CUDA;
   c->last_step_K = K;
   c->last_step_listed = listed;
   if (c->profiling) {

@@ -900,7 +900,7 @@ struct UmmaPlan {
   // next to the forward GEMM (fork / join by events)
   cudaStream_t side;
   cudaEvent_t fork, join;
-  bool side_ok;
+  bool side_ok, side_open;   // open: a copy is on the side stream that nothing has joined yet
   // Test hook.  SFB_TEST_LOSE_SIGNAL=1 in the environment at plan creation: the first GEMM launched through this
   // plan loses one pipeline signal in its first CTA (pair), which must end in SFB_DEV_TIMEOUT after the bounded
   // wait, not in a hang.  The only environment variable the library reads.
@@ -980,7 +980,7 @@ int umma_plan_create(const sfb_desc& d, const Layout& l, UmmaPlan** out) {
       return SFB_ERR_ALLOC;
     }
   }
-  p->side_ok = false;
+  p->side_ok = p->side_open = false;
   {
     if (d.model == SFB_MLR) {
       p->side_ok = cudaStreamCreateWithFlags(&p->side, cudaStreamNonBlocking) == cudaSuccess;
@@ -1262,9 +1262,19 @@ int umma_forward_sc(UmmaPlan* pl, cudaStream_t s, const void* W, RowMap a, RowMa
   return launches + r;
 }
 
+// Every exit of a call (errors included) makes `s` wait for the side stream, so the caller's stream never runs ahead of
+// the copy and a stream capture in progress stays well formed.
+int umma_join(UmmaPlan* pl, cudaStream_t s) {
+  if (!pl->side_open) return SFB_OK;
+  pl->side_open = false;
+  if (cudaEventRecord(pl->join, pl->side) != cudaSuccess || cudaStreamWaitEvent(s, pl->join, 0) != cudaSuccess)
+    return SFB_ERR_CUDA;
+  return SFB_OK;
+}
+
 int umma_forward(UmmaPlan* pl, cudaStream_t s, const void* W, const __nv_bfloat16* w_shadow, const void* X,
                  const sfb_aux* aux, RowMap u, RowMap v, int* dev_status, int workers, bool for_apply,
-                 const FinishExtra& extra_in) {
+                 const FinishExtra& extra_in, bool defer_v) {
   const sfb_desc& d = pl->d;
   const int K = (workers > 0 ? workers : d.P) * d.B;
   int launches = 0, r;
@@ -1299,14 +1309,7 @@ int umma_forward(UmmaPlan* pl, cudaStream_t s, const void* W, const __nv_bfloat1
         return SFB_ERR_CUDA;
       forked = true;
     }
-    // Once forked, every exit (errors included) makes `s` wait for the side stream, so the caller's stream
-    // never runs ahead of the copy and a stream capture in progress stays well formed.
-    auto join_side = [&]() -> int {
-      if (!forked) return 0;
-      if (cudaEventRecord(pl->join, pl->side) != cudaSuccess || cudaStreamWaitEvent(s, pl->join, 0) != cudaSuccess)
-        return SFB_ERR_CUDA;
-      return 0;
-    };
+    pl->side_open = forked;
     auto body = [&]() -> int {
       if (forked) {
         if ((r = launch_copy_rows(pl->side, x_rows, v, K, d.D, cv)) < 0) return r;
@@ -1348,7 +1351,7 @@ int umma_forward(UmmaPlan* pl, cudaStream_t s, const void* W, const __nv_bfloat1
       return 0;
     };
     const int rb = body();
-    const int rj = join_side();
+    const int rj = defer_v && rb >= 0 ? 0 : umma_join(pl, s);
     if (rb < 0 || rj < 0) pl->fresh_u = nullptr;
     if (rb < 0) return rb;
     if (rj < 0) return rj;

@@ -15,10 +15,13 @@ void umma_plan_destroy(UmmaPlan* p);
 // for_apply (compensated path): umma_apply of exactly these u / v rows, all K pairs, follows before anything else
 // changes them: the kernels that write the factors also write the apply's correction operands (one use).
 // workers > 0: only that many workers' samples (X, aux, u, v start at the first of them).
+// defer_v: a copy of the factor v that runs on the side stream is left there; the caller calls umma_join on every path.
 // extra: what the finishing pass does besides (header, flags of nonzero rows).
 int umma_forward(UmmaPlan* p, cudaStream_t s, const void* W, const __nv_bfloat16* w_shadow, const void* X,
                  const sfb_aux* aux, RowMap u, RowMap v, int* dev_status, int workers = 0, bool for_apply = false,
-                 const FinishExtra& extra = FinishExtra());
+                 const FinishExtra& extra = FinishExtra(), bool defer_v = false);
+
+int umma_join(UmmaPlan* p, cudaStream_t s);
 
 // Z rows (fp32) = A rows (the path's value type) times Wop^T on the tensor cores; no epilogue beyond the store.
 // w_corr: on the compensated path, W's correction operand (launch_split_k of W's rows, B side); w_shadow plays
