@@ -106,7 +106,7 @@ __global__ void __launch_bounds__(256) compact_move_kernel(char* buf, char* stre
 // idx[0 .. *n_out) = p * B + r for every worker p < workers and every r < its pair count, in that order.
 __global__ void __launch_bounds__(256) kept_rows_kernel(const char* buf, int B, int workers, int* __restrict__ idx,
                                                         int* __restrict__ n_out) {
-  chain();
+  chain_wait();
   __shared__ int base;
   if (threadIdx.x == 0) base = 0;
   __syncthreads();

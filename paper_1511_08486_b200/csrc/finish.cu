@@ -118,7 +118,8 @@ __device__ __forceinline__ bool wire_nonzero4(const float4& t, int es) {
 __global__ void __launch_bounds__(1024) finish_mlr_kernel(RowMap z, RowMap u, const int32_t* __restrict__ labels,
                                                                  int K, int J, int cache_floats, int* dev_status, int nsplit, long long zstride,
                                                                  float* __restrict__ dual, float sdca_step, CorrOut corr, const __grid_constant__ FinishExtra extra) {
-  chain();
+  if (extra.next_early) chain_next();
+  chain_wait();
   extern __shared__ __align__(16) float cache[];
   __shared__ float red[32];
   const int i = blockIdx.x;
@@ -199,7 +200,8 @@ __global__ void __launch_bounds__(1024) finish_mlr_kernel(RowMap z, RowMap u, co
 __global__ void __launch_bounds__(1024) finish_dml_kernel(RowMap z, RowMap u, const uint8_t* __restrict__ similar,
                                                                  float margin, int K, int J, int cache_floats, int nsplit, long long zstride,
                                                                  uint8_t* __restrict__ active, CorrOut corr, const __grid_constant__ FinishExtra extra) {
-  chain();
+  if (extra.next_early) chain_next();
+  chain_wait();
   extern __shared__ __align__(16) float cache[];
   __shared__ float red[32];
   const int i = blockIdx.x;
@@ -252,7 +254,8 @@ __global__ void __launch_bounds__(256) finish_mlr_fused_kernel(RowMap u, const f
                                                                int part_cols, const int32_t* __restrict__ labels, int K,
                                                                int J, int* dev_status, float* __restrict__ dual,
                                                                float sdca_step, const __grid_constant__ FinishExtra extra) {
-  chain();
+  if (extra.next_early) chain_next();
+  chain_wait();
   extern __shared__ float scale[];   // [n_parts]
   __shared__ float red[32];
   const int i = blockIdx.x;
@@ -510,7 +513,7 @@ int launch_finish_mlr(cudaStream_t s, RowMap z, RowMap u, const int32_t* labels,
 // idx[0 .. n) = the samples i < K with active[i] != 0, in ascending order; *n_out = n.  One block, ordered.
 __global__ void __launch_bounds__(1024) compact_active_kernel(const uint8_t* __restrict__ active, int K, int* __restrict__ idx,
                                                               int* __restrict__ n_out) {
-  chain();
+  chain_wait();
   __shared__ int warp_cnt[32];
   __shared__ int base;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;

@@ -68,7 +68,7 @@ template <int MI, int NI>
 __global__ void __launch_bounds__(256, 2) forward_f32_kernel(const float* __restrict__ W, const float* __restrict__ X,
                                                           const float* __restrict__ Xb, int K, int J, int D,
                                                           RowMap z, RowMap v, int d_per_split, long long split_stride) {
-  chain();
+  chain_wait();
   constexpr int BM = 64 * MI, BN = 64 * NI;
   __shared__ __align__(16) float As[BK][BM + 4];
   __shared__ __align__(16) float Bs[BK][BN + 4];
@@ -157,7 +157,7 @@ __global__ void __launch_bounds__(256, 2) forward_f32_kernel(const float* __rest
 template <int MI, int NI>
 __global__ void __launch_bounds__(256, 2) apply_f32_kernel(float* __restrict__ W, RowMap u, RowMap v, int K, int J,
                                                         int D, float eta, const int* __restrict__ dev_status) {
-  chain();
+  chain_wait();
   constexpr int BM = 64 * MI, BN = 64 * NI;
   __shared__ __align__(16) float As[BK][BM + 4];
   __shared__ __align__(16) float Bs[BK][BN + 4];
@@ -253,7 +253,7 @@ __global__ void __launch_bounds__(256, 2) sgemm_pipe_kernel(float* __restrict__ 
                                                          int D, float eta, const int* __restrict__ dev_status,
                                                          RowMap z, int k_per_range, long long range_stride,
                                                          const int* __restrict__ row_idx, const int* __restrict__ n_rows) {
-  chain();
+  chain_wait();
   constexpr int BM = 128, BN = 128;
   extern __shared__ __align__(16) float ring[];
   if (OUT == 0 && dev_status != nullptr && (*dev_status & SFB_DEV_BAD_HEADER)) return;
@@ -356,7 +356,7 @@ __global__ void __launch_bounds__(256, 2) sgemm_pipe_kernel(float* __restrict__ 
 // zero).  `copy` (optional): the same rows also copied there, pad columns zero (the factor v = x of the MLR model).
 __global__ void __launch_bounds__(256) transpose_rows_kernel(RowMap src, float* __restrict__ dst, int R, int C, int ldr,
                                                              RowMap copy) {
-  chain();
+  chain_wait();
   __shared__ float tile[32][33];
   const int c0 = blockIdx.x * 32, r0 = blockIdx.y * 32;
   const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;   // 32 x 8
@@ -386,7 +386,7 @@ struct TransposeJob {
   RowMap copy;
 };
 __global__ void __launch_bounds__(256) transpose_rows_vec_kernel(TransposeJob j0, TransposeJob j1) {
-  chain();
+  chain_wait();
   __shared__ float tile[64][65];
   const TransposeJob& j = blockIdx.z == 0 ? j0 : j1;
   const int c0 = blockIdx.x * 64, r0 = blockIdx.y * 64;

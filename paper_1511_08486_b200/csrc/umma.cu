@@ -1290,6 +1290,7 @@ int umma_forward(UmmaPlan* pl, cudaStream_t s, const void* W, const __nv_bfloat1
   x_rows.ld = d.D; x_rows.B = d.B; x_rows.es = pl->es;
   x_rows.worker_stride = (long long)d.B * d.D * pl->es;
   FinishExtra extra = extra_in;
+  extra.next_early = true;
   if (d.model == SFB_MLR) {
     const bool bf16 = d.path == SFB_PATH_BF16;
     bool forked = false;
