@@ -202,18 +202,22 @@ int factors_into(sfb_ctx* c, const void* W, const void* X, const sfb_aux* aux, R
     const RowMap part = caller_rows(c->f32_part, c->ldp, d.B, 4);
     const long long sstride = (long long)c->K * c->ldp * 4;
     int ks = 1;
-    if (c->f32_nn_ws != nullptr && (Xb == nullptr || v.base != nullptr)) {
+    if (forward_f32_fused(K, d.J, d.D) || (Xb != nullptr && v.base == nullptr)) {
+      ACC(launch_forward_f32(c->stream, Wf, reinterpret_cast<const float*>(X), Xb, K, d.J, d.D, u, v));
+    } else {
       RowMap src = caller_rows(X, d.D, d.B, 4), copy = v;
       if (Xb != nullptr) {   // pair differences first (they are the factor v), then contracted from there
         ACC(launch_diff_rows(c->stream, reinterpret_cast<const float*>(X), Xb, v, K, d.D));
         src = v;
         copy = RowMap();
       }
-      ACC(launch_forward_f32_nn(c->stream, Wf, src, copy, K, d.J, d.D, c->f32_nn_ws, u, part, sstride, c->f32_splits,
-                                &ks));
-    } else {
-      ACC(launch_forward_f32(c->stream, Wf, reinterpret_cast<const float*>(X), Xb, K, d.J, d.D, u, v, part, sstride,
-                             c->f32_splits, &ks));
+      // a shard of the workers stays within the partial buffers and transposed copies of the whole
+      int want = forward_f32_splits(K, d.J, d.D);
+      if (want > c->f32_splits) want = c->f32_splits;
+      if (forward_f32_transposed(K, d.J, d.D) && c->f32_nn_ws != nullptr)
+        ACC(launch_forward_f32_nn(c->stream, Wf, src, copy, K, d.J, d.D, c->f32_nn_ws, u, part, sstride, want, &ks));
+      else
+        ACC(launch_forward_f32_small(c->stream, Wf, src, copy, K, d.J, d.D, u, part, sstride, want, &ks));
     }
     const RowMap zsrc = ks > 1 ? part : u;
     if (d.model == SFB_MLR)
@@ -306,9 +310,9 @@ int sfb_create(const sfb_desc* desc, void* cuda_stream, sfb_ctx** out) {
       ok = cudaMalloc(&c->dml_active, (size_t)c->K) == cudaSuccess;
       if (ok) ok = cudaMalloc(&c->dml_idx, ((size_t)c->K + 1) * 4) == cudaSuccess;
     }
-    // shapes with at least a tile of work per dimension take the forward through transposed operand copies
+    // large shapes take the forward through transposed operand copies
     const long long nn_floats = forward_f32_nn_workspace_floats(c->K, desc->J, desc->D);
-    if (ok && c->K >= 128 && desc->J >= 64 && desc->D >= 512 && nn_floats * 4 <= (2LL << 30))
+    if (ok && forward_f32_transposed(c->K, desc->J, desc->D) && nn_floats * 4 <= (2LL << 30))
       ok = cudaMalloc(&c->f32_nn_ws, (size_t)nn_floats * 4) == cudaSuccess;
   }
   if (ok) {

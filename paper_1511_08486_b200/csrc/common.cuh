@@ -231,24 +231,29 @@ struct PerDeviceOnce {
 
 // ---- kernel launchers (each returns the number of kernels it launched, or a negative SFB_ERR_*) ----
 
-// Z[i][j] = sum_d A[i][d] * W[j][d] on fp32 CUDA cores, written as fp32 rows through `z`.
-// A = X, or X - Xb (element-wise fp32 subtraction) when Xb != nullptr.  When `v` has a base, the
-// operand rows (X, or the difference) are also written there (the factor v), pad columns zero.
-// With a `part` row map (fp32 rows, split_stride bytes between partial buffers) and nsplit_out, a problem
-// with few tiles has its reduction cut into *nsplit_out ranges whose partial products go to `part` instead
-// of `z` (the finishing pass sums them in range order); forward_f32_splits tells how many in advance.
 // v rows = Xa rows - Xb rows, one fp32 subtraction per element, pad columns zero (the DML factor v).
 int launch_diff_rows(cudaStream_t s, const float* Xa, const float* Xb, RowMap v, int K, int D, CorrOut corr = CorrOut());
+// Z[i][j] = sum_d A[i][d] * W[j][d] on fp32 CUDA cores, written as fp32 rows through `z`.
+// A = X, or X - Xb (element-wise fp32 subtraction) when Xb != nullptr.  When `v` has a base, the
+// operand rows (X, or the difference) are also written there (the factor v), pad columns zero.  One launch: for problems
+// that forward_f32_fused tells are small, and where the difference is not kept.
+bool forward_f32_fused(int K, int J, int D);
+int launch_forward_f32(cudaStream_t s, const float* W, const float* X, const float* Xb, int K, int J, int D,
+                       RowMap z, RowMap v);
+// The same for operand rows a_i behind a row map; copy (optional): those rows also written there.  The reduction is cut
+// into ks ranges (*nsplit_out of them exist) whose partial products go to `part` (fp32 rows, split_stride bytes between
+// partial buffers) instead of `z` if there is more than one; the finishing pass sums them in range order.
+// forward_f32_splits: how many to ask for, at most FORWARD_F32_MAX_SPLITS; forward_f32_transposed: by which of the two.
+//   _small: 64 x 64 tiles, operands in place.  _nn: large tiles through transposed copies of both operands; ws:
+//   forward_f32_nn_workspace_floats(K, J, D) floats.
+constexpr int FORWARD_F32_MAX_SPLITS = 32;
 int forward_f32_splits(int K, int J, int D);
-// The same contraction through transposed copies of both operands (two transposing passes, then the pipelined
-// large-tile kernel).  src: operand rows a_i behind a row map; copy (optional): those rows also written there;
-// ws: forward_f32_nn_workspace_floats(K, J, D) floats.  Needs at least one full 128 x 128 tile of work to pay.
+bool forward_f32_transposed(int K, int J, int D);
+int launch_forward_f32_small(cudaStream_t s, const float* W, RowMap src, RowMap copy, int K, int J, int D, RowMap z,
+                             RowMap part, long long split_stride, int ks, int* nsplit_out);
 long long forward_f32_nn_workspace_floats(int K, int J, int D);
 int launch_forward_f32_nn(cudaStream_t s, const float* W, RowMap src, RowMap copy, int K, int J, int D, float* ws,
-                          RowMap z, RowMap part, long long split_stride, int max_splits, int* nsplit_out);
-int launch_forward_f32(cudaStream_t s, const float* W, const float* X, const float* Xb, int K, int J, int D,
-                       RowMap z, RowMap v, RowMap part = RowMap(), long long split_stride = 0, int max_splits = 1,
-                       int* nsplit_out = nullptr);
+                          RowMap z, RowMap part, long long split_stride, int ks, int* nsplit_out);
 
 // W[j][d] -= eta * sum_{i<K} U[i][j] * V[i][d] on fp32 CUDA cores (fixed summation order).
 int launch_apply_f32(cudaStream_t s, float* W, RowMap u, RowMap v, int K, int J, int D, float eta,

@@ -61,13 +61,14 @@ __device__ __forceinline__ void mma_tile(const float (*As)[64 * MI + 4], const f
   }
 }
 
-// ------------------------------------------------------------------------------------------ forward
+// ------------------------------------------------------------------------------------------ forward, one launch
+// For the smallest problems, and where the pair difference is formed on the way (sfb_loss).
 // Tile rows = samples i (BM = 64*MI), tile columns = classes j (BN = 64*NI), reduction over d.
 // Both operands are contiguous along d, so tiles are transposed while being stored to shared memory.
 template <int MI, int NI>
 __global__ void __launch_bounds__(256, 2) forward_f32_kernel(const float* __restrict__ W, const float* __restrict__ X,
                                                           const float* __restrict__ Xb, int K, int J, int D,
-                                                          RowMap z, RowMap v, int d_per_split, long long split_stride) {
+                                                          RowMap z, RowMap v) {
   chain_wait();
   constexpr int BM = 64 * MI, BN = 64 * NI;
   __shared__ __align__(16) float As[BK][BM + 4];
@@ -119,15 +120,11 @@ __global__ void __launch_bounds__(256, 2) forward_f32_kernel(const float* __rest
     }
   };
 
-  // blockIdx.z takes the reduction range [d_lo, d_hi) and writes its partial products split_stride bytes
-  // after the previous range's (one range: the whole reduction, written to z itself)
-  const int d_lo = blockIdx.z * d_per_split;
-  const int d_hi = min(D, d_lo + d_per_split);
-  fetch(d_lo);
-  for (int d0 = d_lo; d0 < d_hi; d0 += BK) {
+  fetch(0);
+  for (int d0 = 0; d0 < D; d0 += BK) {
     stash();
     __syncthreads();
-    if (d0 + BK < d_hi) fetch(d0 + BK);
+    if (d0 + BK < D) fetch(d0 + BK);
     mma_tile<MI, NI, false>(As, Bs, ty, tx, acc);
     __syncthreads();
   }
@@ -140,93 +137,13 @@ __global__ void __launch_bounds__(256, 2) forward_f32_kernel(const float* __rest
     for (int a = 0; a < 4; ++a) {
       const int i = i0 + mi * 64 + ty * 4 + a;
       if (i >= K) continue;
-      float* zr = reinterpret_cast<float*>(z.row(i) + blockIdx.z * split_stride);
+      float* zr = reinterpret_cast<float*>(z.row(i));
 #pragma unroll
       for (int ni = 0; ni < NI; ++ni) {
         const int j = j0 + ni * 64 + tx * 4;
         if (j < z.ld)   // ld is a multiple of 4, so the whole float4 is inside the row; columns >= J hold 0
           *reinterpret_cast<float4*>(zr + j) = make_float4(acc[mi * 4 + a][ni * 2].x, acc[mi * 4 + a][ni * 2].y,
                                                            acc[mi * 4 + a][ni * 2 + 1].x, acc[mi * 4 + a][ni * 2 + 1].y);
-      }
-    }
-}
-
-// ------------------------------------------------------------------------------------------ apply
-// Tile rows = rows j of W (BM), tile columns = columns d of W (BN), reduction over the K factors.
-// U rows are contiguous along j and V rows along d: tiles go to shared memory as they are.
-template <int MI, int NI>
-__global__ void __launch_bounds__(256, 2) apply_f32_kernel(float* __restrict__ W, RowMap u, RowMap v, int K, int J,
-                                                        int D, float eta, const int* __restrict__ dev_status) {
-  chain_wait();
-  constexpr int BM = 64 * MI, BN = 64 * NI;
-  __shared__ __align__(16) float As[BK][BM + 4];
-  __shared__ __align__(16) float Bs[BK][BN + 4];
-  if (dev_status != nullptr && (*dev_status & SFB_DEV_BAD_HEADER)) return;
-  const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15;
-  const int j0 = blockIdx.y * BM, d0 = blockIdx.x * BN;
-  const int lr = tid >> 4, lc = (tid & 15) * 4;   // loader: factor row within 16, first of 4 columns
-
-  float2 acc[4 * MI][2 * NI];
-#pragma unroll
-  for (int m = 0; m < 4 * MI; ++m)
-#pragma unroll
-    for (int n = 0; n < 2 * NI; ++n) acc[m][n] = make_float2(0.f, 0.f);
-
-  float4 pa[MI], pb[NI];
-  auto fetch = [&](int k0) {
-    const int i = k0 + lr;
-#pragma unroll
-    for (int q = 0; q < MI; ++q) {
-      const int j = j0 + lc + 64 * q;
-      pa[q] = (i < K) ? ld4_guard(reinterpret_cast<const float*>(u.row(i)), j, J, true)
-                      : make_float4(0.f, 0.f, 0.f, 0.f);
-    }
-#pragma unroll
-    for (int q = 0; q < NI; ++q) {
-      const int d = d0 + lc + 64 * q;
-      pb[q] = (i < K) ? ld4_guard(reinterpret_cast<const float*>(v.row(i)), d, D, true)
-                      : make_float4(0.f, 0.f, 0.f, 0.f);
-    }
-  };
-  auto stash = [&]() {
-#pragma unroll
-    for (int q = 0; q < MI; ++q) *reinterpret_cast<float4*>(&As[lr][lc + 64 * q]) = pa[q];
-#pragma unroll
-    for (int q = 0; q < NI; ++q) *reinterpret_cast<float4*>(&Bs[lr][lc + 64 * q]) = pb[q];
-  };
-
-  fetch(0);
-  for (int k0 = 0; k0 < K; k0 += BK) {
-    stash();
-    __syncthreads();
-    if (k0 + BK < K) fetch(k0 + BK);
-    mma_tile<MI, NI, true>(As, Bs, ty, tx, acc);
-    __syncthreads();
-  }
-
-  const bool vec_ok = (D & 3) == 0;
-#pragma unroll
-  for (int mi = 0; mi < MI; ++mi)
-#pragma unroll
-    for (int a = 0; a < 4; ++a) {
-      const int j = j0 + mi * 64 + ty * 4 + a;
-      if (j >= J) continue;
-      float* wr = W + (size_t)j * D;
-#pragma unroll
-      for (int ni = 0; ni < NI; ++ni) {
-        const int d = d0 + ni * 64 + tx * 4;
-        const float c[4] = {acc[mi * 4 + a][ni * 2].x, acc[mi * 4 + a][ni * 2].y, acc[mi * 4 + a][ni * 2 + 1].x,
-                            acc[mi * 4 + a][ni * 2 + 1].y};
-        if (vec_ok && d + 3 < D) {
-          float4 w = *reinterpret_cast<float4*>(wr + d);
-          w.x = fmaf(-eta, c[0], w.x); w.y = fmaf(-eta, c[1], w.y);
-          w.z = fmaf(-eta, c[2], w.z); w.w = fmaf(-eta, c[3], w.w);
-          *reinterpret_cast<float4*>(wr + d) = w;
-        } else {
-#pragma unroll
-          for (int b = 0; b < 4; ++b)
-            if (d + b < D) wr[d + b] = fmaf(-eta, c[b], wr[d + b]);
-        }
       }
     }
 }
@@ -352,6 +269,132 @@ __global__ void __launch_bounds__(256, 2) sgemm_pipe_kernel(float* __restrict__ 
     }
 }
 
+// ---- 64 x 64 tiles, 4 x 4 outputs per thread, the same ring: for problems whose 128 x 128 tiles leave the chip idle.
+//   OUT 0 (apply):   as above (16-byte copies; the row list too).
+//   OUT 1 (forward): A = sample rows (m = sample i), B = rows of W (n = class j), both contiguous along k = feature d, read
+//                    in place: 4-byte asynchronous copies transpose them on the way into shared memory (sixteen lanes
+//                    take 64 contiguous bytes of a row; any D), no transposing pass.  Where the factor v is a copy of the
+//                    sample rows, the blocks of a row of tiles write it from shared memory, each its share of the rows.
+// Bound: the latency of a step's copies (0.9 us for 16 steps of the forward with a block per SM), hence many short
+// ranges.  A step of 100 x 800, K = 160: 98 -> 19 us, of 40 x 15000, K = 800: 312 -> 144, of 300 x 3000, K = 400: 107 -> 69
+// (64 x 64 tiles without a ring, 128 x 128 tiles in 512-step ranges before).
+constexpr int SMALL_STAGE_FLOATS = 2 * BK * (64 + 4);
+
+__device__ __forceinline__ void cp_async4_zfill(float* dst_smem, const void* src, int src_bytes) {
+  const uint32_t d = (uint32_t)__cvta_generic_to_shared(dst_smem);
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(d), "l"(src), "r"(src_bytes) : "memory");
+}
+
+struct SmallArgs {
+  float* W;                 // OUT 0: updated in place; OUT 1: the B operand
+  RowMap a, b;              // OUT 0: u and v rows; OUT 1: a = sample rows
+  int K, M, N, ldw;         // reduction length; output rows, columns; row length of W
+  float eta;
+  const int* dev_status;
+  RowMap z, copy;           // OUT 1: products (+ range stride); optional second destination of the sample rows
+  int k_per_range;
+  long long range_stride;
+  const int* row_idx;       // OUT 0, optional: the factor rows to take
+  const int* n_rows;
+};
+
+template <int OUT>
+__global__ void __launch_bounds__(256, 4) sgemm_small_kernel(const __grid_constant__ SmallArgs p) {
+  chain_wait();
+  constexpr int BT = 64;
+  __shared__ __align__(16) float ring[PIPE * SMALL_STAGE_FLOATS];
+  __shared__ long long a_off[OUT == 1 ? BT : 1];   // byte offset of the tile's sample rows, -1: no such row
+  __shared__ long long c_off[OUT == 1 ? BT : 1];   // ... and of their copies
+  if (OUT == 0 && p.dev_status != nullptr && (*p.dev_status & SFB_DEV_BAD_HEADER)) return;
+  const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15, lane = tid & 31, warp = tid >> 5;
+  const int m0 = blockIdx.y * BT, n0 = blockIdx.x * BT;
+  const int k_lo = (OUT == 1) ? blockIdx.z * p.k_per_range : 0;
+  const int k_hi = (OUT == 1) ? min(p.K, k_lo + p.k_per_range) : (p.n_rows != nullptr ? min(p.K, *p.n_rows) : p.K);
+  if (OUT == 1) {
+    if (tid < BT) {
+      a_off[tid] = m0 + tid < p.M ? (long long)(p.a.row(m0 + tid) - p.a.base) : -1;
+      c_off[tid] = p.copy.base != nullptr && m0 + tid < p.M ? (long long)(p.copy.row(m0 + tid) - p.copy.base) : -1;
+    }
+    __syncthreads();
+  }
+  auto issue = [&](int stage, int k0) {
+    float* As = ring + stage * SMALL_STAGE_FLOATS;
+    float* Bs = As + BK * (BT + 4);
+    if (OUT == 0) {   // thread = (factor row of the step, 4 columns); nothing to read: a valid address all the same
+      const int r = tid >> 4, c = (tid & 15) * 4, i = k0 + r;
+      const bool ok = i < k_hi;
+      const int ii = ok ? (p.row_idx != nullptr ? p.row_idx[i] : i) : 0;
+      const int ub = max(0, min(16, (p.M - m0 - c) * 4)), vb = max(0, min(16, (p.N - n0 - c) * 4));
+      cp_async16_zfill(As + r * (BT + 4) + c, p.a.row(ii) + (ub > 0 ? (size_t)(m0 + c) * 4 : 0), ok ? ub : 0);
+      cp_async16_zfill(Bs + r * (BT + 4) + c, p.b.row(ii) + (vb > 0 ? (size_t)(n0 + c) * 4 : 0), ok ? vb : 0);
+    } else {
+      const int k = lane & 15, half = lane >> 4;
+      const bool ok = k0 + k < k_hi;
+      const char* abase = p.a.base + (ok ? (size_t)(k0 + k) * 4 : 0);
+      const float* wk = p.W + (ok ? k0 + k : 0);
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const int r = q * 16 + warp * 2 + half;
+        const long long off = a_off[r];
+        const bool in = n0 + r < p.N;
+        cp_async4_zfill(As + k * (BT + 4) + r, abase + (off >= 0 ? off : 0), ok && off >= 0 ? 4 : 0);
+        cp_async4_zfill(Bs + k * (BT + 4) + r, wk + (in ? (size_t)(n0 + r) * p.ldw : 0), ok && in ? 4 : 0);
+      }
+    }
+  };
+  float2 acc[4][2];
+#pragma unroll
+  for (int m = 0; m < 4; ++m) acc[m][0] = acc[m][1] = make_float2(0.f, 0.f);
+  const int nk = (k_hi - k_lo + BK - 1) / BK;
+#pragma unroll
+  for (int st = 0; st < PIPE - 1; ++st) {
+    if (st < nk) issue(st, k_lo + st * BK);
+    cp_async_commit();
+  }
+  for (int kt = 0; kt < nk; ++kt) {
+    cp_async_wait<PIPE - 2>();
+    __syncthreads();
+    const int nxt = kt + PIPE - 1;
+    if (nxt < nk) issue(nxt % PIPE, k_lo + nxt * BK);
+    cp_async_commit();
+    const float* As = ring + (kt % PIPE) * SMALL_STAGE_FLOATS;
+    if (OUT == 1 && p.copy.base != nullptr) {   // four steps of a row per thread; rows blockIdx.x, + gridDim.x, ...
+      const int k = (tid & 3) * 4, kk = k_lo + kt * BK + k;
+      for (int r = blockIdx.x + gridDim.x * (tid >> 2); r < BT; r += gridDim.x * 64)
+        if (c_off[r] >= 0 && kk < p.copy.ld)
+          *reinterpret_cast<float4*>(p.copy.base + c_off[r] + (size_t)kk * 4) =
+              make_float4(As[k * (BT + 4) + r], As[(k + 1) * (BT + 4) + r], As[(k + 2) * (BT + 4) + r],
+                          As[(k + 3) * (BT + 4) + r]);
+    }
+    mma_tile<1, 1, true>(reinterpret_cast<const float(*)[BT + 4]>(As),
+                         reinterpret_cast<const float(*)[BT + 4]>(As + BK * (BT + 4)), ty, tx, acc);
+  }
+  cp_async_wait<0>();
+  const int n = n0 + tx * 4;
+#pragma unroll
+  for (int m = 0; m < 4; ++m) {
+    const int i = m0 + ty * 4 + m;
+    if (i >= p.M) continue;
+    const float c[4] = {acc[m][0].x, acc[m][0].y, acc[m][1].x, acc[m][1].y};
+    if (OUT == 1) {   // z.ld is a multiple of 4 and columns N .. z.ld - 1 get zeros
+      if (n < p.z.ld)
+        *reinterpret_cast<float4*>(p.z.row(i) + blockIdx.z * p.range_stride + (size_t)n * 4) = make_float4(c[0], c[1], c[2], c[3]);
+      continue;
+    }
+    float* w = p.W + (size_t)i * p.ldw + n;
+    if ((p.ldw & 3) == 0 && n + 3 < p.N) {
+      float4 t = *reinterpret_cast<float4*>(w);
+      t.x = fmaf(-p.eta, c[0], t.x); t.y = fmaf(-p.eta, c[1], t.y);
+      t.z = fmaf(-p.eta, c[2], t.z); t.w = fmaf(-p.eta, c[3], t.w);
+      *reinterpret_cast<float4*>(w) = t;
+    } else {
+#pragma unroll
+      for (int e = 0; e < 4; ++e)
+        if (n + e < p.N) w[e] = fmaf(-p.eta, c[e], w[e]);
+    }
+  }
+}
+
 // dst[c][r] = src row r, column c (R rows of C values behind a row map; dst rows ldr floats long, columns R .. ldr - 1
 // zero).  `copy` (optional): the same rows also copied there, pad columns zero (the factor v = x of the MLR model).
 __global__ void __launch_bounds__(256) transpose_rows_kernel(RowMap src, float* __restrict__ dst, int R, int C, int ldr,
@@ -414,43 +457,69 @@ __global__ void __launch_bounds__(256) transpose_rows_vec_kernel(TransposeJob j0
 
 }  // namespace
 
-// Few 128 x 128 tiles and a long reduction (e.g. 1024 samples x 1000 classes over 20000 features): the
-// reduction is cut into ranges so that the blocks fill whole waves of two blocks per SM.  Among 1 .. 12 ranges
-// (each at least 512 reduction steps long) the smallest count whose last wave is at least 94 % full is taken,
-// else the count with the fullest waves.
-int forward_f32_splits(int K, int J, int D) {
-  const long long tiles = (long long)((K + 127) / 128) * ((J + 127) / 128);
-  const long long slots = 2 * 148;
-  if (tiles >= 148) return 1;
-  int best = 1;
-  double best_fill = 0.0;
-  for (int ks = 1; ks <= 12 && D / ks >= 512; ++ks) {
-    const long long blocks = tiles * ks;
-    const double fill = (double)blocks / (double)(((blocks + slots - 1) / slots) * slots);
-    if (fill >= 0.94) return ks;
-    if (fill > best_fill + 1e-9) { best_fill = fill; best = ks; }
-  }
+// How a forward is done: in one launch (the smallest problems, whose sums the single-launch step repeats in the same
+// order), on 64 x 64 tiles in place, or on 128 x 128 tiles through transposed copies; and its reduction ranges.
+namespace {
+struct ForwardPlan {
+  int tile, ks;   // tile 0: one launch
+};
+// Estimated microseconds.  64 x 64 tiles run at 40 % of the FMA rate when the SMs are full and at 0.9 us per 16 steps when
+// not; 128 x 128 tiles at 70 %, behind a transposing pass at 4.5 TB/s; a range's partial products go out and come back.
+ForwardPlan plan_forward(int K, int J, int D, int max_ks) {
+  if (step_small_fits(K, J, D)) return {0, 1};
+  const double fma_us = 128 * 1900.0;
+  ForwardPlan best = {64, 1};
+  double best_us = -1;
+  auto consider = [&](int tile, double rate, double step_us, double before) {
+    const double tiles = (double)((K + tile - 1) / tile) * ((J + tile - 1) / tile);
+    for (int ks = 1; ks <= max_ks && (ks == 1 || D / ks >= 64); ++ks) {
+      const int per = ((D + ks - 1) / ks + BK - 1) / BK * BK;
+      const double per_sm = (double)(long long)((tiles * ks + 147) / 148);
+      const double work = per_sm * tile * tile * per / (fma_us * rate), chain = per / 16.0 * step_us;
+      const double us = before + (work > chain ? work : chain) + (ks > 1 ? ks * (double)J * K * 8 / 6e6 : 0.0);
+      if (best_us < 0 || us < best_us) {
+        best_us = us;
+        best = {tile, ks};
+      }
+    }
+  };
+  consider(64, 0.40, 0.9, 0.0);
+  if (K >= 128 && J >= 64 && D >= 512) consider(128, 0.70, 0.9, 4.0 + (double)(J + K) * D * 8 / 4.5e6);
   return best;
 }
+}  // namespace
 
-int launch_forward_f32(cudaStream_t s, const float* W, const float* X, const float* Xb, int K, int J, int D,
-                       RowMap z, RowMap v, RowMap part, long long split_stride, int max_splits, int* nsplit_out) {
-  if (nsplit_out != nullptr) *nsplit_out = 1;
-  const long long big_tiles = (long long)((K + 127) / 128) * ((J + 127) / 128);
-  int ks = (part.base != nullptr && nsplit_out != nullptr) ? forward_f32_splits(K, J, D) : 1;
-  if (ks > max_splits) ks = max_splits;       // the partial buffers the caller owns
-  if (ks > 1) {
-    const int per = ((D + ks - 1) / ks + BK - 1) / BK * BK;
-    dim3 grid((J + 127) / 128, (K + 127) / 128, ks);
-    launch_chained(forward_f32_kernel<2, 2>, grid, 256, 0, s, W, X, Xb, K, J, D, part, v, per, split_stride);
-    *nsplit_out = ks;
-  } else if (big_tiles >= 148) {
-    dim3 grid((J + 127) / 128, (K + 127) / 128);
-    launch_chained(forward_f32_kernel<2, 2>, grid, 256, 0, s, W, X, Xb, K, J, D, z, v, D, 0);
-  } else {
-    dim3 grid((J + 63) / 64, (K + 63) / 64);
-    launch_chained(forward_f32_kernel<1, 1>, grid, 256, 0, s, W, X, Xb, K, J, D, z, v, D, 0);
-  }
+int forward_f32_splits(int K, int J, int D) { return plan_forward(K, J, D, FORWARD_F32_MAX_SPLITS).ks; }
+bool forward_f32_transposed(int K, int J, int D) { return plan_forward(K, J, D, FORWARD_F32_MAX_SPLITS).tile == 128; }
+bool forward_f32_fused(int K, int J, int D) { return plan_forward(K, J, D, 1).tile == 0; }
+
+int launch_forward_f32(cudaStream_t s, const float* W, const float* X, const float* Xb, int K, int J, int D, RowMap z,
+                       RowMap v) {
+  if ((long long)((K + 127) / 128) * ((J + 127) / 128) >= 148)
+    launch_chained(forward_f32_kernel<2, 2>, dim3((J + 127) / 128, (K + 127) / 128), 256, 0, s, W, X, Xb, K, J, D, z, v);
+  else
+    launch_chained(forward_f32_kernel<1, 1>, dim3((J + 63) / 64, (K + 63) / 64), 256, 0, s, W, X, Xb, K, J, D, z, v);
+  return cudaGetLastError() == cudaSuccess ? 1 : SFB_ERR_CUDA;
+}
+
+// No empty range: the finishing pass would add a partial buffer nobody wrote.
+static int range_length(int D, int* ks) {
+  const int per = ((D + *ks - 1) / *ks + BK - 1) / BK * BK;
+  *ks = (D + per - 1) / per;
+  return per;
+}
+
+int launch_forward_f32_small(cudaStream_t s, const float* W, RowMap src, RowMap copy, int K, int J, int D, RowMap z,
+                             RowMap part, long long split_stride, int ks, int* nsplit_out) {
+  SmallArgs p = {};
+  p.k_per_range = range_length(D, &ks);
+  p.W = const_cast<float*>(W);
+  p.a = src; p.copy = copy;
+  p.K = D; p.M = K; p.N = J; p.ldw = D;
+  p.z = ks > 1 ? part : z;
+  p.range_stride = split_stride;
+  *nsplit_out = ks;
+  launch_chained(sgemm_small_kernel<1>, dim3((J + 63) / 64, (K + 63) / 64, ks), 256, 0, s, p);
   return cudaGetLastError() == cudaSuccess ? 1 : SFB_ERR_CUDA;
 }
 
@@ -466,8 +535,14 @@ int launch_apply_f32(cudaStream_t s, float* W, RowMap u, RowMap v, int K, int J,
     launch_chained(sgemm_pipe_kernel<0>, grid, 256, PIPE * PIPE_STAGE_FLOATS * 4, s, W, u, v, K, J, D, eta, dev_status, RowMap(), 0, 0,
                                                                          row_idx, n_rows);
   } else {
-    dim3 grid((D + 63) / 64, (J + 63) / 64);
-    launch_chained(apply_f32_kernel<1, 1>, grid, 256, 0, s, W, u, v, K, J, D, eta, dev_status);
+    SmallArgs p = {};
+    p.W = W;
+    p.a = u; p.b = v;
+    p.K = K; p.M = J; p.N = D; p.ldw = D;
+    p.eta = eta;
+    p.dev_status = dev_status;
+    p.row_idx = row_idx; p.n_rows = n_rows;
+    launch_chained(sgemm_small_kernel<0>, dim3((D + 63) / 64, (J + 63) / 64), 256, 0, s, p);
   }
   return cudaGetLastError() == cudaSuccess ? 1 : SFB_ERR_CUDA;
 }
@@ -481,7 +556,7 @@ long long forward_f32_nn_workspace_floats(int K, int J, int D) {
 }
 
 int launch_forward_f32_nn(cudaStream_t s, const float* W, RowMap src, RowMap copy, int K, int J, int D, float* ws,
-                          RowMap z, RowMap part, long long split_stride, int max_splits, int* nsplit_out) {
+                          RowMap z, RowMap part, long long split_stride, int ks, int* nsplit_out) {
   const int ldk = (K + 3) & ~3, ldj = (J + 3) & ~3;
   float* xt = ws;
   float* wt = ws + (size_t)D * ldk;
@@ -504,10 +579,8 @@ int launch_forward_f32_nn(cudaStream_t s, const float* W, RowMap src, RowMap cop
     launch_chained(transpose_rows_kernel, dim3((D + 31) / 32, (ldk + 31) / 32), 256, 0, s, src, xt, K, D, ldk, copy);
     launch_chained(transpose_rows_kernel, dim3((D + 31) / 32, (ldj + 31) / 32), 256, 0, s, wrows, wt, J, D, ldj, RowMap());
   }
-  int ks = (part.base != nullptr && nsplit_out != nullptr) ? forward_f32_splits(K, J, D) : 1;
-  if (ks > max_splits) ks = max_splits;
-  if (nsplit_out != nullptr) *nsplit_out = ks;
-  const int per = ((D + ks - 1) / ks + BK - 1) / BK * BK;
+  const int per = range_length(D, &ks);
+  *nsplit_out = ks;
   RowMap a, b;
   a.base = reinterpret_cast<char*>(xt); a.worker_stride = 0; a.ld = ldk; a.B = D; a.es = 4;
   b.base = reinterpret_cast<char*>(wt); b.worker_stride = 0; b.ld = ldj; b.B = D; b.es = 4;

@@ -169,8 +169,7 @@ constexpr size_t SMEM_MAX = 96 * 1024;
 // One SM does all of it, so the time grows with K J D (4 us from 2^14 to 2^16) while three launches that spread over the
 // chip start at 14 us: at 2^16 10.5-11.8 us (J 100 / 16, D 64) against about 17, at 2^18 the two would meet.
 bool step_small_fits(int K, int J, int D) {
-  return J <= 128 && (long long)K * J * D <= (1 << 16) && smem_bytes(K, J, D) <= SMEM_MAX &&
-         forward_f32_splits(K, J, D) == 1;   // (a cut reduction is summed in another order)
+  return J <= 128 && (long long)K * J * D <= (1 << 16) && smem_bytes(K, J, D) <= SMEM_MAX;
 }
 
 int launch_step_small(cudaStream_t s, const sfb_desc& d, float* W, const float* X, const sfb_aux* aux, RowMap u, RowMap v,
