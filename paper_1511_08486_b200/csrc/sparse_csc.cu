@@ -8,11 +8,11 @@
 // so inside a column the entries are in sample order whatever the thread schedule.  Every column of a slice is padded
 // with zero entries to a multiple of four, so that a warp reads the entries of consecutive atoms as one stream of groups
 // of four.
-// The apply gives each thread block 64 rows of W at a time and keeps the matching 64 columns of a slice of the
+// The apply gives each thread block 32 rows of W at a time and keeps the matching 32 columns of a slice of the
 // u_i in shared memory (the samples are taken in as few slices as fit).  A warp takes 8 consecutive
-// atoms: it starts the loads of its part of W, walks the atoms' entries (coalesced loads staged through a
+// atoms: it starts the loads of the next part of W, walks the atoms' entries (coalesced loads staged through a
 // small per-warp strip), accumulating a_id * u_i[j0 + 4 q .. + 3] from shared memory, parks the sums
-// in a private 8 x 68 tile, and finally updates W with 32-byte row segments.
+// in a private 8 x 36 tile, and finally updates W with 32-byte row segments.
 // U is read once and W once per slice; no floating-point atomics; every element of W has one owner and a fixed
 // summation order (bit-reproducible); atoms nobody uses get W + (-eta * 0) = W, bit-identical.
 #include "common.cuh"
@@ -157,20 +157,24 @@ __global__ void __launch_bounds__(256) csc_fill_kernel(CsrView codes, int K, int
   }
 }
 
-constexpr int CSC2_JT = 64;     // rows of W per block, four per lane of a half warp
+constexpr int CSC2_JT = 32;     // rows of W per block, four per lane of a quarter warp
 constexpr int CSC2_AB = 8;      // atoms per warp block
-constexpr int CSC2_WARPS = 16;
+constexpr int CSC2_WARPS = 20;
 constexpr int CSC2_STRIP = 128; // entries a warp stages at a time
-constexpr int CSC2_TS = 68;     // row length of the tile: 4 atoms-worth of banks apart, rows 16-byte aligned
-constexpr int CSC2_WARP_FLOATS = 2 * CSC2_STRIP + CSC2_AB * CSC2_TS;   // entry strip + [8][68] tile
+constexpr int CSC2_RS = 32 / CSC2_AB;   // rows of W a warp instruction covers
+constexpr int CSC2_TS = 32 + CSC2_RS;    // row length of the tile: 8 atoms x 4 rows fall on 32 banks
+constexpr int CSC2_WARP_FLOATS = 2 * CSC2_STRIP + CSC2_AB * CSC2_TS;   // entry strip + [8][36] tile
 
-// The work is the list of (block of 64 rows, block of 8 atoms), rows outermost; every thread block takes an equal run
+// The work is the list of (block of 32 rows, block of 8 atoms), rows outermost; every thread block takes an equal run
 // of it, so the SMs are loaded evenly whatever J is (a run rarely touches more than two blocks of rows).
-// A half warp takes every other entry: one 8-byte read of the strip (two addresses) and one 512-byte read of u per two
-// entries, five wavefronts of shared memory, which bounds this kernel.  (Two rows per lane and an entry at a time cost
-// three wavefronts per entry: a 16-byte broadcast read takes two.)
-// 4096 x 10000, K = 1024: 5 % density 742 -> 514 us an apply, 1 % 459 -> 304, against columns staged one by one in rounds
-// of 8, 16 or 32 entries on 64 x 2 blocks with 64-byte segments of W.
+// A quarter warp takes every fourth entry: one 8-byte read of the strip (four addresses) and one 512-byte read of u per
+// four entries, five wavefronts of shared memory, which bounds this kernel where the codes are dense; the four partial
+// sums meet in three shuffles that leave every lane one row.  Where they are sparse the bound is W's way through the
+// memory and the latency of a column's few steps: 32 rows (not 64), so that 1416 samples fit beside the tiles and W is read
+// and written once; the next block's part of W is in flight while this one's entries are summed; a column's last groups
+// are read together; 20 warps (16: 5 % 488 us; 24 or 32, with fewer registers: 461 and 464, small problems 10 % slower).
+// 4096 x 10000, K = 1024, against half warps on 64 rows with W loaded when its block begins: 5 % density 514 -> 443 us an
+// apply, 2 % 355 -> 274, 1 % 304 -> 206 (3000 x 500, K = 320: 21.9 -> 22.5).
 __global__ void __launch_bounds__(CSC2_WARPS * 32) csc_apply_kernel(float* __restrict__ W, RowMap u, int K, int J, int D,
                                                                     float eta, const int* __restrict__ colptr,
                                                                     const int2* __restrict__ ent, int passes, int Kh,
@@ -178,11 +182,13 @@ __global__ void __launch_bounds__(CSC2_WARPS * 32) csc_apply_kernel(float* __res
   chain();
   extern __shared__ __align__(16) float smem[];
   if (status_ro != nullptr && (*status_ro & SFB_DEV_BAD_HEADER)) return;
-  float* Us = smem;                                   // [Kh][64]
+  float* Us = smem;                                   // [Kh][32]
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  float* region = smem + (size_t)Kh * 64 + warp * CSC2_WARP_FLOATS;
+  float* region = smem + (size_t)Kh * CSC2_JT + warp * CSC2_WARP_FLOATS;
   int2* strip = reinterpret_cast<int2*>(region);
-  const int half = lane >> 4, q4 = (lane & 15) * 4;   // this lane's entries and rows
+  const int quarter = lane >> 3, q4 = (lane & 7) * 4; // this lane's entries and rows
+  const bool up1 = (lane & 16) != 0, up0 = (lane & 8) != 0;
+  const int my_row = q4 + (up1 ? 2 : 0) + (up0 ? 1 : 0);   // ... and the row whose sum it ends up with
   float* T = region + 2 * CSC2_STRIP;
   const int nblocks = (D + CSC2_AB - 1) / CSC2_AB;
   const long long work = (long long)((J + CSC2_JT - 1) / CSC2_JT) * nblocks;
@@ -199,15 +205,14 @@ __global__ void __launch_bounds__(CSC2_WARPS * 32) csc_apply_kernel(float* __res
       const int i_n = min(Kh, K - i_lo);
       __syncthreads();                                  // the previous slice is no longer read
       // 16-byte asynchronous copies, all in flight together; rows of u are padded to 16 bytes
-      for (int t = threadIdx.x; t < i_n * 16; t += CSC2_WARPS * 32) {
-        const int i = t >> 4, c = (t & 15) * 4;
-        const uint32_t dst = (uint32_t)__cvta_generic_to_shared(Us + i * 64 + c);
+      for (int t = threadIdx.x; t < i_n * (CSC2_JT / 4); t += CSC2_WARPS * 32) {
+        const int i = t / (CSC2_JT / 4), c = (t % (CSC2_JT / 4)) * 4;
+        const uint32_t dst = (uint32_t)__cvta_generic_to_shared(Us + i * CSC2_JT + c);
         const bool in = c < jn;
         const char* src = u.row(i_lo + i) + (in ? (size_t)(j0 + c) * 4 : 0);
         asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(in ? 16 : 0) : "memory");
       }
-      asm volatile("cp.async.wait_all;" ::: "memory");
-      __syncthreads();
+      asm volatile("cp.async.commit_group;" ::: "memory");
       // entries of the warp's next block, on their way while the current one is summed
       constexpr int PRE = CSC2_STRIP / 32;
       int2 pre[PRE];
@@ -218,13 +223,27 @@ __global__ void __launch_bounds__(CSC2_WARPS * 32) csc_apply_kernel(float* __res
           pre[t] = e < n_ent ? ent[e] : make_int2(0, 0);
         }
       };
+      // the warp's part of W of a block: lane = atom lane % 8, rows lane / 8 + 4 t
+      const int wa = lane & (CSC2_AB - 1), wq = lane / CSC2_AB;
+      constexpr int WN = CSC2_JT * CSC2_AB / 32;
+      float w_next[WN];
+      auto fetch_w = [&](int ab) {
+        const int d = ab * CSC2_AB + wa;
+        const bool in = ab < ab_hi && d < D;
+        const float* wp = W + (size_t)(j0 + wq) * D + (in ? d : 0);
+        const size_t step = (size_t)CSC2_RS * D;
+        const int rows = in ? jn - wq : 0;
+#pragma unroll
+        for (int t = 0; t < WN; ++t, wp += step) w_next[t] = CSC2_RS * t < rows ? *wp : 0.f;
+      };
       // first entry of the atoms of a block: lane a has atom a's, lanes behind the last atom the end of its column
       const int* cols = colptr + (size_t)h * D;
       auto starts = [&](int ab) { return ab < ab_hi ? cols[ab * CSC2_AB + min(lane, min(CSC2_AB, D - ab * CSC2_AB))] : n_ent; };
       int beg_next = starts(ab_lo + warp);
+      fetch_w(ab_lo + warp);
       fetch(__shfl_sync(0xffffffffu, beg_next, 0));
-      // the warp's part of W of a block: lane = atom lane % 8, rows lane / 8 + 4 t
-      const int wa = lane & (CSC2_AB - 1), wq = lane / CSC2_AB;
+      asm volatile("cp.async.wait_all;" ::: "memory");
+      __syncthreads();
       for (int ab = ab_lo + warp; ab < ab_hi; ab += CSC2_WARPS) {
         const int d0 = ab * CSC2_AB;
         const int dn = min(CSC2_AB, D - d0);
@@ -245,48 +264,48 @@ __global__ void __launch_bounds__(CSC2_WARPS * 32) csc_apply_kernel(float* __res
           __syncwarp();
         };
         refill();
-        // W is on its way while the entries are summed
-        float wv[CSC2_JT / 4];
+        float wv[WN];
 #pragma unroll
-        for (int t = 0; t < CSC2_JT / 4; ++t) {
-          const int jj = 4 * t + wq;
-          wv[t] = (wa < dn && jj < jn) ? W[(size_t)(j0 + jj) * D + d0 + wa] : 0.f;
-        }
+        for (int t = 0; t < WN; ++t) wv[t] = w_next[t];
+        fetch_w(ab + CSC2_WARPS);
         for (int dd = 0; dd < dn; ++dd) {
           const int stop = __shfl_sync(0xffffffffu, beg, dd + 1);
           float4 acc0 = make_float4(0.f, 0.f, 0.f, 0.f), acc1 = acc0;
           while (pos < stop) {
             if (pos == strip_hi) refill();              // (warp-uniform)
-            auto four = [&](int k) {
-              const int2 p = strip[k + half], q = strip[k + 2 + half];
-              const float4 u0 = *reinterpret_cast<const float4*>(Us + p.x * 64 + q4);
-              const float4 u1 = *reinterpret_cast<const float4*>(Us + q.x * 64 + q4);
-              const float a0 = __int_as_float(p.y), a1 = __int_as_float(q.y);
-              acc0.x = fmaf(a0, u0.x, acc0.x); acc0.y = fmaf(a0, u0.y, acc0.y);
-              acc0.z = fmaf(a0, u0.z, acc0.z); acc0.w = fmaf(a0, u0.w, acc0.w);
-              acc1.x = fmaf(a1, u1.x, acc1.x); acc1.y = fmaf(a1, u1.y, acc1.y);
-              acc1.z = fmaf(a1, u1.z, acc1.z); acc1.w = fmaf(a1, u1.w, acc1.w);
+            auto four = [&](int k, float4& acc) {
+              const int2 p = strip[k + quarter];
+              const float4 u0 = *reinterpret_cast<const float4*>(Us + p.x * CSC2_JT + q4);
+              const float a0 = __int_as_float(p.y);
+              acc.x = fmaf(a0, u0.x, acc.x); acc.y = fmaf(a0, u0.y, acc.y);
+              acc.z = fmaf(a0, u0.z, acc.z); acc.w = fmaf(a0, u0.w, acc.w);
             };
             const int to = min(stop, strip_hi);         // groups of four never straddle a column or the strip
             int k = pos - strip_lo;
             const int k_end = to - strip_lo;
-            for (; k + 8 <= k_end; k += 8) { four(k); four(k + 4); }
-            if (k < k_end) four(k);
+#pragma unroll 1
+            for (; k + 16 <= k_end; k += 16) { four(k, acc0); four(k + 4, acc1); four(k + 8, acc0); four(k + 12, acc1); }
+            if (k_end - k == 12) { four(k, acc0); four(k + 4, acc1); four(k + 8, acc0); }
+            else if (k_end - k == 8) { four(k, acc0); four(k + 4, acc1); }
+            else if (k < k_end) four(k, acc0);
             pos = to;
           }
           acc0.x += acc1.x; acc0.y += acc1.y; acc0.z += acc1.z; acc0.w += acc1.w;
-          acc0.x += __shfl_xor_sync(0xffffffffu, acc0.x, 16); acc0.y += __shfl_xor_sync(0xffffffffu, acc0.y, 16);
-          acc0.z += __shfl_xor_sync(0xffffffffu, acc0.z, 16); acc0.w += __shfl_xor_sync(0xffffffffu, acc0.w, 16);
-          if (half == 0) *reinterpret_cast<float4*>(T + dd * CSC2_TS + q4) = acc0;
+          // quarters 0, 1 go on with rows q4, q4 + 1 and quarters 2, 3 with the other two; then one row each
+          float lo = up1 ? acc0.z : acc0.x, hi = up1 ? acc0.w : acc0.y;
+          lo += __shfl_xor_sync(0xffffffffu, up1 ? acc0.x : acc0.z, 16);
+          hi += __shfl_xor_sync(0xffffffffu, up1 ? acc0.y : acc0.w, 16);
+          const float sum = (up0 ? hi : lo) + __shfl_xor_sync(0xffffffffu, up0 ? lo : hi, 8);
+          T[dd * CSC2_TS + my_row] = sum;
         }
         __syncwarp();
         // W[j0 + jj][d0 + wa] -= eta * T[wa][jj]: a warp instruction covers four rows x 8 atoms (32-byte segments)
         if (wa < dn) {
+          float* wp = W + (size_t)(j0 + wq) * D + d0 + wa;
+          const size_t step = (size_t)CSC2_RS * D;
 #pragma unroll
-          for (int t = 0; t < CSC2_JT / 4; ++t) {
-            const int jj = 4 * t + wq;
-            if (jj < jn) W[(size_t)(j0 + jj) * D + d0 + wa] = fmaf(-eta, T[wa * CSC2_TS + jj], wv[t]);
-          }
+          for (int t = 0; t < WN; ++t, wp += step)
+            if (CSC2_RS * t < jn - wq) *wp = fmaf(-eta, T[wa * CSC2_TS + CSC2_RS * t + wq], wv[t]);
         }
         __syncwarp();
       }
@@ -294,13 +313,13 @@ __global__ void __launch_bounds__(CSC2_WARPS * 32) csc_apply_kernel(float* __res
   }
 }
 
-// Slices of the samples: the fewest that let Kh x 256 bytes of u sit beside the warps' tiles.
+// Slices of the samples: the fewest that let Kh x 128 bytes of u sit beside the warps' tiles.
 struct CscSlices {
   int passes, Kh;
 };
 CscSlices csc_slices(int K) {
   const int tiles = CSC2_WARPS * CSC2_WARP_FLOATS * 4;
-  const int kh_max = (220 * 1024 - tiles) / 256 / CSC_CHUNK * CSC_CHUNK;
+  const int kh_max = (220 * 1024 - tiles) / (CSC2_JT * 4) / CSC_CHUNK * CSC_CHUNK;
   CscSlices s;
   s.passes = (K + kh_max - 1) / kh_max;
   s.Kh = ((K + s.passes - 1) / s.passes + CSC_CHUNK - 1) / CSC_CHUNK * CSC_CHUNK;
@@ -368,7 +387,7 @@ int launch_sc_csc_apply(cudaStream_t s, float* W, RowMap u, int K, int J, int D,
   const long long work = (long long)((J + CSC2_JT - 1) / CSC2_JT) * ((D + CSC2_AB - 1) / CSC2_AB);
   long long blocks = (work + CSC2_WARPS - 1) / CSC2_WARPS;   // at least one block of atoms per warp
   if (blocks > 148) blocks = 148;
-  const size_t smem = (size_t)sl.Kh * 256 + (size_t)CSC2_WARPS * CSC2_WARP_FLOATS * 4;
+  const size_t smem = (size_t)sl.Kh * (CSC2_JT * 4) + (size_t)CSC2_WARPS * CSC2_WARP_FLOATS * 4;
   launch_chained(csc_apply_kernel, (unsigned)blocks, CSC2_WARPS * 32, smem, s, W, u, K, J, D, eta, w.colptr, w.ent, sl.passes, sl.Kh,
                                                                    dev_status_ro);
   return cudaGetLastError() == cudaSuccess ? 1 : SFB_ERR_CUDA;
