@@ -3,11 +3,15 @@
 //   W[:, d] -= eta * sum_{i : a_id != 0} a_id * u_i        (Section 3 update with v_i = a_i sparse)
 //
 // The codes arrive sample-major (CSR, the factor v_i of each sample).  Per step they are re-sorted by
-// (slice of samples, atom) with a counting sort that is deterministic: counts per (chunk of 8 samples, atom) by integer
-// atomics, prefix sums over chunks and atoms, then every chunk places its samples one after the other,
-// so inside a column the entries are in sample order whatever the thread schedule.  Every column of a slice is padded
-// with zero entries to a multiple of four, so that a warp reads the entries of consecutive atoms as one stream of groups
-// of four.
+// (slice of samples, atom) with a counting sort that is deterministic: per (chunk of 32 samples, atom) a mask of the
+// samples that use the atom (atomic or), prefix sums of the masks' populations over chunks and atoms, and every entry's
+// place follows from the bits below its own, so inside a column the entries are in sample order whatever the thread
+// schedule.  Every column of a slice is padded with zero entries to a multiple of four, so that a warp reads the entries
+// of consecutive atoms as one stream of groups of four.
+// The sort runs beside the forward pass, but below some 1000 x 3000 weights the forward is the shorter of the two: there
+// the latency of its steps counts, hence no loop over samples in any of them (counts per chunk of 8 samples, placed one
+// sample after the other, and a scan of 1024 sums at a time, made the step 65.0 us
+// against 42.3 at 500 x 3000, K = 320, 5 % density, 46.4 against 30.2 at 100 x 400, K = 40, 2 %).
 // The apply gives each thread block 32 rows of W at a time and keeps the matching 32 columns of a slice of the
 // u_i in shared memory (the samples are taken in as few slices as fit).  A warp takes 8 consecutive
 // atoms: it starts the loads of the next part of W, walks the atoms' entries (coalesced loads staged through a
@@ -20,7 +24,7 @@
 namespace sfb {
 namespace {
 
-constexpr int CSC_CHUNK = 8;    // samples per chunk of the counting sort
+constexpr int CSC_CHUNK = 32;   // samples per chunk of the counting sort: the bits of a mask
 
 struct CsrRow2 {
   const uint32_t* idx;
@@ -56,104 +60,114 @@ __device__ __forceinline__ bool entry_ok(const CsrRow2& row, int k, int D) {
   return d < (uint32_t)D && !(k > 0 && row.idx[k - 1] >= d);
 }
 
-// cnt[chunk][d] += 1 for every nonzero (integer atomics: the final counts do not depend on the order)
-__global__ void __launch_bounds__(256) csc_count_kernel(CsrView codes, int K, int D, int* __restrict__ cnt,
-                                                        int* dev_status) {
+// bit i % 32 of mask[i / 32][d]: sample i uses atom d (atomic or: the masks do not depend on the order)
+__global__ void __launch_bounds__(256) csc_mask_kernel(CsrView codes, int K, int D, uint32_t* __restrict__ mask,
+                                                       int* dev_status) {
   const int i = blockIdx.x;
   const CsrRow2 row = csr_row2(codes, i);
-  int* c = cnt + (size_t)(i / CSC_CHUNK) * D;
+  uint32_t* m = mask + (size_t)(i / CSC_CHUNK) * D;
   bool bad = false;
   for (int k = threadIdx.x; k < row.len; k += 256) {
-    if (entry_ok(row, k, D)) atomicAdd(c + row.idx[k], 1);
+    if (entry_ok(row, k, D)) atomicOr(m + row.idx[k], 1u << (i % CSC_CHUNK));
     else bad = true;   // the entry is skipped
   }
   if (bad && dev_status != nullptr) atomicOr(dev_status, SFB_DEV_BAD_INDEX);
 }
 
-// per atom: counts per chunk -> offsets of each chunk inside the column's slice; slice totals, rounded up to fours
-__global__ void __launch_bounds__(256) csc_chunk_offsets_kernel(int nchunks, int chunks_per_slice, int D, int* __restrict__ cnt,
-                                                                int* __restrict__ total) {
-  const int d = blockIdx.x * 256 + threadIdx.x;
+// per atom: populations of the chunks' masks -> offsets of each chunk inside the column's slice; slice totals
+__global__ void __launch_bounds__(64) csc_chunk_offsets_kernel(int nchunks, int chunks_per_slice, int D,
+                                                               const uint32_t* __restrict__ mask, int* __restrict__ off,
+                                                               int* __restrict__ total) {
+  chain();
+  const int d = blockIdx.x * 64 + threadIdx.x;
   if (d >= D) return;
   int run = 0, slice = 0, left = chunks_per_slice;
-  for (int c0 = 0; c0 < nchunks; c0 += 8) {   // eight independent loads in flight, then the running sum
-    int t[8];
+  for (int c0 = 0; c0 < nchunks; c0 += 16) {   // sixteen independent loads in flight, then the running sum
+    uint32_t t[16];
 #pragma unroll
-    for (int q = 0; q < 8; ++q) t[q] = (c0 + q < nchunks) ? cnt[(size_t)(c0 + q) * D + d] : 0;
+    for (int q = 0; q < 16; ++q) t[q] = (c0 + q < nchunks) ? mask[(size_t)(c0 + q) * D + d] : 0u;
 #pragma unroll
-    for (int q = 0; q < 8; ++q) {
+    for (int q = 0; q < 16; ++q) {
       if (c0 + q < nchunks) {
-        cnt[(size_t)(c0 + q) * D + d] = run;
-        run += t[q];
+        off[(size_t)(c0 + q) * D + d] = run;
+        run += __popc(t[q]);
         if (--left == 0) {
-          total[(size_t)slice * D + d] = (run + 3) & ~3;
+          total[(size_t)slice * D + d] = run;
           run = 0; ++slice; left = chunks_per_slice;
         }
       }
     }
   }
-  if (left < chunks_per_slice) total[(size_t)slice * D + d] = (run + 3) & ~3;
+  if (left < chunks_per_slice) total[(size_t)slice * D + d] = run;
 }
 
-// colptr[0 .. n] = exclusive scan of total[0 .. n) (one block, fixed order)
+// colptr[0 .. n] = exclusive scan of total[0 .. n) rounded up to fours (one block, fixed order; eight sums a thread)
 __global__ void __launch_bounds__(1024) csc_scan_kernel(int n, const int* __restrict__ total, int* __restrict__ colptr) {
+  chain();
   __shared__ int warp_sum[32];
-  __shared__ int carry;
-  if (threadIdx.x == 0) carry = 0;
-  __syncthreads();
-  for (int base = 0; base < n; base += 1024) {
-    const int d = base + threadIdx.x;
-    const int v = d < n ? total[d] : 0;
-    int incl = v;
+  constexpr int PER = 8;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  int carry = 0;
+  for (int base = 0; base < n; base += 1024 * PER) {
+    const int d = base + threadIdx.x * PER;
+    int v[PER], sum = 0;
+#pragma unroll
+    for (int q = 0; q < PER; ++q) v[q] = d + q < n ? (total[d + q] + 3) & ~3 : 0;
+#pragma unroll
+    for (int q = 0; q < PER; ++q) sum += v[q];
+    int incl = sum;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
       const int o_ = __shfl_up_sync(0xffffffffu, incl, o);
-      if ((threadIdx.x & 31) >= o) incl += o_;
+      if (lane >= o) incl += o_;
     }
-    if ((threadIdx.x & 31) == 31) warp_sum[threadIdx.x >> 5] = incl;
+    if (lane == 31) warp_sum[warp] = incl;
     __syncthreads();
-    if (threadIdx.x < 32) {
-      int w = warp_sum[threadIdx.x];
+    int w = warp_sum[lane];                       // every warp scans the 32 sums for itself
 #pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const int o_ = __shfl_up_sync(0xffffffffu, w, o);
-        if (threadIdx.x >= o) w += o_;
-      }
-      warp_sum[threadIdx.x] = w;
+    for (int o = 1; o < 32; o <<= 1) {
+      const int o_ = __shfl_up_sync(0xffffffffu, w, o);
+      if (lane >= o) w += o_;
     }
-    __syncthreads();
-    const int before = carry + ((threadIdx.x >> 5) > 0 ? warp_sum[(threadIdx.x >> 5) - 1] : 0) + incl - v;
-    if (d < n) colptr[d] = before;
-    __syncthreads();
-    if (threadIdx.x == 1023) carry = before + v;
-    __syncthreads();
+    const int before = __shfl_sync(0xffffffffu, w, max(warp - 1, 0));
+    int run = carry + (warp > 0 ? before : 0) + incl - sum;
+#pragma unroll
+    for (int q = 0; q < PER; ++q) {
+      if (d + q < n) colptr[d + q] = run;
+      run += v[q];
+    }
+    carry += __shfl_sync(0xffffffffu, w, 31);
+    __syncthreads();                              // the sums are no longer read
   }
   if (threadIdx.x == 0) colptr[n] = carry;
 }
 
-// one block per chunk: its samples are placed one after the other, so a column is in sample order
-// (entry = sample index inside its slice, value)
-__global__ void __launch_bounds__(256) csc_fill_kernel(CsrView codes, int K, int D, int chunks_per_slice,
-                                                       int* __restrict__ cnt, const int* __restrict__ colptr,
+// Blocks 0 .. K - 1: one sample each, every entry to its place (entry = sample index inside its slice, value); the
+// blocks behind them write the zero entries that fill the columns up.
+__global__ void __launch_bounds__(256) csc_fill_kernel(CsrView codes, int K, int D, int passes, int chunks_per_slice,
+                                                       const uint32_t* __restrict__ mask, const int* __restrict__ off,
+                                                       const int* __restrict__ total, const int* __restrict__ colptr,
                                                        int2* __restrict__ ent) {
-  const int c = blockIdx.x;
-  const int slice = c / chunks_per_slice, i_lo = slice * chunks_per_slice * CSC_CHUNK;
-  int* off = cnt + (size_t)c * D;
-  const int* base = colptr + (size_t)slice * D;
-  for (int s = 0; s < CSC_CHUNK; ++s) {
-    const int i = c * CSC_CHUNK + s;
-    if (i < K) {
-      const CsrRow2 row = csr_row2(codes, i);
-      for (int k = threadIdx.x; k < row.len; k += 256) {
-        if (entry_ok(row, k, D)) {  // indices that pass are unique inside a row: one writer per (chunk, atom) per step
-          const uint32_t d = row.idx[k];
-          const int o = off[d];
-          off[d] = o + 1;
-          ent[base[d] + o] = make_int2(i - i_lo, __float_as_int(row.val[k]));
-        }
-      }
+  chain();
+  if (blockIdx.x >= (unsigned)K) {
+    const int c = (blockIdx.x - K) * 256 + threadIdx.x;
+    if (c < passes * D) {
+      const int end = colptr[c + 1];
+      for (int e = colptr[c] + total[c]; e < end; ++e) ent[e] = make_int2(0, 0);
     }
-    __syncthreads();
+    return;
+  }
+  const int i = blockIdx.x, c = i / CSC_CHUNK, slice = c / chunks_per_slice;
+  const int i_in = i - slice * chunks_per_slice * CSC_CHUNK;
+  const uint32_t below = (1u << (i % CSC_CHUNK)) - 1u;
+  const CsrRow2 row = csr_row2(codes, i);
+  for (int k = threadIdx.x; k < row.len; k += 256) {
+    if (entry_ok(row, k, D)) {
+      const uint32_t d = row.idx[k];
+      const size_t cell = (size_t)c * D + d;
+      ent[colptr[(size_t)slice * D + d] + off[cell] + __popc(mask[cell] & below)] =
+          make_int2(i_in, __float_as_int(row.val[k]));
+    }
   }
 }
 
@@ -329,13 +343,14 @@ CscSlices csc_slices(int K) {
 
 }  // namespace
 
-// Scratch of the CSC path: counts [nchunks][D], totals and column starts [slices][D] ints, entries x (nnz_capacity + padding).
+// Scratch of the CSC path: masks and offsets [nchunks][D], totals and column starts [slices][D] ints, entries x
+// (nnz_capacity + padding).
 static long long csc_entries(int K, int D, long long nnz_capacity) {
   return nnz_capacity + 3LL * csc_slices(K).passes * D;
 }
 static long long csc_ints(int K, int D) {
   const long long nchunks = (K + CSC_CHUNK - 1) / CSC_CHUNK;
-  return nchunks * D + 2LL * csc_slices(K).passes * D + 1;
+  return 2LL * nchunks * D + 2LL * csc_slices(K).passes * D + 1;
 }
 long long sc_csc_workspace_bytes(int K, int D, long long nnz_capacity) {
   // (a step over the first workers' samples only takes fewer slices of another length: no more entries or ints)
@@ -347,13 +362,14 @@ bool sc_csc_supported(int K) { return K <= (1 << 14); }
 
 namespace {
 struct CscScratch {
-  int* cnt; int* total; int* colptr; int2* ent;
+  uint32_t* mask; int* off; int* total; int* colptr; int2* ent;
 };
 CscScratch csc_scratch(void* workspace, int K, int D) {
   const int nchunks = (K + CSC_CHUNK - 1) / CSC_CHUNK, passes = csc_slices(K).passes;
   CscScratch w;
-  w.cnt = reinterpret_cast<int*>(workspace);
-  w.total = w.cnt + (size_t)nchunks * D;
+  w.mask = reinterpret_cast<uint32_t*>(workspace);
+  w.off = reinterpret_cast<int*>(w.mask) + (size_t)nchunks * D;
+  w.total = w.off + (size_t)nchunks * D;
   w.colptr = w.total + (size_t)passes * D;
   w.ent = reinterpret_cast<int2*>(reinterpret_cast<char*>(workspace) + pad_to(csc_ints(K, D) * 4, 256));
   return w;
@@ -367,12 +383,13 @@ int launch_sc_csc_build(cudaStream_t s, CsrView codes, int K, int D, long long n
   const int nchunks = (K + CSC_CHUNK - 1) / CSC_CHUNK;
   const CscSlices sl = csc_slices(K);
   const CscScratch w = csc_scratch(workspace, K, D);
-  if (cudaMemsetAsync(w.cnt, 0, (size_t)nchunks * D * 4, s) != cudaSuccess) return SFB_ERR_CUDA;
-  if (cudaMemsetAsync(w.ent, 0, (size_t)csc_entries(K, D, nnz_capacity) * 8, s) != cudaSuccess) return SFB_ERR_CUDA;
-  csc_count_kernel<<<K, 256, 0, s>>>(codes, K, D, w.cnt, dev_status);
-  csc_chunk_offsets_kernel<<<(D + 255) / 256, 256, 0, s>>>(nchunks, sl.Kh / CSC_CHUNK, D, w.cnt, w.total);
-  csc_scan_kernel<<<1, 1024, 0, s>>>(sl.passes * D, w.total, w.colptr);
-  csc_fill_kernel<<<nchunks, 256, 0, s>>>(codes, K, D, sl.Kh / CSC_CHUNK, w.cnt, w.colptr, w.ent);
+  const int cps = sl.Kh / CSC_CHUNK, cols = sl.passes * D;
+  if (cudaMemsetAsync(w.mask, 0, (size_t)nchunks * D * 4, s) != cudaSuccess) return SFB_ERR_CUDA;
+  csc_mask_kernel<<<K, 256, 0, s>>>(codes, K, D, w.mask, dev_status);
+  launch_chained(csc_chunk_offsets_kernel, (D + 63) / 64, 64, 0, s, nchunks, cps, D, w.mask, w.off, w.total);
+  launch_chained(csc_scan_kernel, 1, 1024, 0, s, cols, w.total, w.colptr);
+  launch_chained(csc_fill_kernel, K + (cols + 255) / 256, 256, 0, s, codes, K, D, sl.passes, cps, w.mask, w.off, w.total,
+                 w.colptr, w.ent);
   return cudaGetLastError() == cudaSuccess ? 4 : SFB_ERR_CUDA;
 }
 
