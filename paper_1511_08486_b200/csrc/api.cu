@@ -578,7 +578,11 @@ int sfb_pack(sfb_ctx* c, const void* U, const void* V, const sfb_aux* aux, void*
 static int apply_from(sfb_ctx* c, void* W, const void* sf_buf, float eta, int K, bool check, bool csc_built = false,
                       bool active_rows = false, const RowMap* v_rows = nullptr) {
   const sfb_desc& d = c->d;
-  if (check) ACC(launch_check_header(c->stream, sf_buf, d, c->l, c->dev_status));
+  HeaderCheck hc;
+  if (check) hc = make_check(sf_buf, d, c->l, c->dev_status);
+  // (the compensated path has a kernel in front of its GEMM that can do the check)
+  const bool with_split = !d.v_sparse && d.path == SFB_PATH_TF32X3;
+  if (check && !with_split) ACC(launch_check_header(c->stream, hc));
   if (d.v_sparse && d.path == SFB_PATH_F32 && c->csc_ws != nullptr) {
     if (!csc_built)
       ACC(launch_sc_csc_build(c->stream, stream_codes(c, sf_buf), K, d.D, (long long)d.nnz_capacity, c->csc_ws,
@@ -613,7 +617,7 @@ static int apply_from(sfb_ctx* c, void* W, const void* sf_buf, float eta, int K,
   } else {
     ACC(umma_apply(c->umma, c->stream, W, c->w_shadow, stream_u(c, sf_buf),
                    v_rows != nullptr ? *v_rows : stream_v(c, sf_buf), eta, K, c->dev_status,
-                   d.compact ? reinterpret_cast<const char*>(sf_buf) + 128 : nullptr));
+                   d.compact ? reinterpret_cast<const char*>(sf_buf) + 128 : nullptr, with_split ? &hc : nullptr));
     // The apply epilogue rewrote the shadow from the new W.  (A compacted buffer without a single pair launches no
     // tile: W and a shadow that mirrored it stay as they were; a stale shadow stays stale.)
     if (has_shadow(c) && (!d.compact || c->shadow_of == W)) c->shadow_of = W;

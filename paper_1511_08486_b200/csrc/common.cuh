@@ -111,6 +111,25 @@ struct HeaderImage {   // exactly the first 68 bytes of the 128-byte header
 };
 static_assert(sizeof(HeaderImage) == 72, "header image is 68 bytes of fields plus 4 of tail padding");
 
+// The check of a buffer's header before it is applied, for whichever kernel of a call does it (buf == nullptr: none).
+struct HeaderCheck {
+  const char* buf;
+  HeaderImage h;
+  int* dev_status;
+  __host__ __device__ HeaderCheck() : buf(nullptr), h(), dev_status(nullptr) {}
+};
+#ifdef __CUDACC__
+// one whole warp, t = lane
+__device__ __forceinline__ void check_header(const HeaderCheck& c, int t) {
+  const uint32_t* w = reinterpret_cast<const uint32_t*>(c.buf);
+  const uint32_t* ref = reinterpret_cast<const uint32_t*>(&c.h);
+  bool ok = true;
+  if (t < 17 && t != 7) ok = (w[t] == ref[t]);   // word 7 is the clock: any value is accepted
+  if (t == 2) ok = ((w[t] & ~2u) == ref[t]);      // flag bit 1 (compacted) may be set or not
+  if (!__all_sync(0xffffffffu, ok) && t == 0) atomicOr(c.dev_status, SFB_DEV_BAD_HEADER);
+}
+#endif
+
 // Header and directory of a buffer, for whichever kernel of a call writes them (buf == nullptr: none).
 struct Commit {
   char* buf;
@@ -314,7 +333,8 @@ int launch_count_pairs(cudaStream_t s, void* sf_buf, const sfb_desc& d, const La
 int launch_kept_rows(cudaStream_t s, const void* sf_buf, int B, int workers, int* idx, int* n_out);
 
 // Sets SFB_DEV_BAD_HEADER in *dev_status unless the buffer's header matches the descriptor.
-int launch_check_header(cudaStream_t s, const void* sf_buf, const sfb_desc& d, const Layout& l, int* dev_status);
+HeaderCheck make_check(const void* sf_buf, const sfb_desc& d, const Layout& l, int* dev_status);
+int launch_check_header(cudaStream_t s, const HeaderCheck& check);
 
 // SC forward: u_i = sum_{(d,a) in code i} a * W[:, d] - x_i, codes read from CSR arrays whose row
 // pointers are either global ([K+1]) or per worker stream inside the SF buffer.
@@ -380,7 +400,8 @@ int launch_cast_bf16(cudaStream_t s, const float* W, __nv_bfloat16* Wb, long lon
 // MN-major: dst[block][64][ldc], block = 32 pairs taken as the apply's reduction blocks are (32 rows of one
 // worker, or k_bb rows of each of k_wp workers), ldc a multiple of 64.
 int launch_split_k(cudaStream_t s, RowMap src, int rows, int cols, void* dst, bool a_side);
-int launch_split_mn(cudaStream_t s, RowMap src, int cols, int workers, int k_bb, int k_wp, int k_bpw, int blocks,
-                    void* dst, int ldc, bool a_side);
+struct SplitSide { RowMap src; int cols; void* dst; int ldc; };   // one factor's rows and where they go (dst == nullptr: not)
+int launch_split_mn(cudaStream_t s, const SplitSide& us, const SplitSide& vs, int workers, int k_bb, int k_wp, int k_bpw,
+                    int blocks, const HeaderCheck& check);
 
 }  // namespace sfb

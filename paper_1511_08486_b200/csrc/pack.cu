@@ -25,16 +25,7 @@ HeaderImage make_header(const sfb_desc& d, const Layout& l, uint32_t clock) {
 
 __global__ void write_header_kernel(const __grid_constant__ Commit c) { chain(); write_header(c, threadIdx.x, blockDim.x); }
 
-__global__ void check_header_kernel(const char* buf, HeaderImage h, int* dev_status) {
-  chain();
-  const uint32_t* w = reinterpret_cast<const uint32_t*>(buf);
-  const uint32_t* ref = reinterpret_cast<const uint32_t*>(&h);
-  const int t = threadIdx.x;   // 32 threads
-  bool ok = true;
-  if (t < 17 && t != 7) ok = (w[t] == ref[t]);   // word 7 is the clock: any value is accepted
-  if (t == 2) ok = ((w[t] & ~2u) == ref[t]);      // flag bit 1 (compacted) may be set or not
-  if (!__all_sync(0xffffffffu, ok) && t == 0) atomicOr(dev_status, SFB_DEV_BAD_HEADER);
-}
+__global__ void check_header_kernel(const __grid_constant__ HeaderCheck c) { chain(); check_header(c, threadIdx.x); }
 
 // grid.x = P workers; each block copies its worker's CSR rows into the stream.
 __global__ void __launch_bounds__(256) pack_csr_kernel(char* buf, long long streams_off, long long stream_stride,
@@ -95,8 +86,16 @@ int launch_write_header(cudaStream_t s, void* sf_buf, const sfb_desc& d, const L
   return cudaGetLastError() == cudaSuccess ? 1 : SFB_ERR_CUDA;
 }
 
-int launch_check_header(cudaStream_t s, const void* sf_buf, const sfb_desc& d, const Layout& l, int* dev_status) {
-  launch_chained(check_header_kernel, 1, 32, 0, s, reinterpret_cast<const char*>(sf_buf), make_header(d, l, 0), dev_status);
+HeaderCheck make_check(const void* sf_buf, const sfb_desc& d, const Layout& l, int* dev_status) {
+  HeaderCheck c;
+  c.buf = reinterpret_cast<const char*>(sf_buf);
+  c.h = make_header(d, l, 0);
+  c.dev_status = dev_status;
+  return c;
+}
+
+int launch_check_header(cudaStream_t s, const HeaderCheck& check) {
+  launch_chained(check_header_kernel, 1, 32, 0, s, check);
   return cudaGetLastError() == cudaSuccess ? 1 : SFB_ERR_CUDA;
 }
 

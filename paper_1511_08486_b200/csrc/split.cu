@@ -61,11 +61,20 @@ __global__ void __launch_bounds__(256) split_k_kernel(RowMap src, int rows, int 
   atom[4 + q] = a_side ? val : rem;
 }
 
-// MN-major.  grid = (reduction blocks, groups of 8 units of 8 values along the padded row); block = 32 lines x 8 units.
-__global__ void __launch_bounds__(256) split_mn_kernel(RowMap src, int cols, int workers, int k_bb, int k_wp, int k_bpw,
-                                                       uint4* __restrict__ dst, int ldc, int a_side) {
+// MN-major, both factors in one launch.  grid = (reduction blocks, groups of 8 units of 8 values along the padded rows of
+// u, then of v); block = 32 lines x 8 units.  On its way it checks the header of the buffer that the rows come from.
+// Bound by launches at small sizes: factors, pack and apply of 300 x 3000 pairs, K = 400, take 40.3 us, with a launch for
+// each factor and one for the check 44.0.
+__global__ void __launch_bounds__(256) split_mn_kernel(const __grid_constant__ SplitSide us, const __grid_constant__ SplitSide vs,
+                                                       int u_groups, int workers, int k_bb, int k_wp, int k_bpw,
+                                                       const __grid_constant__ HeaderCheck check) {
   chain();
-  const int unit = blockIdx.y * 8 + (threadIdx.x & 7);   // 8 values = 16 bytes of bf16
+  if (check.buf != nullptr && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x < 32) check_header(check, threadIdx.x);
+  const int a_side = (int)blockIdx.y < u_groups;
+  const RowMap& src = a_side ? us.src : vs.src;
+  const int cols = a_side ? us.cols : vs.cols, ldc = a_side ? us.ldc : vs.ldc;
+  uint4* dst = reinterpret_cast<uint4*>(a_side ? us.dst : vs.dst);
+  const int unit = ((int)blockIdx.y - (a_side ? 0 : u_groups)) * 8 + (threadIdx.x & 7);   // 8 values = 16 bytes of bf16
   const int line = threadIdx.x >> 3;                      // 0..31: pair inside the reduction block
   const int blk = blockIdx.x;
   if (unit * 8 >= ldc) return;
@@ -98,12 +107,19 @@ int launch_split_k(cudaStream_t s, RowMap src, int rows, int cols, void* dst, bo
   return cudaGetLastError() == cudaSuccess ? 1 : SFB_ERR_CUDA;
 }
 
-int launch_split_mn(cudaStream_t s, RowMap src, int cols, int workers, int k_bb, int k_wp, int k_bpw, int blocks,
-                    void* dst, int ldc, bool a_side) {
-  if (blocks <= 0) return 0;
-  const dim3 grid((unsigned)blocks, (unsigned)((ldc / 8 + 7) / 8));
-  launch_chained(split_mn_kernel, grid, 256, 0, s, src, cols, workers, k_bb, k_wp, k_bpw, reinterpret_cast<uint4*>(dst), ldc,
-                                       a_side ? 1 : 0);
+int launch_split_mn(cudaStream_t s, const SplitSide& us, const SplitSide& vs, int workers, int k_bb, int k_wp, int k_bpw,
+                    int blocks, const HeaderCheck& check) {
+  const int u_groups = us.dst != nullptr ? (us.ldc / 8 + 7) / 8 : 0, v_groups = vs.dst != nullptr ? (vs.ldc / 8 + 7) / 8 : 0;
+  if (blocks <= 0 || u_groups + v_groups == 0) return 0;
+  if (u_groups > 0 && v_groups > 0 && u_groups + v_groups > 65535) {   // the grid's limit: one factor at a time
+    const SplitSide none = {RowMap(), 0, nullptr, 0};
+    const int r = launch_split_mn(s, us, none, workers, k_bb, k_wp, k_bpw, blocks, check);
+    if (r < 0) return r;
+    const int r2 = launch_split_mn(s, none, vs, workers, k_bb, k_wp, k_bpw, blocks, HeaderCheck());
+    return r2 < 0 ? r2 : r + r2;
+  }
+  const dim3 grid((unsigned)blocks, (unsigned)(u_groups + v_groups));
+  launch_chained(split_mn_kernel, grid, 256, 0, s, us, vs, u_groups, workers, k_bb, k_wp, k_bpw, check);
   return cudaGetLastError() == cudaSuccess ? 1 : SFB_ERR_CUDA;
 }
 

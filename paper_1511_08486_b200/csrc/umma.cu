@@ -1395,7 +1395,7 @@ int umma_forward(UmmaPlan* pl, cudaStream_t s, const void* W, const __nv_bfloat1
 // already wrote them there
 static int umma_apply_range(UmmaPlan* pl, cudaStream_t s, void* W, __nv_bfloat16* w_shadow, RowMap u_rows, RowMap v_rows,
                             float eta, int K, const int* dev_status, const void* directory, long long blk0, bool have_u,
-                            bool have_v);
+                            bool have_v, const HeaderCheck& check);
 
 void umma_drop_corr(UmmaPlan* pl) {
   pl->fresh_u = pl->fresh_v = nullptr;
@@ -1403,7 +1403,7 @@ void umma_drop_corr(UmmaPlan* pl) {
 }
 
 int umma_apply(UmmaPlan* pl, cudaStream_t s, void* W, __nv_bfloat16* w_shadow, RowMap u_rows, RowMap v_rows, float eta,
-               int K, const int* dev_status, const void* directory) {
+               int K, const int* dev_status, const void* directory, const HeaderCheck* check) {
   const sfb_desc& d = pl->d;
   // correction operands left by the factor stage of the same step, for exactly these rows (one use)
   const bool chunked = pl->x3 && K > X3_PAIRS_PER_APPLY && K > d.B;
@@ -1411,6 +1411,12 @@ int umma_apply(UmmaPlan* pl, cudaStream_t s, void* W, __nv_bfloat16* w_shadow, R
   const bool have_u = usable && pl->fresh_u == u_rows.base, have_v = usable && pl->fresh_v == v_rows.base;
   pl->fresh_u = pl->fresh_v = nullptr;
   pl->fresh_K = 0;
+  HeaderCheck hc;   // taken along by the first pass over the factor rows, if there is one
+  int launches = 0;
+  if (check != nullptr && check->buf != nullptr) {
+    if (pl->x3 && !(have_u && have_v)) hc = *check;
+    else if ((launches = launch_check_header(s, *check)) < 0) return launches;
+  }
   if (chunked) {
     // The accumulator of a tile rounds toward zero once per 8 pairs (about 1.6e-8 of the sum each time), so an update
     // of very many pairs goes to W in several launches of whole worker streams, each added to W in fp32 by the
@@ -1418,7 +1424,6 @@ int umma_apply(UmmaPlan* pl, cudaStream_t s, void* W, __nv_bfloat16* w_shadow, R
     const int workers = K / d.B;
     int per = X3_PAIRS_PER_APPLY / d.B;
     if (per < 1) per = 1;
-    int launches = 0;
     for (int w0 = 0; w0 < workers; w0 += per) {
       const int n = (workers - w0 < per) ? workers - w0 : per;
       RowMap u = u_rows, v = v_rows;
@@ -1426,18 +1431,20 @@ int umma_apply(UmmaPlan* pl, cudaStream_t s, void* W, __nv_bfloat16* w_shadow, R
       v.base += (long long)w0 * v.worker_stride;
       const void* dir = directory != nullptr ? reinterpret_cast<const char*>(directory) + (size_t)w0 * 32 : nullptr;
       const long long blk0 = d.B >= 32 ? (long long)w0 * ((d.B + 31) / 32) : 0;
-      const int r = umma_apply_range(pl, s, W, w_shadow, u, v, eta, n * d.B, dev_status, dir, blk0, have_u, have_v);
+      const int r = umma_apply_range(pl, s, W, w_shadow, u, v, eta, n * d.B, dev_status, dir, blk0, have_u, have_v, hc);
       if (r < 0) return r;
+      hc = HeaderCheck();
       launches += r;
     }
     return launches;
   }
-  return umma_apply_range(pl, s, W, w_shadow, u_rows, v_rows, eta, K, dev_status, directory, 0, have_u, have_v);
+  const int r = umma_apply_range(pl, s, W, w_shadow, u_rows, v_rows, eta, K, dev_status, directory, 0, have_u, have_v, hc);
+  return r < 0 ? r : launches + r;
 }
 
 static int umma_apply_range(UmmaPlan* pl, cudaStream_t s, void* W, __nv_bfloat16* w_shadow, RowMap u_rows, RowMap v_rows,
                             float eta, int K, const int* dev_status, const void* directory, long long blk0, bool have_u,
-                            bool have_v) {
+                            bool have_v, const HeaderCheck& check) {
   const sfb_desc& d = pl->d;
   const int es = pl->es, CH = 128 / es;
   const int workers = K / d.B;
@@ -1500,15 +1507,8 @@ static int umma_apply_range(UmmaPlan* pl, cudaStream_t s, void* W, __nv_bfloat16
     // correction operands of this launch's factor rows, block by block as the kernel takes them (BK = 32 pairs)
     char* uc = reinterpret_cast<char*>(pl->uc) + blk0 * 64 * pl->ldcu * 2;
     char* vc = reinterpret_cast<char*>(pl->vc) + blk0 * 64 * pl->ldcv * 2;
-    int r;
-    if (!have_u) {
-      if ((r = launch_split_mn(s, u_rows, d.J, workers, p.k_bb, p.k_wp, p.k_bpw, p.k_blocks, uc, pl->ldcu, true)) < 0) return r;
-      launches += r;
-    }
-    if (!have_v) {
-      if ((r = launch_split_mn(s, v_rows, d.D, workers, p.k_bb, p.k_wp, p.k_bpw, p.k_blocks, vc, pl->ldcv, false)) < 0) return r;
-      launches += r;
-    }
+    SplitSide us = {u_rows, d.J, have_u ? nullptr : uc, pl->ldcu}, vs = {v_rows, d.D, have_v ? nullptr : vc, pl->ldcv};
+    if ((launches = launch_split_mn(s, us, vs, workers, p.k_bb, p.k_wp, p.k_bpw, p.k_blocks, check)) < 0) return launches;
     if (!encode_corr_mn_map(&tuc, uc, pl->ldcu, (long long)p.k_blocks * 64, BM / 64) ||
         !encode_corr_mn_map(&tvc, vc, pl->ldcv, (long long)p.k_blocks * 64, (v.bn / v.cg) / 64))
       return SFB_ERR_CUDA;

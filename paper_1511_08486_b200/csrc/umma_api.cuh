@@ -46,7 +46,8 @@ void umma_drop_corr(UmmaPlan* p);
 // u_rows / v_rows: the factor rows (normally the U and V blocks of the SF buffer's worker streams).
 // directory (optional): the SF buffer's directory (sf_buf + 128) of a compacted buffer, whose rows behind each
 // worker's pair count are zeros: reduction blocks that hold only such rows are skipped.
+// check (optional, compensated path): the header check of the buffer, done before W is touched.
 int umma_apply(UmmaPlan* p, cudaStream_t s, void* W, __nv_bfloat16* w_shadow, RowMap u_rows, RowMap v_rows, float eta,
-               int K, const int* dev_status, const void* directory = nullptr);
+               int K, const int* dev_status, const void* directory = nullptr, const HeaderCheck* check = nullptr);
 
 }  // namespace sfb
