@@ -63,7 +63,7 @@ __global__ void __launch_bounds__(256) split_k_kernel(RowMap src, int rows, int 
 
 // MN-major, both factors in one launch.  grid = (reduction blocks, groups of 8 units of 8 values along the padded rows of
 // u, then of v); block = 32 lines x 8 units.  On its way it checks the header of the buffer that the rows come from.
-// Bound by launches at small sizes: factors, pack and apply of 300 x 3000 pairs, K = 400, take 40.3 us, with a launch for
+// Bound by launches at small sizes: factors, pack and apply of 600 x 2000, K = 256, take 40.3 us, with a launch for
 // each factor and one for the check 44.0.
 __global__ void __launch_bounds__(256) split_mn_kernel(const __grid_constant__ SplitSide us, const __grid_constant__ SplitSide vs,
                                                        int u_groups, int workers, int k_bb, int k_wp, int k_bpw,
