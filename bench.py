@@ -154,7 +154,7 @@ def algorithmic(cfg, path, inputs=None):
 
 # dram__bytes_read.sum + dram__bytes_write.sum of one apply launch, from the ncu captures summarised
 # under profiles/ (captured at J = 8192 and scaled by J where the full launch is too large to capture).
-NCU_APPLY_TRAFFIC_BYTES = {("C4", "bf16"): 4.03e9, ("C3", "f32"): 6.28e8, ("C1", "tf32"): 2.03e8, ("C2", "tf32"): 1.21e8,
+NCU_APPLY_TRAFFIC_BYTES = {("C4", "bf16"): 4.03e9, ("C3", "f32"): 3.04e8, ("C1", "tf32"): 2.03e8, ("C2", "tf32"): 1.21e8,
                            ("C1", "f32"): 3.39e8, ("C2", "f32"): 1.95e8}
 
 
