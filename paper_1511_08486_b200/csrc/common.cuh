@@ -5,6 +5,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "per_device.cuh"
 #include "sfb.h"
 
 namespace sfb {
@@ -234,19 +235,18 @@ cudaError_t launch_chained(void (*kernel)(P...), dim3 grid, dim3 block, size_t s
 }
 #endif
 
-// cudaFuncSetAttribute acts on the current device only: first() is true once per device (ordinals 0..63)
-// for the static object it is called on.  A repeated call from a racing thread would set the same value.
-struct PerDeviceOnce {
-  unsigned long long done = 0;
-  bool first() {
-    int dev = 0;
-    cudaGetDevice(&dev);
-    const unsigned long long bit = 1ull << (dev & 63);
-    if (done & bit) return false;
-    done |= bit;
-    return true;
-  }
-};
+// cudaFuncSetAttribute acts on the current device only.  False: the set-up failed, nothing may be launched that needs it.
+template <typename F>
+bool set_up_device(PerDeviceOnce& once, F&& setup) {
+  int dev = 0;
+  if (cudaGetDevice(&dev) == cudaSuccess && once.ok(dev, setup)) return true;
+  cudaGetLastError();
+  return false;
+}
+template <typename K>
+bool allow_smem(K* kernel, size_t bytes) {
+  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) == cudaSuccess;
+}
 
 // ---- kernel launchers (each returns the number of kernels it launched, or a negative SFB_ERR_*) ----
 

@@ -500,11 +500,8 @@ int launch_finish_mlr(cudaStream_t s, RowMap z, RowMap u, const int32_t* labels,
                       int nsplit, long long split_stride_bytes, float* dual, float sdca_step, CorrOut corr,
                       const FinishExtra& extra) {
   const int cf = fin_cache_floats(J);
-  static PerDeviceOnce attr_once;   // function attributes are per device
-  if (attr_once.first()) {
-    cudaFuncSetAttribute(finish_mlr_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, ROW_CACHE_FLOATS * 4);
-    cudaFuncSetAttribute(finish_dml_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, ROW_CACHE_FLOATS * 4);
-  }
+  static PerDeviceOnce attr_once;
+  if (!set_up_device(attr_once, [] { return allow_smem(finish_mlr_kernel, ROW_CACHE_FLOATS * 4); })) return SFB_ERR_CUDA;
   launch_chained(finish_mlr_kernel, K, fin_threads(J), (size_t)cf * 4, s, z, u, labels, K, J, cf, dev_status, nsplit, split_stride_bytes / 4,
                                                               dual, sdca_step, corr, extra);
   return cudaGetLastError() == cudaSuccess ? 1 : SFB_ERR_CUDA;
@@ -548,11 +545,8 @@ int launch_compact_active(cudaStream_t s, const uint8_t* active, int K, int* idx
 int launch_finish_dml(cudaStream_t s, RowMap z, RowMap u, const uint8_t* similar, float margin, int K, int J,
                       int nsplit, long long split_stride_bytes, uint8_t* active, CorrOut corr, const FinishExtra& extra) {
   const int cf = fin_cache_floats(J);
-  static PerDeviceOnce attr_once;   // function attributes are per device
-  if (attr_once.first()) {
-    cudaFuncSetAttribute(finish_mlr_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, ROW_CACHE_FLOATS * 4);
-    cudaFuncSetAttribute(finish_dml_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, ROW_CACHE_FLOATS * 4);
-  }
+  static PerDeviceOnce attr_once;
+  if (!set_up_device(attr_once, [] { return allow_smem(finish_dml_kernel, ROW_CACHE_FLOATS * 4); })) return SFB_ERR_CUDA;
   launch_chained(finish_dml_kernel, K, fin_threads(J), (size_t)cf * 4, s, z, u, similar, margin, K, J, cf, nsplit, split_stride_bytes / 4,
                                                               active, corr, extra);
   return cudaGetLastError() == cudaSuccess ? 1 : SFB_ERR_CUDA;

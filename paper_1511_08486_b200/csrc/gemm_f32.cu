@@ -528,10 +528,9 @@ int launch_apply_f32(cudaStream_t s, float* W, RowMap u, RowMap v, int K, int J,
   const long long big_tiles = (long long)((J + 127) / 128) * ((D + 127) / 128);
   if (big_tiles >= 148) {
     dim3 grid((D + 127) / 128, (J + 127) / 128);
-    static PerDeviceOnce attr_once;   // function attributes are per device
-    if (attr_once.first()) {
-      cudaFuncSetAttribute(sgemm_pipe_kernel<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, PIPE * PIPE_STAGE_FLOATS * 4);
-    }
+    static PerDeviceOnce attr_once;
+    if (!set_up_device(attr_once, [] { return allow_smem(sgemm_pipe_kernel<0>, PIPE * PIPE_STAGE_FLOATS * 4); }))
+      return SFB_ERR_CUDA;
     launch_chained(sgemm_pipe_kernel<0>, grid, 256, PIPE * PIPE_STAGE_FLOATS * 4, s, W, u, v, K, J, D, eta, dev_status, RowMap(), 0, 0,
                                                                          row_idx, n_rows);
   } else {
@@ -584,9 +583,9 @@ int launch_forward_f32_nn(cudaStream_t s, const float* W, RowMap src, RowMap cop
   RowMap a, b;
   a.base = reinterpret_cast<char*>(xt); a.worker_stride = 0; a.ld = ldk; a.B = D; a.es = 4;
   b.base = reinterpret_cast<char*>(wt); b.worker_stride = 0; b.ld = ldj; b.B = D; b.es = 4;
-  static PerDeviceOnce attr_once;   // function attributes are per device
-  if (attr_once.first())
-    cudaFuncSetAttribute(sgemm_pipe_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, PIPE * PIPE_STAGE_FLOATS * 4);
+  static PerDeviceOnce attr_once;
+  if (!set_up_device(attr_once, [] { return allow_smem(sgemm_pipe_kernel<1>, PIPE * PIPE_STAGE_FLOATS * 4); }))
+    return SFB_ERR_CUDA;
   // rows of the output tile = samples (M = K), columns = classes (N = J), reduction over the D features
   dim3 grid((J + 127) / 128, (K + 127) / 128, ks);
   launch_chained(sgemm_pipe_kernel<1>, grid, 256, PIPE * PIPE_STAGE_FLOATS * 4, s, nullptr, a, b, D, K, ldj, 0.f, nullptr,

@@ -367,9 +367,8 @@ bool densify_corr_fits(int ld) { return (size_t)ld * 4 <= 200 * 1024; }
 
 int launch_densify_codes_corr(cudaStream_t s, CsrView codes, RowMap a, int K, int D, int* dev_status, CorrOut corr) {
   const size_t smem = (size_t)a.ld * 4;
-  static PerDeviceOnce attr_once;   // function attributes are per device
-  if (attr_once.first())
-    cudaFuncSetAttribute(densify_corr_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+  static PerDeviceOnce attr_once;
+  if (!set_up_device(attr_once, [] { return allow_smem(densify_corr_kernel, 200 * 1024); })) return SFB_ERR_CUDA;
   launch_chained(densify_corr_kernel, K, 256, smem, s, codes, a, K, D, dev_status, corr);
   return cudaGetLastError() == cudaSuccess ? 1 : SFB_ERR_CUDA;
 }
@@ -384,11 +383,12 @@ int launch_finish_sc(cudaStream_t s, RowMap z, RowMap u, const float* Xdata, int
 
 int launch_sc_apply(cudaStream_t s, float* W, CsrView codes, RowMap u, int K, int J, int D, float eta,
                     const int* dev_status_ro, int* /*dev_status*/) {
-  static PerDeviceOnce attr_once;   // function attributes are per device
-  if (attr_once.first()) {
-    cudaFuncSetAttribute(sc_apply_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SLAB_D * SLAB_J * 4);
-    cudaFuncSetAttribute(sc_apply_kernel, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
-  }
+  static PerDeviceOnce attr_once;
+  const bool ready = set_up_device(attr_once, [] {
+    return allow_smem(sc_apply_kernel, SLAB_D * SLAB_J * 4) &&
+           cudaFuncSetAttribute(sc_apply_kernel, cudaFuncAttributePreferredSharedMemoryCarveout, 100) == cudaSuccess;
+  });
+  if (!ready) return SFB_ERR_CUDA;
   dim3 grid((D + SLAB_D - 1) / SLAB_D, (J + SLAB_J - 1) / SLAB_J);
   sc_apply_kernel<<<grid, SLAB_T, SLAB_D * SLAB_J * 4, s>>>(W, codes, u, K, J, D, eta, dev_status_ro);
   return cudaGetLastError() == cudaSuccess ? 1 : SFB_ERR_CUDA;

@@ -398,9 +398,8 @@ int launch_sc_csc_apply(cudaStream_t s, float* W, RowMap u, int K, int J, int D,
                         void* workspace, const int* dev_status_ro) {
   const CscSlices sl = csc_slices(K);
   const CscScratch w = csc_scratch(workspace, K, D);
-  static PerDeviceOnce attr_once;   // function attributes are per device
-  if (attr_once.first())
-    cudaFuncSetAttribute(csc_apply_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024);
+  static PerDeviceOnce attr_once;
+  if (!set_up_device(attr_once, [] { return allow_smem(csc_apply_kernel, 220 * 1024); })) return SFB_ERR_CUDA;
   const long long work = (long long)((J + CSC2_JT - 1) / CSC2_JT) * ((D + CSC2_AB - 1) / CSC2_AB);
   long long blocks = (work + CSC2_WARPS - 1) / CSC2_WARPS;   // at least one block of atoms per warp
   if (blocks > 148) blocks = 148;

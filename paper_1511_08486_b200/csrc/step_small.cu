@@ -174,9 +174,8 @@ bool step_small_fits(int K, int J, int D) {
 
 int launch_step_small(cudaStream_t s, const sfb_desc& d, float* W, const float* X, const sfb_aux* aux, RowMap u, RowMap v,
                       int K, int K_apply, float eta, int* dev_status, const Commit& commit) {
-  static PerDeviceOnce attr_once;   // function attributes are per device
-  if (attr_once.first())
-    cudaFuncSetAttribute(step_small_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_MAX);
+  static PerDeviceOnce attr_once;
+  if (!set_up_device(attr_once, [] { return allow_smem(step_small_kernel, SMEM_MAX); })) return SFB_ERR_CUDA;
   SmallStep p = {};
   p.W = W; p.X = X;
   if (d.model == SFB_DML) {

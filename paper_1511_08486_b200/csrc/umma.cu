@@ -755,14 +755,13 @@ int launch_gemm(cudaStream_t s, const CUtensorMap& a, const CUtensorMap& b, cons
   constexpr int stages = (RING_BYTES / stage_bytes) < MAX_STAGES ? (RING_BYTES / stage_bytes) : MAX_STAGES;
   constexpr int smem = stages * stage_bytes + EPI_STAGE_BYTES + 1024 + (int)sizeof(SharedCtl);
   auto kernel = umma_gemm_kernel<ES, APPLY, BN, CG, KA, FOLD, EPI, SPLIT>;
-  static PerDeviceOnce attr_once;   // function attributes are per device
+  static PerDeviceOnce attr_once;
   static int max_clusters = 0;
-  if (attr_once.first()) {
-    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess)
-      return SFB_ERR_CUDA;
+  const bool ready = set_up_device(attr_once, [&] {
+    if (!allow_smem(kernel, smem)) return false;
     cudaFuncAttributes fa;
-    if (cudaFuncGetAttributes(&fa, kernel) != cudaSuccess) return SFB_ERR_CUDA;
-    if (SPLIT && fa.numRegs != SPLIT_LAUNCH_REGS) return SFB_ERR_CUDA;   // the register split would wait for ever
+    if (cudaFuncGetAttributes(&fa, kernel) != cudaSuccess) return false;
+    if (SPLIT && fa.numRegs != SPLIT_LAUNCH_REGS) return false;   // the register split would wait for ever
     if (CG == 2) {   // how many CTA pairs the device can hold at once
       cudaLaunchConfig_t q;
       memset(&q, 0, sizeof(q));
@@ -778,7 +777,9 @@ int launch_gemm(cudaStream_t s, const CUtensorMap& a, const CUtensorMap& b, cons
         max_clusters = num_sms / 2;
       }
     }
-  }
+    return true;
+  });
+  if (!ready) return SFB_ERR_CUDA;
   const int tiles = p.m_tiles * p.n_tiles * p.k_splits;
   if (CG == 1) {
     const int grid = tiles < num_sms ? tiles : num_sms;
