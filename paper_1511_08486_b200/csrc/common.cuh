@@ -215,7 +215,10 @@ __device__ __forceinline__ float4 sdca_step4(float* dual_row, int j, int J, floa
 // it ends: their blocks, two to four to an SM, would otherwise crowd onto the SMs that run free first.  40 x 15000,
 // K = 800: 318 us a step, 399 with it.)
 // Nothing before the wait reads or writes global memory, and every thread waits, so each grid is complete, its writes
-// visible, before its successor touches memory, exactly as without the overlap.
+// visible, before its successor touches memory, exactly as without the overlap.  That holds for ordinary loads only: the
+// read-only path asks for data that does not change while the kernel runs, which here begins before the wait, and the
+// compiler may move a load from a __restrict__ pointer above it.  So these kernels declare no pointer __restrict__ and
+// use no __ldg, for the caller's arrays neither (their producer may itself have let its successor start early).
 #ifdef __CUDACC__
 __device__ __forceinline__ void chain_next() { asm volatile("griddepcontrol.launch_dependents;"); }
 __device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }

@@ -19,7 +19,7 @@ constexpr int WAVE = 256;         // rows per wave of the move, one per thread
 constexpr int SLICE_UNITS = 8;    // 16-byte units per column slice
 
 // flags[i] = 1 if the wire values of u row i are not all zero (-0 counts as zero).  One warp per row.
-__global__ void __launch_bounds__(256) row_nonzero_kernel(RowMap u, int K, int J, uint8_t* __restrict__ flags) {
+__global__ void __launch_bounds__(256) row_nonzero_kernel(RowMap u, int K, int J, uint8_t* flags) {
   chain();
   const int i = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (i >= K) return;
@@ -46,7 +46,7 @@ __global__ void __launch_bounds__(256) row_nonzero_kernel(RowMap u, int K, int J
 // scan that the finishing pass and this kernel now do on the way).
 __global__ void __launch_bounds__(256) compact_move_kernel(char* buf, char* streams, long long stream_stride, long long v_off,
                                                            int B, int u_units, int v_units, int u_slices,
-                                                           const uint8_t* __restrict__ flags, int* __restrict__ counts,
+                                                           const uint8_t* flags, int* counts,
                                                            int first_worker, int n_workers) {
   chain();
   __shared__ uint4 wave[WAVE * SLICE_UNITS];   // 32 KB
@@ -104,8 +104,8 @@ __global__ void __launch_bounds__(256) compact_move_kernel(char* buf, char* stre
 }
 
 // idx[0 .. *n_out) = p * B + r for every worker p < workers and every r < its pair count, in that order.
-__global__ void __launch_bounds__(256) kept_rows_kernel(const char* buf, int B, int workers, int* __restrict__ idx,
-                                                        int* __restrict__ n_out) {
+__global__ void __launch_bounds__(256) kept_rows_kernel(const char* buf, int B, int workers, int* idx,
+                                                        int* n_out) {
   chain_wait();
   __shared__ int base;
   if (threadIdx.x == 0) base = 0;
@@ -124,7 +124,7 @@ __global__ void __launch_bounds__(256) kept_rows_kernel(const char* buf, int B, 
 
 // One block per worker: n_sf of its directory entry = number of its u rows flagged nonzero (in a compacted stream
 // the kept pairs are exactly the leading rows); block 0 sets the header's "compacted" flag.
-__global__ void __launch_bounds__(256) count_pairs_kernel(const uint8_t* __restrict__ flags, int B, char* buf) {
+__global__ void __launch_bounds__(256) count_pairs_kernel(const uint8_t* flags, int B, char* buf) {
   chain();
   __shared__ int total;
   if (threadIdx.x == 0) total = 0;

@@ -115,15 +115,16 @@ __device__ __forceinline__ bool wire_nonzero4(const float4& t, int es) {
 }
 
 // z rows are fp32 with ld a multiple of 4; values beyond J inside the last float4 are ignored.
-__global__ void __launch_bounds__(1024) finish_mlr_kernel(RowMap z, RowMap u, const int32_t* __restrict__ labels,
+__global__ void __launch_bounds__(1024) finish_mlr_kernel(RowMap z, RowMap u, const int32_t* labels,
                                                                  int K, int J, int cache_floats, int* dev_status, int nsplit, long long zstride,
-                                                                 float* __restrict__ dual, float sdca_step, CorrOut corr, const __grid_constant__ FinishExtra extra) {
+                                                                 float* dual, float sdca_step, CorrOut corr, const __grid_constant__ FinishExtra extra) {
   if (extra.next_early) chain_next();
   chain_wait();
   extern __shared__ __align__(16) float cache[];
   __shared__ float red[32];
   const int i = blockIdx.x;
   if (i >= K) return;
+  const int y = labels[i];   // (early: its latency passes beside the row's)
   finish_extra(extra, i);
   const float* zr = reinterpret_cast<const float*>(z.row(i));
   char* ur = u.row(i);
@@ -164,7 +165,6 @@ __global__ void __launch_bounds__(1024) finish_mlr_kernel(RowMap z, RowMap u, co
   s = block_sum(s, red);
   const float inv = 1.0f / s;
 
-  const int y = labels[i];
   const bool bad = (y < 0) || (y >= J);
   if (bad && threadIdx.x == 0) atomicOr(dev_status, SFB_DEV_BAD_LABEL);
   const int ld4 = u.ld >> 2;   // u.ld is a multiple of 4 (fp32) or 8 (bf16)
@@ -197,15 +197,16 @@ __global__ void __launch_bounds__(1024) finish_mlr_kernel(RowMap z, RowMap u, co
   flag_row(extra, i, any);
 }
 
-__global__ void __launch_bounds__(1024) finish_dml_kernel(RowMap z, RowMap u, const uint8_t* __restrict__ similar,
+__global__ void __launch_bounds__(1024) finish_dml_kernel(RowMap z, RowMap u, const uint8_t* similar,
                                                                  float margin, int K, int J, int cache_floats, int nsplit, long long zstride,
-                                                                 uint8_t* __restrict__ active, CorrOut corr, const __grid_constant__ FinishExtra extra) {
+                                                                 uint8_t* active, CorrOut corr, const __grid_constant__ FinishExtra extra) {
   if (extra.next_early) chain_next();
   chain_wait();
   extern __shared__ __align__(16) float cache[];
   __shared__ float red[32];
   const int i = blockIdx.x;
   if (i >= K) return;
+  const bool sim = similar[i] != 0;   // (early: its latency passes beside the row's)
   finish_extra(extra, i);
   const float* zr = reinterpret_cast<const float*>(z.row(i));
   char* ur = u.row(i);
@@ -223,7 +224,6 @@ __global__ void __launch_bounds__(1024) finish_dml_kernel(RowMap z, RowMap u, co
     n += (t.x * t.x + t.y * t.y) + (t.z * t.z + t.w * t.w);
   }
   n = block_sum(n, red);
-  const bool sim = similar[i] != 0;
   const float g = sim ? 1.f : ((n < margin) ? -1.f : 0.f);   // strict hinge: inactive at equality
   if (active != nullptr && threadIdx.x == 0) active[i] = (g != 0.f) ? 1 : 0;   // u_i is all zeros otherwise
 
@@ -250,9 +250,9 @@ __global__ void __launch_bounds__(1024) finish_dml_kernel(RowMap z, RowMap u, co
 // in the u row (p = the half tile that holds class j) and (m_p, s_p = sum of those exps) per part.
 // Here: m = max_p m_p, s = sum_p s_p exp(m_p - m), u[j] = e[j] * exp(m_p - m) / s - [j == label], in place.
 template <int ES>
-__global__ void __launch_bounds__(256) finish_mlr_fused_kernel(RowMap u, const float2* __restrict__ stats, int n_parts,
-                                                               int part_cols, const int32_t* __restrict__ labels, int K,
-                                                               int J, int* dev_status, float* __restrict__ dual,
+__global__ void __launch_bounds__(256) finish_mlr_fused_kernel(RowMap u, const float2* stats, int n_parts,
+                                                               int part_cols, const int32_t* labels, int K,
+                                                               int J, int* dev_status, float* dual,
                                                                float sdca_step, const __grid_constant__ FinishExtra extra) {
   if (extra.next_early) chain_next();
   chain_wait();
@@ -260,6 +260,7 @@ __global__ void __launch_bounds__(256) finish_mlr_fused_kernel(RowMap u, const f
   __shared__ float red[32];
   const int i = blockIdx.x;
   if (i >= K) return;
+  const int y = labels[i];   // (early: its latency passes beside the row's)
   finish_extra(extra, i);
   const float kLog2e = 1.4426950408889634f;
   const float2* st = stats + (size_t)i * n_parts;
@@ -275,7 +276,6 @@ __global__ void __launch_bounds__(256) finish_mlr_fused_kernel(RowMap u, const f
   }
   ssum = block_sum(ssum, red);   // also orders the writes of scale[] before the reads below
   const float inv = 1.0f / ssum;
-  const int y = labels[i];
   const bool bad = (y < 0) || (y >= J);
   if (bad && threadIdx.x == 0) atomicOr(dev_status, SFB_DEV_BAD_LABEL);
   char* ur = u.row(i);
@@ -341,7 +341,7 @@ __global__ void __launch_bounds__(256) finish_mlr_fused_kernel(RowMap u, const f
 // the 164 MB of the operand, whose stand-alone rebuild before the next forward pass took 45 us.)
 constexpr int PROX_HELD = 16, PROX_THREADS = 256, PROX_ROWS = PROX_THREADS / 8;
 template <bool VEC>
-__global__ void __launch_bounds__(PROX_THREADS, VEC ? 2 : 1) prox_unit_columns_kernel(float* __restrict__ W, int J, int D,
+__global__ void __launch_bounds__(PROX_THREADS, VEC ? 2 : 1) prox_unit_columns_kernel(float* W, int J, int D,
                                                                             int rows_per_cta, __nv_bfloat16* shadow) {
   chain();
   __shared__ float4 part[PROX_ROWS][9];
@@ -450,7 +450,7 @@ __global__ void __launch_bounds__(256) pack_rows_kernel(RowMap u_src, RowMap u_d
 }
 
 // v rows = Xa - Xb (one fp32 subtraction per element), pad columns zero; 4 values per thread.
-__global__ void __launch_bounds__(256) diff_rows_kernel(const float* __restrict__ Xa, const float* __restrict__ Xb, RowMap v,
+__global__ void __launch_bounds__(256) diff_rows_kernel(const float* Xa, const float* Xb, RowMap v,
                                                         int K, int D, CorrOut corr) {
   chain();
   const int units = v.ld >> 2;
@@ -473,7 +473,7 @@ __global__ void __launch_bounds__(256) diff_rows_kernel(const float* __restrict_
   }
 }
 
-__global__ void __launch_bounds__(256) cast_bf16_kernel(const float* __restrict__ W, __nv_bfloat16* __restrict__ Wb,
+__global__ void __launch_bounds__(256) cast_bf16_kernel(const float* W, __nv_bfloat16* Wb,
                                                         long long n4) {
   chain();
   for (long long g = blockIdx.x * (long long)blockDim.x + threadIdx.x; g < n4; g += (long long)gridDim.x * blockDim.x) {
@@ -508,8 +508,8 @@ int launch_finish_mlr(cudaStream_t s, RowMap z, RowMap u, const int32_t* labels,
 }
 
 // idx[0 .. n) = the samples i < K with active[i] != 0, in ascending order; *n_out = n.  One block, ordered.
-__global__ void __launch_bounds__(1024) compact_active_kernel(const uint8_t* __restrict__ active, int K, int* __restrict__ idx,
-                                                              int* __restrict__ n_out) {
+__global__ void __launch_bounds__(1024) compact_active_kernel(const uint8_t* active, int K, int* idx,
+                                                              int* n_out) {
   chain_wait();
   __shared__ int warp_cnt[32];
   __shared__ int base;

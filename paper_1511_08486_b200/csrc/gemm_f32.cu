@@ -66,8 +66,8 @@ __device__ __forceinline__ void mma_tile(const float (*As)[64 * MI + 4], const f
 // Tile rows = samples i (BM = 64*MI), tile columns = classes j (BN = 64*NI), reduction over d.
 // Both operands are contiguous along d, so tiles are transposed while being stored to shared memory.
 template <int MI, int NI>
-__global__ void __launch_bounds__(256, 2) forward_f32_kernel(const float* __restrict__ W, const float* __restrict__ X,
-                                                          const float* __restrict__ Xb, int K, int J, int D,
+__global__ void __launch_bounds__(256, 2) forward_f32_kernel(const float* W, const float* X,
+                                                          const float* Xb, int K, int J, int D,
                                                           RowMap z, RowMap v) {
   chain_wait();
   constexpr int BM = 64 * MI, BN = 64 * NI;
@@ -86,7 +86,12 @@ __global__ void __launch_bounds__(256, 2) forward_f32_kernel(const float* __rest
     for (int n = 0; n < 2 * NI; ++n) acc[m][n] = make_float2(0.f, 0.f);
 
   float4 pa[MI], pb[NI];
-  auto fetch = [&](int d0) {
+  auto fetch = [&](int d0) {   // (W first: its loads do not wait behind the stores of v)
+#pragma unroll
+    for (int q = 0; q < NI; ++q) {
+      const int j = j0 + lr + 64 * q;
+      pb[q] = (j < J) ? ld4_guard(W + (size_t)j * D, d0 + lc, D, vec_ok) : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
 #pragma unroll
     for (int q = 0; q < MI; ++q) {
       const int i = i0 + lr + 64 * q;
@@ -100,11 +105,6 @@ __global__ void __launch_bounds__(256, 2) forward_f32_kernel(const float* __rest
         if (write_v && d0 + lc < v.ld) *reinterpret_cast<float4*>(v.row(i) + (size_t)(d0 + lc) * 4) = a;
       }
       pa[q] = a;
-    }
-#pragma unroll
-    for (int q = 0; q < NI; ++q) {
-      const int j = j0 + lr + 64 * q;
-      pb[q] = (j < J) ? ld4_guard(W + (size_t)j * D, d0 + lc, D, vec_ok) : make_float4(0.f, 0.f, 0.f, 0.f);
     }
   };
   auto stash = [&]() {
@@ -166,10 +166,10 @@ template <int N>
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 
 template <int OUT>
-__global__ void __launch_bounds__(256, 2) sgemm_pipe_kernel(float* __restrict__ W, RowMap u, RowMap v, int K, int J,
-                                                         int D, float eta, const int* __restrict__ dev_status,
+__global__ void __launch_bounds__(256, 2) sgemm_pipe_kernel(float* W, RowMap u, RowMap v, int K, int J,
+                                                         int D, float eta, const int* dev_status,
                                                          RowMap z, int k_per_range, long long range_stride,
-                                                         const int* __restrict__ row_idx, const int* __restrict__ n_rows) {
+                                                         const int* row_idx, const int* n_rows) {
   chain_wait();
   constexpr int BM = 128, BN = 128;
   extern __shared__ __align__(16) float ring[];
@@ -397,7 +397,7 @@ __global__ void __launch_bounds__(256, 4) sgemm_small_kernel(const __grid_consta
 
 // dst[c][r] = src row r, column c (R rows of C values behind a row map; dst rows ldr floats long, columns R .. ldr - 1
 // zero).  `copy` (optional): the same rows also copied there, pad columns zero (the factor v = x of the MLR model).
-__global__ void __launch_bounds__(256) transpose_rows_kernel(RowMap src, float* __restrict__ dst, int R, int C, int ldr,
+__global__ void __launch_bounds__(256) transpose_rows_kernel(RowMap src, float* dst, int R, int C, int ldr,
                                                              RowMap copy) {
   chain_wait();
   __shared__ float tile[32][33];

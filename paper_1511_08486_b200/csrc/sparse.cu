@@ -46,7 +46,7 @@ __device__ __forceinline__ CsrRow csr_row(const CsrView& c, int i) {
 }
 
 // Wt[d][j] = W[j][d]; Wt rows have ldt values (J rounded up to 4), pad columns zero.
-__global__ void __launch_bounds__(256) transpose_kernel(const float* __restrict__ W, float* __restrict__ Wt, int J, int D,
+__global__ void __launch_bounds__(256) transpose_kernel(const float* W, float* Wt, int J, int D,
                                                         int ldt) {
   chain();
   __shared__ float tile[32][33];
@@ -66,8 +66,8 @@ __global__ void __launch_bounds__(256) transpose_kernel(const float* __restrict_
 }
 
 // grid = (K samples, ceil(ldt / 1024)); each thread owns 4 consecutive rows j of W.
-__global__ void __launch_bounds__(256) sc_forward_kernel(const float* __restrict__ Wt, int ldt, CsrView codes,
-                                                         const float* __restrict__ Xdata, RowMap u, int K, int J, int D,
+__global__ void __launch_bounds__(256) sc_forward_kernel(const float* Wt, int ldt, CsrView codes,
+                                                         const float* Xdata, RowMap u, int K, int J, int D,
                                                          int* dev_status) {
   chain();
   __shared__ uint32_t s_idx[256];
@@ -169,7 +169,7 @@ __global__ void __launch_bounds__(256) densify_corr_kernel(CsrView codes, RowMap
   }
 }
 
-__global__ void __launch_bounds__(256) finish_sc_kernel(RowMap zr, RowMap u, const float* __restrict__ Xdata, int K, int J,
+__global__ void __launch_bounds__(256) finish_sc_kernel(RowMap zr, RowMap u, const float* Xdata, int K, int J,
                                                         int nsplit, long long zstride, CorrOut corr) {
   chain();
   const int units = u.ld >> 2;

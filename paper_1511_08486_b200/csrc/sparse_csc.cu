@@ -76,8 +76,8 @@ __global__ void __launch_bounds__(256) csc_mask_kernel(CsrView codes, int K, int
 
 // per atom: populations of the chunks' masks -> offsets of each chunk inside the column's slice; slice totals
 __global__ void __launch_bounds__(64) csc_chunk_offsets_kernel(int nchunks, int chunks_per_slice, int D,
-                                                               const uint32_t* __restrict__ mask, int* __restrict__ off,
-                                                               int* __restrict__ total) {
+                                                               const uint32_t* mask, int* off,
+                                                               int* total) {
   chain();
   const int d = blockIdx.x * 64 + threadIdx.x;
   if (d >= D) return;
@@ -102,7 +102,7 @@ __global__ void __launch_bounds__(64) csc_chunk_offsets_kernel(int nchunks, int 
 }
 
 // colptr[0 .. n] = exclusive scan of total[0 .. n) rounded up to fours (one block, fixed order; eight sums a thread)
-__global__ void __launch_bounds__(1024) csc_scan_kernel(int n, const int* __restrict__ total, int* __restrict__ colptr) {
+__global__ void __launch_bounds__(1024) csc_scan_kernel(int n, const int* total, int* colptr) {
   chain();
   __shared__ int warp_sum[32];
   constexpr int PER = 8;
@@ -145,9 +145,9 @@ __global__ void __launch_bounds__(1024) csc_scan_kernel(int n, const int* __rest
 // Blocks 0 .. K - 1: one sample each, every entry to its place (entry = sample index inside its slice, value); the
 // blocks behind them write the zero entries that fill the columns up.
 __global__ void __launch_bounds__(256) csc_fill_kernel(CsrView codes, int K, int D, int passes, int chunks_per_slice,
-                                                       const uint32_t* __restrict__ mask, const int* __restrict__ off,
-                                                       const int* __restrict__ total, const int* __restrict__ colptr,
-                                                       int2* __restrict__ ent) {
+                                                       const uint32_t* mask, const int* off,
+                                                       const int* total, const int* colptr,
+                                                       int2* ent) {
   chain();
   if (blockIdx.x >= (unsigned)K) {
     const int c = (blockIdx.x - K) * 256 + threadIdx.x;
@@ -189,10 +189,10 @@ constexpr int CSC2_WARP_FLOATS = 2 * CSC2_STRIP + CSC2_AB * CSC2_TS;   // entry 
 // are read together; 20 warps (16: 5 % 488 us; 24 or 32, with fewer registers: 461 and 464, small problems 10 % slower).
 // 4096 x 10000, K = 1024, against half warps on 64 rows with W loaded when its block begins: 5 % density 514 -> 443 us an
 // apply, 2 % 355 -> 274, 1 % 304 -> 206 (3000 x 500, K = 320: 21.9 -> 22.5).
-__global__ void __launch_bounds__(CSC2_WARPS * 32) csc_apply_kernel(float* __restrict__ W, RowMap u, int K, int J, int D,
-                                                                    float eta, const int* __restrict__ colptr,
-                                                                    const int2* __restrict__ ent, int passes, int Kh,
-                                                                    const int* __restrict__ status_ro) {
+__global__ void __launch_bounds__(CSC2_WARPS * 32) csc_apply_kernel(float* W, RowMap u, int K, int J, int D,
+                                                                    float eta, const int* colptr,
+                                                                    const int2* ent, int passes, int Kh,
+                                                                    const int* status_ro) {
   chain();
   extern __shared__ __align__(16) float smem[];
   if (status_ro != nullptr && (*status_ro & SFB_DEV_BAD_HEADER)) return;

@@ -40,7 +40,7 @@ __device__ __forceinline__ void split8(const float4& x0, const float4& x1, uint4
 }
 
 // K-major.  One thread per (row, 8 values); cols is a multiple of 4, rows are 16-byte aligned.
-__global__ void __launch_bounds__(256) split_k_kernel(RowMap src, int rows, int cols, int atoms, uint4* __restrict__ dst,
+__global__ void __launch_bounds__(256) split_k_kernel(RowMap src, int rows, int cols, int atoms, uint4* dst,
                                                       int a_side) {
   chain();
   const long long t = (long long)blockIdx.x * 256 + threadIdx.x;
@@ -50,8 +50,8 @@ __global__ void __launch_bounds__(256) split_k_kernel(RowMap src, int rows, int 
   const int g = (int)(t - row * per_row);   // group of 8 values inside the row
   const float* x = reinterpret_cast<const float*>(src.row((int)row)) + g * 8;
   const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
-  const float4 x0 = (g * 8 < cols) ? __ldg(reinterpret_cast<const float4*>(x)) : zero;
-  const float4 x1 = (g * 8 + 4 < cols) ? __ldg(reinterpret_cast<const float4*>(x) + 1) : zero;
+  const float4 x0 = (g * 8 < cols) ? *reinterpret_cast<const float4*>(x) : zero;
+  const float4 x1 = (g * 8 + 4 < cols) ? reinterpret_cast<const float4*>(x)[1] : zero;
   uint4 val, rem;
   split8(x0, x1, val, rem);
   // atom g / 4 of the row: eight 16-byte units, the first four of one kind and the last four of the other
@@ -85,8 +85,8 @@ __global__ void __launch_bounds__(256) split_mn_kernel(const __grid_constant__ S
   float4 x0 = zero, x1 = zero;
   if (worker < workers && row < src.B) {
     const float* x = reinterpret_cast<const float*>(src.row(worker * src.B + row)) + unit * 8;
-    if (unit * 8 < cols) x0 = __ldg(reinterpret_cast<const float4*>(x));
-    if (unit * 8 + 4 < cols) x1 = __ldg(reinterpret_cast<const float4*>(x) + 1);
+    if (unit * 8 < cols) x0 = *reinterpret_cast<const float4*>(x);
+    if (unit * 8 + 4 < cols) x1 = reinterpret_cast<const float4*>(x)[1];
   }
   uint4 val, rem;
   split8(x0, x1, val, rem);
