@@ -586,7 +586,7 @@ static int apply_from(sfb_ctx* c, void* W, const void* sf_buf, float eta, int K,
   if (d.v_sparse && d.path == SFB_PATH_F32 && c->csc_ws != nullptr) {
     if (!csc_built)
       ACC(launch_sc_csc_build(c->stream, stream_codes(c, sf_buf), K, d.D, (long long)d.nnz_capacity, c->csc_ws,
-                              c->dev_status));
+                              c->dev_status, check ? c->dev_status : nullptr));
     ACC(launch_sc_csc_apply(c->stream, reinterpret_cast<float*>(W), stream_u(c, sf_buf), K, d.J, d.D, eta,
                             (long long)d.nnz_capacity, c->csc_ws, c->dev_status));
   } else if (d.v_sparse && d.path == SFB_PATH_F32) {
@@ -596,7 +596,7 @@ static int apply_from(sfb_ctx* c, void* W, const void* sf_buf, float eta, int K,
     // dense alternative: rebuild the dense code rows from the buffer's CSR streams unless this step just made them
     if (check)
       ACC(launch_densify_codes(c->stream, stream_codes(c, sf_buf), dense_codes(c), K, d.D, c->dev_status,
-                               d.path == SFB_PATH_TF32));
+                               d.path == SFB_PATH_TF32, c->dev_status));
     ACC(umma_apply(c->umma, c->stream, W, has_shadow(c) ? c->w_shadow : nullptr, stream_u(c, sf_buf), dense_codes(c), eta,
                    K, c->dev_status));
     if (has_shadow(c)) c->shadow_of = W;   // the apply epilogue rewrote the shadow from the new W

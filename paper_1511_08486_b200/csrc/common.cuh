@@ -120,6 +120,11 @@ struct HeaderCheck {
   __host__ __device__ HeaderCheck() : buf(nullptr), h(), dev_status(nullptr) {}
 };
 #ifdef __CUDACC__
+// Has the check that precedes this kernel refused the buffer it was given (refused: the status word, or nullptr = not
+// checked)?  Then nothing in that buffer may be followed: row pointers and offsets could lead anywhere.
+__device__ __forceinline__ bool is_refused(const int* refused) {
+  return refused != nullptr && (*refused & SFB_DEV_BAD_HEADER) != 0;
+}
 // one whole warp, t = lane
 __device__ __forceinline__ void check_header(const HeaderCheck& c, int t) {
   const uint32_t* w = reinterpret_cast<const uint32_t*>(c.buf);
@@ -370,14 +375,17 @@ int launch_sc_apply_csc(cudaStream_t s, float* W, CsrView codes, RowMap u, int K
 // pass), the update needs u and the workspace the re-sort filled.
 // dev_status (optional): SFB_DEV_BAD_INDEX is set for entries the re-sort leaves out (atom out of range, row not
 // strictly ascending: the same entries the forward pass skips).
+// refused: see is_refused (no entry is sorted then).
 int launch_sc_csc_build(cudaStream_t s, CsrView codes, int K, int D, long long nnz_capacity, void* workspace,
-                        int* dev_status = nullptr);
+                        int* dev_status = nullptr, const int* refused = nullptr);
 int launch_sc_csc_apply(cudaStream_t s, float* W, RowMap u, int K, int J, int D, float eta, long long nnz_capacity,
                         void* workspace, const int* dev_status_ro);
 
 // Dense fp32 rows a_i of the CSR codes (zeros elsewhere), for the tensor-core sparse-coding path.
 // round_tf32: values rounded to the nearest tf32 (the plain tf32 path, whose tensor cores would truncate them).
-int launch_densify_codes(cudaStream_t s, CsrView codes, RowMap a, int K, int D, int* dev_status, bool round_tf32 = true);
+// refused: see is_refused (the rows stay as they are then).
+int launch_densify_codes(cudaStream_t s, CsrView codes, RowMap a, int K, int D, int* dev_status, bool round_tf32 = true,
+                         const int* refused = nullptr);
 // The same (exact values) with the rows' correction operands written beside them; a row of ld floats must fit in
 // shared memory (densify_corr_fits).
 bool densify_corr_fits(int ld);

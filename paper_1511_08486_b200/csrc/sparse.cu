@@ -124,8 +124,9 @@ __global__ void __launch_bounds__(256) sc_forward_kernel(const float* Wt, int ld
 
 // One block per sample: zero the dense row, then scatter the sample's nonzeros into it.
 __global__ void __launch_bounds__(256) densify_kernel(CsrView codes, RowMap a, int K, int D, int* dev_status,
-                                                      bool round_tf32) {
+                                                      bool round_tf32, const int* refused) {
   chain();
+  if (is_refused(refused)) return;
   const int i = blockIdx.x;
   float* dst = reinterpret_cast<float*>(a.row(i));
   for (int q = threadIdx.x; q < (a.ld >> 2); q += 256) reinterpret_cast<float4*>(dst)[q] = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -358,8 +359,9 @@ int launch_sc_forward_ws(cudaStream_t s, const float* W, float* Wt, CsrView code
   return cudaGetLastError() == cudaSuccess ? 2 : SFB_ERR_CUDA;
 }
 
-int launch_densify_codes(cudaStream_t s, CsrView codes, RowMap a, int K, int D, int* dev_status, bool round_tf32) {
-  launch_chained(densify_kernel, K, 256, 0, s, codes, a, K, D, dev_status, round_tf32);
+int launch_densify_codes(cudaStream_t s, CsrView codes, RowMap a, int K, int D, int* dev_status, bool round_tf32,
+                         const int* refused) {
+  launch_chained(densify_kernel, K, 256, 0, s, codes, a, K, D, dev_status, round_tf32, refused);
   return cudaGetLastError() == cudaSuccess ? 1 : SFB_ERR_CUDA;
 }
 

@@ -62,7 +62,8 @@ __device__ __forceinline__ bool entry_ok(const CsrRow2& row, int k, int D) {
 
 // bit i % 32 of mask[i / 32][d]: sample i uses atom d (atomic or: the masks do not depend on the order)
 __global__ void __launch_bounds__(256) csc_mask_kernel(CsrView codes, int K, int D, uint32_t* __restrict__ mask,
-                                                       int* dev_status) {
+                                                       int* dev_status, const int* refused) {
+  if (is_refused(refused)) return;
   const int i = blockIdx.x;
   const CsrRow2 row = csr_row2(codes, i);
   uint32_t* m = mask + (size_t)(i / CSC_CHUNK) * D;
@@ -147,8 +148,9 @@ __global__ void __launch_bounds__(1024) csc_scan_kernel(int n, const int* total,
 __global__ void __launch_bounds__(256) csc_fill_kernel(CsrView codes, int K, int D, int passes, int chunks_per_slice,
                                                        const uint32_t* mask, const int* off,
                                                        const int* total, const int* colptr,
-                                                       int2* ent) {
+                                                       int2* ent, const int* refused) {
   chain();
+  if (is_refused(refused)) return;   // (every column is empty: no mask was written)
   if (blockIdx.x >= (unsigned)K) {
     const int c = (blockIdx.x - K) * 256 + threadIdx.x;
     if (c < passes * D) {
@@ -379,17 +381,17 @@ CscScratch csc_scratch(void* workspace, int K, int D) {
 // Atom-major re-sort of the codes into the workspace.  Reads the codes only (not u), so it may run beside
 // the forward pass that produces u.
 int launch_sc_csc_build(cudaStream_t s, CsrView codes, int K, int D, long long nnz_capacity, void* workspace,
-                        int* dev_status) {
+                        int* dev_status, const int* refused) {
   const int nchunks = (K + CSC_CHUNK - 1) / CSC_CHUNK;
   const CscSlices sl = csc_slices(K);
   const CscScratch w = csc_scratch(workspace, K, D);
   const int cps = sl.Kh / CSC_CHUNK, cols = sl.passes * D;
   if (cudaMemsetAsync(w.mask, 0, (size_t)nchunks * D * 4, s) != cudaSuccess) return SFB_ERR_CUDA;
-  csc_mask_kernel<<<K, 256, 0, s>>>(codes, K, D, w.mask, dev_status);
+  csc_mask_kernel<<<K, 256, 0, s>>>(codes, K, D, w.mask, dev_status, refused);
   launch_chained(csc_chunk_offsets_kernel, (D + 63) / 64, 64, 0, s, nchunks, cps, D, w.mask, w.off, w.total);
   launch_chained(csc_scan_kernel, 1, 1024, 0, s, cols, w.total, w.colptr);
   launch_chained(csc_fill_kernel, K + (cols + 255) / 256, 256, 0, s, codes, K, D, sl.passes, cps, w.mask, w.off, w.total,
-                 w.colptr, w.ent);
+                 w.colptr, w.ent, refused);
   return cudaGetLastError() == cudaSuccess ? 4 : SFB_ERR_CUDA;
 }
 

@@ -1,0 +1,43 @@
+"""A buffer whose header does not match the descriptor: nothing behind the header is read, W and the context stay sound."""
+import pytest
+import torch
+
+from sfbgen import make_inputs, scaled
+from tests.test_gpu_parity import _workload
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("path", ["f32", "tf32", "tf32x3"])
+def test_codes_of_a_refused_buffer_are_not_read(path):
+    """Its codes hold atoms that do not exist (every read stays inside the buffer): reading them would set BAD_INDEX."""
+    from paper_1511_08486_b200 import binding as B
+    cfg = scaled("C3", J=36, D=100, P=3, B=7, density=0.2)
+    cfg["path"] = path
+    wl = _workload(cfg, make_inputs(cfg), path)
+    try:
+        wl.compute_factors(0)
+        wl.pack(0)
+        good = wl.sf_buf.clone()
+        off, stride = B.sfb_sf_buffer_layout(wl.desc)
+        pad = lambda n: (n + 127) // 128 * 128
+        idx = off + pad(cfg["B"] * wl.ldu * 4) + pad((cfg["B"] + 1) * 4)
+        cap = wl.desc.nnz_capacity // cfg["P"]
+        for p in range(cfg["P"]):
+            wl.sf_buf[idx + p * stride:idx + p * stride + cap * 4] = 0xFF
+        wl.sf_buf[20] ^= 64                                  # J field of the header
+        wl.apply(0.5)
+        assert wl.ctx.status() == B.SFB_DEV_BAD_HEADER
+        assert torch.equal(wl.W, wl.W0)
+        # a right buffer afterwards is applied as if nothing had happened
+        wl.sf_buf.copy_(good)
+        wl.apply(1e-2)
+        assert wl.ctx.status() == 0
+        applied = wl.W.clone()
+        wl.reset()
+        wl.compute_factors(0)
+        wl.pack(0)
+        wl.apply(1e-2)
+        assert torch.equal(applied, wl.W) and not torch.equal(applied, wl.W0)
+    finally:
+        wl.close()
