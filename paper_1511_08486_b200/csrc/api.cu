@@ -578,6 +578,10 @@ int sfb_pack(sfb_ctx* c, const void* U, const void* V, const sfb_aux* aux, void*
 static int apply_from(sfb_ctx* c, void* W, const void* sf_buf, float eta, int K, bool check, bool csc_built = false,
                       bool active_rows = false, const RowMap* v_rows = nullptr) {
   const sfb_desc& d = c->d;
+  // The epilogue of an update that runs rewrites the shadow from the new W, and one that does not run (a refused buffer, a
+  // compacted one without a single pair) leaves W and shadow as they were, which only the device knows: a shadow that
+  // mirrored this W still does, any other is not to be trusted.
+  const bool mirrored = has_shadow(c) && c->shadow_of == W;
   HeaderCheck hc;
   if (check) hc = make_check(sf_buf, d, c->l, c->dev_status);
   // (the compensated path has a kernel in front of its GEMM that can do the check)
@@ -599,7 +603,7 @@ static int apply_from(sfb_ctx* c, void* W, const void* sf_buf, float eta, int K,
                                d.path == SFB_PATH_TF32, c->dev_status));
     ACC(umma_apply(c->umma, c->stream, W, has_shadow(c) ? c->w_shadow : nullptr, stream_u(c, sf_buf), dense_codes(c), eta,
                    K, c->dev_status));
-    if (has_shadow(c)) c->shadow_of = W;   // the apply epilogue rewrote the shadow from the new W
+    if (!mirrored) c->shadow_of = nullptr;
   } else if (d.path == SFB_PATH_F32) {
     const int* idx = nullptr;
     const int* n_idx = nullptr;
@@ -618,10 +622,7 @@ static int apply_from(sfb_ctx* c, void* W, const void* sf_buf, float eta, int K,
     ACC(umma_apply(c->umma, c->stream, W, c->w_shadow, stream_u(c, sf_buf),
                    v_rows != nullptr ? *v_rows : stream_v(c, sf_buf), eta, K, c->dev_status,
                    d.compact ? reinterpret_cast<const char*>(sf_buf) + 128 : nullptr, with_split ? &hc : nullptr));
-    // The apply epilogue rewrote the shadow from the new W.  (A compacted buffer without a single pair launches no
-    // tile: W and a shadow that mirrored it stay as they were; a stale shadow stays stale.)
-    if (has_shadow(c) && (!d.compact || c->shadow_of == W)) c->shadow_of = W;
-    else c->shadow_of = nullptr;
+    if (!mirrored) c->shadow_of = nullptr;
   }
   return SFB_OK;
 }
@@ -668,7 +669,6 @@ int sfb_apply(sfb_ctx* c, void* W, const void* sf_buf, float eta, int32_t K) {
   if (c == nullptr || W == nullptr || sf_buf == nullptr) return SFB_ERR_ARG;
   if (!aligned(W, 16) || !aligned(sf_buf, 128)) return SFB_ERR_ARG;
   if (K <= 0 || K > c->K || (K % c->d.B) != 0) return SFB_ERR_ARG;
-  if (has_shadow(c) && c->shadow_of != W) c->shadow_of = nullptr;
   if (c->umma != nullptr) umma_drop_corr(c->umma);   // the buffer is the caller's: nothing prepared for it counts
   return apply_from(c, W, sf_buf, eta, K, true);
 }

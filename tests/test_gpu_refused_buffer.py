@@ -41,3 +41,37 @@ def test_codes_of_a_refused_buffer_are_not_read(path):
         assert torch.equal(applied, wl.W) and not torch.equal(applied, wl.W0)
     finally:
         wl.close()
+
+
+@pytest.mark.parametrize("path,name,over", [
+    ("bf16", "C4", dict(J=130, D=264, P=2, B=40, pool=1, labels="uniform")), ("tf32x3", "C1", dict(J=130, D=260, P=2, B=40)),
+    ("tf32x3", "C2", dict(J=70, D=132, P=2, B=40)), ("tf32x3", "C3", dict(J=70, D=132, P=2, B=40, density=0.2))])
+def test_a_refused_update_leaves_no_stale_copy_of_w(path, name, over):
+    """The context has not seen W yet, or W has changed since: after a refused update its copy is rebuilt, not trusted."""
+    from paper_1511_08486_b200 import binding as B
+    cfg = scaled(name, **over)
+    cfg["path"] = path
+    inputs = make_inputs(cfg)
+    a, b = _workload(cfg, inputs, path), _workload(cfg, inputs, path)
+    try:
+        for wl in (a, b):                       # b never sees the bad buffer
+            wl.W.mul_(0.5)
+        a.apply(0.5)                            # header of zeros
+        assert a.ctx.status() == B.SFB_DEV_BAD_HEADER and torch.equal(a.W, b.W)
+        for _ in range(2):
+            a.step(0, eta=1e-3)
+            b.step(0, eta=1e-3)
+            assert a.ctx.status() == 0 and torch.equal(a.W, b.W) and torch.equal(a.sf_buf, b.sf_buf)
+            a.sf_buf[20] ^= 64
+            a.apply(0.5)
+            assert a.ctx.status() == B.SFB_DEV_BAD_HEADER
+            a.sf_buf[20] ^= 64
+            for wl in (a, b):
+                wl.W.mul_(0.9)
+                wl.ctx.invalidate()
+            a.sf_buf[20] ^= 64
+            a.apply(0.5)
+            assert a.ctx.status() == B.SFB_DEV_BAD_HEADER
+    finally:
+        a.close()
+        b.close()
