@@ -74,9 +74,10 @@ __global__ void __launch_bounds__(256, 2) forward_f32_kernel(const float* W, con
   __shared__ __align__(16) float As[BK][BM + 4];
   __shared__ __align__(16) float Bs[BK][BN + 4];
   const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15;
-  const int i0 = blockIdx.y * BM, j0 = blockIdx.x * BN;
+  const int jt = (J + BN - 1) / BN;              // tiles one after the other in grid.x: K has no limit of grid.y
+  const int i0 = (int)(blockIdx.x / jt) * BM, j0 = (int)(blockIdx.x % jt) * BN;
   const bool vec_ok = (D & 3) == 0;
-  const bool write_v = (v.base != nullptr) && (blockIdx.x == 0);
+  const bool write_v = (v.base != nullptr) && (j0 == 0);
   const int lr = tid >> 2, lc = (tid & 3) * 4;   // loader: row within 64, first of 4 reduction columns
 
   float2 acc[4 * MI][2 * NI];
@@ -307,7 +308,8 @@ __global__ void __launch_bounds__(256, 4) sgemm_small_kernel(const __grid_consta
   __shared__ long long c_off[OUT == 1 ? BT : 1];   // ... and of their copies
   if (OUT == 0 && p.dev_status != nullptr && (*p.dev_status & SFB_DEV_BAD_HEADER)) return;
   const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15, lane = tid & 31, warp = tid >> 5;
-  const int m0 = blockIdx.y * BT, n0 = blockIdx.x * BT;
+  const int nt = (p.N + BT - 1) / BT;            // tiles one after the other in grid.x: M has no limit of grid.y
+  const int n_tile = (int)(blockIdx.x % nt), m0 = (int)(blockIdx.x / nt) * BT, n0 = n_tile * BT;
   const int k_lo = (OUT == 1) ? blockIdx.z * p.k_per_range : 0;
   const int k_hi = (OUT == 1) ? min(p.K, k_lo + p.k_per_range) : (p.n_rows != nullptr ? min(p.K, *p.n_rows) : p.K);
   if (OUT == 1) {
@@ -358,9 +360,9 @@ __global__ void __launch_bounds__(256, 4) sgemm_small_kernel(const __grid_consta
     if (nxt < nk) issue(nxt % PIPE, k_lo + nxt * BK);
     cp_async_commit();
     const float* As = ring + (kt % PIPE) * SMALL_STAGE_FLOATS;
-    if (OUT == 1 && p.copy.base != nullptr) {   // four steps of a row per thread; rows blockIdx.x, + gridDim.x, ...
+    if (OUT == 1 && p.copy.base != nullptr) {   // four steps of a row per thread; rows n_tile, + nt, ...
       const int k = (tid & 3) * 4, kk = k_lo + kt * BK + k;
-      for (int r = blockIdx.x + gridDim.x * (tid >> 2); r < BT; r += gridDim.x * 64)
+      for (int r = n_tile + nt * (tid >> 2); r < BT; r += nt * 64)
         if (c_off[r] >= 0 && kk < p.copy.ld)
           *reinterpret_cast<float4*>(p.copy.base + c_off[r] + (size_t)kk * 4) =
               make_float4(As[k * (BT + 4) + r], As[(k + 1) * (BT + 4) + r], As[(k + 2) * (BT + 4) + r],
@@ -496,9 +498,9 @@ bool forward_f32_fused(int K, int J, int D) { return plan_forward(K, J, D, 1).ti
 int launch_forward_f32(cudaStream_t s, const float* W, const float* X, const float* Xb, int K, int J, int D, RowMap z,
                        RowMap v) {
   if ((long long)((K + 127) / 128) * ((J + 127) / 128) >= 148)
-    launch_chained(forward_f32_kernel<2, 2>, dim3((J + 127) / 128, (K + 127) / 128), 256, 0, s, W, X, Xb, K, J, D, z, v);
+    launch_chained(forward_f32_kernel<2, 2>, ((J + 127) / 128) * ((K + 127) / 128), 256, 0, s, W, X, Xb, K, J, D, z, v);
   else
-    launch_chained(forward_f32_kernel<1, 1>, dim3((J + 63) / 64, (K + 63) / 64), 256, 0, s, W, X, Xb, K, J, D, z, v);
+    launch_chained(forward_f32_kernel<1, 1>, ((J + 63) / 64) * ((K + 63) / 64), 256, 0, s, W, X, Xb, K, J, D, z, v);
   return cudaGetLastError() == cudaSuccess ? 1 : SFB_ERR_CUDA;
 }
 
@@ -519,7 +521,7 @@ int launch_forward_f32_small(cudaStream_t s, const float* W, RowMap src, RowMap 
   p.z = ks > 1 ? part : z;
   p.range_stride = split_stride;
   *nsplit_out = ks;
-  launch_chained(sgemm_small_kernel<1>, dim3((J + 63) / 64, (K + 63) / 64, ks), 256, 0, s, p);
+  launch_chained(sgemm_small_kernel<1>, dim3(((J + 63) / 64) * ((K + 63) / 64), 1, ks), 256, 0, s, p);
   return cudaGetLastError() == cudaSuccess ? 1 : SFB_ERR_CUDA;
 }
 
@@ -541,7 +543,7 @@ int launch_apply_f32(cudaStream_t s, float* W, RowMap u, RowMap v, int K, int J,
     p.eta = eta;
     p.dev_status = dev_status;
     p.row_idx = row_idx; p.n_rows = n_rows;
-    launch_chained(sgemm_small_kernel<0>, dim3((D + 63) / 64, (J + 63) / 64), 256, 0, s, p);
+    launch_chained(sgemm_small_kernel<0>, ((D + 63) / 64) * ((J + 63) / 64), 256, 0, s, p);
   }
   return cudaGetLastError() == cudaSuccess ? 1 : SFB_ERR_CUDA;
 }
