@@ -202,8 +202,11 @@ int factors_into(sfb_ctx* c, const void* W, const void* X, const sfb_aux* aux, R
     const RowMap part = caller_rows(c->f32_part, c->ldp, d.B, 4);
     const long long sstride = (long long)c->K * c->ldp * 4;
     int ks = 1;
+    // a shard of the workers stays within the partial buffers and transposed copies of the whole
+    int want = forward_f32_splits(K, d.J, d.D);
+    if (want > c->f32_splits) want = c->f32_splits;
     if (forward_f32_fused(K, d.J, d.D) || (Xb != nullptr && v.base == nullptr)) {
-      ACC(launch_forward_f32(c->stream, Wf, reinterpret_cast<const float*>(X), Xb, K, d.J, d.D, u, v));
+      ACC(launch_forward_f32(c->stream, Wf, reinterpret_cast<const float*>(X), Xb, K, d.J, d.D, u, v, part, sstride, want, &ks));
     } else {
       RowMap src = caller_rows(X, d.D, d.B, 4), copy = v;
       if (Xb != nullptr) {   // pair differences first (they are the factor v), then contracted from there
@@ -211,9 +214,6 @@ int factors_into(sfb_ctx* c, const void* W, const void* X, const sfb_aux* aux, R
         src = v;
         copy = RowMap();
       }
-      // a shard of the workers stays within the partial buffers and transposed copies of the whole
-      int want = forward_f32_splits(K, d.J, d.D);
-      if (want > c->f32_splits) want = c->f32_splits;
       if (forward_f32_transposed(K, d.J, d.D) && c->f32_nn_ws != nullptr)
         ACC(launch_forward_f32_nn(c->stream, Wf, src, copy, K, d.J, d.D, c->f32_nn_ws, u, part, sstride, want, &ks));
       else

@@ -261,16 +261,18 @@ bool allow_smem(K* kernel, size_t bytes) {
 // v rows = Xa rows - Xb rows, one fp32 subtraction per element, pad columns zero (the DML factor v).
 int launch_diff_rows(cudaStream_t s, const float* Xa, const float* Xb, RowMap v, int K, int D, CorrOut corr = CorrOut());
 // Z[i][j] = sum_d A[i][d] * W[j][d] on fp32 CUDA cores, written as fp32 rows through `z`.
-// A = X, or X - Xb (element-wise fp32 subtraction) when Xb != nullptr.  When `v` has a base, the
-// operand rows (X, or the difference) are also written there (the factor v), pad columns zero.  One launch: for problems
-// that forward_f32_fused tells are small, and where the difference is not kept.
+// The reduction is cut into ks ranges (*nsplit_out of them exist) whose partial products go to `part` (fp32 rows,
+// split_stride bytes between partial buffers) instead of `z` if there is more than one; the finishing pass sums them in
+// range order.  The sums do not depend on which of the three kernels forms them.
+//   launch_forward_f32: A = X, or X - Xb (element-wise fp32 subtraction) when Xb != nullptr.  When `v` has a base, the
+//   operand rows (X, or the difference) are also written there (the factor v), pad columns zero.  For problems that
+//   forward_f32_fused tells are small, and where the difference is not kept.
 bool forward_f32_fused(int K, int J, int D);
 int launch_forward_f32(cudaStream_t s, const float* W, const float* X, const float* Xb, int K, int J, int D,
-                       RowMap z, RowMap v);
-// The same for operand rows a_i behind a row map; copy (optional): those rows also written there.  The reduction is cut
-// into ks ranges (*nsplit_out of them exist) whose partial products go to `part` (fp32 rows, split_stride bytes between
-// partial buffers) instead of `z` if there is more than one; the finishing pass sums them in range order.
-// forward_f32_splits: how many to ask for, at most FORWARD_F32_MAX_SPLITS; forward_f32_transposed: by which of the two.
+                       RowMap z, RowMap v, RowMap part = RowMap(), long long split_stride = 0, int ks = 1,
+                       int* nsplit_out = nullptr);
+//   The others take operand rows a_i behind a row map; copy (optional): those rows also written there.
+//   forward_f32_splits: how many ranges to ask for, at most FORWARD_F32_MAX_SPLITS; forward_f32_transposed: which of the two.
 //   _small: 64 x 64 tiles, operands in place.  _nn: large tiles through transposed copies of both operands; ws:
 //   forward_f32_nn_workspace_floats(K, J, D) floats.
 constexpr int FORWARD_F32_MAX_SPLITS = 32;

@@ -62,13 +62,15 @@ __device__ __forceinline__ void mma_tile(const float (*As)[64 * MI + 4], const f
 }
 
 // ------------------------------------------------------------------------------------------ forward, one launch
-// For the smallest problems, and where the pair difference is formed on the way (sfb_loss).
+// For the smallest problems, and where the pair difference is formed on the way and not kept (DML factors without v,
+// sfb_loss).  blockIdx.z takes the reduction range [z d_per_range, + d_per_range) and writes its partial products
+// range_stride bytes after the previous range's.
 // Tile rows = samples i (BM = 64*MI), tile columns = classes j (BN = 64*NI), reduction over d.
 // Both operands are contiguous along d, so tiles are transposed while being stored to shared memory.
 template <int MI, int NI>
 __global__ void __launch_bounds__(256, 2) forward_f32_kernel(const float* W, const float* X,
                                                           const float* Xb, int K, int J, int D,
-                                                          RowMap z, RowMap v) {
+                                                          RowMap z, RowMap v, int d_per_range, long long range_stride) {
   chain_wait();
   constexpr int BM = 64 * MI, BN = 64 * NI;
   __shared__ __align__(16) float As[BK][BM + 4];
@@ -121,11 +123,12 @@ __global__ void __launch_bounds__(256, 2) forward_f32_kernel(const float* W, con
     }
   };
 
-  fetch(0);
-  for (int d0 = 0; d0 < D; d0 += BK) {
+  const int d_lo = blockIdx.z * d_per_range, d_hi = min(D, d_lo + d_per_range);
+  fetch(d_lo);
+  for (int d0 = d_lo; d0 < d_hi; d0 += BK) {
     stash();
     __syncthreads();
-    if (d0 + BK < D) fetch(d0 + BK);
+    if (d0 + BK < d_hi) fetch(d0 + BK);
     mma_tile<MI, NI, false>(As, Bs, ty, tx, acc);
     __syncthreads();
   }
@@ -138,7 +141,7 @@ __global__ void __launch_bounds__(256, 2) forward_f32_kernel(const float* W, con
     for (int a = 0; a < 4; ++a) {
       const int i = i0 + mi * 64 + ty * 4 + a;
       if (i >= K) continue;
-      float* zr = reinterpret_cast<float*>(z.row(i));
+      float* zr = reinterpret_cast<float*>(z.row(i) + blockIdx.z * range_stride);
 #pragma unroll
       for (int ni = 0; ni < NI; ++ni) {
         const int j = j0 + ni * 64 + tx * 4;
@@ -495,20 +498,25 @@ int forward_f32_splits(int K, int J, int D) { return plan_forward(K, J, D, FORWA
 bool forward_f32_transposed(int K, int J, int D) { return plan_forward(K, J, D, FORWARD_F32_MAX_SPLITS).tile == 128; }
 bool forward_f32_fused(int K, int J, int D) { return plan_forward(K, J, D, 1).tile == 0; }
 
-int launch_forward_f32(cudaStream_t s, const float* W, const float* X, const float* Xb, int K, int J, int D, RowMap z,
-                       RowMap v) {
-  if ((long long)((K + 127) / 128) * ((J + 127) / 128) >= 148)
-    launch_chained(forward_f32_kernel<2, 2>, ((J + 127) / 128) * ((K + 127) / 128), 256, 0, s, W, X, Xb, K, J, D, z, v);
-  else
-    launch_chained(forward_f32_kernel<1, 1>, ((J + 63) / 64) * ((K + 63) / 64), 256, 0, s, W, X, Xb, K, J, D, z, v);
-  return cudaGetLastError() == cudaSuccess ? 1 : SFB_ERR_CUDA;
-}
-
 // No empty range: the finishing pass would add a partial buffer nobody wrote.
 static int range_length(int D, int* ks) {
   const int per = ((D + *ks - 1) / *ks + BK - 1) / BK * BK;
   *ks = (D + per - 1) / per;
   return per;
+}
+
+int launch_forward_f32(cudaStream_t s, const float* W, const float* X, const float* Xb, int K, int J, int D, RowMap z,
+                       RowMap v, RowMap part, long long split_stride, int ks, int* nsplit_out) {
+  const int per = range_length(D, &ks);
+  if (ks > 1) z = part;
+  if (nsplit_out != nullptr) *nsplit_out = ks;
+  const int big = ((J + 127) / 128) * ((K + 127) / 128);
+  if ((long long)big * ks >= 148)
+    launch_chained(forward_f32_kernel<2, 2>, dim3(big, 1, ks), 256, 0, s, W, X, Xb, K, J, D, z, v, per, split_stride);
+  else
+    launch_chained(forward_f32_kernel<1, 1>, dim3(((J + 63) / 64) * ((K + 63) / 64), 1, ks), 256, 0, s, W, X, Xb, K, J, D, z, v,
+                   per, split_stride);
+  return cudaGetLastError() == cudaSuccess ? 1 : SFB_ERR_CUDA;
 }
 
 int launch_forward_f32_small(cudaStream_t s, const float* W, RowMap src, RowMap copy, int K, int J, int D, RowMap z,
