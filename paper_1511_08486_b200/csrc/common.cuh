@@ -146,7 +146,7 @@ struct Commit {
 };
 Commit make_commit(void* sf_buf, const sfb_desc& d, const Layout& l, uint32_t clock, const uint32_t* rowptr);
 #ifdef __CUDACC__
-// Called by the n threads of one block.
+// Called by n threads, of one block or of several.
 __device__ __forceinline__ void write_header(const Commit& c, int tid, int n) {
   uint32_t* w = reinterpret_cast<uint32_t*>(c.buf);
   const HeaderImage& h = c.h;
@@ -191,7 +191,8 @@ struct FinishExtra {
   int cols;
   CorrOut corr;
   bool next_early;   // see chain_next
-  FinishExtra() : nonzero(nullptr), src(), dst(), cols(0), next_early(false) {}
+  int header_blocks; // blocks in front of the rows' that write the header (set by the launcher)
+  FinishExtra() : nonzero(nullptr), src(), dst(), cols(0), next_early(false), header_blocks(0) {}
 };
 
 #ifdef __CUDACC__

@@ -8,6 +8,8 @@
 // sees one read and one write per value; reductions over the J entries use warp shuffles.
 #include <cooperative_groups.h>
 
+#include <type_traits>
+
 #include "common.cuh"
 
 namespace cg = cooperative_groups;
@@ -95,9 +97,20 @@ __device__ __forceinline__ void copy_unit(const RowMap& src, const RowMap& dst, 
                                                __uint_as_float(val.w)));
 }
 
-// Block i of a finishing pass: row i of the copy, and block 0 the header.
+// The first header_blocks blocks of a finishing pass write the header and the directory; the others take a row each, and
+// row i of the copy.  (In the block of a row they would be on the pass's critical path, and with many workers the longest
+// part of it: 4096 workers of one sample, 64 x 512 in tf32: 77.9 us a step, 53.2 with blocks of their own.)
+__device__ __forceinline__ bool header_block(const FinishExtra& x) {
+  if ((int)blockIdx.x >= x.header_blocks) return false;
+  write_header(x.commit, blockIdx.x * blockDim.x + threadIdx.x, x.header_blocks * blockDim.x);
+  return true;
+}
+int header_blocks(const FinishExtra& x) {
+  if (x.commit.buf == nullptr) return 0;
+  const long long words = (long long)(x.commit.h.streams_off / 4);
+  return (int)(words / 2048 < 1 ? 1 : (words / 2048 > 148 ? 148 : words / 2048));
+}
 __device__ __forceinline__ void finish_extra(const FinishExtra& x, int i) {
-  if (x.commit.buf != nullptr && i == 0) write_header(x.commit, threadIdx.x, blockDim.x);
   if (x.dst.base != nullptr)
     for (int q = threadIdx.x; q < x.dst.ld * x.dst.es / 16; q += blockDim.x) copy_unit(x.src, x.dst, i, q, x.cols, x.corr);
 }
@@ -115,14 +128,16 @@ __device__ __forceinline__ bool wire_nonzero4(const float4& t, int es) {
 }
 
 // z rows are fp32 with ld a multiple of 4; values beyond J inside the last float4 are ignored.
-__global__ void __launch_bounds__(1024) finish_mlr_kernel(RowMap z, RowMap u, const int32_t* labels,
+template <int T, int BLOCKS>
+__global__ void __launch_bounds__(T, BLOCKS) finish_mlr_kernel(RowMap z, RowMap u, const int32_t* labels,
                                                                  int K, int J, int cache_floats, int* dev_status, int nsplit, long long zstride,
                                                                  float* dual, float sdca_step, CorrOut corr, const __grid_constant__ FinishExtra extra) {
   if (extra.next_early) chain_next();
   chain_wait();
   extern __shared__ __align__(16) float cache[];
   __shared__ float red[32];
-  const int i = blockIdx.x;
+  if (header_block(extra)) return;
+  const int i = blockIdx.x - extra.header_blocks;
   if (i >= K) return;
   const int y = labels[i];   // (early: its latency passes beside the row's)
   finish_extra(extra, i);
@@ -133,7 +148,7 @@ __global__ void __launch_bounds__(1024) finish_mlr_kernel(RowMap z, RowMap u, co
   const float kLog2e = 1.4426950408889634f;
 
   float m = -INFINITY;
-  for (int q = threadIdx.x; q < J4; q += blockDim.x) {
+  for (int q = threadIdx.x; q < J4; q += T) {
     float4 t = ldz4(zr, q * 4, nsplit, zstride);
     const int j = q * 4;
     if (j + 1 >= J) t.y = -INFINITY;
@@ -146,7 +161,7 @@ __global__ void __launch_bounds__(1024) finish_mlr_kernel(RowMap z, RowMap u, co
 
   float s = 0.f;
   const float mb = m * kLog2e;
-  for (int q = threadIdx.x; q < J4; q += blockDim.x) {
+  for (int q = threadIdx.x; q < J4; q += T) {
     const int j = q * 4;
     float4 t;
     if (cached) {
@@ -169,7 +184,7 @@ __global__ void __launch_bounds__(1024) finish_mlr_kernel(RowMap z, RowMap u, co
   if (bad && threadIdx.x == 0) atomicOr(dev_status, SFB_DEV_BAD_LABEL);
   const int ld4 = u.ld >> 2;   // u.ld is a multiple of 4 (fp32) or 8 (bf16)
   bool any = false;
-  for (int q = threadIdx.x; q < ld4; q += blockDim.x) {
+  for (int q = threadIdx.x; q < ld4; q += T) {
     const int j = q * 4;
     float4 t = make_float4(0.f, 0.f, 0.f, 0.f);
     if (q < J4 && !bad) {
@@ -197,14 +212,16 @@ __global__ void __launch_bounds__(1024) finish_mlr_kernel(RowMap z, RowMap u, co
   flag_row(extra, i, any);
 }
 
-__global__ void __launch_bounds__(1024) finish_dml_kernel(RowMap z, RowMap u, const uint8_t* similar,
+template <int T, int BLOCKS>
+__global__ void __launch_bounds__(T, BLOCKS) finish_dml_kernel(RowMap z, RowMap u, const uint8_t* similar,
                                                                  float margin, int K, int J, int cache_floats, int nsplit, long long zstride,
                                                                  uint8_t* active, CorrOut corr, const __grid_constant__ FinishExtra extra) {
   if (extra.next_early) chain_next();
   chain_wait();
   extern __shared__ __align__(16) float cache[];
   __shared__ float red[32];
-  const int i = blockIdx.x;
+  if (header_block(extra)) return;
+  const int i = blockIdx.x - extra.header_blocks;
   if (i >= K) return;
   const bool sim = similar[i] != 0;   // (early: its latency passes beside the row's)
   finish_extra(extra, i);
@@ -214,7 +231,7 @@ __global__ void __launch_bounds__(1024) finish_dml_kernel(RowMap z, RowMap u, co
   const bool cached = (J4 * 4) <= cache_floats;
 
   float n = 0.f;
-  for (int q = threadIdx.x; q < J4; q += blockDim.x) {
+  for (int q = threadIdx.x; q < J4; q += T) {
     float4 t = ldz4(zr, q * 4, nsplit, zstride);
     const int j = q * 4;
     if (j + 1 >= J) t.y = 0.f;
@@ -229,7 +246,7 @@ __global__ void __launch_bounds__(1024) finish_dml_kernel(RowMap z, RowMap u, co
 
   const int ld4 = u.ld >> 2;
   bool any = false;
-  for (int q = threadIdx.x; q < ld4; q += blockDim.x) {
+  for (int q = threadIdx.x; q < ld4; q += T) {
     const int j = q * 4;
     float4 t = make_float4(0.f, 0.f, 0.f, 0.f);
     if (q < J4 && g != 0.f) {
@@ -258,7 +275,8 @@ __global__ void __launch_bounds__(256) finish_mlr_fused_kernel(RowMap u, const f
   chain_wait();
   extern __shared__ float scale[];   // [n_parts]
   __shared__ float red[32];
-  const int i = blockIdx.x;
+  if (header_block(extra)) return;
+  const int i = blockIdx.x - extra.header_blocks;
   if (i >= K) return;
   const int y = labels[i];   // (early: its latency passes beside the row's)
   finish_extra(extra, i);
@@ -486,8 +504,20 @@ __global__ void __launch_bounds__(256) cast_bf16_kernel(const float* W, __nv_bfl
   }
 }
 
-// Long rows take a whole SM's worth of shared memory, so one block must supply all the memory parallelism.
-int fin_threads(int J) { return J >= 8192 ? 1024 : 256; }
+// Threads and blocks per SM of a finishing pass.  Long rows take a whole SM's worth of shared memory, so one block must
+// supply all the memory parallelism.  Other rows take 256 threads and the registers that keep a thread's loads of a row, or
+// of its partial products, in flight together, unless there is nothing of the kind (up to 1024 values, one range) and more
+// rows than two waves of such blocks: then the number of rows at work counts, and the registers are held down for it, in
+// half-size blocks where 512 values suffice (same order of the sums: the other warps would add zeros).
+// 10 x 64, K = 65536: 248 us for the factors with 63 registers a thread and 256 threads, 100 with 40 and 128; but 200 x 8000,
+// one sample in 16 ranges: 13.9 us with 63, 17.3 with 40.
+template <typename F>
+int by_rows(int K, int J, int nsplit, F&& go) {
+  if (J >= 8192) return go(std::integral_constant<int, 1024>(), std::integral_constant<int, 1>());
+  if (J > 1024 || nsplit > 1 || K <= 8 * 148) return go(std::integral_constant<int, 256>(), std::integral_constant<int, 4>());
+  if (J > 512) return go(std::integral_constant<int, 256>(), std::integral_constant<int, 6>());
+  return go(std::integral_constant<int, 128>(), std::integral_constant<int, 12>());
+}
 
 int fin_cache_floats(int J) {
   const int need = ((J + 3) / 4) * 4;
@@ -498,13 +528,19 @@ int fin_cache_floats(int J) {
 
 int launch_finish_mlr(cudaStream_t s, RowMap z, RowMap u, const int32_t* labels, int K, int J, int* dev_status,
                       int nsplit, long long split_stride_bytes, float* dual, float sdca_step, CorrOut corr,
-                      const FinishExtra& extra) {
+                      const FinishExtra& extra_in) {
+  FinishExtra extra = extra_in;
+  extra.header_blocks = header_blocks(extra);
   const int cf = fin_cache_floats(J);
-  static PerDeviceOnce attr_once;
-  if (!set_up_device(attr_once, [] { return allow_smem(finish_mlr_kernel, ROW_CACHE_FLOATS * 4); })) return SFB_ERR_CUDA;
-  launch_chained(finish_mlr_kernel, K, fin_threads(J), (size_t)cf * 4, s, z, u, labels, K, J, cf, dev_status, nsplit, split_stride_bytes / 4,
-                                                              dual, sdca_step, corr, extra);
-  return cudaGetLastError() == cudaSuccess ? 1 : SFB_ERR_CUDA;
+  return by_rows(K, J, nsplit, [&](auto threads, auto blocks) -> int {
+    auto kernel = finish_mlr_kernel<threads(), blocks()>;
+    static PerDeviceOnce attr_once;
+    if (threads() == 1024 && !set_up_device(attr_once, [&] { return allow_smem(kernel, ROW_CACHE_FLOATS * 4); }))
+      return SFB_ERR_CUDA;
+    launch_chained(kernel, K + extra.header_blocks, threads(), (size_t)cf * 4, s, z, u, labels, K, J, cf, dev_status, nsplit, split_stride_bytes / 4,
+                   dual, sdca_step, corr, extra);
+    return cudaGetLastError() == cudaSuccess ? 1 : SFB_ERR_CUDA;
+  });
 }
 
 // idx[0 .. n) = the samples i < K with active[i] != 0, in ascending order; *n_out = n.  One block, ordered.
@@ -543,24 +579,32 @@ int launch_compact_active(cudaStream_t s, const uint8_t* active, int K, int* idx
 }
 
 int launch_finish_dml(cudaStream_t s, RowMap z, RowMap u, const uint8_t* similar, float margin, int K, int J,
-                      int nsplit, long long split_stride_bytes, uint8_t* active, CorrOut corr, const FinishExtra& extra) {
+                      int nsplit, long long split_stride_bytes, uint8_t* active, CorrOut corr, const FinishExtra& extra_in) {
+  FinishExtra extra = extra_in;
+  extra.header_blocks = header_blocks(extra);
   const int cf = fin_cache_floats(J);
-  static PerDeviceOnce attr_once;
-  if (!set_up_device(attr_once, [] { return allow_smem(finish_dml_kernel, ROW_CACHE_FLOATS * 4); })) return SFB_ERR_CUDA;
-  launch_chained(finish_dml_kernel, K, fin_threads(J), (size_t)cf * 4, s, z, u, similar, margin, K, J, cf, nsplit, split_stride_bytes / 4,
-                                                              active, corr, extra);
-  return cudaGetLastError() == cudaSuccess ? 1 : SFB_ERR_CUDA;
+  return by_rows(K, J, nsplit, [&](auto threads, auto blocks) -> int {
+    auto kernel = finish_dml_kernel<threads(), blocks()>;
+    static PerDeviceOnce attr_once;
+    if (threads() == 1024 && !set_up_device(attr_once, [&] { return allow_smem(kernel, ROW_CACHE_FLOATS * 4); }))
+      return SFB_ERR_CUDA;
+    launch_chained(kernel, K + extra.header_blocks, threads(), (size_t)cf * 4, s, z, u, similar, margin, K, J, cf, nsplit, split_stride_bytes / 4,
+                   active, corr, extra);
+    return cudaGetLastError() == cudaSuccess ? 1 : SFB_ERR_CUDA;
+  });
 }
 
 int launch_finish_mlr_fused(cudaStream_t s, RowMap u, const float2* stats, int n_parts, int part_cols,
                             const int32_t* labels, int K, int J, int* dev_status, float* dual, float sdca_step,
-                            const FinishExtra& extra) {
+                            const FinishExtra& extra_in) {
+  FinishExtra extra = extra_in;
+  extra.header_blocks = header_blocks(extra);
   const size_t smem = (size_t)n_parts * sizeof(float);
   if (smem > 48 * 1024) return SFB_ERR_SHAPE;
   if (u.es == 4)
-    launch_chained(finish_mlr_fused_kernel<4>, K, 256, smem, s, u, stats, n_parts, part_cols, labels, K, J, dev_status, dual, sdca_step, extra);
+    launch_chained(finish_mlr_fused_kernel<4>, K + extra.header_blocks, 256, smem, s, u, stats, n_parts, part_cols, labels, K, J, dev_status, dual, sdca_step, extra);
   else
-    launch_chained(finish_mlr_fused_kernel<2>, K, 256, smem, s, u, stats, n_parts, part_cols, labels, K, J, dev_status, dual, sdca_step, extra);
+    launch_chained(finish_mlr_fused_kernel<2>, K + extra.header_blocks, 256, smem, s, u, stats, n_parts, part_cols, labels, K, J, dev_status, dual, sdca_step, extra);
   return cudaGetLastError() == cudaSuccess ? 1 : SFB_ERR_CUDA;
 }
 

@@ -44,11 +44,13 @@ def test_chained_kernels_read_through_ordinary_loads():
 
 
 def test_kernels_launched_with_the_overlap_wait():
-    waits, launched = set(), set()
+    waits, names, launched = set(), set(), set()
     for _, text in _sources():
-        waits |= {n for n, _, b in _kernels(text) if re.search(r"\bchain(_wait)?\(\)", b)}
-        launched |= set(re.findall(r"launch_chained\((\w+)", text)) - {"kernel"}
-        launched |= set(re.findall(r"cudaLaunchKernelEx\(&\w+, (\w+)", text)) - {"kernel"}
-        if "launch_chained(kernel" in text:
-            launched |= set(re.findall(r"auto kernel = (\w+)", text))
+        found = list(_kernels(text))
+        names |= {n for n, _, _ in found}
+        waits |= {n for n, _, b in found if re.search(r"\bchain(_wait)?\(\)", b)}
+        # named in the launch itself, or handed to it as `kernel`
+        launched |= set(re.findall(r"(?:launch_chained|\bgo)\((\w+)", text))
+        launched |= set(re.findall(r"cudaLaunchKernelEx\(&\w+, (\w+)", text)) | set(re.findall(r"auto kernel = (\w+)", text))
+    launched &= names
     assert len(launched) >= 20 and launched <= waits, launched - waits
