@@ -25,7 +25,8 @@ struct sfb_ctx {
   cudaEvent_t aux_fork, aux_join;
   bool aux_ok;
   float* f32_part;          // fp32 dense path: partial products [splits][K][ldp] of a split forward reduction
-  int ldp, f32_splits;
+  int ldp;
+  ForwardF32Plan f32_plan;  // fp32 dense path: how the forward of all K samples is done
   // DML, fp32 path: which pairs of the current step contribute (u_i != 0), their ordered list and its length;
   // the step's apply leaves the others out (bit-identical result, fewer multiply-adds)
   uint8_t* dml_active;
@@ -203,10 +204,10 @@ int factors_into(sfb_ctx* c, const void* W, const void* X, const sfb_aux* aux, R
     const long long sstride = (long long)c->K * c->ldp * 4;
     int ks = 1;
     // a shard of the workers stays within the partial buffers and transposed copies of the whole
-    int want = forward_f32_splits(K, d.J, d.D);
-    if (want > c->f32_splits) want = c->f32_splits;
-    if (forward_f32_fused(K, d.J, d.D) || (Xb != nullptr && v.base == nullptr)) {
-      ACC(launch_forward_f32(c->stream, Wf, reinterpret_cast<const float*>(X), Xb, K, d.J, d.D, u, v, part, sstride, want, &ks));
+    const ForwardF32Plan plan = K == c->K ? c->f32_plan : forward_f32_plan(K, d.J, d.D, Xb != nullptr, c->f32_plan.ks,
+                                                                           c->f32_nn_ws != nullptr);
+    if (plan.route == F32_IN_PLACE || (Xb != nullptr && v.base == nullptr)) {
+      ACC(launch_forward_f32(c->stream, Wf, reinterpret_cast<const float*>(X), Xb, K, d.J, d.D, u, v, part, sstride, plan.ks, &ks));
     } else {
       RowMap src = caller_rows(X, d.D, d.B, 4), copy = v;
       if (Xb != nullptr) {   // pair differences first (they are the factor v), then contracted from there
@@ -214,10 +215,10 @@ int factors_into(sfb_ctx* c, const void* W, const void* X, const sfb_aux* aux, R
         src = v;
         copy = RowMap();
       }
-      if (forward_f32_transposed(K, d.J, d.D) && c->f32_nn_ws != nullptr)
-        ACC(launch_forward_f32_nn(c->stream, Wf, src, copy, K, d.J, d.D, c->f32_nn_ws, u, part, sstride, want, &ks));
+      if (plan.route == F32_TRANSPOSED)
+        ACC(launch_forward_f32_nn(c->stream, Wf, src, copy, K, d.J, d.D, c->f32_nn_ws, u, part, sstride, plan.ks, &ks));
       else
-        ACC(launch_forward_f32_small(c->stream, Wf, src, copy, K, d.J, d.D, u, part, sstride, want, &ks));
+        ACC(launch_forward_f32_small(c->stream, Wf, src, copy, K, d.J, d.D, u, part, sstride, plan.ks, &ks));
     }
     const RowMap zsrc = ks > 1 ? part : u;
     if (d.model == SFB_MLR)
@@ -302,18 +303,17 @@ int sfb_create(const sfb_desc* desc, void* cuda_stream, sfb_ctx** out) {
   if (ok && desc->model == SFB_SC && (desc->path == SFB_PATH_TF32 || desc->path == SFB_PATH_TF32X3))
     ok = cudaMalloc(&c->a_dense, (size_t)c->K * c->l.ldv * 4) == cudaSuccess;
   if (ok && desc->model != SFB_SC && desc->path == SFB_PATH_F32) {
-    const int ks = forward_f32_splits(c->K, desc->J, desc->D);
+    // large shapes take the forward through transposed operand copies
+    const long long nn_bytes = forward_f32_nn_workspace_floats(c->K, desc->J, desc->D) * 4;
+    c->f32_plan = forward_f32_plan(c->K, desc->J, desc->D, desc->model == SFB_DML, FORWARD_F32_MAX_SPLITS, nn_bytes <= (2LL << 30));
+    const int ks = c->f32_plan.ks;
     c->ldp = (desc->J + 3) & ~3;
-    c->f32_splits = ks;
     if (ks > 1) ok = cudaMalloc(&c->f32_part, (size_t)ks * c->K * c->ldp * 4) == cudaSuccess;
     if (ok && desc->model == SFB_DML) {
       ok = cudaMalloc(&c->dml_active, (size_t)c->K) == cudaSuccess;
       if (ok) ok = cudaMalloc(&c->dml_idx, ((size_t)c->K + 1) * 4) == cudaSuccess;
     }
-    // large shapes take the forward through transposed operand copies
-    const long long nn_floats = forward_f32_nn_workspace_floats(c->K, desc->J, desc->D);
-    if (ok && forward_f32_transposed(c->K, desc->J, desc->D) && nn_floats * 4 <= (2LL << 30))
-      ok = cudaMalloc(&c->f32_nn_ws, (size_t)nn_floats * 4) == cudaSuccess;
+    if (ok && c->f32_plan.route == F32_TRANSPOSED) ok = cudaMalloc(&c->f32_nn_ws, (size_t)nn_bytes) == cudaSuccess;
   }
   if (ok) {
     if (cudaStreamCreateWithFlags(&c->aux, cudaStreamNonBlocking) == cudaSuccess) {

@@ -265,20 +265,22 @@ int launch_diff_rows(cudaStream_t s, const float* Xa, const float* Xb, RowMap v,
 // The reduction is cut into ks ranges (*nsplit_out of them exist) whose partial products go to `part` (fp32 rows,
 // split_stride bytes between partial buffers) instead of `z` if there is more than one; the finishing pass sums them in
 // range order.  The sums do not depend on which of the three kernels forms them.
-//   launch_forward_f32: A = X, or X - Xb (element-wise fp32 subtraction) when Xb != nullptr.  When `v` has a base, the
-//   operand rows (X, or the difference) are also written there (the factor v), pad columns zero.  For problems that
-//   forward_f32_fused tells are small, and where the difference is not kept.
-bool forward_f32_fused(int K, int J, int D);
+//   launch_forward_f32, one launch: A = X, or X - Xb (element-wise fp32 subtraction) when Xb != nullptr.  When `v` has a
+//   base, the operand rows (X, or the difference) are also written there (the factor v), pad columns zero.
 int launch_forward_f32(cudaStream_t s, const float* W, const float* X, const float* Xb, int K, int J, int D,
                        RowMap z, RowMap v, RowMap part = RowMap(), long long split_stride = 0, int ks = 1,
                        int* nsplit_out = nullptr);
 //   The others take operand rows a_i behind a row map; copy (optional): those rows also written there.
-//   forward_f32_splits: how many ranges to ask for, at most FORWARD_F32_MAX_SPLITS; forward_f32_transposed: which of the two.
 //   _small: 64 x 64 tiles, operands in place.  _nn: large tiles through transposed copies of both operands; ws:
 //   forward_f32_nn_workspace_floats(K, J, D) floats.
+// forward_f32_plan: which of the three, and how many ranges to ask for, at most max_ks.  pair: A = X - Xb.
+enum F32Route { F32_IN_PLACE, F32_SMALL, F32_TRANSPOSED };
+struct ForwardF32Plan {
+  F32Route route;
+  int ks;
+};
 constexpr int FORWARD_F32_MAX_SPLITS = 32;
-int forward_f32_splits(int K, int J, int D);
-bool forward_f32_transposed(int K, int J, int D);
+ForwardF32Plan forward_f32_plan(int K, int J, int D, bool pair, int max_ks, bool transposed_ok);
 int launch_forward_f32_small(cudaStream_t s, const float* W, RowMap src, RowMap copy, int K, int J, int D, RowMap z,
                              RowMap part, long long split_stride, int ks, int* nsplit_out);
 long long forward_f32_nn_workspace_floats(int K, int J, int D);

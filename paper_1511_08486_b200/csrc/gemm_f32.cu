@@ -14,15 +14,15 @@ namespace sfb {
 namespace {
 
 constexpr int BK = 16;
+constexpr int F32_MIN_LARGE_TILES = 100;   // fewer tiles of 128 x 128, and the one-launch forward takes 64 x 64
 
-__device__ __forceinline__ float4 ld4_guard(const float* row, int c, int cols, bool vec_ok) {
-  // row: start of a row; c: first column (multiple of 4); cols: valid columns
-  if (vec_ok && c + 3 < cols) return *reinterpret_cast<const float4*>(row + c);
+__device__ __forceinline__ float4 ld4_left(const float* p, int left, bool vec_ok) {
+  if (vec_ok && left > 3) return *reinterpret_cast<const float4*>(p);
   float4 r = make_float4(0.f, 0.f, 0.f, 0.f);
-  if (c < cols) r.x = row[c];
-  if (c + 1 < cols) r.y = row[c + 1];
-  if (c + 2 < cols) r.z = row[c + 2];
-  if (c + 3 < cols) r.w = row[c + 3];
+  if (left > 0) r.x = p[0];
+  if (left > 1) r.y = p[1];
+  if (left > 2) r.z = p[2];
+  if (left > 3) r.w = p[3];
   return r;
 }
 
@@ -67,8 +67,9 @@ __device__ __forceinline__ void mma_tile(const float (*As)[64 * MI + 4], const f
 // range_stride bytes after the previous range's.
 // Tile rows = samples i (BM = 64*MI), tile columns = classes j (BN = 64*NI), reduction over d.
 // Both operands are contiguous along d, so tiles are transposed while being stored to shared memory.
-template <int MI, int NI>
-__global__ void __launch_bounds__(256, 2) forward_f32_kernel(const float* W, const float* X,
+// PAIR: A = X - Xb.
+template <int MI, int NI, bool PAIR>
+__global__ void __launch_bounds__(256, MI == 1 ? 3 : 2) forward_f32_kernel(const float* W, const float* X,
                                                           const float* Xb, int K, int J, int D,
                                                           RowMap z, RowMap v, int d_per_range, long long range_stride) {
   chain_wait();
@@ -89,25 +90,36 @@ __global__ void __launch_bounds__(256, 2) forward_f32_kernel(const float* W, con
     for (int n = 0; n < 2 * NI; ++n) acc[m][n] = make_float2(0.f, 0.f);
 
   float4 pa[MI], pb[NI];
-  auto fetch = [&](int d0) {   // (W first: its loads do not wait behind the stores of v)
+  const float* xr = X + (size_t)(i0 + lr) * D + lc;
+  const float* wr = W + (size_t)(j0 + lr) * D + lc;
+  auto fetch = [&](int d0) {   // (the stores of v last: no load waits behind them)
+    const int left = D - d0 - lc;
+    float4 sb[PAIR ? MI : 1];
 #pragma unroll
-    for (int q = 0; q < NI; ++q) {
-      const int j = j0 + lr + 64 * q;
-      pb[q] = (j < J) ? ld4_guard(W + (size_t)j * D, d0 + lc, D, vec_ok) : make_float4(0.f, 0.f, 0.f, 0.f);
-    }
+    for (int q = 0; q < NI; ++q)
+      pb[q] = (j0 + lr + 64 * q < J) ? ld4_left(wr + (size_t)(64 * q) * D + d0, left, vec_ok) : make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
     for (int q = 0; q < MI; ++q) {
-      const int i = i0 + lr + 64 * q;
       float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (i < K) {
-        a = ld4_guard(X + (size_t)i * D, d0 + lc, D, vec_ok);
-        if (Xb != nullptr) {
-          const float4 b = ld4_guard(Xb + (size_t)i * D, d0 + lc, D, vec_ok);
-          a.x = __fsub_rn(a.x, b.x); a.y = __fsub_rn(a.y, b.y); a.z = __fsub_rn(a.z, b.z); a.w = __fsub_rn(a.w, b.w);
-        }
-        if (write_v && d0 + lc < v.ld) *reinterpret_cast<float4*>(v.row(i) + (size_t)(d0 + lc) * 4) = a;
+      if (PAIR) sb[PAIR ? q : 0] = a;
+      if (i0 + lr + 64 * q < K) {
+        const float* x = xr + (size_t)(64 * q) * D + d0;
+        a = ld4_left(x, left, vec_ok);
+        if (PAIR) sb[PAIR ? q : 0] = ld4_left(x + (Xb - X), left, vec_ok);
       }
       pa[q] = a;
+    }
+    if (PAIR) {
+#pragma unroll
+      for (int q = 0; q < MI; ++q) {
+        const float4 a = pa[q], b = sb[PAIR ? q : 0];
+        pa[q] = make_float4(__fsub_rn(a.x, b.x), __fsub_rn(a.y, b.y), __fsub_rn(a.z, b.z), __fsub_rn(a.w, b.w));
+      }
+    }
+    if (write_v && d0 + lc < v.ld) {
+#pragma unroll
+      for (int q = 0; q < MI; ++q)
+        if (i0 + lr + 64 * q < K) *reinterpret_cast<float4*>(v.row(i0 + lr + 64 * q) + (size_t)(d0 + lc) * 4) = pa[q];
     }
   };
   auto stash = [&]() {
@@ -462,20 +474,23 @@ __global__ void __launch_bounds__(256) transpose_rows_vec_kernel(TransposeJob j0
 
 }  // namespace
 
-// How a forward is done: in one launch (the smallest problems, whose sums the single-launch step repeats in the same
-// order), on 64 x 64 tiles in place, or on 128 x 128 tiles through transposed copies; and its reduction ranges.
-namespace {
-struct ForwardPlan {
-  int tile, ks;   // tile 0: one launch
-};
-// Estimated microseconds.  64 x 64 tiles run at 40 % of the FMA rate when the SMs are full and at 0.9 us per 16 steps when
-// not; 128 x 128 tiles at 70 %, behind a transposing pass at 4.5 TB/s; a range's partial products go out and come back.
-ForwardPlan plan_forward(int K, int J, int D, int max_ks) {
-  if (step_small_fits(K, J, D)) return {0, 1};
+// How a forward is done, and its reduction ranges.  Estimated microseconds: 64 x 64 tiles run at 40 % of the FMA rate when
+// the SMs are full and at 0.9 us per 16 steps when not; 128 x 128 tiles at 70 %, behind a transposing pass at 4.5 TB/s; a
+// range's partial products go out and come back.
+// Where the transposing pass does not pay (or its workspace is not there), one launch with the operands in place is the
+// faster of the two others
+//   - on 128 x 128 tiles, where there are enough of them and the samples meet more than one tile's width of classes: 3.28 us
+//     per 16 steps for two tiles to an SM, against 0.62 for every 64 x 64 tile (1000 x 256, K = 32768: 569 -> 388 us;
+//     300 x 511, K = 65536, rows of no whole 16-byte units: 721 -> 640; 100 x 64, K = 32768: 22.0 -> 17.4; but
+//     64 x 256, K = 65536: 84 against 131 us);
+//   - for reductions of four stages or less, which would not fill the ring (10 x 64, K = 4096: 5.7 -> 5.1 us);
+//   - for pairs also where the difference, formed on the way, would cost more as a pass of its own.
+ForwardF32Plan forward_f32_plan(int K, int J, int D, bool pair, int max_ks, bool transposed_ok) {
+  if (step_small_fits(K, J, D)) return {F32_IN_PLACE, 1};   // (the single-launch step repeats these sums in this order)
   const double fma_us = 128 * 1900.0;
-  ForwardPlan best = {64, 1};
+  ForwardF32Plan best = {F32_SMALL, 1};
   double best_us = -1;
-  auto consider = [&](int tile, double rate, double step_us, double before) {
+  auto consider = [&](F32Route route, int tile, double rate, double step_us, double before) {
     const double tiles = (double)((K + tile - 1) / tile) * ((J + tile - 1) / tile);
     for (int ks = 1; ks <= max_ks && (ks == 1 || D / ks >= 64); ++ks) {
       const int per = ((D + ks - 1) / ks + BK - 1) / BK * BK;
@@ -484,19 +499,31 @@ ForwardPlan plan_forward(int K, int J, int D, int max_ks) {
       const double us = before + (work > chain ? work : chain) + (ks > 1 ? ks * (double)J * K * 8 / 6e6 : 0.0);
       if (best_us < 0 || us < best_us) {
         best_us = us;
-        best = {tile, ks};
+        best = {route, ks};
       }
     }
   };
-  consider(64, 0.40, 0.9, 0.0);
-  if (K >= 128 && J >= 64 && D >= 512) consider(128, 0.70, 0.9, 4.0 + (double)(J + K) * D * 8 / 4.5e6);
+  consider(F32_SMALL, 64, 0.40, 0.9, 0.0);
+  if (transposed_ok && K >= 128 && J >= 64 && D >= 512)
+    consider(F32_TRANSPOSED, 128, 0.70, 0.9, 4.0 + (double)(J + K) * D * 8 / 4.5e6);
+  if (best.route != F32_SMALL) return best;
+  auto tiles_of = [&](int t) { return (long long)((K + t - 1) / t) * ((J + t - 1) / t); };
+  const long long t64 = tiles_of(64), t128 = tiles_of(128);
+  const double steps = (D + BK - 1) / BK, steps_ks = ((D + best.ks - 1) / best.ks + BK - 1) / BK;
+  const double full = (double)((t64 * best.ks + 147) / 148) * (0.25 + 0.62 * steps_ks), chain = 0.9 * steps_ks;
+  const double small_us = 0.5 + (full > chain ? full : chain) + (best.ks > 1 ? best.ks * (double)J * K * 8 / 6e6 : 0.0) +
+                          (pair ? 3.0 + (double)K * D * 12 / 5e6 : 0.0);
+  const double odd = (D & 3) != 0 ? 1.12 : 1.0;
+  double in_place_us = small_us;
+  if (J > 64 && t128 >= F32_MIN_LARGE_TILES)
+    in_place_us = odd * (t128 > 148 ? (double)((t128 + 295) / 296) * (2.8 + 3.28 * steps) : 2.8 + 2.1 * steps);
+  else if (pair) {
+    const double f = (double)((t64 + 147) / 148) * (0.45 + 0.70 * steps), c = 0.9 * steps;
+    in_place_us = 0.5 + odd * (f > c ? f : c);
+  }
+  if (in_place_us < small_us || (D <= 4 * BK && t64 <= 296)) return {F32_IN_PLACE, 1};
   return best;
 }
-}  // namespace
-
-int forward_f32_splits(int K, int J, int D) { return plan_forward(K, J, D, FORWARD_F32_MAX_SPLITS).ks; }
-bool forward_f32_transposed(int K, int J, int D) { return plan_forward(K, J, D, FORWARD_F32_MAX_SPLITS).tile == 128; }
-bool forward_f32_fused(int K, int J, int D) { return plan_forward(K, J, D, 1).tile == 0; }
 
 // No empty range: the finishing pass would add a partial buffer nobody wrote.
 static int range_length(int D, int* ks) {
@@ -510,12 +537,17 @@ int launch_forward_f32(cudaStream_t s, const float* W, const float* X, const flo
   const int per = range_length(D, &ks);
   if (ks > 1) z = part;
   if (nsplit_out != nullptr) *nsplit_out = ks;
-  const int big = ((J + 127) / 128) * ((K + 127) / 128);
-  if ((long long)big * ks >= 148)
-    launch_chained(forward_f32_kernel<2, 2>, dim3(big, 1, ks), 256, 0, s, W, X, Xb, K, J, D, z, v, per, split_stride);
-  else
-    launch_chained(forward_f32_kernel<1, 1>, dim3(((J + 63) / 64) * ((K + 63) / 64), 1, ks), 256, 0, s, W, X, Xb, K, J, D, z, v,
-                   per, split_stride);
+  const int large = ((J + 127) / 128) * ((K + 127) / 128), small = ((J + 63) / 64) * ((K + 63) / 64);
+  auto go = [&](auto kernel, int tiles) {
+    launch_chained(kernel, dim3(tiles, 1, ks), 256, 0, s, W, X, Xb, K, J, D, z, v, per, split_stride);
+  };
+  if (J > 64 && (long long)large * ks >= F32_MIN_LARGE_TILES) {
+    if (Xb != nullptr) go(forward_f32_kernel<2, 2, true>, large);
+    else go(forward_f32_kernel<2, 2, false>, large);
+  } else {
+    if (Xb != nullptr) go(forward_f32_kernel<1, 1, true>, small);
+    else go(forward_f32_kernel<1, 1, false>, small);
+  }
   return cudaGetLastError() == cudaSuccess ? 1 : SFB_ERR_CUDA;
 }
 
