@@ -46,9 +46,10 @@ __device__ __forceinline__ CsrRow csr_row(const CsrView& c, int i) {
 }
 
 // Wt[d][j] = W[j][d]; Wt rows have ldt values (J rounded up to 4), pad columns zero.
-__global__ void __launch_bounds__(256) transpose_kernel(const float* W, float* Wt, int J, int D,
-                                                        int ldt) {
-  chain();
+// early: the forward pass behind it is let in at once, not when the copy is done.
+__global__ void __launch_bounds__(256) transpose_kernel(const float* W, float* Wt, int J, int D, int ldt, bool early) {
+  if (early) chain_next();
+  chain_wait();
   __shared__ float tile[32][33];
   const int d0 = blockIdx.x * 32, j0 = blockIdx.y * 32;
   const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;   // 32 x 8
@@ -63,6 +64,7 @@ __global__ void __launch_bounds__(256) transpose_kernel(const float* W, float* W
     const int d = d0 + ty + r, j = j0 + tx;
     if (d < D && j < ldt) Wt[(size_t)d * ldt + j] = tile[tx][ty + r];
   }
+  if (!early) chain_next();
 }
 
 // grid = (K samples, ceil(ldt / 1024)); each thread owns 4 consecutive rows j of W.
@@ -352,9 +354,13 @@ int launch_sc_forward_ws(cudaStream_t s, const float* W, float* Wt, CsrView code
                          int J, int D, int* dev_status) {
   const int ldt = (int)pad_to(J, 4);
   dim3 tg((D + 31) / 32, (ldt + 31) / 32);
-  launch_chained(transpose_kernel, tg, 256, 0, s, W, Wt, J, D, ldt);
   const int cols = ldt > u.ld ? ldt : u.ld;   // pad columns of a wider u row are written (as zeros) too
   dim3 grid(K, (cols + 1023) / 1024);
+  // Where the blocks of both do not fit on the chip together (eight to an SM), those of the forward, one per sample and 1024
+  // rows, would crowd onto the SMs that run free first: 1000 x 1000, K = 256, half of the codes nonzero: 80 us for the
+  // factors, 38 when they wait for the end of the copy.  Where they do fit, waiting would cost 1 us of 8 (100 x 400, K = 20).
+  const bool early = (long long)tg.x * tg.y + (long long)grid.x * grid.y <= 8 * 148;
+  launch_chained(transpose_kernel, tg, 256, 0, s, W, Wt, J, D, ldt, early);
   launch_chained(sc_forward_kernel, grid, 256, 0, s, Wt, ldt, codes, Xdata, u, K, J, D, dev_status);
   return cudaGetLastError() == cudaSuccess ? 2 : SFB_ERR_CUDA;
 }
