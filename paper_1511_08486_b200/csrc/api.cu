@@ -19,6 +19,7 @@ struct sfb_ctx {
   float* wt_ws;             // SC, fp32 path: atom-major copy of W for the forward
   float* a_dense;           // SC, tf32 path: dense rows of the codes, [K][ldv]
   void* csc_ws;             // SC, fp32 path: scratch of the atom-major re-sort of the codes (when K fits)
+  uint8_t* sc_flags;        // ... and when it does not: which rows of the codes are malformed
   // sfb_step: work that does not depend on the factors (codes into the buffer, header, atom-major re-sort of
   // the codes) runs on this stream beside the forward pass, forked and joined by events
   cudaStream_t aux;
@@ -300,6 +301,8 @@ int sfb_create(const sfb_desc* desc, void* cuda_stream, sfb_ctx** out) {
     ok = cudaMalloc(&c->wt_ws, (size_t)sc_forward_workspace_bytes(desc->J, desc->D)) == cudaSuccess;
   if (ok && desc->model == SFB_SC && desc->path == SFB_PATH_F32 && sc_csc_supported(c->K))
     ok = cudaMalloc(&c->csc_ws, (size_t)sc_csc_workspace_bytes(c->K, desc->D, (long long)desc->nnz_capacity)) == cudaSuccess;
+  if (ok && desc->model == SFB_SC && desc->path == SFB_PATH_F32 && !sc_csc_supported(c->K))
+    ok = cudaMalloc(&c->sc_flags, (size_t)c->K) == cudaSuccess;
   if (ok && desc->model == SFB_SC && (desc->path == SFB_PATH_TF32 || desc->path == SFB_PATH_TF32X3))
     ok = cudaMalloc(&c->a_dense, (size_t)c->K * c->l.ldv * 4) == cudaSuccess;
   if (ok && desc->model != SFB_SC && desc->path == SFB_PATH_F32) {
@@ -369,6 +372,7 @@ int sfb_destroy(sfb_ctx* c) {
   if (c->wt_ws) cudaFree(c->wt_ws);
   if (c->a_dense) cudaFree(c->a_dense);
   if (c->csc_ws) cudaFree(c->csc_ws);
+  if (c->sc_flags) cudaFree(c->sc_flags);
   if (c->f32_part) cudaFree(c->f32_part);
   if (c->f32_nn_ws) cudaFree(c->f32_nn_ws);
   if (c->compact_ws) cudaFree(c->compact_ws);
@@ -595,7 +599,7 @@ static int apply_from(sfb_ctx* c, void* W, const void* sf_buf, float eta, int K,
                             (long long)d.nnz_capacity, c->csc_ws, c->dev_status));
   } else if (d.v_sparse && d.path == SFB_PATH_F32) {
     ACC(launch_sc_apply(c->stream, reinterpret_cast<float*>(W), stream_codes(c, sf_buf), stream_u(c, sf_buf), K, d.J,
-                        d.D, eta, c->dev_status, c->dev_status));
+                        d.D, eta, c->sc_flags, c->dev_status, check ? c->dev_status : nullptr));
   } else if (d.v_sparse) {
     // dense alternative: rebuild the dense code rows from the buffer's CSR streams unless this step just made them
     if (check)

@@ -367,8 +367,9 @@ int launch_sc_forward_ws(cudaStream_t s, const float* W, float* Wt, CsrView code
                          int J, int D, int* dev_status);
 
 // SC apply: W[:, d] -= eta * sum_{i: a_id != 0} a_id * u_i (sparse-v scatter, no float atomics).
-int launch_sc_apply(cudaStream_t s, float* W, CsrView codes, RowMap u, int K, int J, int D, float eta,
-                    const int* dev_status_ro, int* dev_status);
+// flags: K bytes of scratch.  dev_status: SFB_DEV_BAD_INDEX for rows with entries that are left out; refused: see is_refused.
+int launch_sc_apply(cudaStream_t s, float* W, CsrView codes, RowMap u, int K, int J, int D, float eta, uint8_t* flags,
+                    int* dev_status, const int* refused = nullptr);
 
 // The same update through an atom-major (CSC) re-sort of the codes and shared-memory u columns (faster;
 // needs sc_csc_supported(K) and a workspace of sc_csc_workspace_bytes(K, D, nnz_capacity) bytes).

@@ -124,6 +124,36 @@ __global__ void __launch_bounds__(256) sc_forward_kernel(const float* Wt, int ld
   }
 }
 
+// A row's entries into its dense row, which holds zeros, by one block.  An entry counts if its atom exists and exceeds its
+// predecessor's; in a row that is not ascending an atom may count more than once: the values are added in row order.
+// round: what is stored is the nearest tf32 value.  (The tensor cores drop the low 13 mantissa bits of a tf32 operand; the
+// dense rows are only ever that, the wire keeps the exact CSR values, and rounding halves the error.)
+__device__ __forceinline__ void scatter_row(const CsrRow& row, float* dense, int D, bool round, int* dev_status) {
+  auto counts = [&](int k) { return row.idx[k] < (uint32_t)D && !(k > 0 && row.idx[k - 1] >= row.idx[k]); };
+  auto stored = [&](float a) {
+    uint32_t r = __float_as_uint(a);
+    if (round) asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(r) : "f"(a));
+    return __uint_as_float(r);
+  };
+  bool bad = false;
+  for (int k = threadIdx.x; k < row.len; k += 256) {
+    if (counts(k)) dense[row.idx[k]] = stored(row.val[k]);
+    else bad = true;
+  }
+  if (!__syncthreads_or(bad)) return;
+  if (threadIdx.x == 0) atomicOr(dev_status, SFB_DEV_BAD_INDEX);
+  for (int k = threadIdx.x; k < row.len; k += 256)
+    if (counts(k)) dense[row.idx[k]] = 0.f;
+  __syncthreads();
+  if (threadIdx.x == 0)
+    for (int k = 0; k < row.len; ++k)
+      if (counts(k)) dense[row.idx[k]] += row.val[k];
+  __syncthreads();
+  for (int k = threadIdx.x; k < row.len; k += 256)   // (rounding a second time changes nothing)
+    if (counts(k)) dense[row.idx[k]] = stored(dense[row.idx[k]]);
+  __syncthreads();
+}
+
 // One block per sample: zero the dense row, then scatter the sample's nonzeros into it.
 __global__ void __launch_bounds__(256) densify_kernel(CsrView codes, RowMap a, int K, int D, int* dev_status,
                                                       bool round_tf32, const int* refused) {
@@ -134,17 +164,7 @@ __global__ void __launch_bounds__(256) densify_kernel(CsrView codes, RowMap a, i
   for (int q = threadIdx.x; q < (a.ld >> 2); q += 256) reinterpret_cast<float4*>(dst)[q] = make_float4(0.f, 0.f, 0.f, 0.f);
   __syncthreads();
   const CsrRow row = csr_row(codes, i);
-  for (int k = threadIdx.x; k < row.len; k += 256) {
-    const uint32_t c = row.idx[k];
-    if (c >= (uint32_t)D || (k > 0 && row.idx[k - 1] >= c)) atomicOr(dev_status, SFB_DEV_BAD_INDEX);   // entry skipped
-    else {
-      // the tensor cores drop the low 13 mantissa bits of a tf32 operand: rounding the code value to nearest
-      // here (the dense rows are only ever a tf32 operand; the wire keeps the exact CSR values) halves that error
-      uint32_t r = __float_as_uint(row.val[k]);
-      if (round_tf32) asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(r) : "f"(row.val[k]));
-      dst[c] = __uint_as_float(r);
-    }
-  }
+  scatter_row(row, dst, D, round_tf32, dev_status);
 }
 
 // The same through shared memory (one block per sample, the dense row of a.ld floats staged there), for the
@@ -158,12 +178,7 @@ __global__ void __launch_bounds__(256) densify_corr_kernel(CsrView codes, RowMap
   for (int q = threadIdx.x; q < units; q += 256) reinterpret_cast<float4*>(dense)[q] = make_float4(0.f, 0.f, 0.f, 0.f);
   __syncthreads();
   const CsrRow row = csr_row(codes, i);
-  for (int k = threadIdx.x; k < row.len; k += 256) {
-    const uint32_t c = row.idx[k];
-    if (c >= (uint32_t)D || (k > 0 && row.idx[k - 1] >= c)) atomicOr(dev_status, SFB_DEV_BAD_INDEX);   // entry skipped
-    else dense[c] = row.val[k];
-  }
-  __syncthreads();
+  scatter_row(row, dense, D, false, dev_status);
   float4* dst = reinterpret_cast<float4*>(a.row(i));
   for (int q = threadIdx.x; q < units; q += 256) {
     const float4 t = reinterpret_cast<const float4*>(dense)[q];
@@ -203,14 +218,31 @@ constexpr int SLAB_J = 4 * SLAB_T; // rows of W per block: four consecutive rows
 constexpr int SLAB_CAP = 1024;     // entries applied per pass (more are handled by further passes)
 constexpr int SLAB_BATCH = 8;      // entries whose u values are fetched together
 
+// flags[i] = 1 if row i is not strictly ascending (or holds an atom that does not exist): one warp per row.
+__global__ void __launch_bounds__(256) sc_malformed_kernel(CsrView codes, int K, int D, uint8_t* __restrict__ flags,
+                                                           int* dev_status, const int* refused) {
+  const int i = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  if (i >= K || is_refused(refused)) return;
+  const CsrRow row = csr_row(codes, i);
+  bool bad = false;
+  for (int k = lane; k < row.len; k += 32) bad |= row.idx[k] >= (uint32_t)D || (k > 0 && row.idx[k - 1] >= row.idx[k]);
+  bad = __any_sync(0xffffffffu, bad);
+  if (lane != 0) return;
+  flags[i] = bad ? 1 : 0;
+  if (bad) atomicOr(dev_status, SFB_DEV_BAD_INDEX);
+}
+
 // grid = (ceil(D / 16), ceil(J / 1024)); the block owns the 16-atom x 1024-row slab of W in shared memory.
 // Per round of 256 samples: every thread finds the entries of one sample's sorted CSR row that fall
 // inside the slab (binary search + short scan), a block-wide scan orders them by (sample, atom), and
 // the entries are applied in that order: thread t adds -eta * a * u_i[j] to its own four rows j of
 // the slab, with the u values of 8 entries fetched ahead as independent 16-byte loads.
 // A thread owns its rows for the whole kernel, so there is no race and the summation order is fixed.
+// In a row flagged as malformed every entry is looked at: those that count (atom in the slab, above its predecessor's) are
+// taken in row order.
 __global__ void __launch_bounds__(SLAB_T) sc_apply_kernel(float* __restrict__ W, CsrView codes, RowMap u, int K, int J,
-                                                          int D, float eta, const int* __restrict__ status_ro) {
+                                                          int D, float eta, const uint8_t* __restrict__ malformed,
+                                                          const int* __restrict__ status_ro) {
   extern __shared__ __align__(16) float Ws[];   // 64 KB: Ws[atom * SLAB_J + row]
   __shared__ int s_key[SLAB_CAP];               // sample * 16 + atom-in-slab
   __shared__ float s_val[SLAB_CAP];             // -eta * code value
@@ -254,17 +286,23 @@ __global__ void __launch_bounds__(SLAB_T) sc_apply_kernel(float* __restrict__ W,
     int lo = 0, cnt = 0;
     CsrRow row;
     row.len = 0;
+    bool scan_all = false;
+    auto counts = [&](int k) {
+      return row.idx[k] >= (uint32_t)d0 && row.idx[k] < (uint32_t)(d0 + dn) && !(k > 0 && row.idx[k - 1] >= row.idx[k]);
+    };
     if (i < K) {
       row = csr_row(codes, i);
-      int hi = row.len;
-      while (lo < hi) {   // lower bound of d0
-        const int mid = (lo + hi) >> 1;
-        if (row.idx[mid] < (uint32_t)d0) lo = mid + 1; else hi = mid;
+      scan_all = malformed[i] != 0;
+      if (scan_all) {
+        for (int k = 0; k < row.len; ++k) cnt += counts(k) ? 1 : 0;
+      } else {
+        int hi = row.len;
+        while (lo < hi) {   // lower bound of d0
+          const int mid = (lo + hi) >> 1;
+          if (row.idx[mid] < (uint32_t)d0) lo = mid + 1; else hi = mid;
+        }
+        while (lo + cnt < row.len && cnt < SLAB_D && row.idx[lo + cnt] < (uint32_t)(d0 + dn)) ++cnt;
       }
-      // (the lower bound matters only for rows that are not ascending: nothing outside the slab is ever addressed)
-      while (lo + cnt < row.len && cnt < SLAB_D && row.idx[lo + cnt] >= (uint32_t)d0 &&
-             row.idx[lo + cnt] < (uint32_t)(d0 + dn))
-        ++cnt;
     }
     // (2) block-wide exclusive scan of the counts (fixed order)
     int incl = cnt;
@@ -290,14 +328,14 @@ __global__ void __launch_bounds__(SLAB_T) sc_apply_kernel(float* __restrict__ W,
     __syncthreads();
     // (3) apply, SLAB_CAP entries per pass, in (sample, atom) order
     for (int win = 0; win < total; win += SLAB_CAP) {
-      for (int e = 0; e < cnt; ++e) {
+      for (int e = 0, k = lo; e < cnt; ++k) {
+        if (scan_all && !counts(k)) continue;
         const int pos = base + e - win;
         if (pos >= 0 && pos < SLAB_CAP) {
-          s_key[pos] = i * SLAB_D + ((int)row.idx[lo + e] - d0);
-          // an entry that breaks the ascending order is skipped, as in the forward pass
-          const bool skip = lo + e > 0 && row.idx[lo + e - 1] >= row.idx[lo + e];
-          s_val[pos] = skip ? 0.f : -eta * row.val[lo + e];
+          s_key[pos] = i * SLAB_D + ((int)row.idx[k] - d0);
+          s_val[pos] = -eta * row.val[k];
         }
+        ++e;
       }
       __syncthreads();
       const int n = min(SLAB_CAP, total - win);
@@ -389,8 +427,8 @@ int launch_finish_sc(cudaStream_t s, RowMap z, RowMap u, const float* Xdata, int
   return cudaGetLastError() == cudaSuccess ? 1 : SFB_ERR_CUDA;
 }
 
-int launch_sc_apply(cudaStream_t s, float* W, CsrView codes, RowMap u, int K, int J, int D, float eta,
-                    const int* dev_status_ro, int* /*dev_status*/) {
+int launch_sc_apply(cudaStream_t s, float* W, CsrView codes, RowMap u, int K, int J, int D, float eta, uint8_t* flags,
+                    int* dev_status, const int* refused) {
   static PerDeviceOnce attr_once;
   const bool ready = set_up_device(attr_once, [] {
     return allow_smem(sc_apply_kernel, SLAB_D * SLAB_J * 4) &&
@@ -398,8 +436,9 @@ int launch_sc_apply(cudaStream_t s, float* W, CsrView codes, RowMap u, int K, in
   });
   if (!ready) return SFB_ERR_CUDA;
   dim3 grid((D + SLAB_D - 1) / SLAB_D, (J + SLAB_J - 1) / SLAB_J);
-  sc_apply_kernel<<<grid, SLAB_T, SLAB_D * SLAB_J * 4, s>>>(W, codes, u, K, J, D, eta, dev_status_ro);
-  return cudaGetLastError() == cudaSuccess ? 1 : SFB_ERR_CUDA;
+  sc_malformed_kernel<<<(K + 7) / 8, 256, 0, s>>>(codes, K, D, flags, dev_status, refused);
+  sc_apply_kernel<<<grid, SLAB_T, SLAB_D * SLAB_J * 4, s>>>(W, codes, u, K, J, D, eta, flags, dev_status);
+  return cudaGetLastError() == cudaSuccess ? 2 : SFB_ERR_CUDA;
 }
 
 }  // namespace sfb

@@ -52,9 +52,9 @@ __device__ __forceinline__ CsrRow2 csr_row2(const CsrView& c, int i) {
   return r;
 }
 
-// An entry counts only if its atom exists and the row is strictly ascending up to it: the rule of the forward
-// pass (sc_forward_kernel), so that forward and apply agree on malformed rows, and the reason why a
-// (chunk, atom) cell has at most one writer per sample in the fill below (no repeated atom inside a row).
+// An entry counts only if its atom exists and exceeds its predecessor's: the rule of the forward pass
+// (sc_forward_kernel), so that forward and apply agree on malformed rows.  In a row that is strictly ascending no atom
+// is repeated; in another one an atom may count more than once (5, 3, 5: the fill adds both values, as the forward does).
 __device__ __forceinline__ bool entry_ok(const CsrRow2& row, int k, int D) {
   const uint32_t d = row.idx[k];
   return d < (uint32_t)D && !(k > 0 && row.idx[k - 1] >= d);
@@ -163,13 +163,26 @@ __global__ void __launch_bounds__(256) csc_fill_kernel(CsrView codes, int K, int
   const int i_in = i - slice * chunks_per_slice * CSC_CHUNK;
   const uint32_t below = (1u << (i % CSC_CHUNK)) - 1u;
   const CsrRow2 row = csr_row2(codes, i);
+  auto place = [&](int k) {
+    const uint32_t d = row.idx[k];
+    const size_t cell = (size_t)c * D + d;
+    return ent + colptr[(size_t)slice * D + d] + off[cell] + __popc(mask[cell] & below);
+  };
+  bool bad = false;
   for (int k = threadIdx.x; k < row.len; k += 256) {
-    if (entry_ok(row, k, D)) {
-      const uint32_t d = row.idx[k];
-      const size_t cell = (size_t)c * D + d;
-      ent[colptr[(size_t)slice * D + d] + off[cell] + __popc(mask[cell] & below)] =
-          make_int2(i_in, __float_as_int(row.val[k]));
-    }
+    if (entry_ok(row, k, D)) *place(k) = make_int2(i_in, __float_as_int(row.val[k]));
+    else bad = true;
+  }
+  if (__syncthreads_or(bad)) {   // malformed: an atom that counts twice has one place, its values are added in row order
+    for (int k = threadIdx.x; k < row.len; k += 256)
+      if (entry_ok(row, k, D)) place(k)->y = 0;
+    __syncthreads();
+    if (threadIdx.x == 0)
+      for (int k = 0; k < row.len; ++k)
+        if (entry_ok(row, k, D)) {
+          int2* e = place(k);
+          e->y = __float_as_int(__int_as_float(e->y) + row.val[k]);
+        }
   }
 }
 
