@@ -124,33 +124,35 @@ __global__ void __launch_bounds__(256) sc_forward_kernel(const float* Wt, int ld
   }
 }
 
+__device__ __forceinline__ float nearest_tf32(float a) {
+  uint32_t r;
+  asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(r) : "f"(a));
+  return __uint_as_float(r);
+}
 // A row's entries into its dense row, which holds zeros, by one block.  An entry counts if its atom exists and exceeds its
 // predecessor's; in a row that is not ascending an atom may count more than once: the values are added in row order.
 // round: what is stored is the nearest tf32 value.  (The tensor cores drop the low 13 mantissa bits of a tf32 operand; the
 // dense rows are only ever that, the wire keeps the exact CSR values, and rounding halves the error.)
-__device__ __forceinline__ void scatter_row(const CsrRow& row, float* dense, int D, bool round, int* dev_status) {
-  auto counts = [&](int k) { return row.idx[k] < (uint32_t)D && !(k > 0 && row.idx[k - 1] >= row.idx[k]); };
-  auto stored = [&](float a) {
-    uint32_t r = __float_as_uint(a);
-    if (round) asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(r) : "f"(a));
-    return __uint_as_float(r);
-  };
-  bool bad = false;
+// malformed: a shared word, zero before the block's last barrier.
+__device__ __forceinline__ void scatter_row(const CsrRow& row, float* dense, int D, bool round, int* malformed, int* dev_status) {
   for (int k = threadIdx.x; k < row.len; k += 256) {
-    if (counts(k)) dense[row.idx[k]] = stored(row.val[k]);
-    else bad = true;
+    const uint32_t c = row.idx[k];
+    if (c >= (uint32_t)D || (k > 0 && row.idx[k - 1] >= c)) *malformed = 1;   // entry skipped
+    else dense[c] = round ? nearest_tf32(row.val[k]) : row.val[k];
   }
-  if (!__syncthreads_or(bad)) return;
-  if (threadIdx.x == 0) atomicOr(dev_status, SFB_DEV_BAD_INDEX);
-  for (int k = threadIdx.x; k < row.len; k += 256)
-    if (counts(k)) dense[row.idx[k]] = 0.f;
   __syncthreads();
-  if (threadIdx.x == 0)
-    for (int k = 0; k < row.len; ++k)
-      if (counts(k)) dense[row.idx[k]] += row.val[k];
-  __syncthreads();
-  for (int k = threadIdx.x; k < row.len; k += 256)   // (rounding a second time changes nothing)
-    if (counts(k)) dense[row.idx[k]] = stored(dense[row.idx[k]]);
+  if (*malformed == 0) return;
+  if (threadIdx.x == 0) {
+    atomicOr(dev_status, SFB_DEV_BAD_INDEX);
+    for (int pass = 0; pass < 3; ++pass)   // clear, add, round (a second time changes nothing)
+      for (int k = 0; k < row.len; ++k) {
+        const uint32_t c = row.idx[k];
+        if (c >= (uint32_t)D || (k > 0 && row.idx[k - 1] >= c)) continue;
+        if (pass == 0) dense[c] = 0.f;
+        else if (pass == 1) dense[c] += row.val[k];
+        else if (round) dense[c] = nearest_tf32(dense[c]);
+      }
+  }
   __syncthreads();
 }
 
@@ -159,12 +161,14 @@ __global__ void __launch_bounds__(256) densify_kernel(CsrView codes, RowMap a, i
                                                       bool round_tf32, const int* refused) {
   chain();
   if (is_refused(refused)) return;
+  __shared__ int malformed;
+  if (threadIdx.x == 0) malformed = 0;
   const int i = blockIdx.x;
   float* dst = reinterpret_cast<float*>(a.row(i));
   for (int q = threadIdx.x; q < (a.ld >> 2); q += 256) reinterpret_cast<float4*>(dst)[q] = make_float4(0.f, 0.f, 0.f, 0.f);
   __syncthreads();
   const CsrRow row = csr_row(codes, i);
-  scatter_row(row, dst, D, round_tf32, dev_status);
+  scatter_row(row, dst, D, round_tf32, &malformed, dev_status);
 }
 
 // The same through shared memory (one block per sample, the dense row of a.ld floats staged there), for the
@@ -173,12 +177,14 @@ __global__ void __launch_bounds__(256) densify_corr_kernel(CsrView codes, RowMap
                                                            CorrOut corr) {
   chain();
   extern __shared__ __align__(16) float dense[];
+  __shared__ int malformed;
+  if (threadIdx.x == 0) malformed = 0;
   const int i = blockIdx.x;
   const int units = a.ld >> 2;
   for (int q = threadIdx.x; q < units; q += 256) reinterpret_cast<float4*>(dense)[q] = make_float4(0.f, 0.f, 0.f, 0.f);
   __syncthreads();
   const CsrRow row = csr_row(codes, i);
-  scatter_row(row, dense, D, false, dev_status);
+  scatter_row(row, dense, D, false, &malformed, dev_status);
   float4* dst = reinterpret_cast<float4*>(a.row(i));
   for (int q = threadIdx.x; q < units; q += 256) {
     const float4 t = reinterpret_cast<const float4*>(dense)[q];
@@ -238,8 +244,9 @@ __global__ void __launch_bounds__(256) sc_malformed_kernel(CsrView codes, int K,
 // the entries are applied in that order: thread t adds -eta * a * u_i[j] to its own four rows j of
 // the slab, with the u values of 8 entries fetched ahead as independent 16-byte loads.
 // A thread owns its rows for the whole kernel, so there is no race and the summation order is fixed.
-// In a row flagged as malformed every entry is looked at: those that count (atom in the slab, above its predecessor's) are
-// taken in row order.
+// SCAN: some rows are flagged as malformed.  There every entry is looked at: those that count (atom in the slab, above its
+// predecessor's) are taken in row order.  Both instantiations are launched, the status word tells which one has the work.
+template <bool SCAN>
 __global__ void __launch_bounds__(SLAB_T) sc_apply_kernel(float* __restrict__ W, CsrView codes, RowMap u, int K, int J,
                                                           int D, float eta, const uint8_t* __restrict__ malformed,
                                                           const int* __restrict__ status_ro) {
@@ -247,7 +254,8 @@ __global__ void __launch_bounds__(SLAB_T) sc_apply_kernel(float* __restrict__ W,
   __shared__ int s_key[SLAB_CAP];               // sample * 16 + atom-in-slab
   __shared__ float s_val[SLAB_CAP];             // -eta * code value
   __shared__ int s_warp[SLAB_T / 32];
-  if (status_ro != nullptr && (*status_ro & SFB_DEV_BAD_HEADER)) return;
+  if (*status_ro & SFB_DEV_BAD_HEADER) return;
+  if (((*status_ro & SFB_DEV_BAD_INDEX) != 0) != SCAN) return;   // (no row is flagged without it)
   const int t = threadIdx.x;
   const int d0 = blockIdx.x * SLAB_D, j0 = blockIdx.y * SLAB_J;
   const int dn = min(SLAB_D, D - d0);
@@ -292,7 +300,7 @@ __global__ void __launch_bounds__(SLAB_T) sc_apply_kernel(float* __restrict__ W,
     };
     if (i < K) {
       row = csr_row(codes, i);
-      scan_all = malformed[i] != 0;
+      scan_all = SCAN && malformed[i] != 0;
       if (scan_all) {
         for (int k = 0; k < row.len; ++k) cnt += counts(k) ? 1 : 0;
       } else {
@@ -431,14 +439,18 @@ int launch_sc_apply(cudaStream_t s, float* W, CsrView codes, RowMap u, int K, in
                     int* dev_status, const int* refused) {
   static PerDeviceOnce attr_once;
   const bool ready = set_up_device(attr_once, [] {
-    return allow_smem(sc_apply_kernel, SLAB_D * SLAB_J * 4) &&
-           cudaFuncSetAttribute(sc_apply_kernel, cudaFuncAttributePreferredSharedMemoryCarveout, 100) == cudaSuccess;
+    for (auto kernel : {sc_apply_kernel<false>, sc_apply_kernel<true>})
+      if (!allow_smem(kernel, SLAB_D * SLAB_J * 4) ||
+          cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, 100) != cudaSuccess)
+        return false;
+    return true;
   });
   if (!ready) return SFB_ERR_CUDA;
   dim3 grid((D + SLAB_D - 1) / SLAB_D, (J + SLAB_J - 1) / SLAB_J);
   sc_malformed_kernel<<<(K + 7) / 8, 256, 0, s>>>(codes, K, D, flags, dev_status, refused);
-  sc_apply_kernel<<<grid, SLAB_T, SLAB_D * SLAB_J * 4, s>>>(W, codes, u, K, J, D, eta, flags, dev_status);
-  return cudaGetLastError() == cudaSuccess ? 2 : SFB_ERR_CUDA;
+  sc_apply_kernel<false><<<grid, SLAB_T, SLAB_D * SLAB_J * 4, s>>>(W, codes, u, K, J, D, eta, flags, dev_status);
+  sc_apply_kernel<true><<<grid, SLAB_T, SLAB_D * SLAB_J * 4, s>>>(W, codes, u, K, J, D, eta, flags, dev_status);
+  return cudaGetLastError() == cudaSuccess ? 3 : SFB_ERR_CUDA;
 }
 
 }  // namespace sfb
