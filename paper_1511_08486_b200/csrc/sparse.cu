@@ -203,16 +203,18 @@ __global__ void __launch_bounds__(256) finish_sc_kernel(RowMap zr, RowMap u, con
     const int i = (int)(g / units), j = (int)(g % units) * 4;
     float4* p = reinterpret_cast<float4*>(u.row(i) + (size_t)j * 4);
     const float* zp = reinterpret_cast<const float*>(zr.row(i)) + j;
+    const float* x = Xdata + (size_t)i * J;   // (loaded beside the products, not behind their sum)
+    const float x0 = (j < J) ? x[j] : 0.f, x1 = (j + 1 < J) ? x[j + 1] : 0.f, x2 = (j + 2 < J) ? x[j + 2] : 0.f,
+                x3 = (j + 3 < J) ? x[j + 3] : 0.f;
     float4 z = *reinterpret_cast<const float4*>(zp);
     for (int sp = 1; sp < nsplit; ++sp) {
       const float4 q = *reinterpret_cast<const float4*>(zp + sp * zstride);
       z.x += q.x; z.y += q.y; z.z += q.z; z.w += q.w;
     }
-    const float* x = Xdata + (size_t)i * J;
-    z.x = (j < J) ? z.x - x[j] : 0.f;
-    z.y = (j + 1 < J) ? z.y - x[j + 1] : 0.f;
-    z.z = (j + 2 < J) ? z.z - x[j + 2] : 0.f;
-    z.w = (j + 3 < J) ? z.w - x[j + 3] : 0.f;
+    z.x = (j < J) ? z.x - x0 : 0.f;
+    z.y = (j + 1 < J) ? z.y - x1 : 0.f;
+    z.z = (j + 2 < J) ? z.z - x2 : 0.f;
+    z.w = (j + 3 < J) ? z.w - x3 : 0.f;
     *p = z;
     if (corr.mn != nullptr) corr_store4(corr, i, u.B, j, z);
   }
