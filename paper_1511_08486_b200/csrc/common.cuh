@@ -189,7 +189,6 @@ struct FinishExtra {
   uint8_t* nonzero;  // [rows] or nullptr
   RowMap src, dst;   // dst.base == nullptr: no copy
   int cols;
-  CorrOut corr;
   bool next_early;   // see chain_next
   int header_blocks; // blocks in front of the rows' that write the header (set by the launcher)
   FinishExtra() : nonzero(nullptr), src(), dst(), cols(0), next_early(false), header_blocks(0) {}
@@ -375,12 +374,10 @@ int launch_sc_apply(cudaStream_t s, float* W, CsrView codes, RowMap u, int K, in
 // needs sc_csc_supported(K) and a workspace of sc_csc_workspace_bytes(K, D, nnz_capacity) bytes).
 long long sc_csc_workspace_bytes(int K, int D, long long nnz_capacity);
 bool sc_csc_supported(int K);
-int launch_sc_apply_csc(cudaStream_t s, float* W, CsrView codes, RowMap u, int K, int J, int D, float eta,
-                        long long nnz_capacity, void* workspace, const int* dev_status_ro);
-// The two halves of launch_sc_apply_csc: the re-sort reads only the codes (it can run beside the forward
-// pass), the update needs u and the workspace the re-sort filled.
-// dev_status (optional): SFB_DEV_BAD_INDEX is set for entries the re-sort leaves out (atom out of range, row not
-// strictly ascending: the same entries the forward pass skips).
+// In two halves: the re-sort reads only the codes (it can run beside the forward pass), the update needs u and the
+// workspace the re-sort filled.
+// dev_status (optional): SFB_DEV_BAD_INDEX is set for entries the re-sort leaves out (the same entries the forward
+// pass skips).
 // refused: see is_refused (no entry is sorted then).
 int launch_sc_csc_build(cudaStream_t s, CsrView codes, int K, int D, long long nnz_capacity, void* workspace,
                         int* dev_status = nullptr, const int* refused = nullptr);

@@ -112,7 +112,7 @@ int header_blocks(const FinishExtra& x) {
 }
 __device__ __forceinline__ void finish_extra(const FinishExtra& x, int i) {
   if (x.dst.base != nullptr)
-    for (int q = threadIdx.x; q < x.dst.ld * x.dst.es / 16; q += blockDim.x) copy_unit(x.src, x.dst, i, q, x.cols, x.corr);
+    for (int q = threadIdx.x; q < x.dst.ld * x.dst.es / 16; q += blockDim.x) copy_unit(x.src, x.dst, i, q, x.cols, CorrOut());
 }
 
 // Row i of u written: does it hold a nonzero wire value?  (any: this thread's values do)

@@ -424,12 +424,4 @@ int launch_sc_csc_apply(cudaStream_t s, float* W, RowMap u, int K, int J, int D,
   return cudaGetLastError() == cudaSuccess ? 1 : SFB_ERR_CUDA;
 }
 
-int launch_sc_apply_csc(cudaStream_t s, float* W, CsrView codes, RowMap u, int K, int J, int D, float eta,
-                        long long nnz_capacity, void* workspace, const int* dev_status_ro) {
-  const int a = launch_sc_csc_build(s, codes, K, D, nnz_capacity, workspace, const_cast<int*>(dev_status_ro));
-  if (a < 0) return a;
-  const int b2 = launch_sc_csc_apply(s, W, u, K, J, D, eta, nnz_capacity, workspace, dev_status_ro);
-  return b2 < 0 ? b2 : a + b2;
-}
-
 }  // namespace sfb

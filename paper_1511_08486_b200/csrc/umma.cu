@@ -1305,7 +1305,7 @@ int umma_forward(UmmaPlan* pl, cudaStream_t s, const void* W, const __nv_bfloat1
       if ((r = launch_copy_rows(s, x_rows, v, K, d.D, cv)) < 0) return r;
       launches += r;
     }
-    if (v_inline && !v_first) { extra.src = x_rows; extra.dst = v; extra.cols = d.D; extra.corr = cv; }
+    if (v_inline && !v_first) { extra.src = x_rows; extra.dst = v; extra.cols = d.D; }
     if (v.base != nullptr && !v_inline && !v_first && pl->side_ok) {   // v = x on the side stream, joined before this call returns its work
       if (cudaEventRecord(pl->fork, s) != cudaSuccess || cudaStreamWaitEvent(pl->side, pl->fork, 0) != cudaSuccess)
         return SFB_ERR_CUDA;
@@ -1314,7 +1314,7 @@ int umma_forward(UmmaPlan* pl, cudaStream_t s, const void* W, const __nv_bfloat1
     pl->side_open = forked;
     auto body = [&]() -> int {
       if (forked) {
-        if ((r = launch_copy_rows(pl->side, x_rows, v, K, d.D, cv)) < 0) return r;
+        if ((r = launch_copy_rows(pl->side, x_rows, v, K, d.D)) < 0) return r;
         launches += r;
       }
       // the GEMM epilogue leaves exp(z - local max) in u and (max, sum) per half tile; the finishing
@@ -1347,7 +1347,7 @@ int umma_forward(UmmaPlan* pl, cudaStream_t s, const void* W, const __nv_bfloat1
         launches += r;
       }
       if (!forked && !v_inline && !v_first && v.base != nullptr) {
-        if ((r = launch_copy_rows(s, x_rows, v, K, d.D, cv)) < 0) return r;
+        if ((r = launch_copy_rows(s, x_rows, v, K, d.D)) < 0) return r;
         launches += r;
       }
       return 0;
