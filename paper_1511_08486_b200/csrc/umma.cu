@@ -875,8 +875,16 @@ bool encode_corr_mn_map(CUtensorMap* m, const void* base, long long ldc, long lo
 constexpr int MAX_SPLITS = 16;   // ranges a forward reduction may be cut into (partial buffers of the plan)
 constexpr int X3_MAX_SPLITS = 32;   // ... on the compensated path, where the count is also tuned to fill whole waves
 
+struct PickedVariant {   // what pick_variant chose for one shape (splits 0: empty)
+  int key[6];
+  Variant v;
+  int splits;
+};
+
 struct UmmaPlan {
   sfb_desc d;
+  PickedVariant picked[4];
+  unsigned next_picked;
   Layout l;
   int num_sms;
   int es;
@@ -1033,8 +1041,8 @@ void umma_plan_destroy(UmmaPlan* p) {
 // max_splits > 1: the caller can take partial products, so a problem with few tiles may cut its reduction
 // (k_atoms 128-byte atoms long) into *splits ranges.  CTA pairs on 256 x 256 tiles need half the operand
 // traffic per flop of single 128 x 128 tiles, so they are preferred as soon as pairs x ranges fill the SMs.
-static Variant pick_variant(const UmmaPlan* pl, int m_units, int N, bool dims_chunk_aligned, bool apply, int k_atoms,
-                            int max_splits = 1, int* splits = nullptr) {
+static Variant estimate_variant(const UmmaPlan* pl, int m_units, int N, bool dims_chunk_aligned, bool apply, int k_atoms,
+                                int max_splits, int* splits) {
   Variant v;
   v.split = false;
   if (splits != nullptr) *splits = 1;
@@ -1125,6 +1133,22 @@ static Variant pick_variant(const UmmaPlan* pl, int m_units, int N, bool dims_ch
   // per-stage barrier round trip, not the number of TMA instructions, is what costs
   v.ka = (v.cg == 2 || v.bn == 128) ? STAGE_ATOMS : 1;
   return v;
+}
+
+// The same, estimated once per shape (some 50 candidates): a context has a forward and an update, and a shard's.
+static Variant pick_variant(UmmaPlan* pl, int m_units, int N, bool dims_chunk_aligned, bool apply, int k_atoms,
+                            int max_splits = 1, int* splits = nullptr) {
+  const PickedVariant want = {{m_units, N, dims_chunk_aligned, apply, k_atoms, splits != nullptr ? max_splits : 0}, Variant(), 1};
+  for (const PickedVariant& p : pl->picked)
+    if (p.splits > 0 && memcmp(p.key, want.key, sizeof(p.key)) == 0) {
+      if (splits != nullptr) *splits = p.splits;
+      return p.v;
+    }
+  PickedVariant& slot = pl->picked[pl->next_picked++ & 3];
+  slot = want;
+  slot.v = estimate_variant(pl, m_units, N, dims_chunk_aligned, apply, k_atoms, max_splits, splits);
+  if (splits != nullptr) slot.splits = *splits;
+  return slot.v;
 }
 
 // Z rows (fp32, through `z`) = A rows (through `a`, the path's value type) times W^T.
