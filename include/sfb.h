@@ -111,8 +111,10 @@ enum {
 /* bits of the device status word */
 enum {
   SFB_DEV_BAD_LABEL = 1,    /* MLR label outside [0, J): that sample's u is written as zeros */
-  SFB_DEV_BAD_INDEX = 2,    /* CSR column >= D or not strictly ascending: that entry is skipped */
-  SFB_DEV_BAD_HEADER = 4,   /* SF buffer header does not match the descriptor: apply leaves W untouched */
+  SFB_DEV_BAD_INDEX = 2,    /* CSR column >= D or not above its predecessor's: that entry is skipped (a column that
+                               passes twice, as in 5, 3, 5, counts with the sum of its values) */
+  SFB_DEV_BAD_HEADER = 4,   /* SF buffer header does not match the descriptor: apply leaves W untouched and reads
+                               nothing behind the header that could lead out of the buffer */
   SFB_DEV_CAPACITY = 8,     /* a worker's nonzeros exceed cap_p: that stream's codes are truncated */
   SFB_DEV_TIMEOUT = 16      /* a bounded device-side wait (about a second) ran out: the launch completed, its
                                output is not to be used; the context stays usable */

@@ -3,11 +3,11 @@
 //   forward:  Z[i][j] = sum_d A[i][d] * W[j][d]      (z_i = W a_i for every sample; Section 2, (P))
 //   apply  :  W[j][d] -= eta * sum_i U[i][j] * V[i][d]  (W <- W - eta * sum_i u_i v_i^T; Section 3)
 //
-// Both are register-blocked shared-memory SGEMMs: 256 threads, a (64*MI) x (64*NI) output tile, a
-// reduction step of 16, operands staged k-major in shared memory so that every inner-loop read is
-// a conflict-free 16-byte load, global loads prefetched into registers one step ahead.  The
-// summation order is fixed (ascending reduction index inside one thread), so results are
-// bit-reproducible run to run.
+// All are register-blocked shared-memory SGEMMs: 256 threads, a 128 x 128 or 64 x 64 output tile, a reduction step of 16,
+// operands staged k-major in shared memory so that every inner-loop read is a conflict-free 16-byte load.  The one-launch
+// forward prefetches a step into registers and transposes it on the way to shared memory; the others bring theirs by
+// asynchronous copies through a ring of stages.  The summation order is fixed (ascending reduction index inside one
+// thread), so results are bit-reproducible run to run and, range for range, the same from all of them.
 #include "common.cuh"
 
 namespace sfb {
@@ -62,8 +62,8 @@ __device__ __forceinline__ void mma_tile(const float (*As)[64 * MI + 4], const f
 }
 
 // ------------------------------------------------------------------------------------------ forward, one launch
-// For the smallest problems, and where the pair difference is formed on the way and not kept (DML factors without v,
-// sfb_loss).  blockIdx.z takes the reduction range [z d_per_range, + d_per_range) and writes its partial products
+// For the shapes that forward_f32_plan gives it, and where the pair difference is formed on the way and not kept (DML
+// factors without v, sfb_loss).  blockIdx.z takes the reduction range [z d_per_range, + d_per_range) and writes its partial products
 // range_stride bytes after the previous range's.
 // Tile rows = samples i (BM = 64*MI), tile columns = classes j (BN = 64*NI), reduction over d.
 // Both operands are contiguous along d, so tiles are transposed while being stored to shared memory.
@@ -292,7 +292,7 @@ __global__ void __launch_bounds__(256, 2) sgemm_pipe_kernel(float* W, RowMap u, 
 //                    take 64 contiguous bytes of a row; any D), no transposing pass.  Where the factor v is a copy of the
 //                    sample rows, the blocks of a row of tiles write it from shared memory, each its share of the rows.
 // Bound: the latency of a step's copies (0.9 us for 16 steps of the forward with a block per SM), hence many short
-// ranges.  A step of 100 x 800, K = 160: 98 -> 19 us, of 40 x 15000, K = 800: 312 -> 144, of 300 x 3000, K = 400: 107 -> 69
+// ranges.  A step of 100 x 800, K = 160: 98 -> 19 us, of 40 x 15000, K = 800: 312 -> 132, of 300 x 3000, K = 400: 107 -> 69
 // (64 x 64 tiles without a ring, 128 x 128 tiles in 512-step ranges before).
 constexpr int SMALL_STAGE_FLOATS = 2 * BK * (64 + 4);
 

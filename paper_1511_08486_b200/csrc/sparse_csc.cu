@@ -199,7 +199,7 @@ constexpr int CSC2_WARP_FLOATS = 2 * CSC2_STRIP + CSC2_AB * CSC2_TS;   // entry 
 // A quarter warp takes every fourth entry: one 8-byte read of the strip (four addresses) and one 512-byte read of u per
 // four entries, five wavefronts of shared memory, which bounds this kernel where the codes are dense; the four partial
 // sums meet in three shuffles that leave every lane one row.  Where they are sparse the bound is W's way through the
-// memory and the latency of a column's few steps: 32 rows (not 64), so that 1416 samples fit beside the tiles and W is read
+// memory and the latency of a column's few steps: 32 rows (not 64), so that 1408 samples fit beside the tiles and W is read
 // and written once; the next block's part of W is in flight while this one's entries are summed; a column's last groups
 // are read together; 20 warps (16: 5 % 488 us; 24 or 32, with fewer registers: 461 and 464, small problems 10 % slower).
 // 4096 x 10000, K = 1024, against half warps on 64 rows with W loaded when its block begins: 5 % density 514 -> 443 us an

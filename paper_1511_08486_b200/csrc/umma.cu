@@ -903,7 +903,8 @@ struct UmmaPlan {
   const void* fresh_u;
   const void* fresh_v;
   int fresh_K;
-  float* part_ws;               // partial products of a split reduction, [MAX_SPLITS][K][ldp] fp32 (small forward GEMMs only)
+  float* part_ws;               // partial products of a split reduction, [max_splits][K][ldp] fp32 (forward GEMMs of few
+                                // tiles; the compensated path always)
   int ldp;
   // MLR: the factor v is a copy of x that nothing in the factor stage reads, so it runs on a side stream
   // next to the forward GEMM (fork / join by events)
@@ -954,7 +955,7 @@ int umma_plan_create(const sfb_desc& d, const Layout& l, UmmaPlan** out) {
   {   // forward GEMMs whose 128 x 128 tiles do not fill the SMs may split their reduction
     const long long K_ = (long long)d.P * d.B;
     const long long tiles = ((K_ + 127) / 128) * ((d.J + 127) / 128);
-    // the compensated path tunes the count up to 16, within 4 GB of partial buffers
+    // the compensated path tunes the count up to X3_MAX_SPLITS, within 4 GB of partial buffers
     p->max_splits = MAX_SPLITS;
     if (p->x3) {
       const long long one = K_ * p->ldp * 4;
@@ -1037,10 +1038,9 @@ void umma_plan_destroy(UmmaPlan* p) {
   delete p;
 }
 
-// Tile shape and kernel variant for an M x N output (M counted in 128-row units).
-// max_splits > 1: the caller can take partial products, so a problem with few tiles may cut its reduction
-// (k_atoms 128-byte atoms long) into *splits ranges.  CTA pairs on 256 x 256 tiles need half the operand
-// traffic per flop of single 128 x 128 tiles, so they are preferred as soon as pairs x ranges fill the SMs.
+// Tile shape and kernel variant for an M x N output (M counted in 128-row units): the candidate with the least estimated
+// cost.  max_splits > 1: the caller can take partial products, so the reduction (k_atoms 128-byte atoms long) may be cut
+// into *splits ranges, chosen with the shape.
 static Variant estimate_variant(const UmmaPlan* pl, int m_units, int N, bool dims_chunk_aligned, bool apply, int k_atoms,
                                 int max_splits, int* splits) {
   Variant v;
@@ -1051,8 +1051,8 @@ static Variant estimate_variant(const UmmaPlan* pl, int m_units, int N, bool dim
     // kernels run at the rate L2 delivers their operands, so a candidate shape costs the bytes its busiest SM loads:
     //   256 x 128 pair tiles: 48 KB per stage and CTA; the accumulators (main, corrections) of two tiles fill the
     //     512 columns of tensor memory, so a tile's epilogue overlaps the MMAs of the next;
-    //   256 x 256 pair tiles: 64 KB per stage for twice the work, but one accumulator set: the epilogue is exposed
-    //     (about 8 stages' worth per tile, measured at 4096 x 10000, K = 1024);
+    //   256 x 256 pair tiles: 64 KB per stage for twice the work, but one accumulator set: the next tile's MMAs wait
+    //     until the epilogue has read it (about a stage's worth; the stores run beside them);
     //   128 x 128 single tiles (64 KB per stage): for a single row unit, or when an odd number of row units would
     //     leave the last pair half empty and waves of singles are shorter (an apply of 600 rows).
     // With a split reduction (forward; ranges added in fp32 by the finishing pass) the number of ranges is chosen
