@@ -51,6 +51,7 @@ struct sfb_ctx {
   // (bf16 [value | remainder] per 32 columns, as many bytes as W), rebuilt before a forward pass when stale.
   __nv_bfloat16* w_shadow;
   const void* shadow_of;    // W pointer the shadow currently mirrors (nullptr = stale)
+  F32Tc* f32_tc;            // fp32 path, large dense problems: the contractions on the tensor cores (else nullptr)
   UmmaPlan* umma;           // tensor-core plan (tensor maps), TF32 / BF16 paths
   int64_t launches;
   bool profiling;
@@ -204,6 +205,21 @@ int factors_into(sfb_ctx* c, const void* W, const void* X, const sfb_aux* aux, R
     const RowMap part = caller_rows(c->f32_part, c->ldp, d.B, 4);
     const long long sstride = (long long)c->K * c->ldp * 4;
     int ks = 1;
+    if (c->f32_tc != nullptr) {
+      RowMap z;
+      long long zstride = 0;
+      ACC(f32tc_forward(c->f32_tc, c->stream, Wf, reinterpret_cast<const float*>(X), Xb, K, u, v, c->dev_status, &z, &ks,
+                        &zstride));
+      FinishExtra x = extra;
+      x.take_bad = f32tc_bad_forward(c->f32_tc);
+      if (for_apply) x.give_bad = f32tc_bad_apply(c->f32_tc);
+      if (for_apply && x.nonzero == nullptr) x.nonzero = f32tc_flags(c->f32_tc);
+      if (d.model == SFB_MLR)
+        ACC(launch_finish_mlr(c->stream, z, u, aux->labels, K, d.J, c->dev_status, ks, zstride,
+                              reinterpret_cast<float*>(aux->dual), aux->sdca_step, CorrOut(), x));
+      else ACC(launch_finish_dml(c->stream, z, u, aux->similar, d.margin, K, d.J, ks, zstride, c->dml_active, CorrOut(), x));
+      return SFB_OK;
+    }
     // a shard of the workers stays within the partial buffers and transposed copies of the whole
     const ForwardF32Plan plan = K == c->K ? c->f32_plan : forward_f32_plan(K, d.J, d.D, Xb != nullptr, c->f32_plan.ks,
                                                                            c->f32_nn_ws != nullptr);
@@ -311,12 +327,13 @@ int sfb_create(const sfb_desc* desc, void* cuda_stream, sfb_ctx** out) {
     c->f32_plan = forward_f32_plan(c->K, desc->J, desc->D, desc->model == SFB_DML, FORWARD_F32_MAX_SPLITS, nn_bytes <= (2LL << 30));
     const int ks = c->f32_plan.ks;
     c->ldp = (desc->J + 3) & ~3;
-    if (ks > 1) ok = cudaMalloc(&c->f32_part, (size_t)ks * c->K * c->ldp * 4) == cudaSuccess;
+    if (f32tc_pays(c->K, desc->J, desc->D, desc->model == SFB_DML, c->f32_plan.us)) ok = f32tc_create(*desc, &c->f32_tc) == SFB_OK;
+    if (ok && c->f32_tc == nullptr && ks > 1) ok = cudaMalloc(&c->f32_part, (size_t)ks * c->K * c->ldp * 4) == cudaSuccess;
     if (ok && desc->model == SFB_DML) {
       ok = cudaMalloc(&c->dml_active, (size_t)c->K) == cudaSuccess;
       if (ok) ok = cudaMalloc(&c->dml_idx, ((size_t)c->K + 1) * 4) == cudaSuccess;
     }
-    if (ok && c->f32_plan.route == F32_TRANSPOSED) ok = cudaMalloc(&c->f32_nn_ws, (size_t)nn_bytes) == cudaSuccess;
+    if (ok && c->f32_tc == nullptr && c->f32_plan.route == F32_TRANSPOSED) ok = cudaMalloc(&c->f32_nn_ws, (size_t)nn_bytes) == cudaSuccess;
   }
   if (ok) {
     if (cudaStreamCreateWithFlags(&c->aux, cudaStreamNonBlocking) == cudaSuccess) {
@@ -365,6 +382,7 @@ int sfb_destroy(sfb_ctx* c) {
     cudaStreamDestroy(c->aux);
   }
   if (c->umma) umma_plan_destroy(c->umma);
+  f32tc_destroy(c->f32_tc);
   if (c->prof_have_events)
     for (int i = 0; i < 128; ++i)
       for (int e = 0; e < 3; ++e) cudaEventDestroy(c->prof_ev[i][e]);
@@ -590,6 +608,7 @@ static int apply_from(sfb_ctx* c, void* W, const void* sf_buf, float eta, int K,
   if (check) hc = make_check(sf_buf, d, c->l, c->dev_status);
   // (the compensated path has a kernel in front of its GEMM that can do the check)
   const bool with_split = !d.v_sparse && d.path == SFB_PATH_TF32X3;
+  if (check && c->f32_tc != nullptr) hc.clear = f32tc_bad_apply(c->f32_tc);
   if (check && !with_split) ACC(launch_check_header(c->stream, hc));
   if (d.v_sparse && d.path == SFB_PATH_F32 && c->csc_ws != nullptr) {
     if (!csc_built)
@@ -608,6 +627,17 @@ static int apply_from(sfb_ctx* c, void* W, const void* sf_buf, float eta, int K,
     ACC(umma_apply(c->umma, c->stream, W, has_shadow(c) ? c->w_shadow : nullptr, stream_u(c, sf_buf), dense_codes(c), eta,
                    K, c->dev_status));
     if (!mirrored) c->shadow_of = nullptr;
+  } else if (c->f32_tc != nullptr) {
+    // the rows with nonzero u, in order: a compacted buffer's kept slots, or a list made from the flags of the step's
+    // finishing pass (a buffer of the caller's: from its rows)
+    const RowMap u = stream_u(c, sf_buf);
+    const bool listed = active_rows && c->dml_active != nullptr;
+    if (d.compact) ACC(launch_kept_rows(c->stream, sf_buf, d.B, K / d.B, c->kept_idx, c->kept_idx + c->K));
+    else ACC(f32tc_list(c->f32_tc, c->stream, u, K, !check, listed ? c->dml_active : nullptr, listed ? c->dml_idx + c->K : nullptr));
+    const int* idx = d.compact ? c->kept_idx : nullptr;
+    const int* n_idx = d.compact ? c->kept_idx + c->K : nullptr;
+    ACC(f32tc_apply(c->f32_tc, c->stream, reinterpret_cast<float*>(W), u, stream_v(c, sf_buf), K, eta, c->dev_status, idx, n_idx,
+                    !check, idx, n_idx));
   } else if (d.path == SFB_PATH_F32) {
     const int* idx = nullptr;
     const int* n_idx = nullptr;
@@ -751,7 +781,7 @@ int sfb_step(sfb_ctx* c, void* W, const void* X, const sfb_aux* aux, void* sf_bu
   if (!d.v_sparse) extra.commit = commit;
   if (d.compact) extra.nonzero = compact_flags(c->compact_ws);
   r = factors_into(c, W, X, aux, stream_u(c, sf_buf), d.v_sparse ? RowMap() : stream_v(c, sf_buf), codes, 0,
-                   d.path == SFB_PATH_TF32X3 && !d.compact && K == c->K, extra, defer_v);
+                   c->f32_tc != nullptr || (d.path == SFB_PATH_TF32X3 && !d.compact && K == c->K), extra, defer_v);
   if (forked && cudaStreamWaitEvent(c->stream, c->aux_join, 0) != cudaSuccess) return SFB_ERR_CUDA;
   if (r < 0) return r;   // (umma_forward has joined its side stream)
   // pairs whose u came out as zero are dropped from the message before it is "sent" (and applied)

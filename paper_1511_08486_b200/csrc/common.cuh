@@ -117,7 +117,8 @@ struct HeaderCheck {
   const char* buf;
   HeaderImage h;
   int* dev_status;
-  __host__ __device__ HeaderCheck() : buf(nullptr), h(), dev_status(nullptr) {}
+  int* clear;   // optional: a word to clear on the way
+  __host__ __device__ HeaderCheck() : buf(nullptr), h(), dev_status(nullptr), clear(nullptr) {}
 };
 #ifdef __CUDACC__
 // Has the check that precedes this kernel refused the buffer it was given (refused: the status word, or nullptr = not
@@ -131,6 +132,7 @@ __device__ __forceinline__ void check_header(const HeaderCheck& c, int t) {
   const uint32_t* ref = reinterpret_cast<const uint32_t*>(&c.h);
   bool ok = true;
   if (t < 17 && t != 7) ok = (w[t] == ref[t]);   // word 7 is the clock: any value is accepted
+  if (t == 0 && c.clear != nullptr) *c.clear = 0;
   if (t == 2) ok = ((w[t] & ~2u) == ref[t]);      // flag bit 1 (compacted) may be set or not
   if (!__all_sync(0xffffffffu, ok) && t == 0) atomicOr(c.dev_status, SFB_DEV_BAD_HEADER);
 }
@@ -191,7 +193,9 @@ struct FinishExtra {
   int cols;
   bool next_early;   // see chain_next
   int header_blocks; // blocks in front of the rows' that write the header (set by the launcher)
-  FinishExtra() : nonzero(nullptr), src(), dst(), cols(0), next_early(false), header_blocks(0) {}
+  int* take_bad;     // a word to clear, and (give_bad) another that gets its value first
+  int* give_bad;
+  FinishExtra() : nonzero(nullptr), src(), dst(), cols(0), next_early(false), header_blocks(0), take_bad(nullptr), give_bad(nullptr) {}
 };
 
 #ifdef __CUDACC__
@@ -277,9 +281,13 @@ enum F32Route { F32_IN_PLACE, F32_SMALL, F32_TRANSPOSED };
 struct ForwardF32Plan {
   F32Route route;
   int ks;
+  double us;   // estimated time
 };
 constexpr int FORWARD_F32_MAX_SPLITS = 32;
 ForwardF32Plan forward_f32_plan(int K, int J, int D, bool pair, int max_ks, bool transposed_ok);
+// The products only, in exactly ks ranges (range s to z + s * split_stride; ranges beyond D: zeros), if *only_if != 0.
+int launch_forward_f32_if(cudaStream_t s, const float* W, const float* X, const float* Xb, int K, int J, int D, RowMap z,
+                          long long split_stride, int ks, const int* only_if);
 int launch_forward_f32_small(cudaStream_t s, const float* W, RowMap src, RowMap copy, int K, int J, int D, RowMap z,
                              RowMap part, long long split_stride, int ks, int* nsplit_out);
 long long forward_f32_nn_workspace_floats(int K, int J, int D);
@@ -288,7 +296,9 @@ int launch_forward_f32_nn(cudaStream_t s, const float* W, RowMap src, RowMap cop
 
 // W[j][d] -= eta * sum_{i<K} U[i][j] * V[i][d] on fp32 CUDA cores (fixed summation order).
 int launch_apply_f32(cudaStream_t s, float* W, RowMap u, RowMap v, int K, int J, int D, float eta,
-                     const int* dev_status, const int* row_idx = nullptr, const int* n_rows = nullptr);
+                     const int* dev_status, const int* row_idx = nullptr, const int* n_rows = nullptr,
+                     const int* only_if = nullptr);
+// only_if (optional, device): nothing is done where it is 0.
 // row_idx / n_rows (optional, device): apply only the factor rows row_idx[0 .. *n_rows), in that order, instead of
 // rows 0 .. K-1 (rows that are known to be all zeros can be left out: the result is bit-identical).
 
@@ -340,6 +350,8 @@ int launch_compact(cudaStream_t s, void* sf_buf, const sfb_desc& d, const Layout
                    bool flags_ready = false);   // n_workers > 0: only those workers' streams (a process's shard)
 // flags_ready: the finishing pass that wrote the u rows left its flags (FinishExtra::nonzero) in compact_flags(workspace).
 uint8_t* compact_flags(void* workspace);
+// flags[i] = 1 where row i of u (J values) holds a nonzero one.
+int launch_row_nonzero(cudaStream_t s, RowMap u, int K, int J, uint8_t* flags);
 // Rebuilds the directory's pair counts (and the header flag) from streams that arrived already compacted.
 int launch_count_pairs(cudaStream_t s, void* sf_buf, const sfb_desc& d, const Layout& l, void* workspace);
 int launch_kept_rows(cudaStream_t s, const void* sf_buf, int B, int workers, int* idx, int* n_out);

@@ -173,6 +173,11 @@ int launch_count_pairs(cudaStream_t s, void* sf_buf, const sfb_desc& d, const La
   return cudaGetLastError() == cudaSuccess ? 2 : SFB_ERR_CUDA;
 }
 
+int launch_row_nonzero(cudaStream_t s, RowMap u, int K, int J, uint8_t* flags) {
+  launch_chained(row_nonzero_kernel, (K + 7) / 8, 256, 0, s, u, K, J, flags);
+  return cudaGetLastError() == cudaSuccess ? 1 : SFB_ERR_CUDA;
+}
+
 // first_worker / n_workers: compact only the streams of those workers (n_workers = 0: all P).  Worker indices
 // inside the kernels are relative to first_worker: streams, directory entries, flags, slots and counts alike
 // (counts[p] of the workspace belongs to worker first_worker + p).

@@ -101,6 +101,10 @@ __device__ __forceinline__ void copy_unit(const RowMap& src, const RowMap& dst, 
 // row i of the copy.  (In the block of a row they would be on the pass's critical path, and with many workers the longest
 // part of it: 4096 workers of one sample, 64 x 512 in tf32: 77.9 us a step, 53.2 with blocks of their own.)
 __device__ __forceinline__ bool header_block(const FinishExtra& x) {
+  if (x.take_bad != nullptr && blockIdx.x == 0 && threadIdx.x == 0) {
+    if (x.give_bad != nullptr) *x.give_bad = *x.take_bad;
+    *x.take_bad = 0;
+  }
   if ((int)blockIdx.x >= x.header_blocks) return false;
   write_header(x.commit, blockIdx.x * blockDim.x + threadIdx.x, x.header_blocks * blockDim.x);
   return true;

@@ -71,8 +71,10 @@ __device__ __forceinline__ void mma_tile(const float (*As)[64 * MI + 4], const f
 template <int MI, int NI, bool PAIR>
 __global__ void __launch_bounds__(256, MI == 1 ? 3 : 2) forward_f32_kernel(const float* W, const float* X,
                                                           const float* Xb, int K, int J, int D,
-                                                          RowMap z, RowMap v, int d_per_range, long long range_stride) {
+                                                          RowMap z, RowMap v, int d_per_range, long long range_stride,
+                                                          const int* only_if) {
   chain_wait();
+  if (only_if != nullptr && *only_if == 0) return;
   constexpr int BM = 64 * MI, BN = 64 * NI;
   __shared__ __align__(16) float As[BK][BM + 4];
   __shared__ __align__(16) float Bs[BK][BN + 4];
@@ -185,8 +187,9 @@ template <int OUT>
 __global__ void __launch_bounds__(256, 2) sgemm_pipe_kernel(float* W, RowMap u, RowMap v, int K, int J,
                                                          int D, float eta, const int* dev_status,
                                                          RowMap z, int k_per_range, long long range_stride,
-                                                         const int* row_idx, const int* n_rows) {
+                                                         const int* row_idx, const int* n_rows, const int* only_if) {
   chain_wait();
+  if (OUT == 0 && only_if != nullptr && *only_if == 0) return;
   constexpr int BM = 128, BN = 128;
   extern __shared__ __align__(16) float ring[];
   if (OUT == 0 && dev_status != nullptr && (*dev_status & SFB_DEV_BAD_HEADER)) return;
@@ -312,6 +315,7 @@ struct SmallArgs {
   long long range_stride;
   const int* row_idx;       // OUT 0, optional: the factor rows to take
   const int* n_rows;
+  const int* only_if;       // OUT 0, optional: do nothing where this is 0
 };
 
 template <int OUT>
@@ -321,6 +325,7 @@ __global__ void __launch_bounds__(256, 4) sgemm_small_kernel(const __grid_consta
   __shared__ __align__(16) float ring[PIPE * SMALL_STAGE_FLOATS];
   __shared__ long long a_off[OUT == 1 ? BT : 1];   // byte offset of the tile's sample rows, -1: no such row
   __shared__ long long c_off[OUT == 1 ? BT : 1];   // ... and of their copies
+  if (OUT == 0 && p.only_if != nullptr && *p.only_if == 0) return;
   if (OUT == 0 && p.dev_status != nullptr && (*p.dev_status & SFB_DEV_BAD_HEADER)) return;
   const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15, lane = tid & 31, warp = tid >> 5;
   const int nt = (p.N + BT - 1) / BT;            // tiles one after the other in grid.x: M has no limit of grid.y
@@ -486,10 +491,9 @@ __global__ void __launch_bounds__(256) transpose_rows_vec_kernel(TransposeJob j0
 //   - for reductions of four stages or less, which would not fill the ring (10 x 64, K = 4096: 5.7 -> 5.1 us);
 //   - for pairs also where the difference, formed on the way, would cost more as a pass of its own.
 ForwardF32Plan forward_f32_plan(int K, int J, int D, bool pair, int max_ks, bool transposed_ok) {
-  if (step_small_fits(K, J, D)) return {F32_IN_PLACE, 1};   // (the single-launch step repeats these sums in this order)
+  if (step_small_fits(K, J, D)) return {F32_IN_PLACE, 1, 0.0};   // (the single-launch step repeats these sums in this order)
   const double fma_us = 128 * 1900.0;
-  ForwardF32Plan best = {F32_SMALL, 1};
-  double best_us = -1;
+  ForwardF32Plan best = {F32_SMALL, 1, -1.0};
   auto consider = [&](F32Route route, int tile, double rate, double step_us, double before) {
     const double tiles = (double)((K + tile - 1) / tile) * ((J + tile - 1) / tile);
     for (int ks = 1; ks <= max_ks && (ks == 1 || D / ks >= 64); ++ks) {
@@ -497,10 +501,7 @@ ForwardF32Plan forward_f32_plan(int K, int J, int D, bool pair, int max_ks, bool
       const double per_sm = (double)(long long)((tiles * ks + 147) / 148);
       const double work = per_sm * tile * tile * per / (fma_us * rate), chain = per / 16.0 * step_us;
       const double us = before + (work > chain ? work : chain) + (ks > 1 ? ks * (double)J * K * 8 / 6e6 : 0.0);
-      if (best_us < 0 || us < best_us) {
-        best_us = us;
-        best = {route, ks};
-      }
+      if (best.us < 0 || us < best.us) best = {route, ks, us};
     }
   };
   consider(F32_SMALL, 64, 0.40, 0.9, 0.0);
@@ -521,7 +522,7 @@ ForwardF32Plan forward_f32_plan(int K, int J, int D, bool pair, int max_ks, bool
     const double f = (double)((t64 + 147) / 148) * (0.45 + 0.70 * steps), c = 0.9 * steps;
     in_place_us = 0.5 + odd * (f > c ? f : c);
   }
-  if (in_place_us < small_us || (D <= 4 * BK && t64 <= 296)) return {F32_IN_PLACE, 1};
+  if (in_place_us < small_us || (D <= 4 * BK && t64 <= 296)) return {F32_IN_PLACE, 1, in_place_us < best.us ? in_place_us : best.us};
   return best;
 }
 
@@ -532,14 +533,11 @@ static int range_length(int D, int* ks) {
   return per;
 }
 
-int launch_forward_f32(cudaStream_t s, const float* W, const float* X, const float* Xb, int K, int J, int D, RowMap z,
-                       RowMap v, RowMap part, long long split_stride, int ks, int* nsplit_out) {
-  const int per = range_length(D, &ks);
-  if (ks > 1) z = part;
-  if (nsplit_out != nullptr) *nsplit_out = ks;
+static int forward_in_place(cudaStream_t s, const float* W, const float* X, const float* Xb, int K, int J, int D, RowMap z,
+                            RowMap v, int per, long long split_stride, int ks, const int* only_if) {
   const int large = ((J + 127) / 128) * ((K + 127) / 128), small = ((J + 63) / 64) * ((K + 63) / 64);
   auto go = [&](auto kernel, int tiles) {
-    launch_chained(kernel, dim3(tiles, 1, ks), 256, 0, s, W, X, Xb, K, J, D, z, v, per, split_stride);
+    launch_chained(kernel, dim3(tiles, 1, ks), 256, 0, s, W, X, Xb, K, J, D, z, v, per, split_stride, only_if);
   };
   if (J > 64 && (long long)large * ks >= F32_MIN_LARGE_TILES) {
     if (Xb != nullptr) go(forward_f32_kernel<2, 2, true>, large);
@@ -549,6 +547,19 @@ int launch_forward_f32(cudaStream_t s, const float* W, const float* X, const flo
     else go(forward_f32_kernel<1, 1, false>, small);
   }
   return cudaGetLastError() == cudaSuccess ? 1 : SFB_ERR_CUDA;
+}
+
+int launch_forward_f32(cudaStream_t s, const float* W, const float* X, const float* Xb, int K, int J, int D, RowMap z,
+                       RowMap v, RowMap part, long long split_stride, int ks, int* nsplit_out) {
+  const int per = range_length(D, &ks);
+  if (nsplit_out != nullptr) *nsplit_out = ks;
+  return forward_in_place(s, W, X, Xb, K, J, D, ks > 1 ? part : z, v, per, split_stride, ks, nullptr);
+}
+
+int launch_forward_f32_if(cudaStream_t s, const float* W, const float* X, const float* Xb, int K, int J, int D, RowMap z,
+                          long long split_stride, int ks, const int* only_if) {
+  const int per = ((D + ks - 1) / ks + BK - 1) / BK * BK;
+  return forward_in_place(s, W, X, Xb, K, J, D, z, RowMap(), per, split_stride, ks, only_if);
 }
 
 int launch_forward_f32_small(cudaStream_t s, const float* W, RowMap src, RowMap copy, int K, int J, int D, RowMap z,
@@ -566,7 +577,7 @@ int launch_forward_f32_small(cudaStream_t s, const float* W, RowMap src, RowMap 
 }
 
 int launch_apply_f32(cudaStream_t s, float* W, RowMap u, RowMap v, int K, int J, int D, float eta,
-                     const int* dev_status, const int* row_idx, const int* n_rows) {
+                     const int* dev_status, const int* row_idx, const int* n_rows, const int* only_if) {
   const long long big_tiles = (long long)((J + 127) / 128) * ((D + 127) / 128);
   if (big_tiles >= 148) {
     dim3 grid((D + 127) / 128, (J + 127) / 128);
@@ -574,7 +585,7 @@ int launch_apply_f32(cudaStream_t s, float* W, RowMap u, RowMap v, int K, int J,
     if (!set_up_device(attr_once, [] { return allow_smem(sgemm_pipe_kernel<0>, PIPE * PIPE_STAGE_FLOATS * 4); }))
       return SFB_ERR_CUDA;
     launch_chained(sgemm_pipe_kernel<0>, grid, 256, PIPE * PIPE_STAGE_FLOATS * 4, s, W, u, v, K, J, D, eta, dev_status, RowMap(), 0, 0,
-                                                                         row_idx, n_rows);
+                                                                         row_idx, n_rows, only_if);
   } else {
     SmallArgs p = {};
     p.W = W;
@@ -582,7 +593,7 @@ int launch_apply_f32(cudaStream_t s, float* W, RowMap u, RowMap v, int K, int J,
     p.K = K; p.M = J; p.N = D; p.ldw = D;
     p.eta = eta;
     p.dev_status = dev_status;
-    p.row_idx = row_idx; p.n_rows = n_rows;
+    p.row_idx = row_idx; p.n_rows = n_rows; p.only_if = only_if;
     launch_chained(sgemm_small_kernel<0>, ((D + 63) / 64) * ((J + 63) / 64), 256, 0, s, p);
   }
   return cudaGetLastError() == cudaSuccess ? 1 : SFB_ERR_CUDA;
@@ -631,7 +642,7 @@ int launch_forward_f32_nn(cudaStream_t s, const float* W, RowMap src, RowMap cop
   // rows of the output tile = samples (M = K), columns = classes (N = J), reduction over the D features
   dim3 grid((J + 127) / 128, (K + 127) / 128, ks);
   launch_chained(sgemm_pipe_kernel<1>, grid, 256, PIPE * PIPE_STAGE_FLOATS * 4, s, nullptr, a, b, D, K, ldj, 0.f, nullptr,
-                                                                       ks > 1 ? part : z, per, split_stride, nullptr, nullptr);
+                                                                       ks > 1 ? part : z, per, split_stride, nullptr, nullptr, nullptr);
   return cudaGetLastError() == cudaSuccess ? transposes + 1 : SFB_ERR_CUDA;
 }
 

@@ -122,6 +122,11 @@ __device__ __forceinline__ uint32_t map_to_cta(uint32_t smem_addr, uint32_t rank
 __device__ __forceinline__ void mbar_arrive_cluster(uint32_t bar_cluster_addr) {
   asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar_cluster_addr) : "memory");
 }
+// The same without release semantics: for a signal that says "I have read" and has no memory of its own to publish.  (The
+// release waits for every earlier store of the thread, at cluster scope: 2000 clocks and more behind an epilogue's stores.)
+__device__ __forceinline__ void mbar_arrive_cluster_relaxed(uint32_t bar_cluster_addr) {
+  asm volatile("mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar_cluster_addr) : "memory");
+}
 
 // ---- tcgen05: tensor memory ------------------------------------------------------------------------
 // CG = 1: one CTA owns the MMA.  CG = 2: a pair of CTAs (a cluster of two SMs) shares one MMA of
@@ -198,6 +203,18 @@ __device__ __forceinline__ void mma_commit(uint64_t* bar) {
   else
     asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar))
                  : "memory");
+}
+// The same barrier in both CTAs of a pair, by one instruction.
+__device__ __forceinline__ void mma_commit_pair(uint64_t* bar) {
+  asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;"
+               ::"r"(smem_u32(bar)), "h"((uint16_t)3) : "memory");
+}
+// One lane of a converged warp.  Code behind it keeps warp-uniform values in uniform registers, which tcgen05.mma takes its
+// operands from: an instruction every 39 clocks, against 53 (and more with computed descriptors) behind `lane == 0`.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile("{\n\t.reg .pred q;\n\telect.sync _|q, 0xffffffff;\n\tselp.u32 %0, 1, 0, q;\n\t}" : "=r"(p));
+  return p != 0;
 }
 // 32 lanes x 32 consecutive 32-bit columns: thread t of the warp gets lane (base + t), columns c..c+31.
 __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {

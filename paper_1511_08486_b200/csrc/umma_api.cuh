@@ -50,4 +50,31 @@ void umma_drop_corr(UmmaPlan* p);
 int umma_apply(UmmaPlan* p, cudaStream_t s, void* W, __nv_bfloat16* w_shadow, RowMap u_rows, RowMap v_rows, float eta,
                int K, const int* dev_status, const void* directory = nullptr, const HeaderCheck* check = nullptr);
 
+// fp32 path, large dense problems: the two contractions on the tensor cores, each fp32 operand as three bf16 parts
+// (umma_f32.cu).
+struct F32Tc;
+// Is a whole step estimated to be faster than on the CUDA cores, whose forward takes cores_forward_us?  pair: DML.
+bool f32tc_pays(int K, int J, int D, bool pair, double cores_forward_us);
+// *out = nullptr with SFB_OK: no room for the workspace, the CUDA cores do it.
+int f32tc_create(const sfb_desc& d, F32Tc** out);
+void f32tc_destroy(F32Tc* t);
+// Products of K samples (X, or X - Xb) with W, as `nsplit` partial products of rows *z (which are u itself, or the
+// workspace), and the samples (differences) into v where v.base != nullptr.
+int f32tc_forward(F32Tc* t, cudaStream_t s, const float* W, const float* X, const float* Xb, int K, RowMap u, RowMap v,
+                  int* dev_status, RowMap* z, int* nsplit, long long* split_stride);
+// Words that say operands hold values which bf16 parts cannot carry (infinities, NaN): the CUDA-core kernels then do the
+// work.  The forward's is cleared by the finishing pass behind it, the update's by what precedes it (the finishing pass
+// of the same step, which hands the forward's on, or the header check).
+int* f32tc_bad_forward(F32Tc* t);
+int* f32tc_bad_apply(F32Tc* t);
+uint8_t* f32tc_flags(F32Tc* t);         // where the finishing pass leaves which u rows are nonzero
+// Lists the rows with nonzero u among the first K: f32tc_apply's when it gets no list of its own.
+// active / n_active (optional): how many of these flags are set.
+int f32tc_list(F32Tc* t, cudaStream_t s, RowMap u, int K, bool flags_ready, const uint8_t* active, int* n_active);
+// W -= eta * sum u_i v_i^T over the listed rows, in that order (idx / n_rows, or f32tc_list's).  The sum depends on the listed
+// rows alone, so leaving out zero rows, as a compacted buffer does, changes no bit.
+// v_planes: the forward of the same step made v's planes (all K rows).  core_idx / core_n: the list the CUDA cores get.
+int f32tc_apply(F32Tc* t, cudaStream_t s, float* W, RowMap u, RowMap v, int K, float eta, int* dev_status, const int* idx,
+                const int* n_rows, bool v_planes, const int* core_idx, const int* core_n);
+
 }  // namespace sfb

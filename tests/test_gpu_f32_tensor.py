@@ -1,0 +1,117 @@
+"""The fp32 path of large dense problems, whose products run on the tensor cores as three bf16 parts per operand.
+
+Shapes at the edges of its tiles (256 x 256 and 256 x 128 per CTA pair) and of its chunks of 64 reduction steps, ragged rows, few
+classes and one sample beyond a tile, against the oracle with guard bands; its error against the CUDA cores' own; operands that
+are not finite, which fall back to the CUDA cores for that call only.
+"""
+import numpy as np
+import pytest
+import torch
+
+from oracle import sfb_oracle as orc
+from sfbgen import make_inputs, scaled
+from tests.test_gpu_parity import _workload, check_config
+from tests.util import to_f64
+
+pytestmark = pytest.mark.gpu
+
+# J, D, P, B
+MLR = [(1000, 2003, 8, 100), (257, 5121, 3, 171), (256, 4096, 4, 128), (385, 3333, 5, 103), (129, 8193, 1, 513), (100, 16841, 16, 42), (10, 9174, 10, 254),
+       (3000, 641, 3, 333), (513, 191, 9, 229)]
+DML = [(129, 8193, 1, 513), (600, 2001, 8, 64), (257, 1025, 3, 300), (40, 11625, 14, 85)]
+
+
+def _on_tensor_cores(wl):
+    """Eight launches a step, or nine with the compaction: planes, GEMM and its stand-in, finish, list, planes, GEMM, stand-in."""
+    n = wl.ctx.launch_count()
+    wl.step(0, eta=0.0)
+    return wl.ctx.launch_count() - n >= 8
+
+
+@pytest.mark.parametrize("J,D,P,B", MLR)
+def test_mlr(J, D, P, B):
+    cfg = scaled("C1", J=J, D=D, P=P, B=B, pool=1)
+    wl = _workload(cfg, make_inputs(cfg), "f32")
+    try:
+        assert _on_tensor_cores(wl)
+    finally:
+        wl.close()
+    check_config(cfg, "f32", eta=0.5, steps=2, guard=True)
+
+
+@pytest.mark.parametrize("J,D,P,B", DML)
+def test_dml(J, D, P, B):
+    cfg = scaled("C2", J=J, D=D, P=P, B=B)
+    check_config(cfg, "f32", eta=1e-3, steps=2, guard=True)
+    inputs = make_inputs(cfg)
+    full, comp = _workload(cfg, inputs, "f32"), _workload(dict(cfg, compact=1), inputs, "f32", guard=True)
+    try:
+        assert _on_tensor_cores(full)
+        for t in range(2):
+            full.step(t, eta=1e-3)
+            comp.step(t, eta=1e-3)
+        torch.cuda.synchronize()
+        assert torch.equal(full.W, comp.W) and comp.guards_intact()      # the sums depend on the nonzero pairs alone
+    finally:
+        full.close()
+        comp.close()
+
+
+def test_error_is_below_that_of_fp32_multiply_adds():
+    """u = L d of similar pairs, 300 x 8192: a chain of n fp32 multiply-adds rounds n times, about sqrt(n) 2^-25 of a sum of
+    random signs (8192 / 9 ranges: 9e-7 at worst, 4e-7 measured on the CUDA cores); the chunk sums here are good to 2^-24."""
+    cfg = scaled("C2", J=300, D=8192, P=4, B=96)
+    inputs = make_inputs(cfg)
+    inputs["similar"] = np.ones_like(inputs["similar"])
+    wl = _workload(cfg, inputs, "f32")
+    try:
+        wl.compute_factors(0)
+        assert wl.ctx.status() == 0
+        d = to_f64(wl.V)[:, :8192]
+        assert orc.rel_fro(to_f64(wl.U)[:, :300], d @ inputs["W"].astype(np.float64).T) <= 2.0 ** -22
+    finally:
+        wl.close()
+
+
+@pytest.mark.parametrize("where", ["w", "x", "none"])
+def test_operands_that_are_not_finite(where):
+    """A weight of -inf that meets positive features only is a logit of -inf: class probability 0, everything else finite.  An
+    infinite feature makes its sample's u NaN, and with it W; the next call, on finite values, is again that of a fresh context."""
+    cfg = scaled("C1", J=257, D=2051, P=4, B=128, pool=1)
+    inputs = make_inputs(cfg)
+    wl, fresh = _workload(cfg, inputs, "f32", guard=True), _workload(cfg, inputs, "f32")
+    try:
+        assert _on_tensor_cores(fresh)
+        t = wl.batches[0]
+        x = t["X"].clone()
+        t["X"][:, 7] = t["X"][:, 7].abs() + 0.1
+        W = wl.W.clone()
+        if where == "w":
+            wl.W[31, 7] = -float("inf")
+        elif where == "x":
+            t["X"][100, 9] = float("inf")
+        X64, W64 = to_f64(t["X"]), to_f64(wl.W)
+        wl.step(0, eta=0.25)
+        assert wl.ctx.status() == 0 and wl.guards_intact()
+        h, U, V = orc.unpack(wl.sf_buf.cpu().numpy())
+        with np.errstate(invalid="ignore"):
+            U_or, _ = orc.mlr_factors(W64, X64, t["labels"].cpu().numpy())
+            W_or = W64 - 0.25 * (U_or.T @ X64)
+        assert np.array_equal(np.isnan(U), np.isnan(U_or))
+        ok = np.isfinite(U_or)
+        assert np.linalg.norm((U - U_or)[ok]) <= 1e-5 * np.linalg.norm(U_or[ok])
+        got = to_f64(wl.W)
+        ok = np.isfinite(W_or)
+        assert np.array_equal(np.isfinite(got), ok) and (where == "x") == (not ok.any())
+        if ok.any():
+            assert np.linalg.norm(got[ok] - W_or[ok]) <= 1e-5 * np.linalg.norm(W_or[ok] - W64[ok]) + 2.0 ** -24 * np.linalg.norm(W64[ok])
+        wl.W.copy_(W)
+        t["X"].copy_(x)
+        wl.step(0, eta=0.25)
+        fresh.W.copy_(W)
+        fresh.step(0, eta=0.25)
+        assert wl.ctx.status() == 0
+        assert torch.equal(wl.W, fresh.W) and torch.equal(wl.sf_buf, fresh.sf_buf)
+    finally:
+        wl.close()
+        fresh.close()
