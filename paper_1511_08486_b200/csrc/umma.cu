@@ -177,7 +177,7 @@ umma_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
   float* epi_stage = reinterpret_cast<float*>(tiles + STAGES * STAGE_BYTES);
   SharedCtl* ctl = reinterpret_cast<SharedCtl*>(tiles + STAGES * STAGE_BYTES + EPI_STAGE_BYTES);
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;   // (uniform: see ptx::elect_one)
   chain_next();
 
   const uint32_t rank = (CG == 2) ? ptx::cluster_ctarank() : 0u;   // 0 = the CTA that issues the MMAs
@@ -388,7 +388,7 @@ umma_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
         ok = wait_or_abort(&ctl->full[s], ph, ctl, p.status);
         if (!ok) break;
         ptx::tc_fence_after();
-        if (lane == 0) {
+        if (ptx::elect_one()) {
           const uint32_t a_addr = ptx::smem_u32(tiles + s * STAGE_BYTES);
           const uint32_t b_addr = a_addr + A_STAGE_BYTES;
           if (!APPLY) {
@@ -438,13 +438,14 @@ umma_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
           }
           // (test hook: one lost signal, so that the producer's bounded wait runs out and the abort path is taken)
           const bool lost = p.lose_signal != 0 && cluster_id == 0 && it == 0 && kb == kb_begin;
+          // stage reusable once these MMAs have read it; accumulator complete: in both CTAs of a pair
           if (!lost) {
-            ptx::mma_commit<CG>(&ctl->empty[s]);                   // stage reusable once these MMAs have read it
-            if (CG == 2) ptx::mma_commit_addr<CG>(ptx::map_to_cta(ptx::smem_u32(&ctl->empty[s]), 1));
+            if (CG == 2) ptx::mma_commit_pair(&ctl->empty[s]);
+            else ptx::mma_commit<CG>(&ctl->empty[s]);
           }
-          if (kb == kb_end - 1) {                                  // accumulator complete, in both CTAs
-            ptx::mma_commit<CG>(&ctl->tmem_full[buf]);
-            if (CG == 2) ptx::mma_commit_addr<CG>(ptx::map_to_cta(ptx::smem_u32(&ctl->tmem_full[buf]), 1));
+          if (kb == kb_end - 1) {
+            if (CG == 2) ptx::mma_commit_pair(&ctl->tmem_full[buf]);
+            else ptx::mma_commit<CG>(&ctl->tmem_full[buf]);
           }
         }
         __syncwarp();
@@ -580,7 +581,7 @@ umma_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
         __syncwarp();
         if (lane == 0) {
           if (CG == 1 || rank == 0) ptx::mbar_arrive(&ctl->tmem_empty[buf]);
-          else ptx::mbar_arrive_cluster(ptx::map_to_cta(ptx::smem_u32(&ctl->tmem_empty[buf]), 0));
+          else ptx::mbar_arrive_cluster_relaxed(ptx::map_to_cta(ptx::smem_u32(&ctl->tmem_empty[buf]), 0));
         }
       };
       // Compensated kernels: all of the warp's columns come out of tensor memory first (main accumulator + correction
@@ -679,7 +680,7 @@ umma_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
         __syncwarp();
         if (lane == 0) {   // this warp's part of the accumulator is drained
           if (CG == 1 || rank == 0) ptx::mbar_arrive(&ctl->tmem_empty[buf]);
-          else ptx::mbar_arrive_cluster(ptx::map_to_cta(ptx::smem_u32(&ctl->tmem_empty[buf]), 0));
+          else ptx::mbar_arrive_cluster_relaxed(ptx::map_to_cta(ptx::smem_u32(&ctl->tmem_empty[buf]), 0));
         }
       }
     }

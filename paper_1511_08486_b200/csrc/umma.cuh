@@ -119,11 +119,9 @@ __device__ __forceinline__ uint32_t map_to_cta(uint32_t smem_addr, uint32_t rank
   asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(smem_addr), "r"(rank));
   return r;
 }
-__device__ __forceinline__ void mbar_arrive_cluster(uint32_t bar_cluster_addr) {
-  asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar_cluster_addr) : "memory");
-}
-// The same without release semantics: for a signal that says "I have read" and has no memory of its own to publish.  (The
-// release waits for every earlier store of the thread, at cluster scope: 2000 clocks and more behind an epilogue's stores.)
+// Arrival without release semantics, on a barrier of any CTA of the cluster: for a signal that says "I have read" and has
+// no memory of its own to publish.  (A release waits for every earlier store of the thread, at cluster scope: 2000 clocks
+// and more behind an epilogue's stores.)
 __device__ __forceinline__ void mbar_arrive_cluster_relaxed(uint32_t bar_cluster_addr) {
   asm volatile("mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar_cluster_addr) : "memory");
 }
@@ -184,17 +182,6 @@ __device__ __forceinline__ void mma_tf32(uint32_t d_tmem, uint64_t a_desc, uint6
 }
 // Arrives once on `bar` (a barrier of the issuing CTA) when every tcgen05.mma issued so far by this
 // thread has completed.
-// Same, with the barrier given by its address in the cluster's shared window (it may belong to the
-// other CTA of the pair).
-template <int CG>
-__device__ __forceinline__ void mma_commit_addr(uint32_t bar_cluster_addr) {
-  if (CG == 1)
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar_cluster_addr)
-                 : "memory");
-  else
-    asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar_cluster_addr)
-                 : "memory");
-}
 template <int CG>
 __device__ __forceinline__ void mma_commit(uint64_t* bar) {
   if (CG == 1)
