@@ -56,7 +56,7 @@ struct F32Tc;
 // Is a whole step estimated to be faster than on the CUDA cores, whose forward takes cores_forward_us?  pair: DML.
 bool f32tc_pays(int K, int J, int D, bool pair, double cores_forward_us);
 // *out = nullptr with SFB_OK: no room for the workspace, the CUDA cores do it.
-int f32tc_create(const sfb_desc& d, F32Tc** out);
+int f32tc_create(const sfb_desc& d, cudaStream_t s, F32Tc** out);
 void f32tc_destroy(F32Tc* t);
 // Products of K samples (X, or X - Xb) with W, as `nsplit` partial products of rows *z (which are u itself, or the
 // workspace), and the samples (differences) into v where v.base != nullptr.

@@ -682,7 +682,7 @@ bool f32tc_pays(int K, int J, int D, bool pair, double cores_forward_us) {
   return f.us + a.us + planes + 27.0 < cores;
 }
 
-int f32tc_create(const sfb_desc& d, F32Tc** out) {
+int f32tc_create(const sfb_desc& d, cudaStream_t s, F32Tc** out) {
   *out = nullptr;
   const long long K = (long long)d.P * d.B, ldd = pad_to(d.D, 8), ldj = pad_to(d.J, 8), ldp = pad_to(d.J, 4);
   if (encoder() == nullptr) return SFB_OK;
@@ -701,7 +701,7 @@ int f32tc_create(const sfb_desc& d, F32Tc** out) {
   bool ok = cudaMalloc(&t->xp, (size_t)(6 * K * ldd)) == cudaSuccess && cudaMalloc(&t->wp, (size_t)(6 * d.J * ldd)) == cudaSuccess &&
             cudaMalloc(&t->up, (size_t)(6 * K * ldj)) == cudaSuccess && cudaMalloc(&t->flags, (size_t)K) == cudaSuccess &&
             cudaMalloc(&t->idx, (size_t)K * 4) == cudaSuccess && cudaMalloc(&t->words, 256) == cudaSuccess &&
-            cudaMemset(t->words, 0, 256) == cudaSuccess;
+            cudaMemsetAsync(t->words, 0, 256, s) == cudaSuccess;
   if (ok && part > 0) ok = cudaMalloc(&t->part, (size_t)part) == cudaSuccess;
   if (!ok) {   // the CUDA-core route needs none of this
     cudaGetLastError();
