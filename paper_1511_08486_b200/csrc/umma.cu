@@ -259,7 +259,8 @@ umma_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
       if (by_dir)
         while (kp0 < p.P && ctl->nb[kp0] == 0) ++kp0;
       for (int kb = kb_begin; kb < kb_end; ++kb) {
-        ok = wait_or_abort(&ctl->empty[s], ph ^ 1u, ctl, p.status);
+        // (the first round of the ring is free: no wait, which takes 150 clocks even where there is nothing to wait for)
+        ok = issued < STAGES || wait_or_abort(&ctl->empty[s], ph ^ 1u, ctl, p.status);
         if (!ok) break;
         if (lane == 0) {
           uint8_t* a_dst = tiles + s * STAGE_BYTES;
@@ -379,7 +380,7 @@ umma_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
       const int kb_begin = split * k_per_split, kb_end = min(kb_begin + k_per_split, k_blocks);
       const int buf = it % NBUF;
       const uint32_t acc_ph = (uint32_t)(it / NBUF) & 1u;
-      ok = wait_or_abort(&ctl->tmem_empty[buf], acc_ph ^ 1u, ctl, p.status);
+      ok = it < NBUF || wait_or_abort(&ctl->tmem_empty[buf], acc_ph ^ 1u, ctl, p.status);
       if (!ok) break;
       ptx::tc_fence_after();
       const uint32_t d_tmem = tmem_base + buf * ACC_COLS;
@@ -1132,7 +1133,10 @@ static Variant estimate_variant(const UmmaPlan* pl, int m_units, int N, bool dim
   v.fold = v.cg == 2 && dims_chunk_aligned;
   // two 128-byte atoms of reduction per stage wherever three such stages fit in shared memory: the
   // per-stage barrier round trip, not the number of TMA instructions, is what costs
-  v.ka = (v.cg == 2 || v.bn == 128) ? STAGE_ATOMS : 1;
+  // (but in a forward on pairs with fp32 operands, which L2 cannot bring fast enough, six stages of one atom keep more of
+  // the ring on its way: 1000 x 20000, K = 1024 70 -> 61 us, 600 x 10000, K = 2048 48 -> 42; not in an update, whose rows
+  // then come in more and smaller loads: 600 x 10000, K = 2048 61 -> 89 us)
+  v.ka = (v.cg == 2 && pl->es == 4 && !apply) || (v.cg == 1 && v.bn == 256) ? 1 : STAGE_ATOMS;
   return v;
 }
 

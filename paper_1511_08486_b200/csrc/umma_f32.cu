@@ -203,7 +203,8 @@ umma_f32_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
 #pragma unroll
         for (int q = 0; q < 3; ++q) {
           const int plane = q == 0 ? LO : q == 1 ? MID : HI;
-          ok = wait_or_abort(&ctl->empty[s], ph ^ 1u, ctl, p.status);
+          // (the first round of the ring is free: no wait, which takes 150 clocks even where there is nothing to wait for)
+          ok = it * 3 + q < SLOTS || wait_or_abort(&ctl->empty[s], ph ^ 1u, ctl, p.status);
           if (!ok) break;
           if (lane == 0) {
             uint8_t* a_dst = ring + s * SLOT_BYTES;
@@ -240,7 +241,7 @@ umma_f32_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
       const int k_end = min((w.range + 1) * k_per_range, k_chunks);
       for (int k = w.range * k_per_range; k < k_end && ok; ++k, ++it) {
         const int buf = it % BUFS;
-        ok = wait_or_abort(&ctl->acc_empty[buf], ((uint32_t)(it / BUFS) & 1u) ^ 1u, ctl, p.status);
+        ok = it < BUFS || wait_or_abort(&ctl->acc_empty[buf], ((uint32_t)(it / BUFS) & 1u) ^ 1u, ctl, p.status);
         if (!ok) break;
         const uint32_t acc = tmem_base + buf * BN;
         int slot[3];
