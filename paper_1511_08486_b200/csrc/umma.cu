@@ -823,6 +823,7 @@ int dispatch_es(cudaStream_t s, const Variant& v, const CUtensorMap& a, const CU
       if (v.cg == 2 && v.bn == 256) return launch_gemm<4, APPLY, 256, 2, 1, false, 0, true>(s, a, b, w, ac, bc, p, num_sms);
       if (v.cg == 2 && v.fold) return launch_gemm<4, APPLY, 128, 2, 1, true, 0, true>(s, a, b, w, ac, bc, p, num_sms);
       if (v.cg == 2) return launch_gemm<4, APPLY, 128, 2, 1, false, 0, true>(s, a, b, w, ac, bc, p, num_sms);
+      if (v.bn == 64) return launch_gemm<4, APPLY, 64, 1, 1, false, 0, true>(s, a, b, w, ac, bc, p, num_sms);
       return launch_gemm<4, APPLY, 128, 1, 1, false, 0, true>(s, a, b, w, ac, bc, p, num_sms);
     }
     return SFB_ERR_UNSUPPORTED;
@@ -833,6 +834,7 @@ int dispatch_es(cudaStream_t s, const Variant& v, const CUtensorMap& a, const CU
     if (v.ka == 2) return launch_gemm<ES, APPLY, 256, 2, 2, false, EPI>(s, a, b, w, a, b, p, num_sms);
     return launch_gemm<ES, APPLY, 256, 2, 1, false, EPI>(s, a, b, w, a, b, p, num_sms);
   }
+  if (EPI == 0 && v.bn == 64) return launch_gemm<ES, APPLY, 64, 1, 2, false, 0>(s, a, b, w, a, b, p, num_sms);
   if (v.bn == 256) return launch_gemm<ES, APPLY, 256, 1, 1, false, EPI>(s, a, b, w, a, b, p, num_sms);
   if (v.ka == 2) return launch_gemm<ES, APPLY, 128, 1, 2, false, EPI>(s, a, b, w, a, b, p, num_sms);
   return launch_gemm<ES, APPLY, 128, 1, 1, false, EPI>(s, a, b, w, a, b, p, num_sms);
@@ -1042,9 +1044,9 @@ void umma_plan_destroy(UmmaPlan* p) {
 
 // Tile shape and kernel variant for an M x N output (M counted in 128-row units): the candidate with the least estimated
 // cost.  max_splits > 1: the caller can take partial products, so the reduction (k_atoms 128-byte atoms long) may be cut
-// into *splits ranges, chosen with the shape.
+// into *splits ranges, chosen with the shape.  narrow: tiles of 64 columns will do (plain stores or the write-back of W).
 static Variant estimate_variant(const UmmaPlan* pl, int m_units, int N, bool dims_chunk_aligned, bool apply, int k_atoms,
-                                int max_splits, int* splits) {
+                                int max_splits, int* splits, bool narrow) {
   Variant v;
   v.split = false;
   if (splits != nullptr) *splits = 1;
@@ -1099,6 +1101,10 @@ static Variant estimate_variant(const UmmaPlan* pl, int m_units, int N, bool dim
     } else {
       consider(128, 1);
     }
+    // Where half of the SMs take all tiles of 64 columns, their stores and loads are the shorter (257 x 1000, K = 200: 26.9 ->
+    // 22.7 us); not in place of a long update on pairs that fetch an operand's tile by one load (240 x 320, K = 1264: 48.5, 51).
+    const bool long_pairs = apply && v.cg == 2 && dims_chunk_aligned && k_len > 24;
+    if ((apply || ranged) && !long_pairs && 2LL * m_units * ((N + 63) / 64) * (ranged ? *splits : 1) <= pl->num_sms) { v.bn = 64; v.cg = 1; }
     v.fold = v.cg == 2 && dims_chunk_aligned;
     return v;
   }
@@ -1117,6 +1123,7 @@ static Variant estimate_variant(const UmmaPlan* pl, int m_units, int N, bool dim
     const long long tiles = (long long)((m_units + cg - 1) / cg) * ((N + bn - 1) / bn), slots = pl->num_sms / cg;
     for (int ks = 1; ks <= max_splits && (ks == 1 || k_atoms >= 2 * STAGE_ATOMS * ks); ++ks) {
       const int per = (k_atoms + ks - 1) / ks, ranges = (k_atoms + per - 1) / per;
+      if (bn == 64 && 2 * tiles > slots) break;   // (tiles of 64 columns are for problems that leave SMs without work)
       const double waves = (double)((tiles * ranges + slots - 1) / slots), work = per * t_atom;
       const double cost = waves * (work > epi ? work : epi) + epi + 8000.0 +
                           (ks > 1 ? (double)ranges * m_units * BM * N * 8 / 3400 : 0.0);
@@ -1128,8 +1135,16 @@ static Variant estimate_variant(const UmmaPlan* pl, int m_units, int N, bool dim
     }
   };
   consider(128, 1);
+  // an update cannot cut its reduction: narrow tiles give a small one more SMs and a shorter write-back (257 x 1000, K = 200 in
+  // tf32 19.8 -> 17.2 us a step, 512 x 1024, K = 512 in bf16 18.2 -> 16.5)
+  if (apply) consider(64, 1);
   if (N > 128) consider(256, 1);
   if (N > 128 && m_units >= 2) consider(256, 2);
+  // A forward takes tiles of 64 columns where it keeps its ranges (longer ones cost more than narrow tiles give) and half of
+  // the SMs are enough (209 x 1484, K = 130 in tf32 18.1 -> 17.5 us; but 348 x 8720, K = 42 in bf16, 96 tiles, 23.2 -> 24.4).
+  if (!apply && narrow && v.cg == 1 && v.bn == 128 &&
+      2LL * m_units * ((N + 63) / 64) * (splits != nullptr ? *splits : 1) <= pl->num_sms)
+    v.bn = 64;
   v.fold = v.cg == 2 && dims_chunk_aligned;
   // two 128-byte atoms of reduction per stage wherever three such stages fit in shared memory: the
   // per-stage barrier round trip, not the number of TMA instructions, is what costs
@@ -1142,8 +1157,8 @@ static Variant estimate_variant(const UmmaPlan* pl, int m_units, int N, bool dim
 
 // The same, estimated once per shape (some 50 candidates): a context has a forward and an update, and a shard's.
 static Variant pick_variant(UmmaPlan* pl, int m_units, int N, bool dims_chunk_aligned, bool apply, int k_atoms,
-                            int max_splits = 1, int* splits = nullptr) {
-  const PickedVariant want = {{m_units, N, dims_chunk_aligned, apply, k_atoms, splits != nullptr ? max_splits : 0}, Variant(), 1};
+                            int max_splits = 1, int* splits = nullptr, bool narrow = true) {
+  const PickedVariant want = {{m_units, N, dims_chunk_aligned, apply + 2 * narrow, k_atoms, splits != nullptr ? max_splits : 0}, Variant(), 1};
   for (const PickedVariant& p : pl->picked)
     if (p.splits > 0 && memcmp(p.key, want.key, sizeof(p.key)) == 0) {
       if (splits != nullptr) *splits = p.splits;
@@ -1151,7 +1166,7 @@ static Variant pick_variant(UmmaPlan* pl, int m_units, int N, bool dims_chunk_al
     }
   PickedVariant& slot = pl->picked[pl->next_picked++ & 3];
   slot = want;
-  slot.v = estimate_variant(pl, m_units, N, dims_chunk_aligned, apply, k_atoms, max_splits, splits);
+  slot.v = estimate_variant(pl, m_units, N, dims_chunk_aligned, apply, k_atoms, max_splits, splits, narrow);
   if (splits != nullptr) slot.splits = *splits;
   return slot.v;
 }
@@ -1179,7 +1194,8 @@ int umma_forward_rows(UmmaPlan* pl, cudaStream_t s, const void* Wop, RowMap a, R
   const bool may_split = k_splits_out != nullptr && stats == nullptr && max_splits > 1;
   int ks_pick = 1;
   const Variant v = pick_variant(pl, m_units, d.J, (d.D % CH) == 0 && (a.ld % CH) == 0, false, (d.D + CH - 1) / CH,
-                                 may_split ? (max_splits < pl->max_splits ? max_splits : pl->max_splits) : 1, &ks_pick);
+                                 may_split ? (max_splits < pl->max_splits ? max_splits : pl->max_splits) : 1, &ks_pick,
+                                 stats == nullptr);
   p.m_tiles = (m_units + v.cg - 1) / v.cg;
   p.n_tiles = (d.J + v.bn - 1) / v.bn;
   p.k_blocks = (d.D + CH * v.ka - 1) / (CH * v.ka);
