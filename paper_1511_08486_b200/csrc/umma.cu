@@ -1101,10 +1101,12 @@ static Variant estimate_variant(const UmmaPlan* pl, int m_units, int N, bool dim
     } else {
       consider(128, 1);
     }
-    // Where half of the SMs take all tiles of 64 columns, their stores and loads are the shorter (257 x 1000, K = 200: 26.9 ->
-    // 22.7 us); not in place of a long update on pairs that fetch an operand's tile by one load (240 x 320, K = 1264: 48.5, 51).
+    // Where all tiles of 64 columns run at once (in a forward: on half of the SMs), their stores and loads are the shorter:
+    // 257 x 1000, K = 200 26.9 -> 22.7 us a step, 300 x 3000, K = 300 (141 tiles) 33.8 -> 31.1.  Not in place of a long update on
+    // pairs that fetch an operand's tile by one load (240 x 320, K = 1264: 48.5 us against 51).
+    const long long narrow_tiles = (long long)m_units * ((N + 63) / 64) * (ranged ? *splits : 1);
     const bool long_pairs = apply && v.cg == 2 && dims_chunk_aligned && k_len > 24;
-    if ((apply || ranged) && !long_pairs && 2LL * m_units * ((N + 63) / 64) * (ranged ? *splits : 1) <= pl->num_sms) { v.bn = 64; v.cg = 1; }
+    if ((apply || ranged) && !long_pairs && narrow_tiles <= (apply ? pl->num_sms : pl->num_sms / 2)) { v.bn = 64; v.cg = 1; }
     v.fold = v.cg == 2 && dims_chunk_aligned;
     return v;
   }
