@@ -446,8 +446,11 @@ __device__ __forceinline__ void zero_planes(const PlaneJob& j, int r, int c) {
 #pragma unroll
   for (int s = 0; s < 3; ++s) *reinterpret_cast<uint4*>(d + s * j.plane_bytes) = make_uint4(0u, 0u, 0u, 0u);
 }
+// Operands below this bound have products below 2^120: no instruction and no chunk sum overflows (two infinite products of
+// parts with different signs would make a NaN of a sum that is an infinity).
+constexpr float PARTS_BOUND = 0x1p60f;
 // Eight values of source row i at column c: to row r of the planes (put), or only looked at.  False: one of them is not
-// finite, or beyond the range of bf16.
+// finite, or not below PARTS_BOUND.
 __device__ __forceinline__ bool make_planes(const PlaneJob& j, int i, int r, int c, bool put) {
   float x[8];
   load8(j.src.row(i), c, j.C, j.vec, x);
@@ -472,7 +475,7 @@ __device__ __forceinline__ bool make_planes(const PlaneJob& j, int i, int r, int
       const __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
       const uint32_t u = *reinterpret_cast<const uint32_t*>(&h);
       const float ha = __uint_as_float(u << 16), hb = __uint_as_float(u & 0xffff0000u);
-      if (s == HI) fine = fine && fabsf(ha) < INFINITY && fabsf(hb) < INFINITY;
+      if (s == HI) fine = fine && fabsf(ha) < PARTS_BOUND && fabsf(hb) < PARTS_BOUND;
       w[s][q] = u;
       a -= ha; b -= hb;                              // exact: the parts of a value do not overlap
     }

@@ -73,10 +73,11 @@ def test_error_is_below_that_of_fp32_multiply_adds():
         wl.close()
 
 
-@pytest.mark.parametrize("where", ["w", "x", "none"])
+@pytest.mark.parametrize("where", ["w", "x", "big", "none"])
 def test_operands_that_are_not_finite(where):
-    """A weight of -inf that meets positive features only is a logit of -inf: class probability 0, everything else finite.  An
-    infinite feature makes its sample's u NaN, and with it W; the next call, on finite values, is again that of a fresh context."""
+    """Operands that are not finite or so large that products overflow.  A weight of -inf that meets positive features only is a logit of -inf: class probability 0, everything else finite.  An
+    infinite feature makes its sample's u NaN, and with it W; a finite weight whose product overflows is a logit of -inf too (its
+    first two bf16 parts have different signs: their products would be -inf and +inf).  The next call, on finite values, is again that of a fresh context."""
     cfg = scaled("C1", J=257, D=2051, P=4, B=128, pool=1)
     inputs = make_inputs(cfg)
     wl, fresh = _workload(cfg, inputs, "f32", guard=True), _workload(cfg, inputs, "f32")
@@ -88,6 +89,10 @@ def test_operands_that_are_not_finite(where):
         W = wl.W.clone()
         if where == "w":
             wl.W[31, 7] = -float("inf")
+        elif where == "big":
+            t["X"][:, 7] = 2.0 ** 40
+            wl.W[:, 7] = 0.0
+            wl.W[31, 7] = -(2.0 ** 101) * (1 - 2.0 ** -12)
         elif where == "x":
             t["X"][100, 9] = float("inf")
         X64, W64 = to_f64(t["X"]), to_f64(wl.W)
