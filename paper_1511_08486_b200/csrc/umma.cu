@@ -1104,9 +1104,13 @@ static Variant estimate_variant(const UmmaPlan* pl, int m_units, int N, bool dim
     // Where all tiles of 64 columns run at once (in a forward: on half of the SMs), their stores and loads are the shorter:
     // 257 x 1000, K = 200 26.9 -> 22.7 us a step, 300 x 3000, K = 300 (141 tiles) 33.8 -> 31.1.  Not in place of a long update on
     // pairs that fetch an operand's tile by one load (240 x 320, K = 1264: 48.5 us against 51).
+    // In sparse coding an update with long rows, too, leaves half of the SMs to what is launched behind it, the blocks of the
+    // next call's dense code rows above all, a row of shared memory each (with the prox, K = 200-300, on 128 and on 64 columns:
+    // 80 x 9000 37.0 / 40.3 us, 200 x 4000 34.8 / 35.8; 300 x 2500 37.0 / 36.9, 600 x 1500 33.0 / 30.9).
     const long long narrow_tiles = (long long)m_units * ((N + 63) / 64) * (ranged ? *splits : 1);
     const bool long_pairs = apply && v.cg == 2 && dims_chunk_aligned && k_len > 24;
-    if ((apply || ranged) && !long_pairs && narrow_tiles <= (apply ? pl->num_sms : pl->num_sms / 2)) { v.bn = 64; v.cg = 1; }
+    const int most = apply && (pl->d.model != SFB_SC || N <= 2560) ? pl->num_sms : pl->num_sms / 2;
+    if ((apply || ranged) && !long_pairs && narrow_tiles <= most) { v.bn = 64; v.cg = 1; }
     v.fold = v.cg == 2 && dims_chunk_aligned;
     return v;
   }
