@@ -46,10 +46,12 @@ def tensor_peak(peaks, path, region_s):
     """(peak TFLOP/s, label) for a tensor-core kernel timed inside a region of `region_s` seconds."""
     # tf32 nominal rate is half of bf16; the compensated path spends, per algorithmic product, one tf32 product and
     # one bf16 product of twice the reduction length (as long as a tf32 one): two tf32 products' worth
-    scale = {"bf16": 1.0, "tf32": 0.5, "tf32x3": 0.5 / 2.0}[path]
+    # (f32 on the tensor cores: six bf16 products of parts)
+    scale = {"bf16": 1.0, "tf32": 0.5, "tf32x3": 0.5 / 2.0, "f32": 1.0 / 6.0}[path]
     kind = "burst" if region_s < BURST_REGION_S else "sustained"
     base = peaks["bf16"] if kind == "burst" else peaks["bf16_sustained"]
-    label = (f"{peaks['source']} cuBLAS bf16 {kind} ({base:.1f})" + {"bf16": "", "tf32": " x 0.5 (tf32)", "tf32x3": " x 0.5 (tf32) / 2 (a tf32 product and a bf16 correction product of the same length per multiply-add)"}[path] +
+    label = (f"{peaks['source']} cuBLAS bf16 {kind} ({base:.1f})" + {"bf16": "", "tf32": " x 0.5 (tf32)", "tf32x3": " x 0.5 (tf32) / 2 (a tf32 product and a bf16 correction product of the same length per multiply-add)",
+                                                                    "f32": " / 6 (six products of bf16 parts per multiply-add)"}[path] +
              f": timed region {region_s * 1e3:.0f} ms")
     return base * scale, label, scale
 
@@ -582,6 +584,9 @@ def main():
             # the apply left out pairs whose u is zero: its work is counted on the pairs it multiplied through
             alg["flops_all_pairs"] = alg["flops"]
             out["pairs_applied_last_step"] = applied
+        # large dense fp32 steps: planes, GEMM and its stand-in, finishing pass, list, planes, GEMM, stand-in
+        f32_on_tensor_cores = path == "f32" and alg is not None and not alg["sparse"] and launches >= 8 * args.steps
+        kernel = "umma_f32_kernel" if path == "f32" else "umma_gemm_kernel"
         if alg is not None:
             apply_tflops = alg["flops"] * (applied / K if 0 < applied < K else 1.0) / (a_ms * 1e-3) / 1e12
             fwd_tflops = alg["flops"] / (f_ms * 1e-3) / 1e12
@@ -596,7 +601,7 @@ def main():
                 out["roofline"]["secondary"] = {"bound": "shared-memory operand reads", "achieved": smem_tbs,
                                                 "peak": SMEM_TBS, "unit": "TB/s", "frac": smem_tbs / SMEM_TBS,
                                                 "peak_source": "148 SMs x 128 B/clk x 1.965 GHz"}
-            elif path == "f32":
+            elif path == "f32" and not f32_on_tensor_cores:
                 out["roofline"] = {"bound": "alu", "achieved": apply_tflops, "peak": FP32_FMA_TFLOPS, "unit": "TFLOP/s",
                                    "frac": apply_tflops / FP32_FMA_TFLOPS, "traffic": traffic,
                                    "kernel": "sgemm_pipe_kernel<0> (apply)", "peak_source": "148 SMs x 128 FMA lanes x 1.965 GHz"}
@@ -604,7 +609,7 @@ def main():
                 # the apply is ONE launch per step: its launch duration is the apply stage's event span
                 peak, label, scale = tensor_peak(peaks, path, ms * 1e-3)
                 out["roofline"] = {"bound": "tensor", "achieved": apply_tflops, "peak": peak, "unit": "TFLOP/s",
-                                   "frac": apply_tflops / peak, "traffic": traffic, "kernel": "umma_gemm_kernel (apply)",
+                                   "frac": apply_tflops / peak, "traffic": traffic, "kernel": kernel + " (apply)",
                                    "peak_source": label,
                                    "frac_of_burst": apply_tflops / (peaks["bf16"] * scale),
                                    "frac_of_sustained": apply_tflops / (peaks["bf16_sustained"] * scale),
@@ -617,7 +622,7 @@ def main():
                 out["roofline_factors"] = {"bound": "l2", "achieved": l2_tbs, "peak": L2_TBS, "unit": "TB/s",
                                            "frac": l2_tbs / L2_TBS, "kernel": "sc_forward_kernel",
                                            "peak_source": "ncu: 17.9 TB/s of L2 reads at lts__throughput 73 %"}
-            elif path == "f32":
+            elif path == "f32" and not f32_on_tensor_cores:
                 out["roofline_factors"] = {"bound": "alu", "achieved": fwd_tflops, "peak": FP32_FMA_TFLOPS,
                                            "unit": "TFLOP/s", "frac": fwd_tflops / FP32_FMA_TFLOPS,
                                            "kernel": "fp32 forward kernels + finishing pass"}
@@ -625,7 +630,7 @@ def main():
                 peak, label, scale = tensor_peak(peaks, path, ms * 1e-3)
                 out["roofline_factors"] = {"bound": "tensor", "achieved": fwd_tflops, "peak": peak,
                                            "unit": "TFLOP/s", "frac": fwd_tflops / peak, "peak_source": label,
-                                           "kernel": "umma_gemm_kernel (forward) + finishing pass"}
+                                           "kernel": kernel + " (forward) + finishing pass"}
         if not args.no_cpu_baseline:
             sw = pick_sample_workers(cfg, budget=6e12)
             dt, n = oracle_step_time(cfg, inputs, sw)
