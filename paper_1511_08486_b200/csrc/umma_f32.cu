@@ -20,7 +20,7 @@
 // What bounds the GEMMs: the tensor pipe (six bf16 instructions per product), under the power cap.  A 256 x 256 tile of a
 // CTA pair loads 96 KB per CTA and chunk for 3072 clocks of tensor work, 32 bytes a clock, half of what the tf32 kernels
 // need for a tile of the same shape, because each part meets two or three others: by the clock counter a chunk takes 3072
-// clocks once the pipeline runs.  1000 x 20000, K = 1024: forward 167 us (246 TFLOP of bf16), update 160 us.
+// clocks once the pipeline runs.  1000 x 20000, K = 1024: forward 167 us (246 GFLOP of bf16), update 160 us.
 #include <cuda.h>
 #include <cudaTypedefs.h>
 
