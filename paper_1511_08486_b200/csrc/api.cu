@@ -606,6 +606,7 @@ static int apply_from(sfb_ctx* c, void* W, const void* sf_buf, float eta, int K,
   const bool mirrored = has_shadow(c) && c->shadow_of == W;
   HeaderCheck hc;
   if (check) hc = make_check(sf_buf, d, c->l, c->dev_status);
+  const int* refused = check ? c->dev_status : nullptr;   // for the passes over the buffer in front of the update: see is_refused
   // (the compensated path has a kernel in front of its GEMM that can do the check)
   const bool with_split = !d.v_sparse && d.path == SFB_PATH_TF32X3;
   if (check && c->f32_tc != nullptr) hc.clear = f32tc_bad_apply(c->f32_tc);
@@ -613,17 +614,17 @@ static int apply_from(sfb_ctx* c, void* W, const void* sf_buf, float eta, int K,
   if (d.v_sparse && d.path == SFB_PATH_F32 && c->csc_ws != nullptr) {
     if (!csc_built)
       ACC(launch_sc_csc_build(c->stream, stream_codes(c, sf_buf), K, d.D, (long long)d.nnz_capacity, c->csc_ws,
-                              c->dev_status, check ? c->dev_status : nullptr));
+                              c->dev_status, refused));
     ACC(launch_sc_csc_apply(c->stream, reinterpret_cast<float*>(W), stream_u(c, sf_buf), K, d.J, d.D, eta,
                             (long long)d.nnz_capacity, c->csc_ws, c->dev_status));
   } else if (d.v_sparse && d.path == SFB_PATH_F32) {
     ACC(launch_sc_apply(c->stream, reinterpret_cast<float*>(W), stream_codes(c, sf_buf), stream_u(c, sf_buf), K, d.J,
-                        d.D, eta, c->sc_flags, c->dev_status, check ? c->dev_status : nullptr));
+                        d.D, eta, c->sc_flags, c->dev_status, refused));
   } else if (d.v_sparse) {
     // dense alternative: rebuild the dense code rows from the buffer's CSR streams unless this step just made them
     if (check)
       ACC(launch_densify_codes(c->stream, stream_codes(c, sf_buf), dense_codes(c), K, d.D, c->dev_status,
-                               d.path == SFB_PATH_TF32, c->dev_status));
+                               d.path == SFB_PATH_TF32, refused));
     ACC(umma_apply(c->umma, c->stream, W, has_shadow(c) ? c->w_shadow : nullptr, stream_u(c, sf_buf), dense_codes(c), eta,
                    K, c->dev_status));
     if (!mirrored) c->shadow_of = nullptr;
@@ -632,17 +633,18 @@ static int apply_from(sfb_ctx* c, void* W, const void* sf_buf, float eta, int K,
     // finishing pass (a buffer of the caller's: from its rows)
     const RowMap u = stream_u(c, sf_buf);
     const bool listed = active_rows && c->dml_active != nullptr;
-    if (d.compact) ACC(launch_kept_rows(c->stream, sf_buf, d.B, K / d.B, c->kept_idx, c->kept_idx + c->K));
-    else ACC(f32tc_list(c->f32_tc, c->stream, u, K, !check, listed ? c->dml_active : nullptr, listed ? c->dml_idx + c->K : nullptr));
+    if (d.compact) ACC(launch_kept_rows(c->stream, sf_buf, d.B, K / d.B, c->kept_idx, c->kept_idx + c->K, refused));
+    else ACC(f32tc_list(c->f32_tc, c->stream, u, K, !check, listed ? c->dml_active : nullptr, listed ? c->dml_idx + c->K : nullptr,
+                        refused));
     const int* idx = d.compact ? c->kept_idx : nullptr;
     const int* n_idx = d.compact ? c->kept_idx + c->K : nullptr;
     ACC(f32tc_apply(c->f32_tc, c->stream, reinterpret_cast<float*>(W), u, stream_v(c, sf_buf), K, eta, c->dev_status, idx, n_idx,
-                    !check, idx, n_idx));
+                    !check, idx, n_idx, refused));
   } else if (d.path == SFB_PATH_F32) {
     const int* idx = nullptr;
     const int* n_idx = nullptr;
     if (d.compact) {   // compacted buffer: the kept pairs sit in the first n_sf slots of every worker (directory)
-      ACC(launch_kept_rows(c->stream, sf_buf, d.B, K / d.B, c->kept_idx, c->kept_idx + c->K));
+      ACC(launch_kept_rows(c->stream, sf_buf, d.B, K / d.B, c->kept_idx, c->kept_idx + c->K, refused));
       idx = c->kept_idx;
       n_idx = c->kept_idx + c->K;
     } else if (active_rows && c->dml_active != nullptr) {   // ordered list of the contributing pairs among the first K

@@ -350,11 +350,11 @@ int launch_compact(cudaStream_t s, void* sf_buf, const sfb_desc& d, const Layout
                    bool flags_ready = false);   // n_workers > 0: only those workers' streams (a process's shard)
 // flags_ready: the finishing pass that wrote the u rows left its flags (FinishExtra::nonzero) in compact_flags(workspace).
 uint8_t* compact_flags(void* workspace);
-// flags[i] = 1 where row i of u (J values) holds a nonzero one.
-int launch_row_nonzero(cudaStream_t s, RowMap u, int K, int J, uint8_t* flags);
+// flags[i] = 1 where row i of u (J values) holds a nonzero one.  refused: see is_refused (the flags stay as they are then).
+int launch_row_nonzero(cudaStream_t s, RowMap u, int K, int J, uint8_t* flags, const int* refused = nullptr);
 // Rebuilds the directory's pair counts (and the header flag) from streams that arrived already compacted.
 int launch_count_pairs(cudaStream_t s, void* sf_buf, const sfb_desc& d, const Layout& l, void* workspace);
-int launch_kept_rows(cudaStream_t s, const void* sf_buf, int B, int workers, int* idx, int* n_out);
+int launch_kept_rows(cudaStream_t s, const void* sf_buf, int B, int workers, int* idx, int* n_out, const int* refused = nullptr);
 
 // Sets SFB_DEV_BAD_HEADER in *dev_status unless the buffer's header matches the descriptor.
 HeaderCheck make_check(const void* sf_buf, const sfb_desc& d, const Layout& l, int* dev_status);

@@ -19,10 +19,11 @@ constexpr int WAVE = 256;         // rows per wave of the move, one per thread
 constexpr int SLICE_UNITS = 8;    // 16-byte units per column slice
 
 // flags[i] = 1 if the wire values of u row i are not all zero (-0 counts as zero).  One warp per row.
-__global__ void __launch_bounds__(256) row_nonzero_kernel(RowMap u, int K, int J, uint8_t* flags) {
+// refused: see is_refused.
+__global__ void __launch_bounds__(256) row_nonzero_kernel(RowMap u, int K, int J, uint8_t* flags, const int* refused) {
   chain();
   const int i = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-  if (i >= K) return;
+  if (i >= K || is_refused(refused)) return;
   const int per = 16 / u.es, units = (J + per - 1) / per;     // pad values inside the last unit are zeros
   const uint4* row = reinterpret_cast<const uint4*>(u.row(i));
   const uint32_t mask = u.es == 4 ? 0x7fffffffu : 0x7fff7fffu;
@@ -104,10 +105,12 @@ __global__ void __launch_bounds__(256) compact_move_kernel(char* buf, char* stre
 }
 
 // idx[0 .. *n_out) = p * B + r for every worker p < workers and every r < its pair count, in that order.
+// refused: see is_refused (the list is empty then).
 __global__ void __launch_bounds__(256) kept_rows_kernel(const char* buf, int B, int workers, int* idx,
-                                                        int* n_out) {
+                                                        int* n_out, const int* refused) {
   chain_wait();
   __shared__ int base;
+  if (is_refused(refused)) workers = 0;
   if (threadIdx.x == 0) base = 0;
   __syncthreads();
   for (int p = 0; p < workers; ++p) {
@@ -168,13 +171,13 @@ int launch_count_pairs(cudaStream_t s, void* sf_buf, const sfb_desc& d, const La
   char* buf = reinterpret_cast<char*>(sf_buf);
   RowMap u;
   u.base = buf + l.streams_off; u.worker_stride = l.stream_stride; u.ld = l.ldu; u.B = d.B; u.es = l.es;
-  launch_chained(row_nonzero_kernel, (K + 7) / 8, 256, 0, s, u, K, d.J, w.flags);
+  launch_chained(row_nonzero_kernel, (K + 7) / 8, 256, 0, s, u, K, d.J, w.flags, nullptr);
   launch_chained(count_pairs_kernel, d.P, 256, 0, s, w.flags, d.B, buf);
   return cudaGetLastError() == cudaSuccess ? 2 : SFB_ERR_CUDA;
 }
 
-int launch_row_nonzero(cudaStream_t s, RowMap u, int K, int J, uint8_t* flags) {
-  launch_chained(row_nonzero_kernel, (K + 7) / 8, 256, 0, s, u, K, J, flags);
+int launch_row_nonzero(cudaStream_t s, RowMap u, int K, int J, uint8_t* flags, const int* refused) {
+  launch_chained(row_nonzero_kernel, (K + 7) / 8, 256, 0, s, u, K, J, flags, refused);
   return cudaGetLastError() == cudaSuccess ? 1 : SFB_ERR_CUDA;
 }
 
@@ -190,7 +193,7 @@ int launch_compact(cudaStream_t s, void* sf_buf, const sfb_desc& d, const Layout
   char* streams = buf + l.streams_off + (long long)first_worker * l.stream_stride;
   RowMap u;
   u.base = streams; u.worker_stride = l.stream_stride; u.ld = l.ldu; u.B = d.B; u.es = l.es;
-  if (!flags_ready) launch_chained(row_nonzero_kernel, (K + 7) / 8, 256, 0, s, u, K, d.J, w.flags);
+  if (!flags_ready) launch_chained(row_nonzero_kernel, (K + 7) / 8, 256, 0, s, u, K, d.J, w.flags, nullptr);
   const int u_units = l.ldu * l.es / 16, v_units = l.ldv * l.es / 16;
   const int u_slices = (u_units + SLICE_UNITS - 1) / SLICE_UNITS, v_slices = (v_units + SLICE_UNITS - 1) / SLICE_UNITS;
   launch_chained(compact_move_kernel, n_workers * (u_slices + v_slices), 256, 0, s, buf, streams, l.stream_stride, l.u_bytes, d.B,
@@ -199,8 +202,8 @@ int launch_compact(cudaStream_t s, void* sf_buf, const sfb_desc& d, const Layout
   return cudaGetLastError() == cudaSuccess ? (flags_ready ? 1 : 2) : SFB_ERR_CUDA;
 }
 
-int launch_kept_rows(cudaStream_t s, const void* sf_buf, int B, int workers, int* idx, int* n_out) {
-  launch_chained(kept_rows_kernel, 1, 256, 0, s, reinterpret_cast<const char*>(sf_buf), B, workers, idx, n_out);
+int launch_kept_rows(cudaStream_t s, const void* sf_buf, int B, int workers, int* idx, int* n_out, const int* refused) {
+  launch_chained(kept_rows_kernel, 1, 256, 0, s, reinterpret_cast<const char*>(sf_buf), B, workers, idx, n_out, refused);
   return cudaGetLastError() == cudaSuccess ? 1 : SFB_ERR_CUDA;
 }
 

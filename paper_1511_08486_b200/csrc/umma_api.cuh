@@ -69,12 +69,14 @@ int* f32tc_bad_forward(F32Tc* t);
 int* f32tc_bad_apply(F32Tc* t);
 uint8_t* f32tc_flags(F32Tc* t);         // where the finishing pass leaves which u rows are nonzero
 // Lists the rows with nonzero u among the first K: f32tc_apply's when it gets no list of its own.
-// active / n_active (optional): how many of these flags are set.
-int f32tc_list(F32Tc* t, cudaStream_t s, RowMap u, int K, bool flags_ready, const uint8_t* active, int* n_active);
+// active / n_active (optional): how many of these flags are set.  refused: see is_refused (the list is empty then).
+int f32tc_list(F32Tc* t, cudaStream_t s, RowMap u, int K, bool flags_ready, const uint8_t* active, int* n_active,
+               const int* refused);
 // W -= eta * sum u_i v_i^T over the listed rows, in that order (idx / n_rows, or f32tc_list's).  The sum depends on the listed
 // rows alone, so leaving out zero rows, as a compacted buffer does, changes no bit.
 // v_planes: the forward of the same step made v's planes (all K rows).  core_idx / core_n: the list the CUDA cores get.
+// refused: see is_refused (no row is read then).
 int f32tc_apply(F32Tc* t, cudaStream_t s, float* W, RowMap u, RowMap v, int K, float eta, int* dev_status, const int* idx,
-                const int* n_rows, bool v_planes, const int* core_idx, const int* core_n);
+                const int* n_rows, bool v_planes, const int* core_idx, const int* core_n, const int* refused);
 
 }  // namespace sfb

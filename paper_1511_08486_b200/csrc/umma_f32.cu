@@ -490,9 +490,11 @@ __device__ __forceinline__ bool make_planes(const PlaneJob& j, int i, int r, int
 
 // Bound: HBM.  Eight values a thread at a time: 32 bytes in, 16 bytes to each plane; samples and W of 1000 x 20000,
 // K = 1024 (487 MB) 74 us, 6.6 TB/s.
+// refused: see is_refused.
 __global__ void __launch_bounds__(256) planes_kernel(const __grid_constant__ PlaneJob j0, const __grid_constant__ PlaneJob j1,
-                                                     int* bad) {
+                                                     int* bad, const int* refused) {
   chain();
+  if (is_refused(refused)) return;
   const bool second = (int)blockIdx.x >= j0.blocks;
   const PlaneJob j = second ? j1 : j0;
   const unsigned per_row = j.ldc >> 3, units = j.rows * per_row;   // (the workspace limit keeps them below 2^31)
@@ -510,11 +512,12 @@ __global__ void __launch_bounds__(256) planes_kernel(const __grid_constant__ Pla
 }
 
 // idx[0 .. n): the rows i < K with flags[i] != 0, ascending; idx[n ..): the others.  *n_active (optional): rows with
-// active[i] != 0.  One block; a thread takes K / 1024 consecutive rows.
+// active[i] != 0.  One block; a thread takes K / 1024 consecutive rows.  refused: see is_refused (the list is empty then).
 __global__ void __launch_bounds__(1024) list_rows_kernel(const uint8_t* flags, const uint8_t* active, int K, int* idx,
-                                                         int* n_out, int* n_active) {
+                                                         int* n_out, int* n_active, const int* refused) {
   chain();
   __shared__ int warp_sum[32], act_sum[32];
+  if (is_refused(refused)) K = 0;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int per = (K + 1023) / 1024, lo = min(K, (int)threadIdx.x * per), hi = min(K, lo + per);
   int n = 0, na = 0;
@@ -734,14 +737,14 @@ static RowMap plain_rows(const void* base, int ld, int rows) {
   return m;
 }
 
-static int launch_planes(cudaStream_t s, PlaneJob a, PlaneJob b, int* bad) {
+static int launch_planes(cudaStream_t s, PlaneJob a, PlaneJob b, int* bad, const int* refused) {
   auto blocks = [](const PlaneJob& j) {
     const long long n = ((long long)j.rows * (j.ldc / 8) + 255) / 256;
     return (int)(j.keep_if_all && n > 148 * 16 ? 148 * 16 : n);   // (blocks that most often have nothing to do: 13 -> 5 us)
   };
   a.blocks = blocks(a);
   b.blocks = blocks(b);
-  launch_chained(planes_kernel, a.blocks + b.blocks, 256, 0, s, a, b, bad);
+  launch_chained(planes_kernel, a.blocks + b.blocks, 256, 0, s, a, b, bad, refused);
   return cudaGetLastError() == cudaSuccess ? 1 : SFB_ERR_CUDA;
 }
 
@@ -759,7 +762,7 @@ int f32tc_forward(F32Tc* t, cudaStream_t s, const float* W, const float* X, cons
   jw.dst = t->wp; jw.plane_bytes = (long long)J * t->ldd * 2;
   jw.rows = J; jw.C = D; jw.ldc = t->ldd; jw.vec = vec;
   int r, launches = 0;
-  if ((r = launch_planes(s, jx, jw, f32tc_bad_forward(t))) < 0) return r;
+  if ((r = launch_planes(s, jx, jw, f32tc_bad_forward(t), nullptr)) < 0) return r;
   launches += r;
 
   const int chunks = (D + CHUNK - 1) / CHUNK;
@@ -794,18 +797,19 @@ int f32tc_forward(F32Tc* t, cudaStream_t s, const float* W, const float* X, cons
   return launches;
 }
 
-int f32tc_list(F32Tc* t, cudaStream_t s, RowMap u, int K, bool flags_ready, const uint8_t* active, int* n_active) {
+int f32tc_list(F32Tc* t, cudaStream_t s, RowMap u, int K, bool flags_ready, const uint8_t* active, int* n_active,
+               const int* refused) {
   int r, launches = 0;
   if (!flags_ready) {
-    if ((r = launch_row_nonzero(s, u, K, t->J, t->flags)) < 0) return r;
+    if ((r = launch_row_nonzero(s, u, K, t->J, t->flags, refused)) < 0) return r;
     launches += r;
   }
-  launch_chained(list_rows_kernel, 1, 1024, 0, s, t->flags, active, K, t->idx, t->words, n_active);
+  launch_chained(list_rows_kernel, 1, 1024, 0, s, t->flags, active, K, t->idx, t->words, n_active, refused);
   return cudaGetLastError() == cudaSuccess ? launches + 1 : SFB_ERR_CUDA;
 }
 
 int f32tc_apply(F32Tc* t, cudaStream_t s, float* W, RowMap u, RowMap v, int K, float eta, int* dev_status, const int* idx,
-                const int* n_rows, bool v_planes, const int* core_idx, const int* core_n) {
+                const int* n_rows, bool v_planes, const int* core_idx, const int* core_n, const int* refused) {
   const int D = t->D, J = t->J;
   PlaneJob ju = {}, jv = {};
   ju.src = u; ju.dst = t->up; ju.plane_bytes = (long long)t->K * t->ldj * 2;
@@ -818,7 +822,7 @@ int f32tc_apply(F32Tc* t, cudaStream_t s, float* W, RowMap u, RowMap v, int K, f
   jv.rest = own && !v_planes ? 1 : 0;   // (the pass that made the planes has looked at every row)
   jv.keep_if_all = v_planes ? 1 : 0;
   int r, launches = 0;
-  if ((r = launch_planes(s, ju, jv, f32tc_bad_apply(t))) < 0) return r;
+  if ((r = launch_planes(s, ju, jv, f32tc_bad_apply(t), refused)) < 0) return r;
   launches += r;
   const int chunks = (K + CHUNK - 1) / CHUNK;
   const Geometry g = pick(D, J, chunks, 1, t->num_sms / 2);

@@ -75,3 +75,36 @@ def test_a_refused_update_leaves_no_stale_copy_of_w(path, name, over):
     finally:
         a.close()
         b.close()
+
+
+@pytest.mark.parametrize("name,over", [
+    ("C1", dict(J=1000, D=2003, P=8, B=100, pool=1)), ("C2", dict(J=257, D=1025, P=3, B=300)), ("C2", dict(J=257, D=1025, P=3, B=300, compact=1))])
+def test_large_fp32_update_of_a_refused_buffer(name, over):
+    """Dense fp32 on the tensor cores.  The streams hold NaN (every read stays inside the buffer); afterwards the right buffer is
+    applied, and a step taken, as by a context that never saw the refused one."""
+    from paper_1511_08486_b200 import binding as B
+    cfg = scaled(name, **over)
+    inputs = make_inputs(cfg)
+    wl, fresh = _workload(cfg, inputs, "f32", guard=True), _workload(cfg, inputs, "f32")
+    try:
+        for w in (wl, fresh):
+            w.compute_factors(0)
+            w.pack(0)
+        good = wl.sf_buf.clone()
+        off, _ = B.sfb_sf_buffer_layout(wl.desc)
+        wl.sf_buf[20] ^= 64                                  # J field of the header
+        wl.sf_buf[off:] = 0xFF
+        bad = wl.sf_buf.clone()
+        wl.apply(0.5)
+        assert wl.ctx.status() == B.SFB_DEV_BAD_HEADER
+        assert torch.equal(wl.W, wl.W0) and torch.equal(wl.sf_buf, bad)
+        wl.sf_buf.copy_(good)
+        for w in (wl, fresh):
+            w.apply(1e-4)
+            w.step(0, eta=1e-4)
+            assert w.ctx.status() == 0
+        assert torch.equal(wl.W, fresh.W) and torch.equal(wl.sf_buf, fresh.sf_buf)
+        assert not torch.equal(wl.W, wl.W0) and wl.guards_intact()
+    finally:
+        wl.close()
+        fresh.close()
