@@ -126,15 +126,23 @@ struct HeaderCheck {
 __device__ __forceinline__ bool is_refused(const int* refused) {
   return refused != nullptr && (*refused & SFB_DEV_BAD_HEADER) != 0;
 }
-// one whole warp, t = lane
-__device__ __forceinline__ void check_header(const HeaderCheck& c, int t) {
-  const uint32_t* w = reinterpret_cast<const uint32_t*>(c.buf);
-  const uint32_t* ref = reinterpret_cast<const uint32_t*>(&c.h);
-  bool ok = true;
-  if (t < 17 && t != 7) ok = (w[t] == ref[t]);   // word 7 is the clock: any value is accepted
-  if (t == 0 && c.clear != nullptr) *c.clear = 0;
-  if (t == 2) ok = ((w[t] & ~2u) == ref[t]);      // flag bit 1 (compacted) may be set or not
-  if (!__all_sync(0xffffffffu, ok) && t == 0) atomicOr(c.dev_status, SFB_DEV_BAD_HEADER);
+// Does the buffer's header match the descriptor's?  Every thread for itself: five loads at once, the same for all, and the
+// expected words at fixed offsets.  (A word per lane looks them up one after the other: 0.5 us of the pass that asks.)
+__device__ __forceinline__ bool header_matches(const HeaderCheck& c) {
+  const uint4* q = reinterpret_cast<const uint4*>(c.buf);
+  const uint32_t* r = reinterpret_cast<const uint32_t*>(&c.h);
+  const uint4 w0 = q[0], w1 = q[1], w2 = q[2], w3 = q[3];
+  const uint32_t w16 = reinterpret_cast<const uint32_t*>(c.buf)[16];
+  uint32_t d = (w0.x ^ r[0]) | (w0.y ^ r[1]) | ((w0.z & ~2u) ^ r[2]) | (w0.w ^ r[3]);   // flag bit 1 (compacted): either
+  d |= (w1.x ^ r[4]) | (w1.y ^ r[5]) | (w1.z ^ r[6]);                                   // word 7 is the clock: any value
+  d |= (w2.x ^ r[8]) | (w2.y ^ r[9]) | (w2.z ^ r[10]) | (w2.w ^ r[11]);
+  d |= (w3.x ^ r[12]) | (w3.y ^ r[13]) | (w3.z ^ r[14]) | (w3.w ^ r[15]) | (w16 ^ r[16]);
+  return d == 0u;
+}
+// The outcome written down, by one thread.
+__device__ __forceinline__ void report_header(const HeaderCheck& c, bool matches) {
+  if (c.clear != nullptr) *c.clear = 0;
+  if (!matches) atomicOr(c.dev_status, SFB_DEV_BAD_HEADER);
 }
 #endif
 
@@ -427,7 +435,9 @@ int launch_cast_bf16(cudaStream_t s, const float* W, __nv_bfloat16* Wb, long lon
 // worker, or k_bb rows of each of k_wp workers), ldc a multiple of 64.
 int launch_split_k(cudaStream_t s, RowMap src, int rows, int cols, void* dst, bool a_side);
 struct SplitSide { RowMap src; int cols; void* dst; int ldc; };   // one factor's rows and where they go (dst == nullptr: not)
+// check: done on the way; refused: see is_refused (of a check that came before).  Either way the rows of a buffer that does
+// not match are not read.
 int launch_split_mn(cudaStream_t s, const SplitSide& us, const SplitSide& vs, int workers, int k_bb, int k_wp, int k_bpw,
-                    int blocks, const HeaderCheck& check);
+                    int blocks, const HeaderCheck& check, const int* refused);
 
 }  // namespace sfb

@@ -25,7 +25,10 @@ HeaderImage make_header(const sfb_desc& d, const Layout& l, uint32_t clock) {
 
 __global__ void write_header_kernel(const __grid_constant__ Commit c) { chain(); write_header(c, threadIdx.x, blockDim.x); }
 
-__global__ void check_header_kernel(const __grid_constant__ HeaderCheck c) { chain(); check_header(c, threadIdx.x); }
+__global__ void check_header_kernel(const __grid_constant__ HeaderCheck c) {
+  chain();
+  report_header(c, header_matches(c));
+}
 
 // grid.x = P workers; each block copies its worker's CSR rows into the stream.
 __global__ void __launch_bounds__(256) pack_csr_kernel(char* buf, long long streams_off, long long stream_stride,
@@ -95,7 +98,7 @@ HeaderCheck make_check(const void* sf_buf, const sfb_desc& d, const Layout& l, i
 }
 
 int launch_check_header(cudaStream_t s, const HeaderCheck& check) {
-  launch_chained(check_header_kernel, 1, 32, 0, s, check);
+  launch_chained(check_header_kernel, 1, 1, 0, s, check);
   return cudaGetLastError() == cudaSuccess ? 1 : SFB_ERR_CUDA;
 }
 

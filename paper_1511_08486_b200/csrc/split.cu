@@ -62,14 +62,20 @@ __global__ void __launch_bounds__(256) split_k_kernel(RowMap src, int rows, int 
 }
 
 // MN-major, both factors in one launch.  grid = (reduction blocks, groups of 8 units of 8 values along the padded rows of
-// u, then of v); block = 32 lines x 8 units.  On its way it checks the header of the buffer that the rows come from.
-// Bound by launches at small sizes: factors, pack and apply of 600 x 2000, K = 256, take 40.3 us, with a launch for
+// u, then of v); block = 32 lines x 8 units.  On its way it checks the header of the buffer that the rows come from: every
+// thread for itself, before it reads a row, and block 0 reports.  Bound by launches at small sizes: factors, pack and apply of 600 x 2000, K = 256, take 40.3 us, with a launch for
 // each factor and one for the check 44.0.
 __global__ void __launch_bounds__(256) split_mn_kernel(const __grid_constant__ SplitSide us, const __grid_constant__ SplitSide vs,
                                                        int u_groups, int workers, int k_bb, int k_wp, int k_bpw,
-                                                       const __grid_constant__ HeaderCheck check) {
+                                                       const __grid_constant__ HeaderCheck check, const int* refused) {
   chain();
-  if (check.buf != nullptr && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x < 32) check_header(check, threadIdx.x);
+  if (check.buf != nullptr) {
+    const bool matches = header_matches(check);
+    if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) report_header(check, matches);
+    if (!matches) return;
+  } else if (is_refused(refused)) {
+    return;
+  }
   const int a_side = (int)blockIdx.y < u_groups;
   const RowMap& src = a_side ? us.src : vs.src;
   const int cols = a_side ? us.cols : vs.cols, ldc = a_side ? us.ldc : vs.ldc;
@@ -108,18 +114,18 @@ int launch_split_k(cudaStream_t s, RowMap src, int rows, int cols, void* dst, bo
 }
 
 int launch_split_mn(cudaStream_t s, const SplitSide& us, const SplitSide& vs, int workers, int k_bb, int k_wp, int k_bpw,
-                    int blocks, const HeaderCheck& check) {
+                    int blocks, const HeaderCheck& check, const int* refused) {
   const int u_groups = us.dst != nullptr ? (us.ldc / 8 + 7) / 8 : 0, v_groups = vs.dst != nullptr ? (vs.ldc / 8 + 7) / 8 : 0;
   if (blocks <= 0 || u_groups + v_groups == 0) return 0;
   if (u_groups > 0 && v_groups > 0 && u_groups + v_groups > 65535) {   // the grid's limit: one factor at a time
     const SplitSide none = {RowMap(), 0, nullptr, 0};
-    const int r = launch_split_mn(s, us, none, workers, k_bb, k_wp, k_bpw, blocks, check);
+    const int r = launch_split_mn(s, us, none, workers, k_bb, k_wp, k_bpw, blocks, check, refused);
     if (r < 0) return r;
-    const int r2 = launch_split_mn(s, none, vs, workers, k_bb, k_wp, k_bpw, blocks, HeaderCheck());
+    const int r2 = launch_split_mn(s, none, vs, workers, k_bb, k_wp, k_bpw, blocks, HeaderCheck(), refused);
     return r2 < 0 ? r2 : r + r2;
   }
   const dim3 grid((unsigned)blocks, (unsigned)(u_groups + v_groups));
-  launch_chained(split_mn_kernel, grid, 256, 0, s, us, vs, u_groups, workers, k_bb, k_wp, k_bpw, check);
+  launch_chained(split_mn_kernel, grid, 256, 0, s, us, vs, u_groups, workers, k_bb, k_wp, k_bpw, check, refused);
   return cudaGetLastError() == cudaSuccess ? 1 : SFB_ERR_CUDA;
 }
 

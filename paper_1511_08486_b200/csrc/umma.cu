@@ -198,7 +198,8 @@ umma_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
       if (p.dir != nullptr) {   // only with B >= BK and at most MAX_DIR_WORKERS workers (the host checks)
         chain_wait();
         tot = 0;
-        for (int w = 0; w < p.P; ++w) {
+        const int workers = is_refused(p.status_ro) ? 0 : p.P;   // (the directory of a refused buffer may end earlier)
+        for (int w = 0; w < workers; ++w) {
           const int n = min((int)p.dir[w * 8 + 1], p.B);
           const int nbw = (n + BK - 1) / BK;
           ctl->nb[w] = (uint16_t)nbw;
@@ -1560,7 +1561,8 @@ static int umma_apply_range(UmmaPlan* pl, cudaStream_t s, void* W, __nv_bfloat16
     char* uc = reinterpret_cast<char*>(pl->uc) + blk0 * 64 * pl->ldcu * 2;
     char* vc = reinterpret_cast<char*>(pl->vc) + blk0 * 64 * pl->ldcv * 2;
     SplitSide us = {u_rows, d.J, have_u ? nullptr : uc, pl->ldcu}, vs = {v_rows, d.D, have_v ? nullptr : vc, pl->ldcv};
-    if ((launches = launch_split_mn(s, us, vs, workers, p.k_bb, p.k_wp, p.k_bpw, p.k_blocks, check)) < 0) return launches;
+    if ((launches = launch_split_mn(s, us, vs, workers, p.k_bb, p.k_wp, p.k_bpw, p.k_blocks, check, dev_status)) < 0)
+      return launches;
     if (!encode_corr_mn_map(&tuc, uc, pl->ldcu, (long long)p.k_blocks * 64, BM / 64) ||
         !encode_corr_mn_map(&tvc, vc, pl->ldcv, (long long)p.k_blocks * 64, (v.bn / v.cg) / 64))
       return SFB_ERR_CUDA;
