@@ -630,7 +630,8 @@ static int apply_from(sfb_ctx* c, void* W, const void* sf_buf, float eta, int K,
     if (!mirrored) c->shadow_of = nullptr;
   } else if (c->f32_tc != nullptr) {
     // the rows with nonzero u, in order: a compacted buffer's kept slots, or a list made from the flags of the step's
-    // finishing pass (a buffer of the caller's: from its rows)
+    // finishing pass (a buffer of the caller's: from its rows).  A step's inactive pairs and a compacted buffer's empty slots
+    // are left out on the CUDA cores too, where operands that are not finite lead.
     const RowMap u = stream_u(c, sf_buf);
     const bool listed = active_rows && c->dml_active != nullptr;
     if (d.compact) ACC(launch_kept_rows(c->stream, sf_buf, d.B, K / d.B, c->kept_idx, c->kept_idx + c->K, refused));
@@ -639,7 +640,7 @@ static int apply_from(sfb_ctx* c, void* W, const void* sf_buf, float eta, int K,
     const int* idx = d.compact ? c->kept_idx : nullptr;
     const int* n_idx = d.compact ? c->kept_idx + c->K : nullptr;
     ACC(f32tc_apply(c->f32_tc, c->stream, reinterpret_cast<float*>(W), u, stream_v(c, sf_buf), K, eta, c->dev_status, idx, n_idx,
-                    !check, idx, n_idx, refused));
+                    !check, listed || d.compact, refused));
   } else if (d.path == SFB_PATH_F32) {
     const int* idx = nullptr;
     const int* n_idx = nullptr;

@@ -74,9 +74,11 @@ int f32tc_list(F32Tc* t, cudaStream_t s, RowMap u, int K, bool flags_ready, cons
                const int* refused);
 // W -= eta * sum u_i v_i^T over the listed rows, in that order (idx / n_rows, or f32tc_list's).  The sum depends on the listed
 // rows alone, so leaving out zero rows, as a compacted buffer does, changes no bit.
-// v_planes: the forward of the same step made v's planes (all K rows).  core_idx / core_n: the list the CUDA cores get.
+// v_planes: the forward of the same step made v's planes (all K rows).
+// left_out: rows that are not listed are not part of the update, whatever their v holds; otherwise a row without a nonzero u
+// still makes a NaN of a v that is not finite (the CUDA cores then take all K rows).
 // refused: see is_refused (no row is read then).
 int f32tc_apply(F32Tc* t, cudaStream_t s, float* W, RowMap u, RowMap v, int K, float eta, int* dev_status, const int* idx,
-                const int* n_rows, bool v_planes, const int* core_idx, const int* core_n, const int* refused);
+                const int* n_rows, bool v_planes, bool left_out, const int* refused);
 
 }  // namespace sfb

@@ -809,7 +809,7 @@ int f32tc_list(F32Tc* t, cudaStream_t s, RowMap u, int K, bool flags_ready, cons
 }
 
 int f32tc_apply(F32Tc* t, cudaStream_t s, float* W, RowMap u, RowMap v, int K, float eta, int* dev_status, const int* idx,
-                const int* n_rows, bool v_planes, const int* core_idx, const int* core_n, const int* refused) {
+                const int* n_rows, bool v_planes, bool left_out, const int* refused) {
   const int D = t->D, J = t->J;
   PlaneJob ju = {}, jv = {};
   ju.src = u; ju.dst = t->up; ju.plane_bytes = (long long)t->K * t->ldj * 2;
@@ -841,7 +841,8 @@ int f32tc_apply(F32Tc* t, cudaStream_t s, float* W, RowMap u, RowMap v, int K, f
     return SFB_ERR_CUDA;
   if ((r = launch_gemm<true>(s, ta, tb, p, t->num_sms)) < 0) return r;
   launches += r;
-  if ((r = launch_apply_f32(s, W, u, v, K, J, D, eta, dev_status, core_idx, core_n, p.bad)) < 0) return r;
+  if ((r = launch_apply_f32(s, W, u, v, K, J, D, eta, dev_status, left_out ? ju.idx : nullptr, left_out ? ju.n_rows : nullptr, p.bad)) < 0)
+    return r;
   return launches + r;
 }
 

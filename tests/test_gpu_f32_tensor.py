@@ -120,3 +120,28 @@ def test_operands_that_are_not_finite(where):
     finally:
         wl.close()
         fresh.close()
+
+
+@pytest.mark.parametrize("J,D,P,B", [(300, 8192, 4, 96)])
+def test_inactive_pairs_that_are_not_finite(J, D, P, B):
+    """A dissimilar pair with a NaN or an infinite feature is beyond the margin (no comparison with NaN holds): its u is zero and
+    the step leaves it out, with and without compaction.  W is that of the same pairs with finite features far apart."""
+    cfg = scaled("C2", J=J, D=D, P=P, B=B)
+    inputs = make_inputs(cfg)
+    apart = np.nonzero(inputs["similar"] == 0)[0]
+    full, comp, ref = _workload(cfg, inputs, "f32", guard=True), _workload(dict(cfg, compact=1), inputs, "f32"), _workload(cfg, inputs, "f32")
+    try:
+        for wl, values in ((full, ("nan", "inf", "-inf")), (comp, ("nan", "inf", "-inf")), (ref, (1e4, 1e4, -1e4))):
+            for i, x in zip((apart[0], apart[7], apart[-1]), values):
+                wl.batches[0]["X"][int(i), 5 + int(i) % 7] = float(x)
+            wl.step(0, eta=1e-4)
+            assert wl.ctx.status() == 0
+        assert bool(torch.isfinite(full.W).all()) and torch.equal(full.W, comp.W) and full.guards_intact()
+        assert full.ctx.active_pairs() == comp.ctx.active_pairs() == ref.ctx.active_pairs()
+        dw, want = to_f64(full.W) - inputs["W"].astype(np.float64), to_f64(ref.W) - inputs["W"].astype(np.float64)
+        # two roundings of the sums, and of W, per side
+        assert np.linalg.norm(dw - want) <= 2e-6 * np.linalg.norm(want) + 2.0 ** -23 * np.linalg.norm(inputs["W"])
+    finally:
+        full.close()
+        comp.close()
+        ref.close()
