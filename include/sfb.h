@@ -258,9 +258,11 @@ int sfb_prox(sfb_ctx* ctx, void* W);
 int sfb_loss(sfb_ctx* ctx, const void* W, const void* X, const sfb_aux* aux, double* loss);
 
 /* Number of (u, v) pairs the last sfb_step actually multiplied through.  SFB_DML on SFB_PATH_F32 leaves out the
- * pairs whose u is zero (dissimilar pairs beyond the margin; the update is bit-identical to the sum over all K
- * slots, Section 6 notes that such sparsity can be used), and so does every context with compact = 1 (the count
- * is then the number of pairs the compaction kept); every other model / path applies all K slots and reports K.  Synchronises the stream.  *n is 0 before the first step. */
+ * pairs whose u is zero (dissimilar pairs beyond the margin; Section 6 notes that such sparsity can be used) where
+ * J x D makes 148 tiles of 128 x 128 or the products are formed on the tensor cores, and so does every context with
+ * compact = 1 (the count is then the number of pairs the compaction kept); everything else reports K.  The result depends
+ * on the pairs with nonzero u alone: the same bits with and without the others, wherever these sit and with and
+ * without compaction.  Synchronises the stream.  *n is 0 before the first step. */
 int sfb_active_pairs(sfb_ctx* ctx, int32_t* n);
 
 /* Bytes a broadcast of this committed buffer would carry (Section 5.1 counts them per pair of workers: every

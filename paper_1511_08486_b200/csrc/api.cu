@@ -790,8 +790,9 @@ int sfb_step(sfb_ctx* c, void* W, const void* X, const sfb_aux* aux, void* sf_bu
   // pairs whose u came out as zero are dropped from the message before it is "sent" (and applied)
   if (d.compact) ACC(launch_compact(c->stream, sf_buf, d, c->l, c->compact_ws, 0, 0, true));
   if (c->profiling) cudaEventRecord(c->prof_ev[slot][1], c->stream);
+  // (on the CUDA cores the large-tile update takes the list)
   const bool listed = !d.compact && d.model == SFB_DML && d.path == SFB_PATH_F32 && c->dml_active != nullptr &&
-                      (long long)((d.J + 127) / 128) * ((d.D + 127) / 128) >= 148;   // the large-tile apply takes the list
+                      (c->f32_tc != nullptr || (long long)((d.J + 127) / 128) * ((d.D + 127) / 128) >= 148);
   r = apply_from(c, W, sf_buf, eta, K, false, csc_built, listed, defer_v ? &x_rows : nullptr);
   if (defer_v && umma_join(c->umma, c->stream) < 0 && r >= 0) r = SFB_ERR_CUDA;
   c->last_step_K = K;

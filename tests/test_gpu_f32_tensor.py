@@ -52,6 +52,8 @@ def test_dml(J, D, P, B):
             comp.step(t, eta=1e-3)
         torch.cuda.synchronize()
         assert torch.equal(full.W, comp.W) and comp.guards_intact()      # the sums depend on the nonzero pairs alone
+        _, U, _ = orc.unpack(full.sf_buf.cpu().numpy())
+        assert full.ctx.active_pairs() == comp.ctx.active_pairs() == int(U.any(axis=1).sum()) < cfg["K"]
     finally:
         full.close()
         comp.close()
@@ -122,7 +124,7 @@ def test_operands_that_are_not_finite(where):
         fresh.close()
 
 
-@pytest.mark.parametrize("J,D,P,B", [(300, 8192, 4, 96)])
+@pytest.mark.parametrize("J,D,P,B", [(300, 8192, 4, 96), (600, 2001, 8, 64)])
 def test_inactive_pairs_that_are_not_finite(J, D, P, B):
     """A dissimilar pair with a NaN or an infinite feature is beyond the margin (no comparison with NaN holds): its u is zero and
     the step leaves it out, with and without compaction.  W is that of the same pairs with finite features far apart."""
