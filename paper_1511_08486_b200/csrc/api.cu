@@ -327,7 +327,7 @@ int sfb_create(const sfb_desc* desc, void* cuda_stream, sfb_ctx** out) {
     c->f32_plan = forward_f32_plan(c->K, desc->J, desc->D, desc->model == SFB_DML, FORWARD_F32_MAX_SPLITS, nn_bytes <= (2LL << 30));
     const int ks = c->f32_plan.ks;
     c->ldp = (desc->J + 3) & ~3;
-    if (f32tc_pays(c->K, desc->J, desc->D, desc->model == SFB_DML, c->f32_plan.us)) ok = f32tc_create(*desc, c->stream, &c->f32_tc) == SFB_OK;
+    ok = f32tc_create(*desc, c->stream, c->f32_plan.us, &c->f32_tc) == SFB_OK;
     if (ok && c->f32_tc == nullptr && ks > 1) ok = cudaMalloc(&c->f32_part, (size_t)ks * c->K * c->ldp * 4) == cudaSuccess;
     if (ok && desc->model == SFB_DML) {
       ok = cudaMalloc(&c->dml_active, (size_t)c->K) == cudaSuccess;

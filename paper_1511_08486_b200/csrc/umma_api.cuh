@@ -53,10 +53,9 @@ int umma_apply(UmmaPlan* p, cudaStream_t s, void* W, __nv_bfloat16* w_shadow, Ro
 // fp32 path, large dense problems: the two contractions on the tensor cores, each fp32 operand as three bf16 parts
 // (umma_f32.cu).
 struct F32Tc;
-// Is a whole step estimated to be faster than on the CUDA cores, whose forward takes cores_forward_us?  pair: DML.
-bool f32tc_pays(int K, int J, int D, bool pair, double cores_forward_us);
-// *out = nullptr with SFB_OK: no room for the workspace, the CUDA cores do it.
-int f32tc_create(const sfb_desc& d, cudaStream_t s, F32Tc** out);
+// *out = nullptr with SFB_OK: the CUDA cores do it.  A whole step is not estimated to be faster than theirs, whose forward takes
+// cores_forward_us, or there is no room for the workspace, or the kernels cannot be set up on this device.
+int f32tc_create(const sfb_desc& d, cudaStream_t s, double cores_forward_us, F32Tc** out);
 void f32tc_destroy(F32Tc* t);
 // Products of K samples (X, or X - Xb) with W, as `nsplit` partial products of rows *z (which are u itself, or the
 // workspace), and the samples (differences) into v where v.base != nullptr.

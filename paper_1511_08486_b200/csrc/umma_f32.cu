@@ -680,22 +680,25 @@ struct F32Tc {
 // billion multiply-adds; the line lies near 200 million for a few hundred samples, lower where few tiles leave the
 // CUDA cores a long serial reduction).  87 of the 200 go to the tensor cores, none of them slower, the median 1.6 times
 // faster; 600 x 10000, K = 2048 950 -> 318 us, 1000 x 20000, K = 1024 1737 -> 479.
-bool f32tc_pays(int K, int J, int D, bool pair, double cores_forward_us) {
+static bool pays(int K, int J, int D, bool pair, double cores_forward_us, int pairs) {
   if (D < 2 * CHUNK) return false;
-  const Geometry f = pick(K, J, (D + CHUNK - 1) / CHUNK, F32TC_MAX_RANGES, 74), a = pick(D, J, (K + CHUNK - 1) / CHUNK, 1, 74);
+  const Geometry f = pick(K, J, (D + CHUNK - 1) / CHUNK, F32TC_MAX_RANGES, pairs), a = pick(D, J, (K + CHUNK - 1) / CHUNK, 1, pairs);
   const double planes = ((double)K * D * 14 + (double)J * D * 10 + (double)K * J * 10) / 5e6;
   const double chain = 0.68 * K / 16, rate = 2.0 * K * (double)J * D / 46e6;
   const double cores = 13.0 + 1.05 * cores_forward_us + (chain > rate ? chain : rate) + (pair ? 10.0 + (double)K * D * 12 / 4e6 : 0.0);
   return f.us + a.us + planes + 27.0 < cores;
 }
 
-int f32tc_create(const sfb_desc& d, cudaStream_t s, F32Tc** out) {
+int f32tc_create(const sfb_desc& d, cudaStream_t s, double cores_forward_us, F32Tc** out) {
   *out = nullptr;
   const long long K = (long long)d.P * d.B, ldd = pad_to(d.D, 8), ldj = pad_to(d.J, 8), ldp = pad_to(d.J, 4);
   if (encoder() == nullptr) return SFB_OK;
   int dev = 0, sms = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  if (!pays((int)K, d.J, d.D, d.model == SFB_DML, cores_forward_us, sms / 2)) return SFB_OK;
+  // a kernel that cannot run here (see pairs_at_once) is found out now: the CUDA cores have their workspaces or not from here on
+  if (pairs_at_once<false>(sms) < 1 || pairs_at_once<true>(sms) < 1) return SFB_OK;
   const Geometry f = pick((int)K, d.J, (d.D + CHUNK - 1) / CHUNK, F32TC_MAX_RANGES, sms / 2);
   const long long part = f.t.ranges > 1 ? f.t.ranges * K * ldp * 4 : 0;
   if (6 * (K * ldd + d.J * ldd + K * ldj) > F32TC_MAX_BYTES) return SFB_OK;
@@ -737,10 +740,10 @@ static RowMap plain_rows(const void* base, int ld, int rows) {
   return m;
 }
 
-static int launch_planes(cudaStream_t s, PlaneJob a, PlaneJob b, int* bad, const int* refused) {
-  auto blocks = [](const PlaneJob& j) {
+static int launch_planes(cudaStream_t s, PlaneJob a, PlaneJob b, int num_sms, int* bad, const int* refused) {
+  auto blocks = [=](const PlaneJob& j) {
     const long long n = ((long long)j.rows * (j.ldc / 8) + 255) / 256;
-    return (int)(j.keep_if_all && n > 148 * 16 ? 148 * 16 : n);   // (blocks that most often have nothing to do: 13 -> 5 us)
+    return (int)(j.keep_if_all && n > num_sms * 16 ? num_sms * 16 : n);   // (blocks that most often have nothing to do: 13 -> 5 us)
   };
   a.blocks = blocks(a);
   b.blocks = blocks(b);
@@ -762,7 +765,7 @@ int f32tc_forward(F32Tc* t, cudaStream_t s, const float* W, const float* X, cons
   jw.dst = t->wp; jw.plane_bytes = (long long)J * t->ldd * 2;
   jw.rows = J; jw.C = D; jw.ldc = t->ldd; jw.vec = vec;
   int r, launches = 0;
-  if ((r = launch_planes(s, jx, jw, f32tc_bad_forward(t), nullptr)) < 0) return r;
+  if ((r = launch_planes(s, jx, jw, t->num_sms, f32tc_bad_forward(t), nullptr)) < 0) return r;
   launches += r;
 
   const int chunks = (D + CHUNK - 1) / CHUNK;
@@ -822,7 +825,7 @@ int f32tc_apply(F32Tc* t, cudaStream_t s, float* W, RowMap u, RowMap v, int K, f
   jv.rest = own && !v_planes ? 1 : 0;   // (the pass that made the planes has looked at every row)
   jv.keep_if_all = v_planes ? 1 : 0;
   int r, launches = 0;
-  if ((r = launch_planes(s, ju, jv, f32tc_bad_apply(t), refused)) < 0) return r;
+  if ((r = launch_planes(s, ju, jv, t->num_sms, f32tc_bad_apply(t), refused)) < 0) return r;
   launches += r;
   const int chunks = (K + CHUNK - 1) / CHUNK;
   const Geometry g = pick(D, J, chunks, 1, t->num_sms / 2);

@@ -4,6 +4,7 @@ Behind it stand checks without which a kernel may not run at all (a register spl
 never come free), so a second call must be refused like the first.
 """
 import os
+import re
 import subprocess
 
 CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_1511_08486_b200", "csrc")
@@ -36,3 +37,13 @@ def test_a_failed_set_up_stays_failed(tmp_path):
     subprocess.run(["g++", "-std=c++17", "-I", CSRC, str(src), "-o", str(exe)], check=True)
     r = subprocess.run([str(exe)], capture_output=True, text=True)
     assert r.returncode == 0, r.stdout
+
+
+def test_a_route_is_taken_only_where_its_kernels_can_be_set_up():
+    """The context of a large fp32 problem has either the tensor cores' workspace or the CUDA cores': both kernels' set-up is
+    asked for before the first of it is allocated, while the other route is still open."""
+    text = open(os.path.join(CSRC, "umma_f32.cu")).read()
+    create = text[re.search(r"^int f32tc_create\(", text, flags=re.M).start():]
+    create = create[:create.index("\n}\n")]
+    for kernel in ("pairs_at_once<false>(", "pairs_at_once<true>("):
+        assert 0 <= create.find(kernel) < create.index("cudaMalloc")
