@@ -42,9 +42,10 @@
  * Arithmetic paths (sfb_desc.path)
  *   SFB_PATH_F32   fp32 arithmetic; X, U, V fp32.  Multiply-adds on the CUDA cores, or, for dense problems large enough
  *                  to gain by it (decided once, in sfb_create, from the shape), on the tensor cores with every operand
- *                  as the exact sum of three bf16 values and sums of 64 products at a time, added in fp32: errors against
+ *                  as the exact sum of three scaled bf16 values and sums of 64 products at a time, added in fp32: errors against
  *                  exact arithmetic are no larger than those of a chain of fp32 multiply-adds.  Operands that this
- *                  cannot carry (infinities, NaN) are found on the device, and the CUDA cores then do that product.
+ *                  cannot carry (infinities, NaN, magnitudes of 2^36 and more) are found on the device, and the CUDA
+ *                  cores then do that product.
  *                  Nothing of W is kept from one call to the next.
  *   SFB_PATH_TF32  tensor cores (tcgen05, kind::tf32), fp32 accumulate; X, U, V fp32 in memory.
  *   SFB_PATH_BF16  tensor cores (tcgen05, kind::f16 with bf16 inputs), fp32 accumulate; X, U, V

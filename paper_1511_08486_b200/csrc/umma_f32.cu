@@ -3,8 +3,12 @@
 //   forward:  Z[i][j] = sum_d A[i][d] * W[j][d]          (z_i = W a_i; Section 2, problem (P))
 //   apply  :  W[j][d] -= eta * sum_i U[i][j] * V[i][d]   (W <- W - eta * sum_i u_i v_i^T; Section 3)
 //
-// Every fp32 operand x is the exact sum of three bf16 values (24 significant bits in three times 8): hi = bf16(x),
-// mid = bf16(x - hi), lo = x - hi - mid.  A product is formed from six of the nine products of parts,
+// Every fp32 operand x below 2^36 is 2^-24 times the exact sum of three bf16 values (24 significant bits in three times 8):
+// hi = bf16(2^24 x), mid = bf16(2^24 x - hi), lo = 2^24 x - hi - mid.  (With no factor, operands below 2^-109 lose bits under
+// bf16's smallest subnormal; the last bit of fp32's own subnormals asks for 2^16.  The tensor cores' power depends on how many
+// bits of the parts' exponents change from one value to the next: 1000 x 20000, K = 1024 478.5 us a step with no factor,
+// 482.5 with 2^16, 480.5 with 2^24, 479 with 2^32, which leaves operands below 2^28 only.)
+// A product is formed from six of the nine products of parts,
 //   a b = hi hi + (hi mid + mid hi) + mid mid + (hi lo + lo hi),
 // what is left out (mid lo, lo mid, lo lo) is below 2^-24 of it and of either sign.  The tensor core's fp32 accumulator
 // rounds toward zero once per instruction of 16 reduction steps, about 2^-26 of the sum each time, so it only ever holds
@@ -36,6 +40,8 @@ namespace {
 constexpr int BM = 128;                      // accumulator rows of a CTA (tensor memory lanes)
 constexpr int BN = 256;                      // columns of a whole tile; a half tile has 128
 constexpr int CHUNK = 64;                    // reduction steps an accumulator takes
+constexpr float PARTS_SCALE = 0x1p24f;       // of the parts, on both sides of a product
+constexpr float SUM_SCALE = 0x1p-48f;        // takes a chunk's sum back
 constexpr int THREADS = 384;                 // TMA warp, MMA warp, two idle ones (whole warpgroups), 8 epilogue warps
 constexpr int LAUNCH_REGS = 168;             // per thread: 384 of them fill the register file
 constexpr int A_BYTES = BM * 128, SLOT_BYTES = 2 * A_BYTES;   // one plane of a chunk: 128 rows of A, up to 128 columns of B
@@ -290,6 +296,7 @@ umma_f32_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
     // registers (an output row per thread) while the chunks are added up.
     const int e = warp - 4, quarter = warp & 3, half = e >> 2;
     float* stage = stages + e * 1024;
+    const float2 back = make_float2(SUM_SCALE, SUM_SCALE);
     int it = 0;
     bool ok = true;
     for (int i = 0; work && ok && item_of(p.t, pair, pairs, i, w); ++i) {
@@ -326,8 +333,8 @@ umma_f32_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
           }
 #pragma unroll
           for (int q = 0; q < 16; ++q) {
-            acc[b][q] = __fadd2_rn(acc[b][q], make_float2(__uint_as_float(v0[2 * q]), __uint_as_float(v0[2 * q + 1])));
-            acc[b + 1][q] = __fadd2_rn(acc[b + 1][q], make_float2(__uint_as_float(v1[2 * q]), __uint_as_float(v1[2 * q + 1])));
+            acc[b][q] = __ffma2_rn(make_float2(__uint_as_float(v0[2 * q]), __uint_as_float(v0[2 * q + 1])), back, acc[b][q]);
+            acc[b + 1][q] = __ffma2_rn(make_float2(__uint_as_float(v1[2 * q]), __uint_as_float(v1[2 * q + 1])), back, acc[b + 1][q]);
           }
         }
         if (APPLY && k == max(k_begin, k_end - 3) && row0 < p.M)   // W's part of the tile on its way to L2: a row of W per lane
@@ -446,11 +453,11 @@ __device__ __forceinline__ void zero_planes(const PlaneJob& j, int r, int c) {
 #pragma unroll
   for (int s = 0; s < 3; ++s) *reinterpret_cast<uint4*>(d + s * j.plane_bytes) = make_uint4(0u, 0u, 0u, 0u);
 }
-// Operands below this bound have products below 2^120: no instruction and no chunk sum overflows (two infinite products of
-// parts with different signs would make a NaN of a sum that is an infinity).
+// Parts below this bound, operands below 2^36, have products below 2^120: no instruction and no chunk sum overflows (two
+// infinite products of parts with different signs would make a NaN of a sum that is an infinity).
 constexpr float PARTS_BOUND = 0x1p60f;
 // Eight values of source row i at column c: to row r of the planes (put), or only looked at.  False: one of them is not
-// finite, or not below PARTS_BOUND.
+// finite, or not below 2^36.
 __device__ __forceinline__ bool make_planes(const PlaneJob& j, int i, int r, int c, bool put) {
   float x[8];
   load8(j.src.row(i), c, j.C, j.vec, x);
@@ -469,7 +476,7 @@ __device__ __forceinline__ bool make_planes(const PlaneJob& j, int i, int r, int
   bool fine = true;
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
-    float a = x[2 * q], b = x[2 * q + 1];
+    float a = x[2 * q] * PARTS_SCALE, b = x[2 * q + 1] * PARTS_SCALE;
 #pragma unroll
     for (int s = 0; s < 3; ++s) {
       const __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
@@ -793,7 +800,7 @@ int f32tc_forward(F32Tc* t, cudaStream_t s, const float* W, const float* X, cons
     return SFB_ERR_CUDA;
   if ((r = launch_gemm<false>(s, ta, tb, p, t->num_sms)) < 0) return r;
   launches += r;
-  // operands with infinities or NaN (or beyond bf16's range): the same products on the CUDA cores
+  // operands that are not finite, or not below 2^36: the same products on the CUDA cores
   if ((r = launch_forward_f32_if(s, W, X, Xb, K, J, D, p.z, p.range_stride, g.t.ranges, p.bad)) < 0) return r;
   launches += r;
   *z = p.z; *nsplit = g.t.ranges; *split_stride = p.range_stride;

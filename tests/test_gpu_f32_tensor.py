@@ -75,6 +75,34 @@ def test_error_is_below_that_of_fp32_multiply_adds():
         wl.close()
 
 
+@pytest.mark.parametrize("exponent", [-100, -113, -126, -140])
+def test_small_operands_keep_all_their_bits(exponent):
+    """W, then u, of about 2^exponent (fp32's own subnormals at -140) against samples of about 2^30: every operand's 24 bits count,
+    so the errors are those of ordinary operands (the bound is the one above)."""
+    cfg = scaled("C2", J=300, D=8192, P=4, B=96)
+    inputs = make_inputs(cfg)
+    inputs["similar"] = np.ones_like(inputs["similar"])
+    rng = np.random.default_rng(5)
+    wl = _workload(cfg, inputs, "f32")
+    try:
+        assert _on_tensor_cores(wl)
+        wl.batches[0]["X"].mul_(2.0 ** 30)
+        wl.batches[0]["Xb"].mul_(2.0 ** 30)
+        small = lambda *shape: torch.from_numpy(np.ldexp(rng.standard_normal(shape), exponent).astype(np.float32)).cuda()
+        wl.W.copy_(small(300, 8192))
+        wl.compute_factors(0)
+        d, w = to_f64(wl.V)[:, :8192], to_f64(wl.W)
+        assert orc.rel_fro(to_f64(wl.U)[:, :300], d @ w.T) <= 2.0 ** -22
+        wl.U[:, :300] = small(384, 300)
+        wl.pack(0)
+        wl.W.zero_()
+        wl.apply(-1.0)
+        assert wl.ctx.status() == 0
+        assert orc.rel_fro(to_f64(wl.W), to_f64(wl.U)[:, :300].T @ d) <= 2.0 ** -22
+    finally:
+        wl.close()
+
+
 @pytest.mark.parametrize("where", ["w", "x", "big", "none"])
 def test_operands_that_are_not_finite(where):
     """Operands that are not finite or so large that products overflow.  A weight of -inf that meets positive features only is a logit of -inf: class probability 0, everything else finite.  An
