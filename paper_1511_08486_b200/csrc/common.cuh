@@ -305,8 +305,8 @@ int launch_forward_f32_nn(cudaStream_t s, const float* W, RowMap src, RowMap cop
 // W[j][d] -= eta * sum_{i<K} U[i][j] * V[i][d] on fp32 CUDA cores (fixed summation order).
 int launch_apply_f32(cudaStream_t s, float* W, RowMap u, RowMap v, int K, int J, int D, float eta,
                      const int* dev_status, const int* row_idx = nullptr, const int* n_rows = nullptr,
-                     const int* only_if = nullptr);
-// only_if (optional, device): nothing is done where it is 0.
+                     const int* only_if = nullptr, int full_if = 0);
+// only_if (optional, device): nothing is done where it is 0; all K rows instead of the listed ones where it has a bit of full_if.
 // row_idx / n_rows (optional, device): apply only the factor rows row_idx[0 .. *n_rows), in that order, instead of
 // rows 0 .. K-1 (rows that are known to be all zeros can be left out: the result is bit-identical).
 

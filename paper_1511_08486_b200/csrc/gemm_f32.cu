@@ -187,9 +187,14 @@ template <int OUT>
 __global__ void __launch_bounds__(256, 2) sgemm_pipe_kernel(float* W, RowMap u, RowMap v, int K, int J,
                                                          int D, float eta, const int* dev_status,
                                                          RowMap z, int k_per_range, long long range_stride,
-                                                         const int* row_idx, const int* n_rows, const int* only_if) {
+                                                         const int* row_idx, const int* n_rows, const int* only_if,
+                                                         int full_if) {
   chain_wait();
-  if (OUT == 0 && only_if != nullptr && *only_if == 0) return;
+  if (OUT == 0 && only_if != nullptr) {
+    const int word = *only_if;
+    if (word == 0) return;
+    if (word & full_if) row_idx = n_rows = nullptr;
+  }
   constexpr int BM = 128, BN = 128;
   extern __shared__ __align__(16) float ring[];
   if (OUT == 0 && dev_status != nullptr && (*dev_status & SFB_DEV_BAD_HEADER)) return;
@@ -316,6 +321,7 @@ struct SmallArgs {
   const int* row_idx;       // OUT 0, optional: the factor rows to take
   const int* n_rows;
   const int* only_if;       // OUT 0, optional: do nothing where this is 0
+  int full_if;              // ... and take all rows where it has a bit of this
 };
 
 template <int OUT>
@@ -325,13 +331,18 @@ __global__ void __launch_bounds__(256, 4) sgemm_small_kernel(const __grid_consta
   __shared__ __align__(16) float ring[PIPE * SMALL_STAGE_FLOATS];
   __shared__ long long a_off[OUT == 1 ? BT : 1];   // byte offset of the tile's sample rows, -1: no such row
   __shared__ long long c_off[OUT == 1 ? BT : 1];   // ... and of their copies
-  if (OUT == 0 && p.only_if != nullptr && *p.only_if == 0) return;
+  const int *row_idx = p.row_idx, *n_rows = p.n_rows;
+  if (OUT == 0 && p.only_if != nullptr) {
+    const int word = *p.only_if;
+    if (word == 0) return;
+    if (word & p.full_if) row_idx = n_rows = nullptr;
+  }
   if (OUT == 0 && p.dev_status != nullptr && (*p.dev_status & SFB_DEV_BAD_HEADER)) return;
   const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15, lane = tid & 31, warp = tid >> 5;
   const int nt = (p.N + BT - 1) / BT;            // tiles one after the other in grid.x: M has no limit of grid.y
   const int n_tile = (int)(blockIdx.x % nt), m0 = (int)(blockIdx.x / nt) * BT, n0 = n_tile * BT;
   const int k_lo = (OUT == 1) ? blockIdx.z * p.k_per_range : 0;
-  const int k_hi = (OUT == 1) ? min(p.K, k_lo + p.k_per_range) : (p.n_rows != nullptr ? min(p.K, *p.n_rows) : p.K);
+  const int k_hi = (OUT == 1) ? min(p.K, k_lo + p.k_per_range) : (n_rows != nullptr ? min(p.K, *n_rows) : p.K);
   if (OUT == 1) {
     if (tid < BT) {
       a_off[tid] = m0 + tid < p.M ? (long long)(p.a.row(m0 + tid) - p.a.base) : -1;
@@ -345,7 +356,7 @@ __global__ void __launch_bounds__(256, 4) sgemm_small_kernel(const __grid_consta
     if (OUT == 0) {   // thread = (factor row of the step, 4 columns); nothing to read: a valid address all the same
       const int r = tid >> 4, c = (tid & 15) * 4, i = k0 + r;
       const bool ok = i < k_hi;
-      const int ii = ok ? (p.row_idx != nullptr ? p.row_idx[i] : i) : 0;
+      const int ii = ok ? (row_idx != nullptr ? row_idx[i] : i) : 0;
       const int ub = max(0, min(16, (p.M - m0 - c) * 4)), vb = max(0, min(16, (p.N - n0 - c) * 4));
       cp_async16_zfill(As + r * (BT + 4) + c, p.a.row(ii) + (ub > 0 ? (size_t)(m0 + c) * 4 : 0), ok ? ub : 0);
       cp_async16_zfill(Bs + r * (BT + 4) + c, p.b.row(ii) + (vb > 0 ? (size_t)(n0 + c) * 4 : 0), ok ? vb : 0);
@@ -577,7 +588,7 @@ int launch_forward_f32_small(cudaStream_t s, const float* W, RowMap src, RowMap 
 }
 
 int launch_apply_f32(cudaStream_t s, float* W, RowMap u, RowMap v, int K, int J, int D, float eta,
-                     const int* dev_status, const int* row_idx, const int* n_rows, const int* only_if) {
+                     const int* dev_status, const int* row_idx, const int* n_rows, const int* only_if, int full_if) {
   const long long big_tiles = (long long)((J + 127) / 128) * ((D + 127) / 128);
   if (big_tiles >= 148) {
     dim3 grid((D + 127) / 128, (J + 127) / 128);
@@ -585,7 +596,7 @@ int launch_apply_f32(cudaStream_t s, float* W, RowMap u, RowMap v, int K, int J,
     if (!set_up_device(attr_once, [] { return allow_smem(sgemm_pipe_kernel<0>, PIPE * PIPE_STAGE_FLOATS * 4); }))
       return SFB_ERR_CUDA;
     launch_chained(sgemm_pipe_kernel<0>, grid, 256, PIPE * PIPE_STAGE_FLOATS * 4, s, W, u, v, K, J, D, eta, dev_status, RowMap(), 0, 0,
-                                                                         row_idx, n_rows, only_if);
+                                                                         row_idx, n_rows, only_if, full_if);
   } else {
     SmallArgs p = {};
     p.W = W;
@@ -593,7 +604,7 @@ int launch_apply_f32(cudaStream_t s, float* W, RowMap u, RowMap v, int K, int J,
     p.K = K; p.M = J; p.N = D; p.ldw = D;
     p.eta = eta;
     p.dev_status = dev_status;
-    p.row_idx = row_idx; p.n_rows = n_rows; p.only_if = only_if;
+    p.row_idx = row_idx; p.n_rows = n_rows; p.only_if = only_if; p.full_if = full_if;
     launch_chained(sgemm_small_kernel<0>, ((D + 63) / 64) * ((J + 63) / 64), 256, 0, s, p);
   }
   return cudaGetLastError() == cudaSuccess ? 1 : SFB_ERR_CUDA;
@@ -642,7 +653,7 @@ int launch_forward_f32_nn(cudaStream_t s, const float* W, RowMap src, RowMap cop
   // rows of the output tile = samples (M = K), columns = classes (N = J), reduction over the D features
   dim3 grid((J + 127) / 128, (K + 127) / 128, ks);
   launch_chained(sgemm_pipe_kernel<1>, grid, 256, PIPE * PIPE_STAGE_FLOATS * 4, s, nullptr, a, b, D, K, ldj, 0.f, nullptr,
-                                                                       ks > 1 ? part : z, per, split_stride, nullptr, nullptr, nullptr);
+                                                                       ks > 1 ? part : z, per, split_stride, nullptr, nullptr, nullptr, 0);
   return cudaGetLastError() == cudaSuccess ? transposes + 1 : SFB_ERR_CUDA;
 }
 

@@ -61,8 +61,8 @@ void f32tc_destroy(F32Tc* t);
 // workspace), and the samples (differences) into v where v.base != nullptr.
 int f32tc_forward(F32Tc* t, cudaStream_t s, const float* W, const float* X, const float* Xb, int K, RowMap u, RowMap v,
                   int* dev_status, RowMap* z, int* nsplit, long long* split_stride);
-// Words that say operands hold values which bf16 parts cannot carry (infinities, NaN, 2^36 and more): the CUDA-core kernels
-// then do the work.  The forward's is cleared by the finishing pass behind it, the update's by what precedes it (the finishing pass
+// Words that say operands hold values which bf16 parts cannot carry (infinities, NaN, 2^36 and more), or that an update has very
+// few rows: the CUDA-core kernels then do the work.  The forward's is cleared by the finishing pass behind it, the update's by what precedes it (the finishing pass
 // of the same step, which hands the forward's on, or the header check).
 int* f32tc_bad_forward(F32Tc* t);
 int* f32tc_bad_apply(F32Tc* t);

@@ -50,6 +50,12 @@ constexpr int FULL = 3;                      // chunks that may be on their way 
 constexpr uint32_t WAIT_LIMIT = 1u << 20;    // polls of a bounded wait, about 1.4 s
 enum Plane { HI = 0, MID = 1, LO = 2 };
 
+// Why the CUDA cores do a product (bits of its word): an operand that the parts cannot carry; an update of so few rows that the
+// truncation of a chunk's sum shows, as it does not in longer ones (update of 300 x 8192 by 1, 2, 4, 5, 6, 8 rows: 4.6e-8
+// at all of them from its 64-bit value, multiply-adds 2.5e-8, 3.2e-8, 4.0e-8, 4.4e-8, 4.7e-8, 5.3e-8).
+enum Bad { BAD_VALUE = 1, BAD_FEW = 2 };
+constexpr int FEW_ROWS = 6;
+
 // Work of one launch: m_tiles x (columns / 256) whole tiles in every range of the reduction, of which the last ones
 // are cut in two, and one half tile per row tile where the columns end within the first half of a tile.
 struct Tiles {
@@ -70,7 +76,7 @@ struct TcParams {
   float* W;                    // apply: updated in place (rows of M values: output row = column of W)
   float eta;
   const int* n_rows;           // apply: factor rows in the planes (device)
-  const int* bad;              // operands that are not finite: nothing is done here
+  const int* bad;              // not zero: the CUDA cores do it, nothing is done here
   const int* status_ro;        // apply: a refused buffer
   int* status;
 };
@@ -506,6 +512,7 @@ __global__ void __launch_bounds__(256) planes_kernel(const __grid_constant__ Pla
   const PlaneJob j = second ? j1 : j0;
   const unsigned per_row = j.ldc >> 3, units = j.rows * per_row;   // (the workspace limit keeps them below 2^31)
   const int n = j.n_rows != nullptr ? min(*j.n_rows, j.rows) : j.rows;
+  if (j.n_rows != nullptr && n > 0 && n < FEW_ROWS && blockIdx.x == 0 && threadIdx.x == 0) atomicOr(bad, BAD_FEW);
   if (j.keep_if_all && n == j.rows) return;
   const int n_chunk = (n + CHUNK - 1) / CHUNK * CHUNK;
   bool fine = true;
@@ -515,7 +522,7 @@ __global__ void __launch_bounds__(256) planes_kernel(const __grid_constant__ Pla
     if (r >= n && !j.rest) continue;
     fine = make_planes(j, j.idx != nullptr ? j.idx[r] : r, r, c, r < n) && fine;
   }
-  if (!fine) atomicOr(bad, 1);
+  if (!fine) atomicOr(bad, BAD_VALUE);
 }
 
 // idx[0 .. n): the rows i < K with flags[i] != 0, ascending; idx[n ..): the others.  *n_active (optional): rows with
@@ -851,8 +858,7 @@ int f32tc_apply(F32Tc* t, cudaStream_t s, float* W, RowMap u, RowMap v, int K, f
     return SFB_ERR_CUDA;
   if ((r = launch_gemm<true>(s, ta, tb, p, t->num_sms)) < 0) return r;
   launches += r;
-  if ((r = launch_apply_f32(s, W, u, v, K, J, D, eta, dev_status, left_out ? ju.idx : nullptr, left_out ? ju.n_rows : nullptr, p.bad)) < 0)
-    return r;
+  if ((r = launch_apply_f32(s, W, u, v, K, J, D, eta, dev_status, ju.idx, ju.n_rows, p.bad, left_out ? 0 : BAD_VALUE)) < 0) return r;
   return launches + r;
 }
 

@@ -175,3 +175,45 @@ def test_inactive_pairs_that_are_not_finite(J, D, P, B):
         full.close()
         comp.close()
         ref.close()
+
+
+@pytest.mark.parametrize("compact", [0, 1])
+@pytest.mark.parametrize("n", [1, 5, 6])
+def test_update_by_few_pairs(n, compact):
+    """Fewer than six rows with nonzero u: the CUDA cores' multiply-adds, bit for bit those of a context (96 columns) that has only
+    these; from six on the tensor cores.  A v that is not finite makes NaN where its u is zero, too, unless the pair is left out."""
+    J, D, P, B = 300, 8192, 4, 96
+    cfg = scaled("C2", J=J, D=D, P=P, B=B, compact=compact)
+    small = scaled("C2", J=J, D=96, P=P, B=B, compact=compact)
+    wide, narrow = _workload(cfg, make_inputs(cfg), "f32", guard=True), _workload(small, make_inputs(small), "f32")
+    rng = np.random.default_rng(3)
+    try:
+        assert _on_tensor_cores(wide) and not _on_tensor_cores(narrow)
+        wide.V.copy_(torch.from_numpy(rng.standard_normal((P * B, D)).astype(np.float32)))
+        narrow.V.copy_(wide.V[:, :96])
+        rows = torch.from_numpy(rng.permutation(P * B)[:n])
+        for wl in (wide, narrow):
+            wl.U.zero_()
+            wl.W.zero_()
+        wide.U[rows, :J] = torch.from_numpy(rng.standard_normal((n, J)).astype(np.float32)).cuda()
+        narrow.U.copy_(wide.U)
+        for wl in (wide, narrow):
+            wl.pack(0)
+            wl.apply(-1.0)
+            assert wl.ctx.status() == 0
+        assert torch.equal(wide.W[:, :96], narrow.W) == (n < 6)
+        assert orc.rel_fro(to_f64(wide.W), to_f64(wide.U)[:, :J].T @ to_f64(wide.V)) <= 2.0 ** -24
+        other = next(i for i in range(P * B) if i not in rows)
+        wide.V[other, 70] = float("nan")
+        W = wide.W.clone()
+        wide.W.zero_()
+        wide.pack(0)
+        wide.apply(-1.0)
+        assert wide.ctx.status() == 0 and wide.guards_intact()
+        if compact:
+            assert torch.equal(wide.W, W)
+        else:
+            assert bool(wide.W[:, 70].isnan().all()) and int(wide.W.isnan().sum()) == J
+    finally:
+        wide.close()
+        narrow.close()
