@@ -68,7 +68,7 @@ int* f32tc_bad_forward(F32Tc* t);
 int* f32tc_bad_apply(F32Tc* t);
 uint8_t* f32tc_flags(F32Tc* t);         // where the finishing pass leaves which u rows are nonzero
 // Lists the rows with nonzero u among the first K: f32tc_apply's when it gets no list of its own.
-// active / n_active (optional): how many of these flags are set.  refused: see is_refused (the list is empty then).
+// active / n_active (optional): how many of these flags are set.  refused: see is_refused (u is not read, the list not to be used).
 int f32tc_list(F32Tc* t, cudaStream_t s, RowMap u, int K, bool flags_ready, const uint8_t* active, int* n_active,
                const int* refused);
 // W -= eta * sum u_i v_i^T over the listed rows, in that order (idx / n_rows, or f32tc_list's).  The sum depends on the listed

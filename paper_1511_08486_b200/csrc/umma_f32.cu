@@ -507,11 +507,12 @@ __device__ __forceinline__ bool make_planes(const PlaneJob& j, int i, int r, int
 __global__ void __launch_bounds__(256) planes_kernel(const __grid_constant__ PlaneJob j0, const __grid_constant__ PlaneJob j1,
                                                      int* bad, const int* refused) {
   chain();
-  if (is_refused(refused)) return;
   const bool second = (int)blockIdx.x >= j0.blocks;
   const PlaneJob j = second ? j1 : j0;
   const unsigned per_row = j.ldc >> 3, units = j.rows * per_row;   // (the workspace limit keeps them below 2^31)
-  const int n = j.n_rows != nullptr ? min(*j.n_rows, j.rows) : j.rows;
+  const int n_listed = j.n_rows != nullptr ? *j.n_rows : j.rows;   // (asked for together with the status word)
+  if (is_refused(refused)) return;
+  const int n = min(n_listed, j.rows);
   if (j.n_rows != nullptr && n > 0 && n < FEW_ROWS && blockIdx.x == 0 && threadIdx.x == 0) atomicOr(bad, BAD_FEW);
   if (j.keep_if_all && n == j.rows) return;
   const int n_chunk = (n + CHUNK - 1) / CHUNK * CHUNK;
@@ -526,12 +527,11 @@ __global__ void __launch_bounds__(256) planes_kernel(const __grid_constant__ Pla
 }
 
 // idx[0 .. n): the rows i < K with flags[i] != 0, ascending; idx[n ..): the others.  *n_active (optional): rows with
-// active[i] != 0.  One block; a thread takes K / 1024 consecutive rows.  refused: see is_refused (the list is empty then).
+// active[i] != 0.  One block; a thread takes K / 1024 consecutive rows.
 __global__ void __launch_bounds__(1024) list_rows_kernel(const uint8_t* flags, const uint8_t* active, int K, int* idx,
-                                                         int* n_out, int* n_active, const int* refused) {
+                                                         int* n_out, int* n_active) {
   chain();
   __shared__ int warp_sum[32], act_sum[32];
-  if (is_refused(refused)) K = 0;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int per = (K + 1023) / 1024, lo = min(K, (int)threadIdx.x * per), hi = min(K, lo + per);
   int n = 0, na = 0;
@@ -821,7 +821,7 @@ int f32tc_list(F32Tc* t, cudaStream_t s, RowMap u, int K, bool flags_ready, cons
     if ((r = launch_row_nonzero(s, u, K, t->J, t->flags, refused)) < 0) return r;
     launches += r;
   }
-  launch_chained(list_rows_kernel, 1, 1024, 0, s, t->flags, active, K, t->idx, t->words, n_active, refused);
+  launch_chained(list_rows_kernel, 1, 1024, 0, s, t->flags, active, K, t->idx, t->words, n_active);
   return cudaGetLastError() == cudaSuccess ? launches + 1 : SFB_ERR_CUDA;
 }
 
