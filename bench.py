@@ -584,8 +584,7 @@ def main():
             # the apply left out pairs whose u is zero: its work is counted on the pairs it multiplied through
             alg["flops_all_pairs"] = alg["flops"]
             out["pairs_applied_last_step"] = applied
-        # large dense fp32 steps: planes, GEMM and its stand-in, finishing pass, list, planes, GEMM, stand-in
-        f32_on_tensor_cores = path == "f32" and alg is not None and not alg["sparse"] and launches >= 8 * args.steps
+        f32_on_tensor_cores = path == "f32" and alg is not None and not alg["sparse"] and wl.ctx.on_tensor_cores()
         kernel = "umma_f32_kernel" if path == "f32" else "umma_gemm_kernel"
         if alg is not None:
             apply_tflops = alg["flops"] * (applied / K if 0 < applied < K else 1.0) / (a_ms * 1e-3) / 1e12

@@ -292,6 +292,9 @@ int sfb_stage_ms(sfb_ctx* ctx, float* factors_ms, float* apply_ms, int32_t* step
 /* Number of kernels this context has launched so far (for launch accounting). */
 int64_t sfb_launch_count(const sfb_ctx* ctx);
 
+/* 1 if the context's contractions were set up for the tensor cores (SFB_PATH_F32: see above), 0 for the CUDA cores. */
+int sfb_on_tensor_cores(const sfb_ctx* ctx);
+
 const char* sfb_strerror(int code);
 
 /* Halton-sequence broadcast (Section 4.3): the Q workers that worker p (zero-based) of P would

@@ -25,7 +25,7 @@ EXPORTS = (
     "sfb_profile", "sfb_stage_ms", "sfb_sc_factors_noalloc", "sfb_noalloc_max_scratch_floats",
     "sfb_halton_peers", "sfb_ssp_may_proceed", "sfb_prox", "sfb_step_host",
     "sfb_loss", "sfb_factors_shard", "sfb_commit_header", "sfb_sf_buffer_layout", "sfb_active_pairs",
-    "sfb_wire_bytes",
+    "sfb_wire_bytes", "sfb_on_tensor_cores",
 )
 
 
@@ -98,6 +98,8 @@ def load_library(path: str | None = None) -> C.CDLL:
     lib.sfb_status.restype = C.c_int
     lib.sfb_launch_count.argtypes = [vp]
     lib.sfb_launch_count.restype = C.c_int64
+    lib.sfb_on_tensor_cores.argtypes = [vp]
+    lib.sfb_on_tensor_cores.restype = C.c_int
     lib.sfb_profile.argtypes = [vp, C.c_int]
     lib.sfb_profile.restype = C.c_int
     lib.sfb_stage_ms.argtypes = [vp, C.POINTER(C.c_float), C.POINTER(C.c_float), C.POINTER(C.c_int32)]
@@ -284,6 +286,10 @@ class Context:
 
     def launch_count(self) -> int:
         return int(self._lib.sfb_launch_count(self._h))
+
+    def on_tensor_cores(self) -> bool:
+        """Whether the contractions were set up for the tensor cores (fp32: large dense problems)."""
+        return bool(self._lib.sfb_on_tensor_cores(self._h))
 
     def destroy(self):
         if self._h is not None and self._h.value:

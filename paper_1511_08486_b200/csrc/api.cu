@@ -519,6 +519,8 @@ int sfb_invalidate(sfb_ctx* c) {
 
 int64_t sfb_launch_count(const sfb_ctx* c) { return c ? c->launches : 0; }
 
+int sfb_on_tensor_cores(const sfb_ctx* c) { return c != nullptr && (c->f32_tc != nullptr || c->umma != nullptr) ? 1 : 0; }
+
 int sfb_profile(sfb_ctx* c, int enable) {
   if (c == nullptr) return SFB_ERR_ARG;
   if (enable && !c->prof_have_events) {

@@ -25,6 +25,8 @@ CASES = [
     ("C1", "f32", dict(J=200, D=1024, P=4, B=128), 1e-2),          # large enough for the transposed-operand forward
     ("C2", "f32", dict(J=128, D=1024, P=4, B=64), 1e-3),
     ("C2", "f32", dict(J=40, D=300, P=4, B=6), 1e-3),
+    ("C1", "f32", dict(J=257, D=2051, P=4, B=128), 1e-2),          # fp32 on the tensor cores, and the next
+    ("C2", "f32", dict(J=600, D=2001, P=8, B=64), 1e-3),
     ("C2", "tf32", dict(J=64, D=512, P=4, B=64), 1e-3),
     ("C3", "f32", dict(J=70, D=333, P=4, B=5, density=0.1), 1e-2),
     ("C3", "tf32", dict(J=512, D=2000, P=4, B=32), 1e-3),

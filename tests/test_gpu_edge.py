@@ -158,9 +158,10 @@ def test_saturated_softmax(path, over):
 
 
 def test_dml_step_leaves_out_inactive_pairs_bit_identically():
-    """The fp32 DML step applies only the pairs with u != 0 (an ordered index list built on the device); the
-    result must equal, bit for bit, the staged calls that multiply the zero rows through."""
-    cfg = scaled("C2", J=300, D=8192, P=4, B=96)              # 3 x 64 large tiles: the pipelined apply kernel
+    """The fp32 DML step applies only the pairs with u != 0 (an ordered list built on the device from the finishing pass's
+    flags); the result must equal, bit for bit, that of the staged calls, which find these pairs in the buffer's rows, and
+    both the sum over all K pairs."""
+    cfg = scaled("C2", J=300, D=8192, P=4, B=96)
     inputs = make_inputs(cfg)
     wl = _workload(cfg, inputs, "f32")
     try:
@@ -178,6 +179,9 @@ def test_dml_step_leaves_out_inactive_pairs_bit_identically():
         wl.apply(1e-4)
         assert wl.ctx.status() == 0
         assert torch.equal(wl.sf_buf, buf_step) and torch.equal(wl.W, W_step)
+        U, V = (x.astype(np.float64) for x in orc.unpack(buf_step.cpu().numpy())[1:])
+        dW, dW_or = to_f64(W_step) - inputs["W"].astype(np.float64), -1e-4 * (U.T @ V)
+        assert np.linalg.norm(dW - dW_or) <= 1e-6 * np.linalg.norm(dW_or) + 2.0 ** -24 * np.linalg.norm(inputs["W"])
         # partial apply inside the step: only the first two workers' streams
         wl.reset()
         wl.step(0, eta=1e-4, K=2 * cfg["B"])

@@ -21,19 +21,12 @@ MLR = [(1000, 2003, 8, 100), (257, 5121, 3, 171), (256, 4096, 4, 128), (385, 333
 DML = [(129, 8193, 1, 513), (600, 2001, 8, 64), (257, 1025, 3, 300), (40, 11625, 14, 85)]
 
 
-def _on_tensor_cores(wl):
-    """Eight launches a step, or nine with the compaction: planes, GEMM and its stand-in, finish, list, planes, GEMM, stand-in."""
-    n = wl.ctx.launch_count()
-    wl.step(0, eta=0.0)
-    return wl.ctx.launch_count() - n >= 8
-
-
 @pytest.mark.parametrize("J,D,P,B", MLR)
 def test_mlr(J, D, P, B):
     cfg = scaled("C1", J=J, D=D, P=P, B=B, pool=1)
     wl = _workload(cfg, make_inputs(cfg), "f32")
     try:
-        assert _on_tensor_cores(wl)
+        assert wl.ctx.on_tensor_cores()
     finally:
         wl.close()
     check_config(cfg, "f32", eta=0.5, steps=2, guard=True)
@@ -46,7 +39,7 @@ def test_dml(J, D, P, B):
     inputs = make_inputs(cfg)
     full, comp = _workload(cfg, inputs, "f32"), _workload(dict(cfg, compact=1), inputs, "f32", guard=True)
     try:
-        assert _on_tensor_cores(full)
+        assert full.ctx.on_tensor_cores() and comp.ctx.on_tensor_cores()
         for t in range(2):
             full.step(t, eta=1e-3)
             comp.step(t, eta=1e-3)
@@ -85,7 +78,7 @@ def test_small_operands_keep_all_their_bits(exponent):
     rng = np.random.default_rng(5)
     wl = _workload(cfg, inputs, "f32")
     try:
-        assert _on_tensor_cores(wl)
+        assert wl.ctx.on_tensor_cores()
         wl.batches[0]["X"].mul_(2.0 ** 30)
         wl.batches[0]["Xb"].mul_(2.0 ** 30)
         small = lambda *shape: torch.from_numpy(np.ldexp(rng.standard_normal(shape), exponent).astype(np.float32)).cuda()
@@ -112,7 +105,7 @@ def test_operands_that_are_not_finite(where):
     inputs = make_inputs(cfg)
     wl, fresh = _workload(cfg, inputs, "f32", guard=True), _workload(cfg, inputs, "f32")
     try:
-        assert _on_tensor_cores(fresh)
+        assert fresh.ctx.on_tensor_cores()
         t = wl.batches[0]
         x = t["X"].clone()
         t["X"][:, 7] = t["X"][:, 7].abs() + 0.1
@@ -188,7 +181,7 @@ def test_update_by_few_pairs(n, compact):
     wide, narrow = _workload(cfg, make_inputs(cfg), "f32", guard=True), _workload(small, make_inputs(small), "f32")
     rng = np.random.default_rng(3)
     try:
-        assert _on_tensor_cores(wide) and not _on_tensor_cores(narrow)
+        assert wide.ctx.on_tensor_cores() and not narrow.ctx.on_tensor_cores()
         wide.V.copy_(torch.from_numpy(rng.standard_normal((P * B, D)).astype(np.float32)))
         narrow.V.copy_(wide.V[:, :96])
         rows = torch.from_numpy(rng.permutation(P * B)[:n])
@@ -217,3 +210,46 @@ def test_update_by_few_pairs(n, compact):
     finally:
         wide.close()
         narrow.close()
+
+
+@pytest.mark.parametrize("where", ["u", "v", "v of a zero u"])
+def test_separate_update_of_values_that_are_not_finite(where):
+    """Separate calls: the update finds them itself, in listed rows and in a v whose u is zero (0 times infinity is a NaN of
+    that column).  The next update, of finite rows, is that of a fresh context."""
+    cfg = scaled("C1", J=257, D=2051, P=4, B=128, pool=1)
+    inputs = make_inputs(cfg)
+    wl, fresh = _workload(cfg, inputs, "f32", guard=True), _workload(cfg, inputs, "f32")
+    try:
+        assert wl.ctx.on_tensor_cores()
+        for w in (wl, fresh):
+            w.compute_factors(0)
+            w.U[300] = 0.0
+        U, V = wl.U.clone(), wl.V.clone()
+        if where == "u":
+            wl.U[17, 5] = float("inf")
+        elif where == "v":
+            wl.V[17, 9] = float("nan")
+        else:
+            wl.V[300, 9] = -float("inf")
+        wl.pack(0)
+        wl.apply(0.25)
+        assert wl.ctx.status() == 0 and wl.guards_intact()
+        with np.errstate(invalid="ignore"):
+            u, v = to_f64(wl.U)[:, :257], to_f64(wl.V)[:, :2051]
+            W_or = inputs["W"].astype(np.float64) - 0.25 * (u.T @ v)
+        got, ok = to_f64(wl.W), np.isfinite(W_or)
+        assert not ok.all() and np.array_equal(np.isnan(got), np.isnan(W_or)) and np.array_equal(np.isfinite(got), ok)
+        # a chain of 512 multiply-adds rounds 512 times: sqrt(512) 2^-25 = 6.7e-7 of a change of random signs; then W's own rounding
+        dw = np.linalg.norm(W_or[ok] - inputs["W"].astype(np.float64)[ok])
+        assert np.linalg.norm(got[ok] - W_or[ok]) <= 2.0 ** -20 * dw + 2.0 ** -24 * np.linalg.norm(W_or[ok])
+        wl.U.copy_(U)
+        wl.V.copy_(V)
+        wl.W.copy_(wl.W0)
+        for w in (wl, fresh):
+            w.pack(0)
+            w.apply(0.25)
+            assert w.ctx.status() == 0
+        assert torch.equal(wl.W, fresh.W) and bool(torch.isfinite(wl.W).all())
+    finally:
+        wl.close()
+        fresh.close()

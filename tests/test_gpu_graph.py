@@ -15,6 +15,8 @@ CASES = [
     ("C2", "tf32", dict(J=64, D=512, P=2, B=64)),
     ("C3", "f32", dict(J=70, D=333, P=3, B=5, density=0.1)),
     ("C4", "bf16", dict(J=512, D=1024, P=4, B=128, pool=1, labels="uniform")),
+    ("C1", "f32", dict(J=257, D=2051, P=4, B=128)),             # fp32 on the tensor cores, and the next
+    ("C2", "f32", dict(J=600, D=2001, P=8, B=64)),
 ]
 
 
@@ -51,7 +53,7 @@ def test_captured_step_replays_to_the_same_weights(name, path, over):
             wl.close()
 
 
-@pytest.mark.parametrize("name,path,over", [CASES[1], CASES[2], CASES[4]])
+@pytest.mark.parametrize("name,path,over", [CASES[1], CASES[2], CASES[4], CASES[6], CASES[7]])
 def test_captured_stage_calls_replay_to_the_same_weights(name, path, over):
     """The separate entry points in one graph: factors + pack + apply, and shard factors + header + apply."""
     from paper_1511_08486_b200.workload import DeviceWorkload

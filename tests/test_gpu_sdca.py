@@ -24,6 +24,7 @@ def _ldd(J):
 @pytest.mark.parametrize("path,over", [
     ("f32", dict(J=37, D=203, P=3, B=7)),
     ("f32", dict(J=300, D=1024, P=4, B=64)),
+    ("f32", dict(J=257, D=2051, P=4, B=128)),          # on the tensor cores
     ("tf32", dict(J=300, D=1024, P=4, B=64)),          # split reduction + plain softmax pass
     ("tf32", dict(J=1024, D=512, P=32, B=128)),        # fused softmax epilogue
     ("tf32x3", dict(J=300, D=1024, P=4, B=64)),
