@@ -881,7 +881,7 @@ constexpr int MAX_SPLITS = 16;   // ranges a forward reduction may be cut into (
 constexpr int X3_MAX_SPLITS = 32;   // ... on the compensated path, where the count is also tuned to fill whole waves
 
 struct PickedVariant {   // what pick_variant chose for one shape (splits 0: empty)
-  int key[6];
+  int key[7];
   Variant v;
   int splits;
 };
@@ -1046,8 +1046,9 @@ void umma_plan_destroy(UmmaPlan* p) {
 // Tile shape and kernel variant for an M x N output (M counted in 128-row units): the candidate with the least estimated
 // cost.  max_splits > 1: the caller can take partial products, so the reduction (k_atoms 128-byte atoms long) may be cut
 // into *splits ranges, chosen with the shape.  narrow: tiles of 64 columns will do (plain stores or the write-back of W).
+// blocks32: blocks of up to 32 pairs that an update's reduction takes (blocks begin with a worker).
 static Variant estimate_variant(const UmmaPlan* pl, int m_units, int N, bool dims_chunk_aligned, bool apply, int k_atoms,
-                                int max_splits, int* splits, bool narrow) {
+                                int max_splits, int* splits, bool narrow, int blocks32) {
   Variant v;
   v.split = false;
   if (splits != nullptr) *splits = 1;
@@ -1103,13 +1104,14 @@ static Variant estimate_variant(const UmmaPlan* pl, int m_units, int N, bool dim
       consider(128, 1);
     }
     // Where all tiles of 64 columns run at once (in a forward: on half of the SMs), their stores and loads are the shorter:
-    // 257 x 1000, K = 200 26.9 -> 22.7 us a step, 300 x 3000, K = 300 (141 tiles) 33.8 -> 31.1.  Not in place of a long update on
-    // pairs that fetch an operand's tile by one load (240 x 320, K = 1264: 48.5 us against 51).
+    // 257 x 1000, K = 200 26.9 -> 22.7 us a step, 300 x 3000, K = 300 (141 tiles) 33.8 -> 31.1.  Not in place of an update of
+    // more than 14 blocks of pairs on CTA pairs that fetch an operand's tile by one load (18 shapes, wide against narrow on average: K = 384
+    // +2 %, 448 0, 512 -0.7, 576 -1.4, 640 -3, 768 -4.5; 256 x 2048, K = 384, 640, 768: 29.6 / 29.9, 34.7 / 35.9, 37.4 / 39.3 us).
     // In sparse coding an update with long rows, too, leaves half of the SMs to what is launched behind it, the blocks of the
     // next call's dense code rows above all, a row of shared memory each (with the prox, K = 200-300, on 128 and on 64 columns:
     // 80 x 9000 37.0 / 40.3 us, 200 x 4000 34.8 / 35.8; 300 x 2500 37.0 / 36.9, 600 x 1500 33.0 / 30.9).
     const long long narrow_tiles = (long long)m_units * ((N + 63) / 64) * (ranged ? *splits : 1);
-    const bool long_pairs = apply && v.cg == 2 && dims_chunk_aligned && k_len > 24;
+    const bool long_pairs = apply && v.cg == 2 && dims_chunk_aligned && blocks32 > 14;
     const int most = apply && (pl->d.model != SFB_SC || N <= 2560) ? pl->num_sms : pl->num_sms / 2;
     if ((apply || ranged) && !long_pairs && narrow_tiles <= most) { v.bn = 64; v.cg = 1; }
     v.fold = v.cg == 2 && dims_chunk_aligned;
@@ -1164,8 +1166,9 @@ static Variant estimate_variant(const UmmaPlan* pl, int m_units, int N, bool dim
 
 // The same, estimated once per shape (some 50 candidates): a context has a forward and an update, and a shard's.
 static Variant pick_variant(UmmaPlan* pl, int m_units, int N, bool dims_chunk_aligned, bool apply, int k_atoms,
-                            int max_splits = 1, int* splits = nullptr, bool narrow = true) {
-  const PickedVariant want = {{m_units, N, dims_chunk_aligned, apply + 2 * narrow, k_atoms, splits != nullptr ? max_splits : 0}, Variant(), 1};
+                            int max_splits = 1, int* splits = nullptr, bool narrow = true, int blocks32 = 0) {
+  const PickedVariant want = {{m_units, N, dims_chunk_aligned, apply + 2 * narrow, k_atoms, splits != nullptr ? max_splits : 0, blocks32},
+                              Variant(), 1};
   for (const PickedVariant& p : pl->picked)
     if (p.splits > 0 && memcmp(p.key, want.key, sizeof(p.key)) == 0) {
       if (splits != nullptr) *splits = p.splits;
@@ -1173,7 +1176,7 @@ static Variant pick_variant(UmmaPlan* pl, int m_units, int N, bool dims_chunk_al
     }
   PickedVariant& slot = pl->picked[pl->next_picked++ & 3];
   slot = want;
-  slot.v = estimate_variant(pl, m_units, N, dims_chunk_aligned, apply, k_atoms, max_splits, splits, narrow);
+  slot.v = estimate_variant(pl, m_units, N, dims_chunk_aligned, apply, k_atoms, max_splits, splits, narrow, blocks32);
   if (splits != nullptr) slot.splits = *splits;
   return slot.v;
 }
@@ -1510,7 +1513,9 @@ static int umma_apply_range(UmmaPlan* pl, cudaStream_t s, void* W, __nv_bfloat16
   // stream (the next row, or the stream's V block: always inside the buffer), which only feeds accumulator rows
   // j >= J, and those are never written.  (The V block of the last stream ends the buffer, hence no such
   // licence for D.)
-  const Variant v = pick_variant(pl, m_units, d.D, (d.D % CH) == 0, true, (K + CH - 1) / CH);
+  const int bb = pow2_at_least(d.B);
+  const int blocks32 = d.B >= 32 ? workers * ((d.B + 31) / 32) : (workers + 32 / bb - 1) / (32 / bb);
+  const Variant v = pick_variant(pl, m_units, d.D, (d.D % CH) == 0, true, (K + CH - 1) / CH, 1, nullptr, true, blocks32);
   const int BK = CH * v.ka;
   if (d.B >= BK) { p.k_bb = BK; p.k_wp = 1; p.k_bpw = (d.B + BK - 1) / BK; p.k_blocks = workers * p.k_bpw; }
   else { p.k_bb = pow2_at_least(d.B); p.k_wp = BK / p.k_bb; p.k_bpw = 1; p.k_blocks = (workers + p.k_wp - 1) / p.k_wp; }

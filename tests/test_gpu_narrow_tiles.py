@@ -58,3 +58,12 @@ def test_the_shapes_above_take_narrow_tiles(path):
         pytest.skip("no kernel names from the profiler here")
     assert all(update == [64] for _, update in widths), widths
     assert 2 * sum(forward == [64] for forward, _ in widths) > len(SHAPES), widths
+
+
+@pytest.mark.parametrize("J,D,P,B", [(256, 2048, 5, 128), (300, 1280, 10, 33)])
+def test_long_compensated_updates_on_pairs_keep_wide_tiles(J, D, P, B):
+    """More than 14 reduction blocks of up to 32 pairs, rows of whole 128-byte units: narrow tiles lose."""
+    _, update = _tile_widths("tf32x3", J, D, P, B)
+    if not update:
+        pytest.skip("no kernel names from the profiler here")
+    assert 64 not in update, update
