@@ -1107,9 +1107,11 @@ static Variant estimate_variant(const UmmaPlan* pl, int m_units, int N, bool dim
     // 257 x 1000, K = 200 26.9 -> 22.7 us a step, 300 x 3000, K = 300 (141 tiles) 33.8 -> 31.1.  Not in place of an update of
     // more than 14 blocks of pairs on CTA pairs that fetch an operand's tile by one load (18 shapes, wide against narrow on average: K = 384
     // +2 %, 448 0, 512 -0.7, 576 -1.4, 640 -3, 768 -4.5; 256 x 2048, K = 384, 640, 768: 29.6 / 29.9, 34.7 / 35.9, 37.4 / 39.3 us).
-    // In sparse coding an update with long rows, too, leaves half of the SMs to what is launched behind it, the blocks of the
-    // next call's dense code rows above all, a row of shared memory each (with the prox, K = 200-300, on 128 and on 64 columns:
-    // 80 x 9000 37.0 / 40.3 us, 200 x 4000 34.8 / 35.8; 300 x 2500 37.0 / 36.9, 600 x 1500 33.0 / 30.9).
+    // In sparse coding an update with long rows, too, leaves half of the SMs to what is launched behind it: the blocks of the
+    // next call's dense code rows, a row of shared memory each.  (Steps without the prox between them, K = 200, 5 % dense, on 128
+    // and on 64 columns: 80 x 9000 36.3 / 40.7 us, 80 x 7000 34.8 / 36.9, 200 x 4000 31.8 / 33.7, 300 x 2688 30.8 / 31.6, 300 x 3100
+    // 34.9 / 34.4; up to 2560 none slower, 300 x 2500 32.8 / 32.8, 300 x 1800 29.6 / 26.7.  With the prox there narrow tiles
+    // are 3 to 9 % faster at every one of these, but the update does not know what follows.)
     const long long narrow_tiles = (long long)m_units * ((N + 63) / 64) * (ranged ? *splits : 1);
     const bool long_pairs = apply && v.cg == 2 && dims_chunk_aligned && blocks32 > 14;
     const int most = apply && (pl->d.model != SFB_SC || N <= 2560) ? pl->num_sms : pl->num_sms / 2;
