@@ -16,7 +16,6 @@
 // Every wait on an mbarrier is bounded; a wait that runs out sets SFB_DEV_TIMEOUT and the CTA leaves
 // through the common exit (TMEM freed) instead of hanging.
 #include <cuda.h>
-#include <cudaTypedefs.h>
 
 #include <cstdio>
 #include <cstdlib>
@@ -43,7 +42,6 @@ constexpr int EPI_STAGE_BYTES = 8 * 4096;  // one swizzled 32 x 32 fp32 block pe
 constexpr int RING_BYTES = 192 * 1024;   // shared memory given to the operand ring
 constexpr int MAX_STAGES = 8;
 constexpr int MAX_DIR_WORKERS = 256;      // workers whose pair counts the apply can take from the directory
-constexpr uint32_t WAIT_LIMIT = 1u << 20;   // polls of a bounded wait: a failed poll suspends about 1.4 us, so about 1.4 s
 
 struct GemmParams {
   int m_tiles, n_tiles, k_blocks;   // m_tiles counts tiles of 128*CG rows; k_blocks counts blocks of BK reduction steps
@@ -82,16 +80,6 @@ struct SharedCtl {
   uint16_t nb[MAX_DIR_WORKERS];   // apply with a directory: reduction blocks of each worker
 };
 
-__device__ __forceinline__ bool wait_or_abort(uint64_t* bar, uint32_t parity, SharedCtl* ctl, int* status) {
-  for (uint32_t it = 0; it < WAIT_LIMIT; ++it) {
-    if (ptx::mbar_try_wait(bar, parity)) return true;
-    if ((it & 1023u) == 1023u && ctl->abort) return false;
-  }
-  ctl->abort = 1;
-  if (status != nullptr) atomicOr(status, SFB_DEV_TIMEOUT);
-  return false;
-}
-
 // Tile order.  m_fastest = 0: consecutive tiles walk `group` column tiles, then the next row tile,
 // and only after all row tiles the next group of columns; so one wave of CTAs touches few B slabs
 // (they stay in L2 across waves) while the A slabs stream.  m_fastest = 1: the same with rows and
@@ -123,8 +111,8 @@ __device__ __forceinline__ void tile_coords(const GemmParams& p, int tile, int& 
 //          CTA loads its own 128 rows of A and its own half of B's columns, the even CTA issues
 //          tcgen05.mma.cta_group::2 (M = 256) for the pair, each CTA drains its own 128 accumulator
 //          rows.  TMA bytes of both CTAs are credited to the even CTA's "full" barrier; "stage free"
-//          and "accumulator ready" are committed (tcgen05.commit) once to the even CTA's barrier and
-//          once to the odd CTA's; both epilogues arrive on the even CTA's "accumulator drained" barrier.
+//          and "accumulator ready" are one tcgen05.commit each, which signals both CTAs' barriers;
+//          both epilogues arrive on the even CTA's "accumulator drained" barrier.
 //   KA     128-byte atoms of the reduction index per pipeline stage (BK = KA * CH reduction steps).
 //   EPI    forward epilogue: 0 = store the products z; 1 = multiclass-logistic epilogue: store
 //          exp(z - m) with m the row maximum over this warp's half tile, in the factor's storage
@@ -699,18 +687,6 @@ umma_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
 }
 
 // ------------------------------------------------------------------------------------------- host side
-PFN_cuTensorMapEncodeTiled_v12000 get_encode() {
-  static PFN_cuTensorMapEncodeTiled_v12000 fn = nullptr;
-  if (fn == nullptr) {
-    void* ptr = nullptr;
-    cudaDriverEntryPointQueryResult q;
-    if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &ptr, cudaEnableDefault, &q) == cudaSuccess &&
-        q == cudaDriverEntryPointSuccess)
-      fn = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(ptr);
-  }
-  return fn;
-}
-
 // Tensor map over factor-like rows (row r of worker w at base + w * worker_stride + r * row_stride).
 //   fold == false: 3-D (value, row, worker); box = {CH values, box_rows, box_workers}.
 //   fold == true : 4-D (value within a 128-byte chunk, row, worker, chunk) with the chunk dimension
@@ -719,7 +695,7 @@ PFN_cuTensorMapEncodeTiled_v12000 get_encode() {
 bool encode_rows_map(CUtensorMap* m, int es, const void* base, long long cols, long long rows, long long workers,
                      long long row_stride_bytes, long long worker_stride_bytes, int box_rows, int box_workers,
                      bool fold, int box_chunks, bool atom32) {
-  auto fn = get_encode();
+  auto fn = tensor_map_encoder();
   if (fn == nullptr) return false;
   const int CH = 128 / es;
   const CUtensorMapDataType dt = es == 2 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32;
@@ -765,21 +741,7 @@ int launch_gemm(cudaStream_t s, const CUtensorMap& a, const CUtensorMap& b, cons
     cudaFuncAttributes fa;
     if (cudaFuncGetAttributes(&fa, kernel) != cudaSuccess) return false;
     if (SPLIT && fa.numRegs != SPLIT_LAUNCH_REGS) return false;   // the register split would wait for ever
-    if (CG == 2) {   // how many CTA pairs the device can hold at once
-      cudaLaunchConfig_t q;
-      memset(&q, 0, sizeof(q));
-      cudaLaunchAttribute qa[1];
-      qa[0].id = cudaLaunchAttributeClusterDimension;
-      qa[0].val.clusterDim.x = 2; qa[0].val.clusterDim.y = 1; qa[0].val.clusterDim.z = 1;
-      q.gridDim = dim3(num_sms & ~1, 1, 1);
-      q.blockDim = dim3(threads, 1, 1);
-      q.dynamicSmemBytes = smem;
-      q.attrs = qa; q.numAttrs = 1;
-      if (cudaOccupancyMaxActiveClusters(&max_clusters, kernel, &q) != cudaSuccess || max_clusters < 1) {
-        cudaGetLastError();
-        max_clusters = num_sms / 2;
-      }
-    }
+    if (CG == 2) max_clusters = cta_pairs_at_once(kernel, threads, smem, num_sms);
     return true;
   });
   if (!ready) return SFB_ERR_CUDA;
@@ -852,7 +814,7 @@ int dispatch_gemm(cudaStream_t s, int es, const Variant& v, const CUtensorMap& a
 // K-major: dst[row][atom][64] as (value, row, worker, atom), rows of all workers consecutive.
 bool encode_corr_k_map(CUtensorMap* m, const void* base, long long rows_per_worker, long long workers, long long atoms,
                        int box_rows, int box_workers) {
-  auto fn = get_encode();
+  auto fn = tensor_map_encoder();
   if (fn == nullptr) return false;
   cuuint64_t dims[4] = {64, (cuuint64_t)rows_per_worker, (cuuint64_t)workers, (cuuint64_t)atoms};
   cuuint64_t strides[3] = {(cuuint64_t)atoms * 128, (cuuint64_t)rows_per_worker * atoms * 128, 128};
@@ -864,7 +826,7 @@ bool encode_corr_k_map(CUtensorMap* m, const void* base, long long rows_per_work
 }
 // MN-major: dst[line][ldc] as (value within a chunk of 64, line, chunk); a box is 64 lines of box_chunks chunks.
 bool encode_corr_mn_map(CUtensorMap* m, const void* base, long long ldc, long long lines, int box_chunks) {
-  auto fn = get_encode();
+  auto fn = tensor_map_encoder();
   if (fn == nullptr) return false;
   cuuint64_t dims[3] = {64, (cuuint64_t)lines, (cuuint64_t)(ldc / 64)};
   cuuint64_t strides[2] = {(cuuint64_t)ldc * 2, 128};
@@ -940,7 +902,7 @@ constexpr int EPI_STAGES = 10;   // stages whose time a tile's stores take
 constexpr int X3_PAIRS_PER_APPLY = 1024;
 
 int umma_plan_create(const sfb_desc& d, const Layout& l, UmmaPlan** out) {
-  if (get_encode() == nullptr) return SFB_ERR_CUDA;
+  if (tensor_map_encoder() == nullptr) return SFB_ERR_CUDA;
   UmmaPlan* p = new UmmaPlan();
   p->d = d; p->l = l;
   p->es = (d.path == SFB_PATH_BF16) ? 2 : 4;
@@ -1556,7 +1518,7 @@ static int umma_apply_range(UmmaPlan* pl, cudaStream_t s, void* W, __nv_bfloat16
     cuuint64_t strides[1] = {(cuuint64_t)d.D * 4};
     cuuint32_t box[2] = {32, 32};
     cuuint32_t estr[2] = {1, 1};
-    if (get_encode()(&tw, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, W, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+    if (tensor_map_encoder()(&tw, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, W, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
                      CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_NONE,
                      CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
       return SFB_ERR_CUDA;

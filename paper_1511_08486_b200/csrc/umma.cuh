@@ -4,7 +4,12 @@
 #pragma once
 
 #include <cuda.h>
+#include <cudaTypedefs.h>
 #include <stdint.h>
+
+#include <cstring>
+
+#include "common.cuh"
 
 namespace sfb {
 namespace ptx {
@@ -241,4 +246,53 @@ __host__ __device__ constexpr uint32_t instr_desc(uint32_t fmt, uint32_t a_mn_ma
 }
 
 }  // namespace ptx
+
+// ---- what the tensor-core kernels and their launchers share ------------------------------------------------------------
+constexpr uint32_t WAIT_LIMIT = 1u << 20;   // polls of a bounded wait: a failed poll suspends about 1.4 us, so about 1.4 s
+
+// False: the wait ran out, or another role of the CTA (ctl->abort) gave up.
+template <typename Ctl>
+__device__ __forceinline__ bool wait_or_abort(uint64_t* bar, uint32_t parity, Ctl* ctl, int* status) {
+  for (uint32_t it = 0; it < WAIT_LIMIT; ++it) {
+    if (ptx::mbar_try_wait(bar, parity)) return true;
+    if ((it & 1023u) == 1023u && ctl->abort) return false;
+  }
+  ctl->abort = 1;
+  if (status != nullptr) atomicOr(status, SFB_DEV_TIMEOUT);
+  return false;
+}
+
+// cuTensorMapEncodeTiled, or nullptr where the driver does not have it.
+inline PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder() {
+  static PFN_cuTensorMapEncodeTiled_v12000 fn = nullptr;
+  if (fn == nullptr) {
+    void* ptr = nullptr;
+    cudaDriverEntryPointQueryResult q;
+    if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &ptr, cudaEnableDefault, &q) == cudaSuccess &&
+        q == cudaDriverEntryPointSuccess)
+      fn = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(ptr);
+  }
+  return fn;
+}
+
+// How many CTA pairs of a kernel, whose shared memory has been allowed, the device holds at once.
+template <typename Kernel>
+int cta_pairs_at_once(Kernel kernel, int threads, int smem, int num_sms) {
+  cudaLaunchConfig_t cfg;
+  memset(&cfg, 0, sizeof(cfg));
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = 2; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
+  cfg.gridDim = dim3(num_sms & ~1, 1, 1);
+  cfg.blockDim = dim3(threads, 1, 1);
+  cfg.dynamicSmemBytes = smem;
+  cfg.attrs = at; cfg.numAttrs = 1;
+  int n = 0;
+  if (cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess || n < 1) {
+    cudaGetLastError();
+    n = num_sms / 2;
+  }
+  return n;
+}
+
 }  // namespace sfb

@@ -26,7 +26,6 @@
 // need for a tile of the same shape, because each part meets two or three others: by the clock counter a chunk takes 3072
 // clocks once the pipeline runs.  1000 x 20000, K = 1024: forward 167 us (246 GFLOP of bf16), update 160 us.
 #include <cuda.h>
-#include <cudaTypedefs.h>
 
 #include <cstring>
 #include <new>
@@ -47,7 +46,6 @@ constexpr int LAUNCH_REGS = 168;             // per thread: 384 of them fill the
 constexpr int A_BYTES = BM * 128, SLOT_BYTES = 2 * A_BYTES;   // one plane of a chunk: 128 rows of A, up to 128 columns of B
 constexpr int BUFS = 2;                      // accumulators in tensor memory
 constexpr int FULL = 3;                      // chunks that may be on their way at a time, a barrier each
-constexpr uint32_t WAIT_LIMIT = 1u << 20;    // polls of a bounded wait, about 1.4 s
 enum Plane { HI = 0, MID = 1, LO = 2 };
 
 // Why the CUDA cores do a product (bits of its word): an operand that the parts cannot carry; an update of so few rows that the
@@ -132,16 +130,6 @@ __device__ __forceinline__ bool item_of(const Tiles& t, int pair, int pairs, int
   if (w >= 2 * t.cut + t.ends) return false;
   out = half_tile(t, w);
   return true;
-}
-
-__device__ __forceinline__ bool wait_or_abort(uint64_t* bar, uint32_t parity, Ctl* ctl, int* status) {
-  for (uint32_t it = 0; it < WAIT_LIMIT; ++it) {
-    if (ptx::mbar_try_wait(bar, parity)) return true;
-    if ((it & 1023u) == 1023u && ctl->abort) return false;
-  }
-  ctl->abort = 1;
-  if (status != nullptr) atomicOr(status, SFB_DEV_TIMEOUT);
-  return false;
 }
 
 // CTA pairs (tcgen05.mma.cta_group::2, 256 rows) on tiles of 256 or 128 columns.  A ring slot holds one plane of a chunk:
@@ -563,20 +551,9 @@ __global__ void __launch_bounds__(1024) list_rows_kernel(const uint8_t* flags, c
   }
 }
 
-PFN_cuTensorMapEncodeTiled_v12000 encoder() {
-  static PFN_cuTensorMapEncodeTiled_v12000 fn = [] {
-    void* ptr = nullptr;
-    cudaDriverEntryPointQueryResult q;
-    const bool ok = cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &ptr, cudaEnableDefault, &q) == cudaSuccess &&
-                    q == cudaDriverEntryPointSuccess;
-    return ok ? reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(ptr) : nullptr;
-  }();
-  return fn;
-}
-
 // planes as (column, row, plane), boxes of 64 columns x box_rows rows of one plane
 bool encode_planes(CUtensorMap* m, const void* base, int C, int rows, int ldc, long long plane_bytes, int box_rows) {
-  auto fn = encoder();
+  auto fn = tensor_map_encoder();
   if (fn == nullptr) return false;
   cuuint64_t dims[3] = {(cuuint64_t)C, (cuuint64_t)rows, 3};
   cuuint64_t strides[2] = {(cuuint64_t)ldc * 2, (cuuint64_t)plane_bytes};
@@ -598,21 +575,7 @@ int pairs_at_once(int num_sms) {
     cudaFuncAttributes fa;
     if (!allow_smem(kernel, smem) || cudaFuncGetAttributes(&fa, kernel) != cudaSuccess) return false;
     if (fa.numRegs != LAUNCH_REGS) return false;   // the register split would wait for ever
-    cudaLaunchConfig_t cfg;
-    memset(&cfg, 0, sizeof(cfg));
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = 2; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
-    cfg.gridDim = dim3(num_sms & ~1, 1, 1);
-    cfg.blockDim = dim3(THREADS, 1, 1);
-    cfg.dynamicSmemBytes = smem;
-    cfg.attrs = at; cfg.numAttrs = 1;
-    int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess || n < 1) {
-      cudaGetLastError();
-      n = num_sms / 2;
-    }
-    pairs = n;
+    pairs = cta_pairs_at_once(kernel, THREADS, smem, num_sms);
     return true;
   });
   return ready ? pairs : 0;
@@ -707,7 +670,7 @@ static bool pays(int K, int J, int D, bool pair, double cores_forward_us, int pa
 int f32tc_create(const sfb_desc& d, cudaStream_t s, double cores_forward_us, F32Tc** out) {
   *out = nullptr;
   const long long K = (long long)d.P * d.B, ldd = pad_to(d.D, 8), ldj = pad_to(d.J, 8), ldp = pad_to(d.J, 4);
-  if (encoder() == nullptr) return SFB_OK;
+  if (tensor_map_encoder() == nullptr) return SFB_OK;
   int dev = 0, sms = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
