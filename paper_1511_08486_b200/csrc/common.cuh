@@ -126,11 +126,23 @@ struct HeaderCheck {
 __device__ __forceinline__ bool is_refused(const int* refused) {
   return refused != nullptr && (*refused & SFB_DEV_BAD_HEADER) != 0;
 }
-// Does the buffer's header match the descriptor's?  Every thread for itself: five loads at once, the same for all, and the
-// expected words at fixed offsets.  (A word per lane looks them up one after the other: 0.5 us of the pass that asks.)
-__device__ __forceinline__ bool header_matches(const HeaderCheck& c) {
-  const uint4* q = reinterpret_cast<const uint4*>(c.buf);
+// Does the buffer's header match the descriptor's?  Every thread for itself: five loads at once, the same for all, against
+// the expected words in registers, which a kernel whose other work waits for the answer has fetched before.  (A word per lane
+// looks the expected ones up one after the other: 0.5 us of the pass that asks.)
+struct HeaderWords { uint32_t w[17]; };
+__device__ __forceinline__ HeaderWords expected_header(const HeaderCheck& c) {
   const uint32_t* r = reinterpret_cast<const uint32_t*>(&c.h);
+  HeaderWords e;
+#pragma unroll
+  for (int t = 0; t < 17; ++t) {
+    e.w[t] = r[t];
+    asm volatile("" : "+r"(e.w[t]));   // (now, not where it is used)
+  }
+  return e;
+}
+__device__ __forceinline__ bool header_matches(const HeaderCheck& c, const HeaderWords& e) {
+  const uint4* q = reinterpret_cast<const uint4*>(c.buf);
+  const uint32_t* r = e.w;
   const uint4 w0 = q[0], w1 = q[1], w2 = q[2], w3 = q[3];
   const uint32_t w16 = reinterpret_cast<const uint32_t*>(c.buf)[16];
   uint32_t d = (w0.x ^ r[0]) | (w0.y ^ r[1]) | ((w0.z & ~2u) ^ r[2]) | (w0.w ^ r[3]);   // flag bit 1 (compacted): either

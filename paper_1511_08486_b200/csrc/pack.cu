@@ -27,7 +27,7 @@ __global__ void write_header_kernel(const __grid_constant__ Commit c) { chain();
 
 __global__ void check_header_kernel(const __grid_constant__ HeaderCheck c) {
   chain();
-  report_header(c, header_matches(c));
+  report_header(c, header_matches(c, expected_header(c)));
 }
 
 // grid.x = P workers; each block copies its worker's CSR rows into the stream.

@@ -68,14 +68,8 @@ __global__ void __launch_bounds__(256) split_k_kernel(RowMap src, int rows, int 
 __global__ void __launch_bounds__(256) split_mn_kernel(const __grid_constant__ SplitSide us, const __grid_constant__ SplitSide vs,
                                                        int u_groups, int workers, int k_bb, int k_wp, int k_bpw,
                                                        const __grid_constant__ HeaderCheck check, const int* refused) {
-  chain();
-  if (check.buf != nullptr) {
-    const bool matches = header_matches(check);
-    if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) report_header(check, matches);
-    if (!matches) return;
-  } else if (is_refused(refused)) {
-    return;
-  }
+  chain_next();
+  const HeaderWords expected = expected_header(check);
   const int a_side = (int)blockIdx.y < u_groups;
   const RowMap& src = a_side ? us.src : vs.src;
   const int cols = a_side ? us.cols : vs.cols, ldc = a_side ? us.ldc : vs.ldc;
@@ -83,17 +77,25 @@ __global__ void __launch_bounds__(256) split_mn_kernel(const __grid_constant__ S
   const int unit = ((int)blockIdx.y - (a_side ? 0 : u_groups)) * 8 + (threadIdx.x & 7);   // 8 values = 16 bytes of bf16
   const int line = threadIdx.x >> 3;                      // 0..31: pair inside the reduction block
   const int blk = blockIdx.x;
-  if (unit * 8 >= ldc) return;
   int worker, row;
   if (k_wp == 1) { worker = blk / k_bpw; row = (blk % k_bpw) * 32 + line; }        // 32 rows of one worker
   else { worker = blk * k_wp + line / k_bb; row = line % k_bb; }                  // k_bb rows of each of k_wp workers
+  const bool in = worker < workers && row < src.B;
+  const float* x = reinterpret_cast<const float*>(src.base + (long long)worker * src.worker_stride + (long long)row * src.ld * src.es) + unit * 8;
+  asm volatile("" : "+l"(x));   // all of the above is done before the wait
+  chain_wait();
+  if (check.buf != nullptr) {
+    const bool matches = header_matches(check, expected);
+    if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) report_header(check, matches);
+    if (!matches) return;
+  } else if (is_refused(refused)) {
+    return;
+  }
+  if (unit * 8 >= ldc) return;
   const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
   float4 x0 = zero, x1 = zero;
-  if (worker < workers && row < src.B) {
-    const float* x = reinterpret_cast<const float*>(src.row(worker * src.B + row)) + unit * 8;
-    if (unit * 8 < cols) x0 = *reinterpret_cast<const float4*>(x);
-    if (unit * 8 + 4 < cols) x1 = reinterpret_cast<const float4*>(x)[1];
-  }
+  if (in && unit * 8 < cols) x0 = *reinterpret_cast<const float4*>(x);
+  if (in && unit * 8 + 4 < cols) x1 = reinterpret_cast<const float4*>(x)[1];
   uint4 val, rem;
   split8(x0, x1, val, rem);
   const size_t units_per_line = (size_t)ldc / 8;

@@ -16,7 +16,7 @@ READS = {
     "row_nonzero_kernel": ROWS, "kept_rows_kernel": r"\(buf \+", "planes_kernel": r"make_planes\(",
     "umma_f32_kernel": r"tma_load", "sgemm_pipe_kernel": ROWS, "sgemm_small_kernel": ROWS, "densify_kernel": ROWS,
     "csc_mask_kernel": ROWS, "csc_fill_kernel": ROWS, "csc_apply_kernel": ROWS, "sc_malformed_kernel": ROWS, "sc_apply_kernel": ROWS,
-    "split_mn_kernel": ROWS, "umma_gemm_kernel": r"p\.dir\[",
+    "split_mn_kernel": r"\*reinterpret_cast<const float4\*>\(x\)", "umma_gemm_kernel": r"p\.dir\[",
 }
 
 
