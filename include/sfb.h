@@ -44,8 +44,8 @@
  *                  to gain by it (decided once, in sfb_create, from the shape), on the tensor cores with every operand
  *                  as the exact sum of three scaled bf16 values and sums of 64 products at a time, added in fp32: errors against
  *                  exact arithmetic are no larger than those of a chain of fp32 multiply-adds in updates, and in forward
- *                  products of samples with some 200 nonzero features or more (at most 1.3e-7 of the norm in all of them; with
- *                  1, 16, 64 nonzero features 4.6e-8, 7.9e-8, 9.3e-8, multiply-adds 2.5e-8, 6.9e-8, 8.7e-8).  Operands
+ *                  products of samples with some 200 nonzero features or more (300 x 8192: 1.2e-7 of the norm with all nonzero; with
+ *                  1, 16, 64 of them 4.6e-8, 7.9e-8, 9.3e-8, multiply-adds 2.5e-8, 6.9e-8, 8.7e-8).  Operands
  *                  that this cannot carry (infinities, NaN, magnitudes of 2^36 and more) are found on the device, and so
  *                  are updates of fewer than six pairs with nonzero u; the CUDA cores then do that product.
  *                  Nothing of W is kept from one call to the next.

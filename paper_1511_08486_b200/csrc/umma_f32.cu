@@ -4,18 +4,22 @@
 //   apply  :  W[j][d] -= eta * sum_i U[i][j] * V[i][d]   (W <- W - eta * sum_i u_i v_i^T; Section 3)
 //
 // Every fp32 operand x below 2^36 is 2^-24 times the exact sum of three bf16 values (24 significant bits in three times 8):
-// hi = bf16(2^24 x), mid = bf16(2^24 x - hi), lo = 2^24 x - hi - mid.  (With no factor, operands below 2^-109 lose bits under
-// bf16's smallest subnormal; the last bit of fp32's own subnormals asks for 2^16.  The tensor cores' power depends on how many
-// bits of the parts' exponents change from one value to the next: 1000 x 20000, K = 1024 478.5 us a step with no factor,
-// 482.5 with 2^16, 480.5 with 2^24, 479 with 2^32, which leaves operands below 2^28 only.)
+// hi = bf16(2^24 x), mid = bf16(2^24 x - hi), lo = 2^24 x - hi - mid.  (The scheme is that of G. Henry, P. T. P. Tang,
+// A. Heinecke, "Leveraging the bfloat16 Artificial Intelligence Datatype For Higher-Precision Computations", ARITH 2019.)
+// With no factor, operands below 2^-109 lose bits under bf16's smallest subnormal; the last bit of fp32's own subnormals
+// asks for 2^16.  The tensor cores' power depends on how many bits of the parts' exponents change from one value to the
+// next: 1000 x 20000, K = 1024 478.5 us a step with no factor, 482.5 with 2^16, 480.5 with 2^24, 479 with 2^32, which leaves
+// operands below 2^28 only.
 // A product is formed from six of the nine products of parts,
 //   a b = hi hi + (hi mid + mid hi) + mid mid + (hi lo + lo hi),
 // what is left out (mid lo, lo mid, lo lo) is below 2^-24 of it and of either sign.  The tensor core's fp32 accumulator
 // rounds toward zero once per instruction of 16 reduction steps, about 2^-26 of the sum each time, so it only ever holds
 // the sum of ONE chunk of 64 reduction steps, small products first and the four hi hi instructions last; the chunk
-// sums are added in registers, rounded to nearest.  That makes sums of a chunk good to about 6e-8 and the whole better than
+// sums are added in registers, rounded to nearest.  That makes sums of a chunk good to about 6e-8 and long sums better than
 // a chain of fp32 multiply-adds, which rounds after every step: u of 600 x 10000, K = 2048 is 1.3e-7 from its 64-bit value
-// (multiply-adds: 5.4e-7), of 129 x 2050, K = 195 1.1e-7 (2.0e-7).
+// (multiply-adds: 5.4e-7), of 129 x 2050, K = 195 1.1e-7 (2.0e-7).  Sums of few products are less exact than multiply-adds: for
+// updates see FEW_ROWS; u = L d of 300 x 8192 with 1, 16, 64, 256 nonzero features 4.6e-8, 7.9e-8, 9.3e-8, 1.03e-7 (2.5e-8,
+// 6.9e-8, 8.7e-8, 1.08e-7).
 //
 // The parts ("planes") are written by a bandwidth-bound pass: [3][rows][row length padded to 8] bf16 in the order of
 // `Plane`.  The same planes of the samples serve the forward (contiguous along the reduction: K-major) and the update
@@ -24,7 +28,8 @@
 // What bounds the GEMMs: the tensor pipe (six bf16 instructions per product), under the power cap.  A 256 x 256 tile of a
 // CTA pair loads 96 KB per CTA and chunk for 3072 clocks of tensor work, 32 bytes a clock, half of what the tf32 kernels
 // need for a tile of the same shape, because each part meets two or three others: by the clock counter a chunk takes 3072
-// clocks once the pipeline runs.  1000 x 20000, K = 1024: forward 167 us (246 GFLOP of bf16), update 160 us.
+// clocks once the pipeline runs.  1000 x 20000, K = 1024: forward 164.5 us (246 GFLOP of bf16), update 174.0, each alone and on
+// cold caches.
 #include <cuda.h>
 
 #include <cstring>
@@ -640,7 +645,10 @@ Geometry pick(int M, int N, long long chunks, long long max_ranges, int pairs) {
 }  // namespace
 
 constexpr int F32TC_MAX_RANGES = 16;
-constexpr long long F32TC_MAX_BYTES = 2LL << 30;   // planes a context may hold
+// Planes a context may hold: six bytes for every value of samples, W and u, beside the caller's own four.  The limit is a choice
+// and no measured line: the largest problems keep that memory.  (planes_kernel counts units of eight values in 32 bits and
+// relies on it.)
+constexpr long long F32TC_MAX_BYTES = 2LL << 30;
 
 struct F32Tc {
   int J, D, K, B, num_sms;
